@@ -728,10 +728,11 @@ template <int MODE> __device__ void make_kv_item(const TcBwdParams &p, uint32_t 
     } else {
         int bt = tile - p.main_key_tiles;
         if (!is_main && S > 1) bt = bt * S + rank;           // a cluster holds S branch key tiles
+        const bool past = !is_main && bt >= p.branch_key_tiles;      // the last cluster has ranks to spare: no rows
         if (!is_main && p.depth) { kdepth = bt / p.branch_tiles_per_depth; bt %= p.branch_tiles_per_depth; }
         step = is_main ? kTile : p.step_kb;
         it.row0 = is_main ? (int)p.r.kv_begin + tile * step : (int)p.r.tok_begin + bt * step;
-        it.row_end = min(it.row0 + step, (int)(is_main ? p.r.kv_end : p.r.tok_end));
+        it.row_end = past ? it.row0 : min(it.row0 + step, (int)(is_main ? p.r.kv_end : p.r.tok_end));
     }
     it.srow0 = is_main ? it.row0 : n + (kDq ? 0 : kdepth * p.num_branches) + it.row0;
     it.m0 = it.m1 = it.b0 = it.b1 = 0;
@@ -1461,6 +1462,7 @@ int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
         int64_t kbt = (r.parts & BA_PART_BRANCH) ? (br_n + p.step_kb - 1) / p.step_kb : 0;
         p.branch_tiles_per_depth = (int)kbt;
         if (depth) kbt *= depth;    // the tokens of depths 1 .. depth of the selected branches are keys
+        p.branch_key_tiles = (int)kbt;
         // Share main key tiles between the CTAs of a cluster until they fill the SMs once, as long as an average
         // part keeps eight 64-row steps: 2,048 tokens, 8 KV heads (128 tiles) take 122 us whole, 130 us in two
         // parts, 153 us in four.

@@ -35,7 +35,7 @@ struct TcBwdParams {
     int main_tiles, total_tiles;      // dQ kernel: query row tiles
     int hp, head_chunks, tok;         // dQ with packed heads: heads per tile, chunks of hp heads per group, tokens per tile
     int main_key_tiles, total_key_tiles;  // dK/dV and fused kernels: key tiles
-    int step_kb;                      // branch tokens per branch key tile
+    int branch_key_tiles, step_kb;    // dK/dV: branch key tiles; branch tokens per branch key tile
     int splits, tile_major;           // dK/dV: CTAs per main key tile (cluster size), order of the key tiles
     // Step-major (per-depth) call of the dK/dV kernel: depth > 0.  Query rows are the
     // depth-`depth` tokens of branches [r.tok_begin, r.tok_end) (branch indices), Q / dO / dQ and

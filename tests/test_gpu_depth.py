@@ -172,3 +172,47 @@ def test_stepwise_equals_all_depths_call_full_size(ba):
         err = np.abs(f32(lse0).astype(np.float64) - np.log(want_count[:, depth - 1].astype(np.float64))[:, None])
         assert err.max() <= 2e-5, f"depth {depth}: q=0 LSE closed form off by {err.max():.2e}"
     plan.check()
+
+
+# One sequence with few key tiles: clusters of two, four and eight CTAs share a main key tile, and the branch key
+# tiles (a multiple of 9, 17 or 11 per call) do not fill the last cluster.
+@pytest.mark.parametrize("tokens,h_q,h_kv,length,br_range", [
+    (600, 4, 1, 3, None), (1100, 32, 8, 3, None), (2100, 16, 2, 2, None), (1300, 16, 1, 4, None),
+    (1100, 32, 8, 3, (130, 1001)), (2100, 16, 2, 2, (1, 1500)),
+])
+def test_backward_of_a_depth_touches_its_own_rows_only(ba, tokens, h_q, h_kv, length, br_range):
+    p = chain_problem([tokens], range(tokens), length, h_q, h_kv)
+    n, a = p.n_main, p.num_branches
+    b0, b1 = br_range or (0, a)
+    t = W.make_tensors(p, seed=33, std=0.5)
+    t["d_o"][:n] = 0
+    d = to_dev(p, t)
+    plan = ba.Plan(p, impl=ba.IMPL_TC)
+    o, lse = ba.branch_attn_fwd(plan, d["q_main"], d["q_branch"], d["k"], d["v"])
+    want = [torch.zeros(s, device="cuda") for s in ((n, h_q, 128), (p.n_branch, h_q, 128), (p.rows, h_kv, 128), (p.rows, h_kv, 128))]
+    ba.branch_attn_bwd(plan, d["q_main"], d["q_branch"], d["k"], d["v"], o, lse, d["d_o"], br_range=(b0, b1), qm_range=(0, 0),
+                       accumulate=True, grads=want)
+    k, v = depth_major(d["k"], n, a, length), depth_major(d["v"], n, a, length)
+    split = lambda x: [y.contiguous() for y in x.reshape(a, length, *x.shape[1:]).unbind(1)]
+    q_d, o_d, lse_d, go_d = split(d["q_branch"]), split(o[n:]), split(lse[n:]), split(d["d_o"][n:])
+    guard = 256                                      # rows behind the gradients: more than a key tile
+    g = torch.Generator(device="cuda").manual_seed(7)
+    sums = [torch.zeros((p.rows, h_kv, 128), device="cuda") for _ in range(2)]
+    for depth in range(1, length + 1):
+        bufs = [torch.randn((p.rows + guard, h_kv, 128), generator=g, device="cuda") for _ in range(2)]
+        before = [b.clone() for b in bufs]
+        dq = ba.branch_attn_bwd_depth(plan, depth, q_d[depth - 1], k, v, o_d[depth - 1], lse_d[depth - 1], go_d[depth - 1],
+                                      bufs[0][:p.rows], bufs[1][:p.rows], br_range=(b0, b1))
+        plan.check()
+        mine = torch.zeros(p.rows + guard, dtype=torch.bool, device="cuda")      # rows that the call may change
+        mine[:n] = True
+        for j in range(depth):
+            mine[n + j * a + b0:n + j * a + b1] = True
+        for name, b, x, s in zip(("dK", "dV"), bufs, before, sums):
+            assert torch.equal(b[~mine], x[~mine]), f"{name} depth {depth}: rows of other depths, branches or buffers changed"
+            s += (b - x)[:p.rows]
+        assert_close(f"dQ depth {depth}", f32(dq)[b0:b1], f32(want[1].reshape(a, length, h_q, 128)[b0:b1, depth - 1]), 2e-2)
+    # (differences of sums of order 1 in fp32: 1e-7 each)
+    for name, s, w in zip(("dK", "dV"), sums, want[2:]):
+        got, ref = f32(branch_major(s, n, a, length)), f32(w)
+        assert np.abs(got - ref).max() <= 2e-2 and np.linalg.norm(got - ref) <= 1e-2 * np.linalg.norm(ref), name
