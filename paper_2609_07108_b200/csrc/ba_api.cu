@@ -235,10 +235,11 @@ extern "C" int branch_attn_bwd_depth(const ba_plan_t *plan, int depth, const voi
 
 // ---------------------------------------------------------------- ring steps on a received K/V shard
 
-// The kernels address keys by their global row; a shard holds only rows [kv_begin, kv_end).
-// Tiles of 128 keys start at multiples of 128, so with both ends on such a multiple every row a
-// kernel touches lies inside the shard, and the shard can be addressed as if it were the full
-// tensor by moving its base back by kv_begin rows (no byte before the shard is ever read).
+// The kernels address keys by their global row; a shard holds only rows [kv_begin, kv_end) and is addressed as
+// if it were the full tensor, by moving its base back by kv_begin rows.  No byte outside the shard is read: key
+// tiles start at kv_begin or, where a tile starts at a row's first visible key, at max(that key, kv_begin); and a
+// call without own-branch keys gives the tensor maps of K and V kv_end rows, so that the rows of a tile beyond
+// them arrive as zeros (the plain-FMA kernels load live rows only).
 static int shard_ok(const ba_plan_t *plan, int64_t kv_begin, int64_t kv_end) {
     if (!plan) return BA_EINVAL;
     if (kv_begin < 0 || kv_end < kv_begin || kv_end > plan->prob.n_main) return BA_EINVAL;

@@ -1397,7 +1397,9 @@ int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
     p.num_branches = pr.num_branches;
     p.branch_len = pr.uniform_len;
     const uint64_t all_rows = (uint64_t)(pr.n_main + pr.n_branch);
-    const uint64_t kv_rows = depth ? (uint64_t)(pr.n_main + (int64_t)depth * pr.num_branches) : all_rows;
+    // (without own-branch keys nothing beyond kv_end is needed: a received shard ends there)
+    const uint64_t kv_rows = depth ? (uint64_t)(pr.n_main + (int64_t)depth * pr.num_branches)
+                             : (r.parts & BA_PART_BRANCH) ? all_rows : (uint64_t)(r.kv_end > 0 ? r.kv_end : 1);
     const uint64_t go_rows = depth ? (uint64_t)pr.num_branches : all_rows;
     const void *qm = q_main ? q_main : q_branch;
     const void *qb = (q_branch && pr.n_branch > 0) ? q_branch : q_main;
@@ -1442,15 +1444,12 @@ int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
             q.wide = p.wide;
             q.status = p.status;
             if (grid > INT_MAX) return BA_EUNSUPPORTED;
-            // without own-branch keys nothing beyond kv_end is needed (a received shard ends there)
-            const uint64_t key_rows = (r.parts & BA_PART_BRANCH) ? kv_rows : (uint64_t)(r.kv_end > 0 ? r.kv_end : 1);
-            CUtensorMap km[4];
-            if (!maps(tm, q.tok, q.hp, kTile) || !make_tmap_rhd(&km[0], k, key_rows, pr.h_kv, D, kTile) ||
-                !make_tmap_rhd(&km[1], v, key_rows, pr.h_kv, D, kTile) || !make_tmap_rhd(&km[2], k, key_rows, pr.h_kv, D, 32) ||
-                !make_tmap_rhd(&km[3], v, key_rows, pr.h_kv, D, 32))
+            CUtensorMap k32, v32;
+            if (!maps(tm, q.tok, q.hp, kTile) || !make_tmap_rhd(&k32, k, kv_rows, pr.h_kv, D, 32) ||
+                !make_tmap_rhd(&v32, v, kv_rows, pr.h_kv, D, 32))
                 return BA_EINVAL;
             if (grid > 0) {
-                tc_dq_kernel<<<(unsigned)grid, kDqThreads, sizeof(DqSmem), st>>>(tm[0], tm[1], tm[2], km[0], km[1], km[2], km[3], q);
+                tc_dq_kernel<<<(unsigned)grid, kDqThreads, sizeof(DqSmem), st>>>(tm[0], tm[1], tm[2], tm[3], tm[4], k32, v32, q);
                 int rc = ba_check_launch();
                 if (rc != BA_OK) return rc;
             }

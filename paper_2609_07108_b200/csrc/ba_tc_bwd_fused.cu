@@ -690,11 +690,13 @@ int ba_tc_bwd_fused(const ba_plan *pl, const BaRange &r, const void *q_main, con
 
     CUtensorMap tq_main, tq_branch, tgo, tk, tv;
     const uint64_t all_rows = (uint64_t)(pr.n_main + pr.n_branch);
+    // without own-branch keys nothing beyond kv_end is needed (a received shard ends there)
+    const uint64_t kv_rows = (r.parts & BA_PART_BRANCH) ? all_rows : (uint64_t)(r.kv_end > 0 ? r.kv_end : 1);
     const void *qm = q_main ? q_main : q_branch;
     const void *qb = (q_branch && pr.n_branch > 0) ? q_branch : q_main;
     const uint64_t qm_rows = q_main ? (uint64_t)pr.n_main : (uint64_t)pr.n_branch;
     const uint64_t qb_rows = (q_branch && pr.n_branch > 0) ? (uint64_t)pr.n_branch : (uint64_t)pr.n_main;
-    if (!make_tmap_rhd(&tk, k, all_rows, pr.h_kv, 128, kTile) || !make_tmap_rhd(&tv, v, all_rows, pr.h_kv, 128, kTile) ||
+    if (!make_tmap_rhd(&tk, k, kv_rows, pr.h_kv, 128, kTile) || !make_tmap_rhd(&tv, v, kv_rows, pr.h_kv, 128, kTile) ||
         !make_tmap_rhd(&tgo, d_o, all_rows, pr.h_q, 128, kTile) || !make_tmap_rhd(&tq_main, qm, qm_rows, pr.h_q, 128, kTile) ||
         !make_tmap_rhd(&tq_branch, qb, qb_rows, pr.h_q, 128, kTile))
         return BA_EINVAL;

@@ -74,3 +74,44 @@ def test_shard_calls_check_their_ranges(ba):
                                        ba._stream())
         assert rc == -1, kv
     torch.cuda.synchronize()
+
+
+# Two sequences, the second one starting inside a shard; N no multiple of 32 or 128.  Behind each shard (in the same
+# allocation) lie rows of NaN: a kernel that read them, and multiplied them with a weight of zero, would show.
+@pytest.mark.parametrize("head_dim", [64, 128])
+@pytest.mark.parametrize("kv", [(0, 256), (256, 512), (256, 733), (640, 733), (0, 733)])
+def test_nothing_outside_a_shard_is_read(ba, head_dim, kv):
+    n = 733
+    p = W.Problem(W.cu_from_lengths([300, 433]), np.arange(0, n, 4, dtype=np.int32), W.uniform_branch_offsets(184, 3), W.CHAIN, None,
+                  4, 2, head_dim, dtype="bf16")
+    plan = ba.Plan(p)
+    g = torch.Generator(device="cuda").manual_seed(53)
+    draw = lambda rows, heads, std: (torch.randn((rows, heads, head_dim), generator=g, device="cuda") * std).to(torch.bfloat16)
+    qm, qb, k, v, go = draw(n, 4, 0.5), draw(p.n_branch, 4, 0.5), draw(p.rows, 2, 0.5), draw(p.rows, 2, 0.5), draw(p.rows, 4, 0.1)
+
+    def shard(x):
+        buf = torch.full((kv[1] - kv[0] + 128, *x.shape[1:]), float("nan"), dtype=x.dtype, device="cuda")
+        buf[:kv[1] - kv[0]] = x[kv[0]:kv[1]]
+        return buf[:kv[1] - kv[0]]
+
+    qm_range, br = (0, n), (0, p.num_branches)
+    o_want, l_want = ba.branch_attn_fwd_partial(plan, qm, qb, k, v, qm_range, br, kv, ba.PART_MAIN)
+    acc_o, acc_l = torch.full_like(o_want, 7.0), torch.full_like(l_want, 7.0)
+    ba.branch_attn_fwd_shard(plan, qm, qb, shard(k), shard(v), qm_range, br, kv, acc_o, acc_l, merge=False)
+    assert torch.equal(acc_o, o_want) and torch.equal(acc_l, l_want)
+    o, lse = ba.branch_attn_fwd(plan, qm, qb, k, v)
+    zeros = lambda rows, heads: torch.zeros((rows, heads, head_dim), device="cuda")
+    for stages in (ba.STAGE_ALL, ba.STAGE_ALL_FUSED):
+        if head_dim == 64 and stages == ba.STAGE_ALL_FUSED:
+            continue                                   # the one-kernel backward needs head_dim 128
+        want = (zeros(n, 4), zeros(p.n_branch, 4), zeros(p.rows, 2), zeros(p.rows, 2))
+        ba.branch_attn_bwd(plan, qm, qb, k, v, o, lse, go, qm_range, br, kv, ba.PART_MAIN, accumulate=True, grads=want, stages=stages)
+        dq, db, dk, dv = zeros(n, 4), zeros(p.n_branch, 4), zeros(kv[1] - kv[0], 2), zeros(kv[1] - kv[0], 2)
+        ba.branch_attn_bwd_shard(plan, qm, qb, shard(k), shard(v), o, lse, go, qm_range, br, kv, dq, db, dk, dv, stages=stages)
+        plan.check()
+        assert torch.equal(dk, want[2][kv[0]:kv[1]]) and torch.equal(dv, want[3][kv[0]:kv[1]])
+        for a, b in ((dq, want[0]), (db, want[1])):
+            if stages == ba.STAGE_ALL:
+                assert torch.equal(a, b)
+            else:          # fp32 atomic adds of up to six key tiles: the order moves the last bits
+                assert float((a - b).abs().max()) <= 6 * 2.0 ** -23 * float(b.abs().max())
