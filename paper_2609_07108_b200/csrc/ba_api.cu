@@ -31,6 +31,7 @@ int make_range(const ba_plan *pl, int64_t qm_begin, int64_t qm_end, int64_t br_b
     if (parts < 0 || parts > (BA_PART_MAIN | BA_PART_BRANCH)) return BA_EINVAL;
     r->qm_begin = qm_begin; r->qm_end = qm_end;
     r->kv_begin = kv_begin; r->kv_end = kv_end;
+    r->kv_base = 0;
     r->parts = parts;
     return token_range(pl, br_begin, br_end, &r->tok_begin, &r->tok_end);
 }
@@ -112,18 +113,19 @@ extern "C" int branch_attn_bwd(const ba_plan_t *plan, const void *q_main, const 
                                   ws_bytes, stream, BA_STAGE_ALL);
 }
 
-extern "C" int branch_attn_bwd_stages(const ba_plan_t *plan, const void *q_main, const void *q_branch,
-                                      const void *k, const void *v, const void *O, const float *LSE,
-                                      const void *dO, int64_t qm_begin, int64_t qm_end, int64_t br_begin,
-                                      int64_t br_end, int64_t kv_begin, int64_t kv_end, int parts,
-                                      int accumulate, void *dQ_main, void *dQ_branch, void *dK, void *dV,
-                                      void *workspace, size_t ws_bytes, void *stream, int stages) {
+// kv_base: first row that k, v, dK and dV hold
+static int bwd_common(const ba_plan_t *plan, const void *q_main, const void *q_branch, const void *k, const void *v,
+                      const void *O, const float *LSE, const void *dO, int64_t qm_begin, int64_t qm_end,
+                      int64_t br_begin, int64_t br_end, int64_t kv_begin, int64_t kv_end, int64_t kv_base, int parts,
+                      int accumulate, void *dQ_main, void *dQ_branch, void *dK, void *dV, void *workspace,
+                      size_t ws_bytes, void *stream, int stages) {
     if (!plan) return BA_EINVAL;
     if (stages <= 0 || stages > (BA_STAGE_ALL | BA_STAGE_FUSED)) return BA_EINVAL;
     if ((stages & BA_STAGE_FUSED) && (stages & (BA_STAGE_DQ | BA_STAGE_DKDV))) return BA_EINVAL;
     BaRange r;
     int rc = make_range(plan, qm_begin, qm_end, br_begin, br_end, kv_begin, kv_end, parts, &r);
     if (rc != BA_OK) return rc;
+    r.kv_base = kv_base;
     if (!q_main) r.qm_end = r.qm_begin;  // branch queries only
     const bool has_main_q = r.qm_end > r.qm_begin;
     const bool has_branch_q = r.tok_end > r.tok_begin;
@@ -183,6 +185,16 @@ extern "C" int branch_attn_bwd_stages(const ba_plan_t *plan, const void *q_main,
                        st, stages);
 }
 
+extern "C" int branch_attn_bwd_stages(const ba_plan_t *plan, const void *q_main, const void *q_branch,
+                                      const void *k, const void *v, const void *O, const float *LSE,
+                                      const void *dO, int64_t qm_begin, int64_t qm_end, int64_t br_begin,
+                                      int64_t br_end, int64_t kv_begin, int64_t kv_end, int parts,
+                                      int accumulate, void *dQ_main, void *dQ_branch, void *dK, void *dV,
+                                      void *workspace, size_t ws_bytes, void *stream, int stages) {
+    return bwd_common(plan, q_main, q_branch, k, v, O, LSE, dO, qm_begin, qm_end, br_begin, br_end, kv_begin, kv_end, 0,
+                      parts, accumulate, dQ_main, dQ_branch, dK, dV, workspace, ws_bytes, stream, stages);
+}
+
 // ---------------------------------------------------------------- step-major (per-depth) calls
 
 static int depth_range(const ba_plan_t *plan, int depth, int64_t br_begin, int64_t br_end, BaRange *r) {
@@ -195,6 +207,7 @@ static int depth_range(const ba_plan_t *plan, int depth, int64_t br_begin, int64
     r->qm_begin = r->qm_end = 0;
     r->tok_begin = br_begin; r->tok_end = br_end;   // branch indices: one query row per branch
     r->kv_begin = 0; r->kv_end = pr.n_main;
+    r->kv_base = 0;
     r->parts = BA_PART_MAIN | BA_PART_BRANCH;
     return BA_OK;
 }
@@ -235,20 +248,17 @@ extern "C" int branch_attn_bwd_depth(const ba_plan_t *plan, int depth, const voi
 
 // ---------------------------------------------------------------- ring steps on a received K/V shard
 
-// The kernels address keys by their global row; a shard holds only rows [kv_begin, kv_end) and is addressed as
-// if it were the full tensor, by moving its base back by kv_begin rows.  No byte outside the shard is read: key
-// tiles start at kv_begin or, where a tile starts at a row's first visible key, at max(that key, kv_begin); and a
-// call without own-branch keys gives the tensor maps of K and V kv_end rows, so that the rows of a tile beyond
-// them arrive as zeros (the plain-FMA kernels load live rows only).
+// The kernels number keys by their global row; K, V (and dK, dV) of these calls start at row kv_base = kv_begin.
+// Nothing outside the shard is read: key tiles start at kv_begin or, where a tile starts at a row's first visible
+// key, at max(that key, kv_begin), and without own-branch keys the tensor maps hold rows [kv_begin, kv_end) only, so
+// that the rows of a tile beyond them arrive as zeros (the plain-FMA kernels load live rows only).  No pointer is
+// formed outside the shard either: maps that started kv_begin rows before it, at an address that need not be
+// mapped, ended in a fault once.
 static int shard_ok(const ba_plan_t *plan, int64_t kv_begin, int64_t kv_end) {
     if (!plan) return BA_EINVAL;
     if (kv_begin < 0 || kv_end < kv_begin || kv_end > plan->prob.n_main) return BA_EINVAL;
     if ((kv_begin % 128) != 0 || ((kv_end % 128) != 0 && kv_end != plan->prob.n_main)) return BA_EINVAL;
     return BA_OK;
-}
-
-static inline const void *rebase(const void *shard, int64_t rows_back, size_t row_bytes) {
-    return shard ? (const void *)((const char *)shard - (size_t)rows_back * row_bytes) : nullptr;
 }
 
 extern "C" int branch_attn_fwd_shard(const ba_plan_t *plan, const void *q_main, const void *q_branch,
@@ -259,14 +269,11 @@ extern "C" int branch_attn_fwd_shard(const ba_plan_t *plan, const void *q_main, 
     if (rc != BA_OK) return rc;
     if (merge != 0 && merge != 1) return BA_EINVAL;
     if (kv_end > kv_begin && (!k_shard || !v_shard)) return BA_EINVAL;
-    const size_t esz = plan->prob.dtype == BA_FP32 ? 4 : 2;
-    const size_t row_bytes = (size_t)plan->prob.h_kv * plan->prob.head_dim * esz;
-    const void *k = rebase(k_shard, kv_begin, row_bytes), *v = rebase(v_shard, kv_begin, row_bytes);
-    if (merge)
-        return branch_attn_fwd_partial_merge(plan, q_main, q_branch, k, v, qm_begin, qm_end, br_begin, br_end,
-                                             kv_begin, kv_end, BA_PART_MAIN, O_acc, LSE_acc, nullptr, 0, stream);
-    return branch_attn_fwd_partial(plan, q_main, q_branch, k, v, qm_begin, qm_end, br_begin, br_end, kv_begin,
-                                   kv_end, BA_PART_MAIN, O_acc, LSE_acc, nullptr, 0, stream);
+    BaRange r;
+    if ((rc = make_range(plan, qm_begin, qm_end, br_begin, br_end, kv_begin, kv_end, BA_PART_MAIN, &r)) != BA_OK) return rc;
+    if (!q_main && qm_end > qm_begin) return BA_EINVAL;
+    r.kv_base = kv_begin;
+    return fwd_common(plan, r, q_main, q_branch, k_shard, v_shard, O_acc, LSE_acc, merge ? 2 : 1, stream);
 }
 
 extern "C" int branch_attn_bwd_shard(const ba_plan_t *plan, const void *q_main, const void *q_branch,
@@ -278,12 +285,7 @@ extern "C" int branch_attn_bwd_shard(const ba_plan_t *plan, const void *q_main, 
     int rc = shard_ok(plan, kv_begin, kv_end);
     if (rc != BA_OK) return rc;
     if (kv_end > kv_begin && (!k_shard || !v_shard || !dK_shard || !dV_shard)) return BA_EINVAL;
-    const size_t esz = plan->prob.dtype == BA_FP32 ? 4 : 2;
-    const size_t row_elems = (size_t)plan->prob.h_kv * plan->prob.head_dim;
-    const void *k = rebase(k_shard, kv_begin, row_elems * esz), *v = rebase(v_shard, kv_begin, row_elems * esz);
-    void *dk = (void *)rebase(dK_shard, kv_begin, row_elems * sizeof(float));
-    void *dv = (void *)rebase(dV_shard, kv_begin, row_elems * sizeof(float));
-    return branch_attn_bwd_stages(plan, q_main, q_branch, k, v, O, LSE, dO, qm_begin, qm_end, br_begin, br_end,
-                                  kv_begin, kv_end, BA_PART_MAIN, 1, dQ_main, dQ_branch, dk, dv, workspace,
-                                  ws_bytes, stream, stages);
+    return bwd_common(plan, q_main, q_branch, k_shard, v_shard, O, LSE, dO, qm_begin, qm_end, br_begin, br_end, kv_begin,
+                      kv_end, kv_begin, BA_PART_MAIN, 1, dQ_main, dQ_branch, dK_shard, dV_shard, workspace, ws_bytes,
+                      stream, stages);
 }

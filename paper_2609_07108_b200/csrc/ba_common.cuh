@@ -37,6 +37,7 @@ struct BaRange {
     int64_t qm_begin, qm_end;     // main query rows
     int64_t tok_begin, tok_end;   // branch tokens (query side and branch-key side)
     int64_t kv_begin, kv_end;     // main keys
+    int64_t kv_base;              // first row that K, V (and dK, dV) hold: 0, or kv_begin on a received shard
     int parts;
 };
 

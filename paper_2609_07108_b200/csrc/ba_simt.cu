@@ -271,14 +271,14 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const SimtArgs a) {
         const T *src1 = MODE == kDkdv ? (const T *)a.k : is_main ? (const T *)a.q_main : (const T *)a.q_branch;
         load_rows<T, D, kRows>(sm.st1, src1, [&](int r) -> int64_t {
             if (!live_row(r)) return -1;
-            if (MODE == kDkdv) return (((is_main ? 0 : n) + base + r) * a.h_kv + g) * D;
+            if (MODE == kDkdv) return (((is_main ? -a.r.kv_base : n) + base + r) * a.h_kv + g) * D;
             return (row_tok(r) * a.h_q + h0 + r % a.hp) * D;
         });
         if (MODE != kFwd) {
             const T *src2 = MODE == kDkdv ? (const T *)a.v : (const T *)a.d_o;
             load_rows<T, D, kRows>(sm.st2, src2, [&](int r) -> int64_t {
                 if (!live_row(r)) return -1;
-                if (MODE == kDkdv) return (((is_main ? 0 : n) + base + r) * a.h_kv + g) * D;
+                if (MODE == kDkdv) return (((is_main ? -a.r.kv_base : n) + base + r) * a.h_kv + g) * D;
                 return (((is_main ? 0 : n) + row_tok(r)) * a.h_q + h0 + r % a.hp) * D;
             });
         }
@@ -334,15 +334,15 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const SimtArgs a) {
             }
         } else {
             load_rows<T, D, kBN>(dst, (const T *)a.k,
-                            [&](int r) -> int64_t { return r < x.cnt ? (((x.main ? 0 : n) + x.r0 + r) * a.h_kv + g) * D : -1; });
+                            [&](int r) -> int64_t { return r < x.cnt ? (((x.main ? -a.r.kv_base : n) + x.r0 + r) * a.h_kv + g) * D : -1; });
         }
     };
     auto load_x2 = [&](int t) {
         if (t >= t_end) return;
         const Tile x = tile_of(t);
-        const int64_t heads = MODE == kDkdv ? a.h_q : a.h_kv;
+        const int64_t heads = MODE == kDkdv ? a.h_q : a.h_kv, row0 = !x.main ? n : MODE == kDkdv ? 0 : -a.r.kv_base;
         load_rows<T, D, kBN>(sm.x2, MODE == kDkdv ? (const T *)a.d_o : (const T *)a.v,
-                        [&](int r) -> int64_t { return r < x.cnt ? (((x.main ? 0 : n) + x.r0 + r) * heads + x.h) * D : -1; });
+                        [&](int r) -> int64_t { return r < x.cnt ? ((row0 + x.r0 + r) * heads + x.h) * D : -1; });
     };
 
     // ---- per-thread views: score lanes hold rows 2 rg + i and columns cg + 8 j of the warp's WR x 32 tile,
@@ -559,7 +559,7 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const SimtArgs a) {
             }
             x.x *= a.scale; x.y *= a.scale; x.z *= a.scale; x.w *= a.scale;
             void *dst0 = MODE == kDkdv ? a.dk : is_main ? a.dq_main : a.dq_branch;
-            const size_t off = MODE == kDkdv ? ((size_t)gr * a.h_kv + g) * D + ch : ((size_t)t * a.h_q + h0 + r % a.hp) * D + ch;
+            const size_t off = MODE == kDkdv ? ((size_t)(is_main ? t - a.r.kv_base : gr) * a.h_kv + g) * D + ch : ((size_t)t * a.h_q + h0 + r % a.hp) * D + ch;
             if (a.accumulate) {
                 const float4 o = load4<float>((float *)dst0 + off);
                 store4<float>((float *)dst0 + off, make_float4(o.x + x.x, o.y + x.y, o.z + x.z, o.w + x.w));

@@ -219,7 +219,7 @@ tc_dq_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                             auto load = [&](uint8_t *dst, const CUtensorMap *m128, const CUtensorMap *m32, uint64_t *bar) {
                                 mbar_expect_tx(bar, (uint32_t)(nch * 8192));
                                 if (j < it.n_full) {
-                                    for (int hf = 0; hf < 2; ++hf) tma_load_3d(dst + hf * 16384, m128, hf * 64, it.g, it.lo_min + j * kTile, bar);
+                                    for (int hf = 0; hf < 2; ++hf) tma_load_3d(dst + hf * 16384, m128, hf * 64, it.g, full_row(p, it, j), bar);
                                 } else {
                                     for (int c = 0; c < nch; ++c) {
                                         const int row = chunk_row(p, it, 4 * (j - it.n_full) + c);
@@ -734,7 +734,7 @@ template <int MODE> __device__ void make_kv_item(const TcBwdParams &p, uint32_t 
         it.row0 = is_main ? (int)p.r.kv_begin + tile * step : (int)p.r.tok_begin + bt * step;
         it.row_end = past ? it.row0 : min(it.row0 + step, (int)(is_main ? p.r.kv_end : p.r.tok_end));
     }
-    it.srow0 = is_main ? it.row0 : n + (kDq ? 0 : kdepth * p.num_branches) + it.row0;
+    it.srow0 = is_main ? it.row0 - (kDq ? 0 : (int)p.r.kv_base) : n + (kDq ? 0 : kdepth * p.num_branches) + it.row0;
     it.m0 = it.m1 = it.b0 = it.b1 = 0;
     const int first = it.row0, last = it.row_end - 1;
     if (last >= first) {
@@ -914,7 +914,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                     SubMeta &mt = sm.meta[st];
                     if (kDq) {
                         if (lane == 0) {
-                            const int kr = seg_main ? r0 : (int)p.meta.n_main + r0;
+                            const int kr = seg_main ? r0 - (int)p.r.kv_base : (int)p.meta.n_main + r0;
                             mbar_expect_tx(&sm.x_full[st], 2 * kSubBytes);
                             for (int half = 0; half < kHalves; ++half) {
                                 tma_load_3d(sm.xs[st] + half * 8192, &tm_k, half * 64, it.g, kr, &sm.x_full[st]);
@@ -1399,7 +1399,7 @@ int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
     const uint64_t all_rows = (uint64_t)(pr.n_main + pr.n_branch);
     // (without own-branch keys nothing beyond kv_end is needed: a received shard ends there)
     const uint64_t kv_rows = depth ? (uint64_t)(pr.n_main + (int64_t)depth * pr.num_branches)
-                             : (r.parts & BA_PART_BRANCH) ? all_rows : (uint64_t)(r.kv_end > 0 ? r.kv_end : 1);
+                             : (r.parts & BA_PART_BRANCH) ? all_rows : (uint64_t)(r.kv_end > r.kv_base ? r.kv_end - r.kv_base : 1);
     const uint64_t go_rows = depth ? (uint64_t)pr.num_branches : all_rows;
     const void *qm = q_main ? q_main : q_branch;
     const void *qb = (q_branch && pr.n_branch > 0) ? q_branch : q_main;

@@ -180,7 +180,7 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_
     const int64_t key0 = main_keys ? p.r.kv_begin + (int64_t)tile * kTile
                                    : p.r.tok_begin + (int64_t)(tile - p.main_key_tiles) * p.step_kb;
     const int64_t key_end = main_keys ? p.r.kv_end : min(p.r.tok_end, key0 + p.step_kb);
-    const int64_t gkey0 = main_keys ? key0 : n + key0;
+    const int64_t gkey0 = main_keys ? key0 - p.r.kv_base : n + key0;      // its row in the key tensors
 
     if (tid == 0) {
         mbar_init(&sm.kv_full, 1);
@@ -691,7 +691,7 @@ int ba_tc_bwd_fused(const ba_plan *pl, const BaRange &r, const void *q_main, con
     CUtensorMap tq_main, tq_branch, tgo, tk, tv;
     const uint64_t all_rows = (uint64_t)(pr.n_main + pr.n_branch);
     // without own-branch keys nothing beyond kv_end is needed (a received shard ends there)
-    const uint64_t kv_rows = (r.parts & BA_PART_BRANCH) ? all_rows : (uint64_t)(r.kv_end > 0 ? r.kv_end : 1);
+    const uint64_t kv_rows = (r.parts & BA_PART_BRANCH) ? all_rows : (uint64_t)(r.kv_end > r.kv_base ? r.kv_end - r.kv_base : 1);
     const void *qm = q_main ? q_main : q_branch;
     const void *qb = (q_branch && pr.n_branch > 0) ? q_branch : q_main;
     const uint64_t qm_rows = q_main ? (uint64_t)pr.n_main : (uint64_t)pr.n_branch;

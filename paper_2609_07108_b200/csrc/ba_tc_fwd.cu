@@ -413,7 +413,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
                                 if (j < it.n_full) {
                                     for (int hf = 0; hf < kHalves; ++hf)
                                         tma_load_3d(sm.kv[s] + hf * 16384, kv ? &tm_v : &tm_k, hf * 64, it.g,
-                                                    it.lo_min + j * kTile, &sm.kv_full[s]);
+                                                    full_row(p, it, j), &sm.kv_full[s]);
                                 } else {
                                     for (int c = 0; c < nch; ++c) {
                                         const int row = chunk_row(p, it, 4 * (j - it.n_full) + c);
@@ -946,7 +946,7 @@ int ba_tc_fwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
     // own-branch keys nothing beyond kv_end is needed (a received shard ends there).
     const uint64_t kv_rows = depth ? (uint64_t)(pr.n_main + (int64_t)depth * pr.num_branches)
                              : (r.parts & BA_PART_BRANCH) ? (uint64_t)(pr.n_main + pr.n_branch)
-                                                          : (uint64_t)(r.kv_end > 0 ? r.kv_end : 1);
+                                                          : (uint64_t)(r.kv_end > r.kv_base ? r.kv_end - r.kv_base : 1);
     // an absent query tensor still needs a valid map object: alias the other one
     const void *qm = q_main ? q_main : q_branch;
     const void *qb = (q_branch && pr.n_branch > 0) ? q_branch : q_main;

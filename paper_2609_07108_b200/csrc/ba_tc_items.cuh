@@ -131,9 +131,10 @@ __device__ void make_item(const ItemParams &p, uint32_t work, int rank, Item &it
     it.je = (int)((int64_t)it.T * (rank + 1) / p.splits);
 }
 
-// first key row (of the [N + M] key tensor) of tail chunk c
+// first row of full key tile j / of tail chunk c in the key tensors
+__device__ __forceinline__ int full_row(const ItemParams &p, const Item &it, int j) { return it.lo_min - (int)p.r.kv_base + j * kTile; }
 __device__ __forceinline__ int chunk_row(const ItemParams &p, const Item &it, int c) {
-    if (c < it.n_mc) return it.tail_k + 32 * c;
+    if (c < it.n_mc) return it.tail_k - (int)p.r.kv_base + 32 * c;
     c -= it.n_mc;
     if (!p.depth) return (int)p.meta.n_main + it.bs + 32 * c;
     const int cpd = (it.rows + 31) / 32;
