@@ -55,7 +55,9 @@ enum { BA_STAGE_PREP = 1, BA_STAGE_DQ = 2, BA_STAGE_DKDV = 4, BA_STAGE_ALL = 7,
 
 /* Which kernels a plan uses: the tensor-core (tcgen05) path where the shape
  * allows it (bf16), or the plain-FMA path (any supported shape; the only path
- * for fp32).  BA_STAGE_FUSED and the per-depth calls need head_dim 128. */
+ * for fp32).  BA_STAGE_FUSED and the per-depth calls need head_dim 128.  At head_dim
+ * 64 a tensor-core plan runs calls with fp32 results (partial forwards, accumulate = 1,
+ * shard calls) on the plain-FMA kernels, whose probabilities are fp32 too. */
 enum { BA_IMPL_AUTO = 0, BA_IMPL_SIMT = 1, BA_IMPL_TC = 2 };
 
 typedef struct ba_problem {

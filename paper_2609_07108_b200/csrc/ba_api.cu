@@ -57,9 +57,9 @@ static int fwd_common(const ba_plan_t *plan, const BaRange &r, const void *q_mai
     if (!k || !v || !o || !lse) return BA_EINVAL;
     if (has_branch_q && !q_branch) return BA_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
-    if (plan->impl == BA_IMPL_TC) return ba_tc_fwd(plan, r, q_main, q_branch, k, v, o, lse, partial, st);
-    if (partial == 2) return BA_EUNSUPPORTED;   // merge in the epilogue: tensor-core kernel only
-    return ba_simt_fwd(plan, r, q_main, q_branch, k, v, o, lse, partial != 0, st);
+    if (ba_use_tc(plan, partial != 0)) return ba_tc_fwd(plan, r, q_main, q_branch, k, v, o, lse, partial, st);
+    if (partial == 2 && plan->impl != BA_IMPL_TC) return BA_EUNSUPPORTED;   // merge in the epilogue: tensor-core plans only
+    return ba_simt_fwd(plan, r, q_main, q_branch, k, v, o, lse, partial, st);
 }
 
 extern "C" int branch_attn_fwd(const ba_plan_t *plan, const void *q_main, const void *q_branch,
@@ -178,7 +178,7 @@ static int bwd_common(const ba_plan_t *plan, const void *q_main, const void *q_b
             return rc;
         return BA_OK;
     }
-    if (plan->impl == BA_IMPL_TC)
+    if (ba_use_tc(plan, accumulate != 0))
         return ba_tc_bwd(plan, r, qm, q_branch, k, v, LSE, delta, dO, accumulate, dQ_main, dQ_branch, dK,
                          dV, st, stages);
     return ba_simt_bwd(plan, r, qm, q_branch, k, v, LSE, delta, dO, accumulate, dQ_main, dQ_branch, dK, dV,

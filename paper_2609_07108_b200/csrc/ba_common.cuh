@@ -61,10 +61,23 @@ static inline int ba_check_launch() {
     return BA_OK;
 }
 
+// weights of Eq. (lse-merge) for merging (lse_p, O_p * inv) into the running pair with lse_a
+__device__ __forceinline__ void merge_weights(float lse_a, float lse_p, float inv, float &lse_out, float &w_old, float &w_new) {
+    const float mx = fmaxf(lse_a, lse_p);
+    if (mx == -INFINITY) {
+        lse_out = -INFINITY; w_new = 0.f; w_old = 0.f;
+    } else {
+        const float ea = expf(lse_a - mx), ep = expf(lse_p - mx), s = ea + ep;
+        lse_out = mx + logf(s);
+        w_old = ea / s;
+        w_new = ep / s * inv;
+    }
+}
+
 // --- kernels implemented in the other translation units -------------------
-// Plain-FMA path (ba_simt.cu)
+// Plain-FMA path (ba_simt.cu); partial_out as in ba_tc_fwd
 int ba_simt_fwd(const ba_plan *pl, const BaRange &r, const void *q_main, const void *q_branch,
-                const void *k, const void *v, void *o, float *lse, bool partial_out,
+                const void *k, const void *v, void *o, float *lse, int partial_out,
                 cudaStream_t st);
 int ba_simt_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const void *q_branch,
                 const void *k, const void *v, const float *lse, const float *delta,
@@ -87,6 +100,13 @@ int ba_tc_bwd_fused(const ba_plan *pl, const BaRange &r, const void *q_main, con
                     int accumulate, void *dq_main, void *dq_branch, void *dk, void *dv,
                     cudaStream_t st);
 bool ba_tc_supported(const ba_problem_t *p);
+// Head_dim 64 with fp32 results (partial forwards, accumulated gradients) stays on the plain-FMA kernels: the
+// tensor-core kernels carry P and dS as bf16 pairs (16 bits of mantissa), which bf16 results do not show and fp32
+// results do.  Against fp64, 1,600 .. 3,000 tokens with chains, plain FMA / tensor cores, 2-norm: O 1e-7 .. 3e-7 /
+// 2e-6, dQ 2e-7 .. 5e-7 / 3e-6, dK and dV 4e-7 .. 7e-7 / 4e-6 .. 1.4e-5.
+static inline bool ba_use_tc(const ba_plan *pl, bool fp32_out) {
+    return pl->impl == BA_IMPL_TC && !(pl->prob.head_dim == 64 && fp32_out);
+}
 // Elementwise (ba_elementwise.cu)
 // Backward preprocess into head-major scratch [h_q, row_pitch]:
 //   delta_t[h, r] = <dO[r, h], O[r, h]>,  nlse2_t[h, r] = -LSE[r, h] * log2(e)

@@ -66,7 +66,7 @@ struct SimtArgs {
     void *dq_main, *dq_branch, *dk, *dv;
     int h_q, h_kv, group;
     float scale, scale_log2;
-    int partial_out;  // forward: compact fp32 outputs
+    int partial_out;  // forward: compact fp32 outputs (2: merged in place)
     int accumulate;   // backward: fp32 += outputs
     int hp, head_chunks, tok;      // forward, dQ: heads per tile, chunks of hp heads per group, tokens per tile
     int main_tiles, total_tiles;   // stationary tiles (of one KV head and head chunk)
@@ -524,8 +524,18 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const SimtArgs a) {
     const int rows_mine = kRows / a.splits;
     for (int idx = tid; idx < rows_mine * CPR; idx += kThreads) {
         const int r = rank * rows_mine + idx / CPR, ch = (idx % CPR) * 4;
-        if (!live_row(r)) continue;
+        const bool live = live_row(r);
         const int64_t t = row_tok(r), gr = is_main ? t : n + t;
+        int64_t orow = gr;
+        float lse_a = -INFINITY;
+        if (MODE == kFwd && a.partial_out) {
+            orow = is_main ? t - a.r.qm_begin : (a.r.qm_end - a.r.qm_begin) + (t - a.r.tok_begin);
+            if (a.partial_out == 2) {      // the lanes of a row (of one warp) read the old LSE before one replaces it
+                if (live) lse_a = a.lse_out[orow * a.h_q + h0 + r % a.hp];
+                __syncwarp();
+            }
+        }
+        if (!live) continue;
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
         const uint32_t src0 = smem_u32(out0 + r * P + ch), src1 = smem_u32(out1 + r * P + ch), src_ml = smem_u32(&sm.ml[r]);
         if (MODE == kFwd) {
@@ -540,12 +550,16 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const SimtArgs a) {
                 x.x += w * v.x; x.y += w * v.y; x.z += w * v.z; x.w += w * v.w;
             }
             const float inv = l > 0.f ? 1.0f / l : 0.f;
-            x.x *= inv; x.y *= inv; x.z *= inv; x.w *= inv;
             const int h = h0 + r % a.hp;
-            int64_t orow = gr;
-            if (a.partial_out) orow = is_main ? t - a.r.qm_begin : (a.r.qm_end - a.r.qm_begin) + (t - a.r.tok_begin);
-            if (ch == 0) a.lse_out[orow * a.h_q + h] = l > 0.f ? (mx + log2f(l)) * kLn2 : -INFINITY;
+            float lse_new = l > 0.f ? (mx + log2f(l)) * kLn2 : -INFINITY, w_new = inv, w_old = 0.f;
+            if (a.partial_out == 2) merge_weights(lse_a, lse_new, inv, lse_new, w_old, w_new);
+            x.x *= w_new; x.y *= w_new; x.z *= w_new; x.w *= w_new;
+            if (ch == 0) a.lse_out[orow * a.h_q + h] = lse_new;
             const size_t off = ((size_t)orow * a.h_q + h) * D + ch;
+            if (w_old != 0.f) {
+                const float4 o = load4<float>((float *)a.o + off);
+                x.x += o.x * w_old; x.y += o.y * w_old; x.z += o.z * w_old; x.w += o.w * w_old;
+            }
             if (a.partial_out) store4<float>((float *)a.o + off, x);
             else store4<T>((T *)a.o + off, x);
         } else {
@@ -680,11 +694,11 @@ SimtArgs base_args(const ba_plan *pl, const BaRange &r) {
 }  // namespace
 
 int ba_simt_fwd(const ba_plan *pl, const BaRange &r, const void *q_main, const void *q_branch,
-                const void *k, const void *v, void *o, float *lse, bool partial_out,
+                const void *k, const void *v, void *o, float *lse, int partial_out,
                 cudaStream_t st) {
     SimtArgs a = base_args(pl, r);
     a.q_main = q_main; a.q_branch = q_branch; a.k = k; a.v = v;
-    a.o = o; a.lse_out = lse; a.partial_out = partial_out ? 1 : 0;
+    a.o = o; a.lse_out = lse; a.partial_out = partial_out;
     return dispatch<kFwd>(pl, a, st);
 }
 

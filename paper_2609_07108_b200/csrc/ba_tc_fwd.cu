@@ -137,19 +137,6 @@ __device__ __forceinline__ void merge_row_chunk(void *o, size_t elem_off, const 
     }
 }
 
-// weights of Eq. (lse-merge) for merging (lse_p, O_p * inv) into the running pair with lse_a
-__device__ __forceinline__ void merge_weights(float lse_a, float lse_p, float inv, float &lse_out, float &w_old, float &w_new) {
-    const float mx = fmaxf(lse_a, lse_p);
-    if (mx == -INFINITY) {
-        lse_out = -INFINITY; w_new = 0.f; w_old = 0.f;
-    } else {
-        const float ea = expf(lse_a - mx), ep = expf(lse_p - mx), s = ea + ep;
-        lse_out = mx + logf(s);
-        w_old = ea / s;
-        w_new = ep / s * inv;
-    }
-}
-
 // max over one 32-column chunk of scores
 __device__ __forceinline__ float chunk_max(const uint32_t (&r)[32], float m) {
     float mm[4] = {m, -INFINITY, -INFINITY, -INFINITY};
