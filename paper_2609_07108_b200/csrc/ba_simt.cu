@@ -32,6 +32,7 @@
 #include <string.h>
 
 #include "ba_common.cuh"
+#include "ba_exact.cuh"
 #include "ba_sm100.cuh"
 
 using sm100::cluster_ld_f2;
@@ -55,17 +56,11 @@ constexpr float kLn2 = 0.6931471805599453f;
 
 enum { kFwd = 0, kDq = 1, kDkdv = 2 };
 
-struct SimtArgs {
-    BaMeta meta;
-    BaRange r;
-    const void *q_main, *q_branch, *k, *v, *d_o;
-    const float *lse_in, *delta;  // delta: head-major [h_q, delta_pitch]
-    int64_t delta_pitch;
+struct SimtArgs : RowArgs {
+    const float *lse_in;
     void *o;          // forward output
     float *lse_out;
     void *dq_main, *dq_branch, *dk, *dv;
-    int h_q, h_kv, group;
-    float scale, scale_log2;
     int partial_out;  // forward: compact fp32 outputs (2: merged in place)
     int accumulate;   // backward: fp32 += outputs
     int hp, head_chunks, tok;      // forward, dQ: heads per tile, chunks of hp heads per group, tokens per tile
@@ -94,6 +89,13 @@ template <> __device__ __forceinline__ void store4<__nv_bfloat16>(__nv_bfloat16 
     r.y = *reinterpret_cast<uint32_t *>(&hi);
     *reinterpret_cast<uint2 *>(p) = r;
 }
+
+// NaN or opposite infinities among four results: their row is to be formed again, pair by pair (ba_exact.cuh)
+__device__ __forceinline__ bool not_finite(float4 x) {
+    const float s = x.x + x.y + x.z + x.w;
+    return s != s;
+}
+__device__ __forceinline__ float4 row4(const Cols<4> &c) { return make_float4(c.v[0], c.v[1], c.v[2], c.v[3]); }
 
 // four elements global -> shared as fp32 (zeros when !live): asynchronous for fp32 sources
 __device__ __forceinline__ void copy4(float *dst, const float *src, bool live) {
@@ -211,11 +213,12 @@ template <int D, int MODE> struct SimtSmem {
 };
 
 template <typename T, int D, int MODE>
-__global__ void __launch_bounds__(kThreads, 3) simt_kernel(const SimtArgs a) {
+__global__ void __launch_bounds__(kThreads, 3) simt_kernel(const __grid_constant__ SimtArgs a) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     using Smem = SimtSmem<D, MODE>;
     Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
     constexpr int WR = kRows / 4, AR = 4;     // rows per warp, per accumulator lane
+    constexpr bool kMerges = MODE == kFwd && D == 64 && sizeof(T) == 2;      // partial results merged in place
     constexpr int P = pitch<D>();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t n = a.meta.n_main;
@@ -326,7 +329,7 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const SimtArgs a) {
                 const bool live = tid < x.cnt;
                 const int64_t row = x.r0 + tid, gr = (x.main ? 0 : n) + row;
                 sm.lse2[tid] = live ? a.lse_in[gr * a.h_q + x.h] * kLog2e : 0.f;
-                sm.dlt[tid] = live ? a.delta[(size_t)x.h * a.delta_pitch + gr] : 0.f;
+                sm.dlt[tid] = live ? a.delta_t[(size_t)x.h * a.row_pitch + gr] : 0.f;
                 sm.lo[tid] = live ? a.meta.row_lo[gr] : INT_MAX;
                 sm.hi[tid] = live ? a.meta.row_hi[gr] : -1;
                 sm.bst[tid] = live && !x.main ? a.meta.br_start[row] : 0;
@@ -374,7 +377,7 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const SimtArgs a) {
             if (!is_main && (a.r.parts & BA_PART_BRANCH)) { bst[i] = a.meta.br_start[t]; mask[i] = a.meta.br_mask[t]; }
             if (MODE == kDq) {
                 lse2[i] = a.lse_in[gr * a.h_q + h] * kLog2e;
-                dlt[i] = a.delta[(size_t)h * a.delta_pitch + gr];
+                dlt[i] = a.delta_t[(size_t)h * a.row_pitch + gr];
             }
         }
     }
@@ -524,18 +527,16 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const SimtArgs a) {
     const int rows_mine = kRows / a.splits;
     for (int idx = tid; idx < rows_mine * CPR; idx += kThreads) {
         const int r = rank * rows_mine + idx / CPR, ch = (idx % CPR) * 4;
-        const bool live = live_row(r);
         const int64_t t = row_tok(r), gr = is_main ? t : n + t;
-        int64_t orow = gr;
+        auto out_row = [&]() -> int64_t {
+            return a.partial_out ? is_main ? t - a.r.qm_begin : (a.r.qm_end - a.r.qm_begin) + (t - a.r.tok_begin) : gr;
+        };
         float lse_a = -INFINITY;
-        if (MODE == kFwd && a.partial_out) {
-            orow = is_main ? t - a.r.qm_begin : (a.r.qm_end - a.r.qm_begin) + (t - a.r.tok_begin);
-            if (a.partial_out == 2) {      // the lanes of a row (of one warp) read the old LSE before one replaces it
-                if (live) lse_a = a.lse_out[orow * a.h_q + h0 + r % a.hp];
-                __syncwarp();
-            }
+        if (kMerges && a.partial_out == 2) {      // the lanes of a row (of one warp) read the old LSE before one replaces it
+            if (live_row(r)) lse_a = a.lse_out[out_row() * a.h_q + h0 + r % a.hp];
+            __syncwarp();
         }
-        if (!live) continue;
+        if (!live_row(r)) continue;
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
         const uint32_t src0 = smem_u32(out0 + r * P + ch), src1 = smem_u32(out1 + r * P + ch), src_ml = smem_u32(&sm.ml[r]);
         if (MODE == kFwd) {
@@ -551,12 +552,14 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const SimtArgs a) {
             }
             const float inv = l > 0.f ? 1.0f / l : 0.f;
             const int h = h0 + r % a.hp;
+            if (not_finite(x)) x = row4(exact_query_row<T, D, false, 4>(a, is_main, (int)t, h, -mx, ch));
             float lse_new = l > 0.f ? (mx + log2f(l)) * kLn2 : -INFINITY, w_new = inv, w_old = 0.f;
-            if (a.partial_out == 2) merge_weights(lse_a, lse_new, inv, lse_new, w_old, w_new);
+            if (kMerges && a.partial_out == 2) merge_weights(lse_a, lse_new, inv, lse_new, w_old, w_new);
             x.x *= w_new; x.y *= w_new; x.z *= w_new; x.w *= w_new;
+            const int64_t orow = out_row();
             if (ch == 0) a.lse_out[orow * a.h_q + h] = lse_new;
             const size_t off = ((size_t)orow * a.h_q + h) * D + ch;
-            if (w_old != 0.f) {
+            if (kMerges && w_old != 0.f) {
                 const float4 o = load4<float>((float *)a.o + off);
                 x.x += o.x * w_old; x.y += o.y * w_old; x.z += o.z * w_old; x.w += o.w * w_old;
             }
@@ -571,6 +574,11 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const SimtArgs a) {
                     y.x += u.x; y.y += u.y; y.z += u.z; y.w += u.w;
                 }
             }
+            if (MODE == kDq && not_finite(x))
+                x = row4(exact_query_row<T, D, true, 4>(a, is_main, (int)t, h0 + r % a.hp,
+                                                        a.nlse2_t[(h0 + r % a.hp) * a.row_pitch + gr], ch));
+            if (MODE == kDkdv && not_finite(x)) x = row4(exact_key_row<T, D, 4>(a, is_main, (int)t, g, false, ch));
+            if (MODE == kDkdv && not_finite(y)) y = row4(exact_key_row<T, D, 4>(a, is_main, (int)t, g, true, ch));
             x.x *= a.scale; x.y *= a.scale; x.z *= a.scale; x.w *= a.scale;
             void *dst0 = MODE == kDkdv ? a.dk : is_main ? a.dq_main : a.dq_branch;
             const size_t off = MODE == kDkdv ? ((size_t)(is_main ? t - a.r.kv_base : gr) * a.h_kv + g) * D + ch : ((size_t)t * a.h_q + h0 + r % a.hp) * D + ch;
@@ -708,7 +716,8 @@ int ba_simt_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const v
                 void *dv, cudaStream_t st, int stages) {
     SimtArgs a = base_args(pl, r);
     a.q_main = q_main; a.q_branch = q_branch; a.k = k; a.v = v; a.d_o = d_o;
-    a.lse_in = lse; a.delta = delta; a.delta_pitch = pl->row_pitch; a.accumulate = accumulate;
+    a.lse_in = lse; a.delta_t = delta; a.row_pitch = pl->row_pitch; a.accumulate = accumulate;
+    a.nlse2_t = delta + (size_t)pl->row_pitch * a.h_q;
     a.dq_main = dq_main; a.dq_branch = dq_branch; a.dk = dk; a.dv = dv;
     int rc = BA_OK;
     if (stages & BA_STAGE_DQ) rc = dispatch<kDq>(pl, a, st);

@@ -1,0 +1,103 @@
+"""A NaN or an infinity in one row reaches only the results whose definition contains that row: the plain-FMA
+kernels leave every other row as it is.  What a row may reach follows from the oracle's visibility matrix alone."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2609_07108_b200 import workloads as W
+from helpers import TOL, REL_RMS, f32, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ba():
+    from paper_2609_07108_b200 import binding
+    assert torch.cuda.is_available()
+    return binding
+
+
+def problem(kind, head_dim, dtype, lens, anchors, blen, h_q=4, h_kv=2):
+    anchors = np.sort(np.asarray(anchors, np.int32))
+    rng = np.random.default_rng(11)
+    parent = None
+    if kind == W.TREE:
+        parent = np.concatenate([W.random_tree_parents(rng, blen, 4) for _ in anchors]).astype(np.int32)
+    return W.Problem(W.cu_from_lengths(lens), anchors, W.uniform_branch_offsets(len(anchors), blen), kind, parent, h_q, h_kv,
+                     head_dim, dtype=dtype)
+
+
+# (kind, head_dim, dtype, plain-FMA kernels?): lengths that leave sequences, branches and the poisoned rows in the
+# middle of 32-, 64- and 128-row tiles; few rows (tiles shared by clusters) and enough rows to leave tiles whole
+SMALL = dict(lens=[70, 131, 300], anchors=list(range(0, 501, 9)), blen=5)
+LARGE = dict(lens=[1500, 333, 2200], anchors=list(range(0, 4033, 5)), blen=3, h_q=8, h_kv=8)
+CASES = [(W.CHAIN, 64, "fp32", False, SMALL), (W.TREE, 128, "fp32", False, SMALL), (W.BLOCK, 64, "fp32", False, LARGE),
+         (W.CHAIN, 64, "bf16", True, SMALL), (W.BLOCK, 128, "bf16", True, SMALL)]
+
+
+def poisoned(p, d, name, row, value):
+    """Tensors with row `row` (global numbering) of tensor `name` set to `value` in the last query / KV head."""
+    d = {k: v.clone() for k, v in d.items()}
+    if name == "q":
+        t, row = (d["q_main"], row) if row < p.n_main else (d["q_branch"], row - p.n_main)
+    else:
+        t = d[name]
+    t[row, -1, 3:7] = value
+    return d
+
+
+def check(name, got, want, hit, dtype):
+    """`hit`: [rows, heads] results that the poisoned row may reach (and, all together, does); the others are what
+    they were.  (Two sums in another order: bf16 results may round the other way, fp32 sums differ in the last bits.)"""
+    bad = ~np.isfinite(got).all(axis=-1)
+    assert not (bad & ~hit).any(), f"{name}: {int((bad & ~hit).sum())} rows out of reach are not finite"
+    assert bad[hit].any(), f"{name}: the poison reached nothing"
+    g, w = got[~hit].astype(np.float64), want[~hit].astype(np.float64)
+    assert np.abs(g - w).max() <= TOL[dtype]
+    assert np.linalg.norm(g - w) <= REL_RMS[dtype] * np.linalg.norm(w), name
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+@pytest.mark.parametrize("kind,head_dim,dtype,simt,size", CASES)
+def test_a_poisoned_row_reaches_what_contains_it_only(ba, oracle, kind, head_dim, dtype, simt, size, value):
+    p = problem(kind, head_dim, dtype, **size)
+    d = to_dev(p, W.make_tensors(p, seed=61, std=0.5))
+    plan = ba.Plan(p, impl=ba.IMPL_SIMT if simt else ba.IMPL_AUTO)
+    n, group = p.n_main, p.h_q // p.h_kv
+    vis = oracle.visibility(p)                          # [query row, key row]
+    o, lse = ba.branch_attn_fwd(plan, d["q_main"], d["q_branch"], d["k"], d["v"])
+
+    def backward(d, o):
+        g = ba.branch_attn_bwd(plan, d["q_main"], d["q_branch"], d["k"], d["v"], o, lse, d["d_o"])
+        return [np.concatenate([f32(g[0]), f32(g[1])]), f32(g[2]), f32(g[3])]
+
+    clean_o, clean = f32(o), backward(d, o)
+    q_head = np.arange(p.h_q) >= p.h_q - group          # query heads of the poisoned KV head
+    kv_head = np.arange(p.h_kv) >= p.h_kv - 1
+    last_q = np.arange(p.h_q) >= p.h_q - 1
+    none_q, none_k = np.zeros((p.rows, p.h_q), bool), np.zeros((p.rows, p.h_kv), bool)
+    # a key in the middle of a sequence, the first key of the next one, a branch key
+    for x in (int(p.cu_seqlens[1]) + 37, int(p.cu_seqlens[2]), n + 2 * (p.n_branch // 5)):
+        viewers = vis[:, x]
+        q_hit = viewers[:, None] & q_head
+        k_hit = (np.arange(p.rows) == x)[:, None] & kv_head
+        for name in ("k", "v"):
+            dd = poisoned(p, d, name, x, value)
+            po, pl = ba.branch_attn_fwd(plan, dd["q_main"], dd["q_branch"], dd["k"], dd["v"])
+            check(f"O, poisoned {name}[{x}]", f32(po), clean_o, q_hit, dtype)
+            assert torch.equal(pl[torch.from_numpy(~q_hit).cuda()], lse[torch.from_numpy(~q_hit).cuda()])
+            dq, dk, dv = backward(dd, o)
+            check(f"dQ, poisoned {name}[{x}]", dq, clean[0], q_hit, dtype)
+            check(f"dK, poisoned {name}[{x}]", dk, clean[1], k_hit, dtype)
+            if name == "k":
+                check(f"dV, poisoned k[{x}]", dv, clean[2], k_hit, dtype)
+    # a query row: late in a sequence, the last of one, a branch row
+    for r in (int(p.cu_seqlens[2]) - 20, int(p.cu_seqlens[1]) - 1, n + p.n_branch // 3):
+        q_hit = (np.arange(p.rows) == r)[:, None] & last_q
+        k_hit = vis[r][:, None] & kv_head
+        for name in ("q", "d_o"):
+            dq, dk, dv = backward(poisoned(p, d, name, r, value), o)
+            check(f"dQ, poisoned {name}[{r}]", dq, clean[0], q_hit, dtype)
+            check(f"dK, poisoned {name}[{r}]", dk, clean[1], k_hit, dtype)
+            check(f"dV, poisoned {name}[{r}]", dv, clean[2], k_hit, dtype)
+    plan.check()
