@@ -68,16 +68,6 @@ struct SimtArgs : RowArgs {
     int splits;                    // CTAs per tile (cluster size)
 };
 
-template <typename T> __device__ __forceinline__ float4 load4(const T *p);
-template <> __device__ __forceinline__ float4 load4<float>(const float *p) {
-    return *reinterpret_cast<const float4 *>(p);
-}
-template <> __device__ __forceinline__ float4 load4<__nv_bfloat16>(const __nv_bfloat16 *p) {
-    const uint2 raw = *reinterpret_cast<const uint2 *>(p);
-    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&raw.x));
-    const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&raw.y));
-    return make_float4(a.x, a.y, b.x, b.y);
-}
 template <typename T> __device__ __forceinline__ void store4(T *p, float4 x);
 template <> __device__ __forceinline__ void store4<float>(float *p, float4 x) {
     *reinterpret_cast<float4 *>(p) = x;
@@ -90,12 +80,14 @@ template <> __device__ __forceinline__ void store4<__nv_bfloat16>(__nv_bfloat16 
     *reinterpret_cast<uint2 *>(p) = r;
 }
 
-// NaN or opposite infinities among four results: their row is to be formed again, pair by pair (ba_exact.cuh)
+// NaN or opposite infinities among four results
 __device__ __forceinline__ bool not_finite(float4 x) {
     const float s = x.x + x.y + x.z + x.w;
     return s != s;
 }
-__device__ __forceinline__ float4 row4(const Cols<4> &c) { return make_float4(c.v[0], c.v[1], c.v[2], c.v[3]); }
+__device__ __forceinline__ uint64_t nan_bits(float4 x) {
+    return (x.x != x.x ? 1u : 0u) | (x.y != x.y ? 2u : 0u) | (x.z != x.z ? 4u : 0u) | (x.w != x.w ? 8u : 0u);
+}
 
 // four elements global -> shared as fp32 (zeros when !live): asynchronous for fp32 sources
 __device__ __forceinline__ void copy4(float *dst, const float *src, bool live) {
@@ -531,12 +523,12 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const __grid_constant
         auto out_row = [&]() -> int64_t {
             return a.partial_out ? is_main ? t - a.r.qm_begin : (a.r.qm_end - a.r.qm_begin) + (t - a.r.tok_begin) : gr;
         };
+        const bool live = live_row(r);
         float lse_a = -INFINITY;
         if (kMerges && a.partial_out == 2) {      // the lanes of a row (of one warp) read the old LSE before one replaces it
-            if (live_row(r)) lse_a = a.lse_out[out_row() * a.h_q + h0 + r % a.hp];
+            if (live) lse_a = a.lse_out[out_row() * a.h_q + h0 + r % a.hp];
             __syncwarp();
         }
-        if (!live_row(r)) continue;
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
         const uint32_t src0 = smem_u32(out0 + r * P + ch), src1 = smem_u32(out1 + r * P + ch), src_ml = smem_u32(&sm.ml[r]);
         if (MODE == kFwd) {
@@ -552,7 +544,9 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const __grid_constant
             }
             const float inv = l > 0.f ? 1.0f / l : 0.f;
             const int h = h0 + r % a.hp;
-            if (not_finite(x)) x = row4(exact_query_row<T, D, false, 4>(a, is_main, (int)t, h, -mx, ch));
+            if (__any_sync(0xffffffffu, live && not_finite(x)))      // does it hold what it does not see (ba_exact.cuh)?
+                x = repair_query4<T, D, false>(a, is_main, (int)t, h, g, -mx, ch, live ? nan_bits(x) : 0, x);
+            if (!live) continue;
             float lse_new = l > 0.f ? (mx + log2f(l)) * kLn2 : -INFINITY, w_new = inv, w_old = 0.f;
             if (kMerges && a.partial_out == 2) merge_weights(lse_a, lse_new, inv, lse_new, w_old, w_new);
             x.x *= w_new; x.y *= w_new; x.z *= w_new; x.w *= w_new;
@@ -574,11 +568,19 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const __grid_constant
                     y.x += u.x; y.y += u.y; y.z += u.z; y.w += u.w;
                 }
             }
-            if (MODE == kDq && not_finite(x))
-                x = row4(exact_query_row<T, D, true, 4>(a, is_main, (int)t, h0 + r % a.hp,
-                                                        a.nlse2_t[(h0 + r % a.hp) * a.row_pitch + gr], ch));
-            if (MODE == kDkdv && not_finite(x)) x = row4(exact_key_row<T, D, 4>(a, is_main, (int)t, g, false, ch));
-            if (MODE == kDkdv && not_finite(y)) y = row4(exact_key_row<T, D, 4>(a, is_main, (int)t, g, true, ch));
+            // do they hold rows out of their reach (ba_exact.cuh)?
+            if (MODE == kDq && __any_sync(0xffffffffu, live && not_finite(x))) {
+                const int h = h0 + r % a.hp;
+                const float nl = live ? a.nlse2_t[h * a.row_pitch + gr] : 0.f;
+                x = repair_query4<T, D, true>(a, is_main, (int)t, h, g, nl, ch, live ? nan_bits(x) : 0, x);
+            }
+            if (MODE == kDkdv) {
+                if (__any_sync(0xffffffffu, live && not_finite(x)))
+                    x = repair_key4<T, D>(a, is_main, (int)t, g, false, ch, live ? nan_bits(x) : 0, x);
+                if (__any_sync(0xffffffffu, live && not_finite(y)))
+                    y = repair_key4<T, D>(a, is_main, (int)t, g, true, ch, live ? nan_bits(y) : 0, y);
+            }
+            if (!live) continue;
             x.x *= a.scale; x.y *= a.scale; x.z *= a.scale; x.w *= a.scale;
             void *dst0 = MODE == kDkdv ? a.dk : is_main ? a.dq_main : a.dq_branch;
             const size_t off = MODE == kDkdv ? ((size_t)(is_main ? t - a.r.kv_base : gr) * a.h_kv + g) * D + ch : ((size_t)t * a.h_q + h0 + r % a.hp) * D + ch;

@@ -65,6 +65,9 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
 // wait would sit on the critical path of each producer/consumer handoff); the
 // limit is in SM cycles, about two seconds.
 constexpr long long kWaitLimitCycles = 4000000000ll;
+// Kernels whose warps may have to form result rows one by one (ba_exact.cuh) while the others wait: some
+// hundred cycles per pair, a second or two for a key with some million query rows.
+constexpr long long kSlowWaitLimitCycles = 30 * kWaitLimitCycles;
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag,
                                           long long limit_cycles = kWaitLimitCycles) {
     long long t0 = 0;
@@ -356,6 +359,27 @@ __device__ __forceinline__ float2 fmul2(float2 a, float2 b) {
         : "=l"(d)
         : "l"(*reinterpret_cast<const uint64_t *>(&a)), "l"(*reinterpret_cast<const uint64_t *>(&b)));
     return *reinterpret_cast<float2 *>(&d);
+}
+
+// bit e: element e is NaN
+__device__ __forceinline__ bool is_nan(float x) { return x != x; }
+__device__ __forceinline__ bool is_nan(uint32_t r) { return is_nan(__uint_as_float(r)); }
+template <typename R, int N> __device__ __forceinline__ uint64_t nan_mask(const R (&r)[N]) {
+    uint64_t m = 0;
+#pragma unroll
+    for (int e = 0; e < N; ++e) m |= is_nan(r[e]) ? 1ull << e : 0ull;
+    return m;
+}
+
+// sum of 32 registers as fp32 (four packed chains: it is asked only whether the sum is NaN)
+__device__ __forceinline__ float sum32(const uint32_t (&r)[32]) {
+    float2 s[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s[i] = make_float2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
+#pragma unroll
+    for (int e = 8; e < 32; e += 2) s[(e >> 1) & 3] = fadd2(s[(e >> 1) & 3], make_float2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])));
+    const float2 t = fadd2(fadd2(s[0], s[1]), fadd2(s[2], s[3]));
+    return t.x + t.y;
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {

@@ -784,7 +784,7 @@ template <int D, int MODE, bool SPLIT>
 __global__ void __launch_bounds__(kKvThreads, 1)
 tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constant__ CUtensorMap tm_q_branch,
              const __grid_constant__ CUtensorMap tm_go, const __grid_constant__ CUtensorMap tm_k,
-             const __grid_constant__ CUtensorMap tm_v, const TcBwdParams p) {
+             const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ TcBwdParams p) {
     using Smem = KvSmem<D>;
     constexpr bool kDq = MODE == kModeDq, kHL = D == 64;
     constexpr uint32_t kSubBytes = Smem::kSubBytes;
@@ -793,6 +793,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
     Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     volatile int *abort_flag = &sm.abort_flag;
+    constexpr long long kLimit = D == 64 ? kSlowWaitLimitCycles : kWaitLimitCycles;
     if (smem_u32(smem_raw) & 1023u) {   // the swizzled tiles need 1024-byte alignment
         if (tid == 0) atomicExch(p.status, BA_EUNSUPPORTED);
         return;
@@ -838,7 +839,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
             for (int n_item = 0, n_clc = 0;;) {
                 const int s = n_item & 1, cs = n_clc & 1;
                 bool ok = true;
-                if (n_item >= 2) ok = mbar_wait(&sm.item_empty[s], ((n_item >> 1) - 1) & 1, abort_flag);
+                if (n_item >= 2) ok = mbar_wait(&sm.item_empty[s], ((n_item >> 1) - 1) & 1, abort_flag, kLimit);
                 if (!__all_sync(0xffffffffu, ok)) break;
                 if (!more) {
                     if (lane == 0) {
@@ -861,7 +862,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                     }
                 } else {
                     if (lane == 0) mbar_arrive(&sm.item_full[s]);
-                    if (!SPLIT) ok = mbar_wait(&sm.loads_out, n_item & 1, abort_flag);
+                    if (!SPLIT) ok = mbar_wait(&sm.loads_out, n_item & 1, abort_flag, kLimit);
                     if (!__all_sync(0xffffffffu, ok)) break;
                     ++n_item;
                 }
@@ -873,7 +874,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                         mbar_expect_tx(&sm.clc_full[cs], 16);
                         clc_try_cancel(&sm.clc[cs], &sm.clc_full[cs]);
                     }
-                    ok = mbar_wait(&sm.clc_full[cs], (n_clc >> 1) & 1, abort_flag);
+                    ok = mbar_wait(&sm.clc_full[cs], (n_clc >> 1) & 1, abort_flag, kLimit);
                     if (!__all_sync(0xffffffffu, ok)) {
                         uint32_t spins = 0;      // leave no answer in flight
                         while (!mbar_try_wait(&sm.clc_full[cs], (n_clc >> 1) & 1) && ++spins < (1u << 22)) {}
@@ -890,7 +891,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
             uint32_t t = 0, n_st = 0;      // streamed tiles and stationary tiles loaded so far
             for (int n_item = 0; ok; ++n_item) {
                 const int sl = n_item & 1;
-                ok = __all_sync(0xffffffffu, mbar_wait(&sm.item_full[sl], (n_item >> 1) & 1, abort_flag));
+                ok = __all_sync(0xffffffffu, mbar_wait(&sm.item_full[sl], (n_item >> 1) & 1, abort_flag, kLimit));
                 if (!ok) break;
                 const KvItem it = sm.item[sl];
                 __syncwarp();
@@ -905,7 +906,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                     if (++ps == it.n_sub) { ps = 0; ++ph; }
                 for (int i = 0; i < it.n_iter; ++i, ++t) {
                     const int st = t % kQStages;
-                    if (t >= (uint32_t)kQStages) ok = mbar_wait(&sm.x_empty[st], ((t / kQStages) - 1) & 1, abort_flag);
+                    if (t >= (uint32_t)kQStages) ok = mbar_wait(&sm.x_empty[st], ((t / kQStages) - 1) & 1, abort_flag, kLimit);
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                     if (lane == 0 && i == max(it.n_iter - 1 - kKvFetchLead, 0)) mbar_arrive(&sm.loads_out);
@@ -963,7 +964,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                     }
                     if (i == 0) {
                         // the stationary pair, once the last S, dP of the item before have been formed
-                        if (n_st > 0) ok = mbar_wait(&sm.st_empty, (n_st - 1) & 1, abort_flag);
+                        if (n_st > 0) ok = mbar_wait(&sm.st_empty, (n_st - 1) & 1, abort_flag, kLimit);
                         ok = __all_sync(0xffffffffu, ok);
                         if (!ok) { ++t; break; }
                         if (lane == 0) {
@@ -1027,7 +1028,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                     x.first = false;
                     while (left == 0 && !done) {
                         const int sl = n_item & 1;
-                        ok = ok && mbar_wait(&sm.item_full[sl], (n_item >> 1) & 1, abort_flag);
+                        ok = ok && mbar_wait(&sm.item_full[sl], (n_item >> 1) & 1, abort_flag, kLimit);
                         if (!ok) { done = true; break; }
                         left = sm.item[sl].n_iter;
                         mbar_arrive(&sm.item_empty[sl]);
@@ -1042,7 +1043,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                 uint32_t n_st = 0, n_acc = 0;
                 auto issue_sd = [&](const Step &x, uint32_t t) {
                     const uint32_t km = xs_km0 + (t % kQStages) * kStageStep, xs = tmem + 256 + (t & 1) * 128;
-                    if (x.first) ok = mbar_wait(&sm.st_full, n_st++ & 1, abort_flag);
+                    if (x.first) ok = mbar_wait(&sm.st_full, n_st++ & 1, abort_flag, kLimit);
                     if (!ok) return;
                     tc_fence_after();
                     issue_t(xs, st1_km, km);                        // S
@@ -1052,21 +1053,21 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                 };
                 Step s0, s1, s2;
                 advance(s0);
-                if (s0.valid && ok && (ok = mbar_wait(&sm.x_full[0], 0, abort_flag))) issue_sd(s0, 0);
+                if (s0.valid && ok && (ok = mbar_wait(&sm.x_full[0], 0, abort_flag, kLimit))) issue_sd(s0, 0);
                 s1.valid = false;
                 if (s0.valid && ok) {
                     advance(s1);
-                    if (s1.valid && ok && (ok = mbar_wait(&sm.x_full[1], 0, abort_flag))) issue_sd(s1, 1);
+                    if (s1.valid && ok && (ok = mbar_wait(&sm.x_full[1], 0, abort_flag, kLimit))) issue_sd(s1, 1);
                 }
                 for (uint32_t t = 0; ok && s0.valid; ++t, s0 = s1, s1 = s2) {
                     const int b = t & 1;
                     const uint32_t stage_mn = xs_mn0 + (t % kQStages) * kStageStep, xs = tmem + 256 + b * 128;
                     s2.valid = false;
                     if (s1.valid) advance(s2);
-                    if (ok && s2.valid) ok = mbar_wait(&sm.x_full[(t + 2) % kQStages], ((t + 2) / kQStages) & 1, abort_flag);
+                    if (ok && s2.valid) ok = mbar_wait(&sm.x_full[(t + 2) % kQStages], ((t + 2) / kQStages) & 1, abort_flag, kLimit);
                     // the accumulators of the item before have been read out
-                    if (ok && s0.first && n_acc > 0) ok = mbar_wait(&sm.acc_free, (n_acc - 1) & 1, abort_flag);
-                    if (ok) ok = mbar_wait(&sm.pd_done[b], (t >> 1) & 1, abort_flag);
+                    if (ok && s0.first && n_acc > 0) ok = mbar_wait(&sm.acc_free, (n_acc - 1) & 1, abort_flag, kLimit);
+                    if (ok) ok = mbar_wait(&sm.pd_done[b], (t >> 1) & 1, abort_flag, kLimit);
                     if (!ok) break;
                     tc_fence_after();
                     if (!kDq) issue_acc(tmem + D, xs, stage_mn + kHalfStage, !s0.first);     // dV += P^T dO
@@ -1107,7 +1108,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
         } w, nx;
         auto fetch = [&](int n_item, Work &f) -> bool {
             const int sl = n_item & 1;
-            if (!mbar_wait(&sm.item_full[sl], (n_item >> 1) & 1, abort_flag)) return false;
+            if (!mbar_wait(&sm.item_full[sl], (n_item >> 1) & 1, abort_flag, kLimit)) return false;
             const KvItem &im = sm.item[sl];
             f.n_iter = im.n_iter; f.n_sub = im.n_sub; f.n_sub_main = im.n_sub_main; f.s_beg = im.s_beg; f.g = im.g;
             f.row0 = im.row0; f.row_end = im.row_end; f.srow = im.srow0 + r_in;
@@ -1165,7 +1166,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                 // --- which of the 64 streamed rows (columns) my row sees, or is seen by (needs only the
                 // stage's scalars, so it runs while the MMAs are still in flight)
                 if (!kDq) {
-                    ok = mbar_wait(&sm.x_full[st], (t / kQStages) & 1, abort_flag);
+                    ok = mbar_wait(&sm.x_full[st], (t / kQStages) & 1, abort_flag, kLimit);
                     if (!ok) break;
                 }
                 uint64_t vis = 0ull;
@@ -1188,7 +1189,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                     }
                 }
                 const bool masked = !__all_sync(0xffffffffu, vis == ~0ull);
-                ok = mbar_wait(&sm.sd_full[b], (t >> 1) & 1, abort_flag);
+                ok = mbar_wait(&sm.sd_full[b], (t >> 1) & 1, abort_flag, kLimit);
                 if (!ok) break;
                 tc_fence_after();
                 // --- P, dS 16 columns at a time, the next pair of loads in flight behind the math
@@ -1232,7 +1233,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
             // --- epilogue: dK/dV: warpgroup 0 takes dK (x scale), warpgroup 1 dV; dQ: half the columns each
             const bool any = w.n_iter > 0;
             if (any) {
-                if (!(ok = mbar_wait(&sm.acc_full, n_acc & 1, abort_flag))) break;
+                if (!(ok = mbar_wait(&sm.acc_full, n_acc & 1, abort_flag, kLimit))) break;
                 ++n_acc;
                 tc_fence_after();
             }
@@ -1259,6 +1260,13 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
 #pragma unroll
                     for (int e = 0; e < 32; ++e) r[e] = 0u;
                 }
+                bool not_finite = false;
+                uint64_t nans = 0;
+                if (D == 64 && !shared_tile) {
+                    const float s = sum32(r);
+                    not_finite = __any_sync(0xffffffffu, w.valid && s != s);
+                    if (not_finite && w.valid) nans = nan_mask(r);
+                }
                 if (shared_tile) {
 #pragma unroll
                     for (int e = 0; e < 8; ++e)      // 16-byte chunks swizzled by the row: no bank conflicts
@@ -1268,6 +1276,11 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                 } else if (w.valid) {
                     if (p.accumulate) store_grad_chunk<true>(dst, base + c * 32, r, mul);
                     else store_grad_chunk<false>(dst, base + c * 32, r, mul, p.wide);
+                }
+                if (D == 64 && not_finite) {      // does it hold rows out of its reach (ba_exact.cuh; bf16 results only)?
+                    __nv_bfloat16 *row = (__nv_bfloat16 *)dst + base + c * 32;
+                    if (kDq) repair_query_row<true, 8>(p.rows, w.is_main, w.row, w.h, w.g, w.nl, b * 32, 32, nans, mul, row);
+                    else repair_key_row<8>(p.rows, w.is_main, w.row, w.g, b == 1, c * 32, 32, nans, mul, row);
                 }
             }
             if (SPLIT) break;
@@ -1281,6 +1294,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
         if (warp < 8 && shared_tile && !*abort_flag) {
             const KvItem &it = sm.item[0];
             const int rows_mine = kTile / S;
+            float chk = 0.f;      // NaN: some result is
             for (int idx = tid; idx < 2 * rows_mine * (D / 4); idx += 256) {
                 const int ch = idx % (D / 4), rr = idx / (D / 4);
                 const int which = rr / rows_mine, r = rank * rows_mine + rr % rows_mine;    // dK / dV
@@ -1304,6 +1318,18 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                     *d4 = make_float4(o.x + x.x, o.y + x.y, o.z + x.z, o.w + x.w);
                 } else {
                     *reinterpret_cast<uint2 *>((__nv_bfloat16 *)dst + off) = make_uint2(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w));
+                }
+                if (D == 64) chk += x.x + x.y + x.z + x.w;
+            }
+            if (D == 64 && __any_sync(0xffffffffu, chk != chk)) {      // do they hold rows out of their reach (ba_exact.cuh; bf16 results only)?
+#pragma unroll 1
+                for (int idx = tid; idx < 2 * rows_mine * (D / 4); idx += 256) {
+                    const int ch = idx % (D / 4), rr = idx / (D / 4), which = rr / rows_mine, r = rank * rows_mine + rr % rows_mine;
+                    __nv_bfloat16 *row = (__nv_bfloat16 *)(which == 0 ? p.dk : p.dv) + ((size_t)(it.srow0 + r) * p.h_kv + it.g) * D + ch * 4;
+                    uint64_t nans = 0;
+                    if (it.row0 + r < it.row_end)
+                        for (int e = 0; e < 4; ++e) nans |= is_nan(__bfloat162float(row[e])) ? 1ull << e : 0ull;
+                    repair_key_row<4>(p.rows, true, it.row0 + r, it.g, which == 1, ch * 4, 4, nans, which == 0 ? p.scale : 1.0f, row);
                 }
             }
         }
@@ -1391,6 +1417,11 @@ int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
     p.has_main_q = q_main != nullptr;
     p.status = pl->dev_status;
     p.splits = 1;
+    p.rows.meta = pl->meta; p.rows.r = r;
+    p.rows.q_main = q_main; p.rows.q_branch = q_branch; p.rows.k = k; p.rows.v = v; p.rows.d_o = d_o;
+    p.rows.nlse2_t = p.nlse2_t; p.rows.delta_t = p.delta_t; p.rows.row_pitch = p.row_pitch;
+    p.rows.h_q = p.h_q; p.rows.h_kv = p.h_kv; p.rows.group = p.group;
+    p.rows.scale_log2 = p.scale_log2;
 
     // depth mode: key rows of depths <= depth only (later rows read as zero); Q, dO hold one row per branch
     p.depth = depth;

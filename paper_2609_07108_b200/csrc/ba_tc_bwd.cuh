@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include "ba_common.cuh"
+#include "ba_exact.cuh"
 #include "ba_sm100.cuh"
 #include "ba_tc_items.cuh"
 
@@ -43,6 +44,7 @@ struct TcBwdParams {
     // main rows: token (depth j + 1, branch b) is key row N + j * num_branches + b.
     int depth, num_branches, branch_len, branch_tiles_per_depth;
     int *status;
+    RowArgs rows;                     // head_dim 64: rows that are formed again one by one
 };
 
 // Branch tokens per branch key tile.  Branches of one length: a tile that starts and ends with a branch is seen

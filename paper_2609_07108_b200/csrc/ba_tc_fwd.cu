@@ -39,6 +39,7 @@
 #include <string.h>
 
 #include "ba_common.cuh"
+#include "ba_exact.cuh"
 #include "ba_sm100.cuh"
 #include "ba_tc_items.cuh"
 
@@ -84,6 +85,7 @@ struct TcFwdParams : ItemParams {
     int wide;                    // outputs are 32-byte aligned
     int warp_tok;                // > 0: a full warp of rows is this many tokens and leaves through a TMA store
     int *status;
+    RowArgs rows;                // head_dim 64: rows that are formed again one by one
 };
 
 
@@ -238,15 +240,18 @@ __device__ __forceinline__ void combine_parts(const TcFwdParams &p, FwdSmem<D> &
             }
         }
     }
-    if (!valid) return;
+    bool not_finite = false;
+    const uint64_t nans = D == 64 && valid ? nan_mask(acc) : 0;
+    if (D == 64) not_finite = __any_sync(0xffffffffu, nans != 0);
+    if (!valid && !not_finite) return;
     const float inv = sum > 0.f ? 1.0f / sum : 0.f;
     const float lse_p = sum > 0.f ? (mx + log2f(sum)) * kLn2 : -INFINITY;
     float lse_out = lse_p, w_new = inv, w_old = 0.f;
     if (p.partial_out == 2) merge_weights(lse_a, lse_p, inv, lse_out, w_old, w_new);
     const size_t base = ((size_t)orow * p.h_q + h) * D + part * kCols;
-    if (part == 0) p.lse[orow * p.h_q + h] = lse_out;
+    if (valid && part == 0) p.lse[orow * p.h_q + h] = lse_out;
 #pragma unroll
-    for (int e = 0; e < kVec; ++e) {
+    for (int e = 0; valid && e < kVec; ++e) {
         float4 v = make_float4(acc[4 * e] * w_new, acc[4 * e + 1] * w_new, acc[4 * e + 2] * w_new, acc[4 * e + 3] * w_new);
         if (p.partial_out == 0) {
             *reinterpret_cast<uint2 *>((__nv_bfloat16 *)p.o + base + 4 * e) = make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
@@ -259,6 +264,8 @@ __device__ __forceinline__ void combine_parts(const TcFwdParams &p, FwdSmem<D> &
             *dst = v;
         }
     }
+    if (D == 64 && not_finite)      // does O hold what the row does not see (ba_exact.cuh; bf16 results only)?
+        repair_query_row<false, kCols < 8 ? kCols : 8>(p.rows, it.is_main, my_row, h, it.g, -mx, part * kCols, kCols, nans, inv, (__nv_bfloat16 *)p.o + base);
 }
 
 template <int D, bool SPLIT>
@@ -266,7 +273,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constant__ CUtensorMap tm_q_branch,
               const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
               const __grid_constant__ CUtensorMap tm_k32, const __grid_constant__ CUtensorMap tm_v32,
-              const __grid_constant__ CUtensorMap tm_o, const TcFwdParams p) {
+              const __grid_constant__ CUtensorMap tm_o, const __grid_constant__ TcFwdParams p) {
     using Smem = FwdSmem<D>;
     constexpr int kStages = Smem::kStages;
     constexpr uint32_t kTileBytes = Smem::kTileBytes;
@@ -276,6 +283,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
     Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     volatile int *abort_flag = &sm.abort_flag;
+    constexpr long long kLimit = D == 64 ? kSlowWaitLimitCycles : kWaitLimitCycles;
     if (smem_u32(smem_raw) & 1023u) {   // the swizzled tiles need 1024-byte alignment
         if (tid == 0) atomicExch(p.status, BA_EUNSUPPORTED);
         return;
@@ -320,7 +328,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
             for (int n_item = 0, n_clc = 0;;) {
                 const int s = n_item & 1, cs = n_clc & 1;
                 bool ok = true;
-                if (n_item >= 2) ok = mbar_wait(&sm.item_empty[s], ((n_item >> 1) - 1) & 1, abort_flag);
+                if (n_item >= 2) ok = mbar_wait(&sm.item_empty[s], ((n_item >> 1) - 1) & 1, abort_flag, kLimit);
                 if (!__all_sync(0xffffffffu, ok)) break;
                 if (!more) {
                     if (lane == 0) {
@@ -335,7 +343,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
                     store_empty_item<D>(p, sm.item[s], lane);
                 } else {
                     if (lane == 0) mbar_arrive(&sm.item_full[s]);
-                    if (!SPLIT) ok = mbar_wait(&sm.loads_out, n_item & 1, abort_flag);
+                    if (!SPLIT) ok = mbar_wait(&sm.loads_out, n_item & 1, abort_flag, kLimit);
                     if (!__all_sync(0xffffffffu, ok)) break;
                     ++n_item;
                 }
@@ -350,7 +358,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
                         mbar_expect_tx(&sm.clc_full[cs], 16);
                         clc_try_cancel(&sm.clc[cs], &sm.clc_full[cs]);
                     }
-                    ok = mbar_wait(&sm.clc_full[cs], (n_clc >> 1) & 1, abort_flag);
+                    ok = mbar_wait(&sm.clc_full[cs], (n_clc >> 1) & 1, abort_flag, kLimit);
                     if (!__all_sync(0xffffffffu, ok)) {
                         uint32_t spins = 0;      // leave no answer in flight
                         while (!mbar_try_wait(&sm.clc_full[cs], (n_clc >> 1) & 1) && ++spins < (1u << 22)) {}
@@ -376,11 +384,11 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
                 bool ok = true;
                 for (int n = 0; ok; ++n) {
                     const int sl = n & 1;
-                    if (!mbar_wait(&sm.item_full[sl], (n >> 1) & 1, abort_flag)) break;
+                    if (!mbar_wait(&sm.item_full[sl], (n >> 1) & 1, abort_flag, kLimit)) break;
                     const Item &it = sm.item[sl];
                     if (it.T < 0) break;
                     if (it.je > it.jb) {
-                        if (nq > 0 && !(ok = mbar_wait(&sm.q_empty, (nq - 1) & 1, abort_flag))) break;
+                        if (nq > 0 && !(ok = mbar_wait(&sm.q_empty, (nq - 1) & 1, abort_flag, kLimit))) break;
                         ++nq;
                         const CUtensorMap *tq = it.is_main ? &tm_q_main : &tm_q_branch;
                         mbar_expect_tx(&sm.q_full, q_bytes * (it.live[0] + it.live[1]));
@@ -394,7 +402,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
                             if (j == max(it.je - 1 - kFetchLead, it.jb)) mbar_arrive(&sm.loads_out);
                             for (int kv = 0; kv < 2; ++kv, ++kvi) {
                                 const int s = kvi % kStages;
-                                if (kvi >= (uint32_t)kStages) ok = mbar_wait(&sm.kv_empty[s], ((kvi / kStages) - 1) & 1, abort_flag);
+                                if (kvi >= (uint32_t)kStages) ok = mbar_wait(&sm.kv_empty[s], ((kvi / kStages) - 1) & 1, abort_flag, kLimit);
                                 if (!ok) break;
                                 mbar_expect_tx(&sm.kv_full[s], (uint32_t)(nch * 32 * D * 2));
                                 if (j < it.n_full) {
@@ -471,7 +479,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
                     ++j_cur;
                     while (j_cur >= it.je && !done) {       // next item with keys
                         const int sl = n_item & 1;
-                        ok = ok && mbar_wait(&sm.item_full[sl], (n_item >> 1) & 1, abort_flag);
+                        ok = ok && mbar_wait(&sm.item_full[sl], (n_item >> 1) & 1, abort_flag, kLimit);
                         if (!ok) { done = true; break; }
                         const Item &im = sm.item[sl];
                         it.T = im.T; it.je = im.je; it.n_full = im.n_full; it.n_ch = im.n_ch;
@@ -494,7 +502,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
                 Step cur, nxt;
                 advance(cur);
                 if (ok && !done) {
-                    ok = mbar_wait(&sm.q_full, 0, abort_flag) && mbar_wait(&sm.kv_full[0], 0, abort_flag);
+                    ok = mbar_wait(&sm.q_full, 0, abort_flag, kLimit) && mbar_wait(&sm.kv_full[0], 0, abort_flag, kLimit);
                     nq = 1;
                     if (ok) {
                         tc_fence_after();
@@ -513,14 +521,14 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
                     // (its S was released by the P V issued before).
                     const bool early = SPLIT && more && !(nxt.live & cur.live);
                     if (early) {
-                        ok = ok && mbar_wait(&sm.kv_full[sk], ((kvi + 2) / kStages) & 1, abort_flag);
+                        ok = ok && mbar_wait(&sm.kv_full[sk], ((kvi + 2) / kStages) & 1, abort_flag, kLimit);
                         if (!ok) break;
                         tc_fence_after();
                         if (nxt.live & 1u) issue_qk(0, k_km, nxt.idesc);
                         if (nxt.live & 2u) issue_qk(1, k_km, nxt.idesc);
                         tc_commit(&sm.kv_empty[sk]);
                     }
-                    ok = ok && mbar_wait(&sm.kv_full[sv], ((kvi + 1) / kStages) & 1, abort_flag);
+                    ok = ok && mbar_wait(&sm.kv_full[sv], ((kvi + 1) / kStages) & 1, abort_flag, kLimit);
 #pragma unroll
                     for (int i = 0; i < 2; ++i) {
                         if (!ok) break;
@@ -528,20 +536,20 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
                         if (live) {
                             const bool acc = (started >> i) & 1u;
                             // O of the item before has been read out
-                            if (!acc && ((used_o >> i) & 1u) && !(ok = mbar_wait(&sm.o_free[i], ((par_o >> i) & 1u) ^ 1u, abort_flag))) break;
-                            if (!(ok = mbar_wait(&sm.p_half[i], (par_p >> i) & 1u, abort_flag))) break;
+                            if (!acc && ((used_o >> i) & 1u) && !(ok = mbar_wait(&sm.o_free[i], ((par_o >> i) & 1u) ^ 1u, abort_flag, kLimit))) break;
+                            if (!(ok = mbar_wait(&sm.p_half[i], (par_p >> i) & 1u, abort_flag, kLimit))) break;
                             tc_fence_after();
                             issue_pv(i, v_mn, 0, acc);          // keys 0-63 while the softmax warps finish keys 64-127
                             if (cur.nch > 1) issue_pv(i, v_mn, 2, true);
                             started |= 1u << i;
                         }
                         if (i == 0 && more && !early) {
-                            ok = mbar_wait(&sm.kv_full[sk], ((kvi + 2) / kStages) & 1, abort_flag);
-                            if (ok && nxt.first) ok = mbar_wait(&sm.q_full, nq & 1, abort_flag);
+                            ok = mbar_wait(&sm.kv_full[sk], ((kvi + 2) / kStages) & 1, abort_flag, kLimit);
+                            if (ok && nxt.first) ok = mbar_wait(&sm.q_full, nq & 1, abort_flag, kLimit);
                             if (!ok) break;
                         }
                         if (live) {
-                            if (!(ok = mbar_wait(&sm.p_full[i], (par_p >> i) & 1u, abort_flag))) break;
+                            if (!(ok = mbar_wait(&sm.p_full[i], (par_p >> i) & 1u, abort_flag, kLimit))) break;
                             par_p ^= 1u << i;
                             tc_fence_after();
                             if (cur.nch > 2) issue_pv(i, v_mn, 4, true);
@@ -587,14 +595,14 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
         // registers (a shared-memory load of these warps waits several hundred clocks behind the operand
         // reads of the Q K^T MMAs), and the next item is read while O of the current one is awaited.
         struct Work {
-            int T, jb, je, n_full, lo_min, n_mc, n_ch, bs, va, vb, wa, wb, rows, cnt, h, my_row;
+            int T, jb, je, n_full, lo_min, n_mc, n_ch, bs, va, vb, wa, wb, rows, cnt, h, g, my_row;
             bool is_main, valid;
             int lo, hi, br_start;
             uint64_t bmask;
         } w, nx;
         auto fetch = [&](int nit, Work &f) -> bool {
             const int sl = nit & 1;
-            if (!mbar_wait(&sm.item_full[sl], (nit >> 1) & 1, abort_flag)) return false;
+            if (!mbar_wait(&sm.item_full[sl], (nit >> 1) & 1, abort_flag, kLimit)) return false;
             const Item &im = sm.item[sl];
             f.T = im.T; f.je = im.je; f.n_full = im.n_full; f.lo_min = im.lo_min; f.n_mc = im.n_mc; f.n_ch = im.n_ch;
             f.bs = im.bs; f.va = im.va[i]; f.vb = im.vb[i]; f.wa = im.wa[i]; f.wb = im.wb[i];
@@ -603,6 +611,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
             f.is_main = im.is_main;
             const int off1 = tile1_off(p, f.is_main);
             f.h = im.h0 + my_head;
+            f.g = im.g;
             f.cnt = tile_tokens(p, f.is_main, i, f.rows);     // tokens of my query tile
             f.valid = my_tok < f.cnt && f.h < (im.g + 1) * p.group;
             f.my_row = im.row0 + my_tok + (i ? off1 : 0);
@@ -641,7 +650,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
                 if (j < n_full && (j < w.va || j >= w.vb)) continue;      // no row of this tile sees it
                 if (SPLIT && p.same_rows && (j & 1) != i) continue;
                 const int nch = j < n_full ? 4 : min(4, w.n_ch - 4 * (j - n_full));
-                ok = mbar_wait(&sm.s_full[i], n_s & 1, abort_flag);
+                ok = mbar_wait(&sm.s_full[i], n_s & 1, abort_flag, kLimit);
                 ++n_s;
                 if (!ok) break;
                 tc_fence_after();
@@ -735,7 +744,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
             if (!SPLIT && !(ok = fetch(nit + 1, nx))) break;
             // --- epilogue: O / l and LSE
             if (started) {
-                ok = mbar_wait(&sm.o_full[i], n_o & 1, abort_flag);
+                ok = mbar_wait(&sm.o_full[i], n_o & 1, abort_flag, kLimit);
                 ++n_o;
                 if (!ok) break;
                 tc_fence_after();
@@ -773,7 +782,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
             // A warp whose rows are all live hands 64 columns at a time to a TMA store: row by row from
             // registers, a warp instruction touches 32 cache lines and the stores of an item took 4,000
             // (32-byte) to 6,000 clocks (16-byte), as long as two key tiles; this way an epilogue takes 2,500.
-            const bool by_tma = p.warp_tok > 0 && ((warp & 3) + 1) * p.warp_tok <= w.cnt;
+            bool by_tma = p.warp_tok > 0 && ((warp & 3) + 1) * p.warp_tok <= w.cnt;
             const uint32_t stage = smem_u32(sm.out[warp]) + lane * 128;
 #pragma unroll 1
             for (int hf = 0; hf < D / 64; ++hf) {
@@ -789,6 +798,16 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
                 } else {
 #pragma unroll
                     for (int e = 0; e < 32; ++e) ra[e] = rb[e] = 0u;
+                }
+                bool not_finite = false;
+                uint64_t nans = 0;
+                if (D == 64) {
+                    const float s = sum32(ra) + sum32(rb);
+                    not_finite = __any_sync(0xffffffffu, w.valid && s != s);
+                    if (not_finite) {
+                        if (w.valid) nans = nan_mask(ra) | nan_mask(rb) << 32;
+                        by_tma = false;
+                    }
                 }
                 if (by_tma) {
                     if (lane == 0) tma_store_wait_read();
@@ -819,6 +838,8 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
                         store_row_chunk<false>(p.o, off + 32, rb, inv, p.wide);
                     }
                 }
+                if (D == 64 && not_finite)      // does O hold what the row does not see (ba_exact.cuh; bf16 results only)?
+                    repair_query_row<false, 8>(p.rows, w.is_main, w.my_row, w.h, w.g, neg_ms, 0, 64, nans, inv, (__nv_bfloat16 *)p.o + base);
             }
         }
         if (lane == 0) tma_store_wait_all();
@@ -908,6 +929,10 @@ int ba_tc_fwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
     p.partial_out = partial_out;   // 0 final layout, 1 compact fp32, 2 compact fp32 merged in place
     p.wide = ((uintptr_t)o & 31) == 0;
     p.status = pl->dev_status;
+    p.rows.meta = pl->meta; p.rows.r = r;
+    p.rows.q_main = q_main; p.rows.q_branch = q_branch; p.rows.k = k; p.rows.v = v;
+    p.rows.h_q = pr.h_q; p.rows.h_kv = pr.h_kv; p.rows.group = pr.h_q / pr.h_kv;
+    p.rows.scale_log2 = p.scale_log2;
     // Few items and long key ranges (a handful of branches on long sequences): split the keys of an item over a
     // cluster until the SMs are busy, as long as a part keeps at least four tiles.  With branches of different
     // sequences in the two query tiles (same_rows), an item per sequence's rows and both tiles on them, unless two

@@ -1,5 +1,6 @@
 """A NaN or an infinity in one row reaches only the results whose definition contains that row: the plain-FMA
-kernels leave every other row as it is.  What a row may reach follows from the oracle's visibility matrix alone."""
+kernels (fp32, any shape) and the head_dim 64 tensor-core kernels leave every other row as it is.  What a row may
+reach follows from the oracle's visibility matrix alone."""
 import numpy as np
 import pytest
 import torch
@@ -32,7 +33,8 @@ def problem(kind, head_dim, dtype, lens, anchors, blen, h_q=4, h_kv=2):
 SMALL = dict(lens=[70, 131, 300], anchors=list(range(0, 501, 9)), blen=5)
 LARGE = dict(lens=[1500, 333, 2200], anchors=list(range(0, 4033, 5)), blen=3, h_q=8, h_kv=8)
 CASES = [(W.CHAIN, 64, "fp32", False, SMALL), (W.TREE, 128, "fp32", False, SMALL), (W.BLOCK, 64, "fp32", False, LARGE),
-         (W.CHAIN, 64, "bf16", True, SMALL), (W.BLOCK, 128, "bf16", True, SMALL)]
+         (W.TREE, 64, "bf16", False, SMALL), (W.CHAIN, 64, "bf16", False, LARGE), (W.CHAIN, 64, "bf16", True, SMALL),
+         (W.BLOCK, 128, "bf16", True, SMALL)]
 
 
 def poisoned(p, d, name, row, value):
