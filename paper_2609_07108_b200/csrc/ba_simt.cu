@@ -328,16 +328,17 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const __grid_constant
                 sm.mask[tid] = live && !x.main ? a.meta.br_mask[row] : 0ull;
             }
         } else {
+            const int row0 = (int)((x.main ? -a.r.kv_base : n) + x.r0);      // in the key tensors
             load_rows<T, D, kBN>(dst, (const T *)a.k,
-                            [&](int r) -> int64_t { return r < x.cnt ? (((x.main ? -a.r.kv_base : n) + x.r0 + r) * a.h_kv + g) * D : -1; });
+                            [&](int r) -> int64_t { return r < x.cnt ? ((int64_t)(row0 + r) * a.h_kv + g) * D : -1; });
         }
     };
     auto load_x2 = [&](int t) {
         if (t >= t_end) return;
         const Tile x = tile_of(t);
-        const int64_t heads = MODE == kDkdv ? a.h_q : a.h_kv, row0 = !x.main ? n : MODE == kDkdv ? 0 : -a.r.kv_base;
+        const int heads = MODE == kDkdv ? a.h_q : a.h_kv, row0 = (int)((!x.main ? n : MODE == kDkdv ? 0 : -a.r.kv_base) + x.r0);
         load_rows<T, D, kBN>(sm.x2, MODE == kDkdv ? (const T *)a.d_o : (const T *)a.v,
-                        [&](int r) -> int64_t { return r < x.cnt ? ((row0 + x.r0 + r) * heads + x.h) * D : -1; });
+                        [&](int r) -> int64_t { return r < x.cnt ? ((int64_t)(row0 + r) * heads + x.h) * D : -1; });
     };
 
     // ---- per-thread views: score lanes hold rows 2 rg + i and columns cg + 8 j of the warp's WR x 32 tile,
