@@ -784,7 +784,8 @@ template <int D, int MODE, bool SPLIT>
 __global__ void __launch_bounds__(kKvThreads, 1)
 tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constant__ CUtensorMap tm_q_branch,
              const __grid_constant__ CUtensorMap tm_go, const __grid_constant__ CUtensorMap tm_k,
-             const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ TcBwdParams p) {
+             const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_go_branch,
+             const __grid_constant__ TcBwdParams p) {
     using Smem = KvSmem<D>;
     constexpr bool kDq = MODE == kModeDq, kHL = D == 64;
     constexpr uint32_t kSubBytes = Smem::kSubBytes;
@@ -926,11 +927,12 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                         const int h = it.g * p.group + hh;
                         const int gr0 = seg_main ? r0 : qbase + r0;
                         if (lane == 0) {
-                            const CUtensorMap *tq = seg_main ? &tm_q_main : &tm_q_branch;
+                            // (a branch tile may start up to three rows before branch row 0: no rows of these maps)
+                            const CUtensorMap *tq = seg_main ? &tm_q_main : &tm_q_branch, *tg = seg_main ? &tm_go : &tm_go_branch;
                             mbar_expect_tx(&sm.x_full[st], 2 * kSubBytes + 2 * kSub * 4);
                             for (int half = 0; half < kHalves; ++half) {
                                 tma_load_3d(sm.xs[st] + half * 8192, tq, half * 64, h, r0, &sm.x_full[st]);
-                                tma_load_3d(sm.xs[st] + kSubBytes + half * 8192, &tm_go, half * 64, h, gr0, &sm.x_full[st]);
+                                tma_load_3d(sm.xs[st] + kSubBytes + half * 8192, tg, half * 64, h, r0, &sm.x_full[st]);
                             }
                             const size_t off = (size_t)h * p.row_pitch + gr0;
                             bulk_load(mt.neg_lse2, p.nlse2_t + off, kSub * 4, &sm.x_full[st]);
@@ -940,10 +942,10 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                                 const bool main2 = ps < it.n_sub_main;
                                 const int r2 = main2 ? it.ma + ps * kSub : it.ba + (ps - it.n_sub_main) * kSub;
                                 const int g2 = main2 ? r2 : qbase + r2;
-                                const CUtensorMap *tq2 = main2 ? &tm_q_main : &tm_q_branch;
+                                const CUtensorMap *tq2 = main2 ? &tm_q_main : &tm_q_branch, *tg2 = main2 ? &tm_go : &tm_go_branch;
                                 for (int half = 0; half < kHalves; ++half) {
                                     tma_prefetch_3d(tq2, half * 64, h2, r2);
-                                    tma_prefetch_3d(&tm_go, half * 64, h2, g2);
+                                    tma_prefetch_3d(tg2, half * 64, h2, r2);
                                 }
                                 const size_t off2 = (size_t)h2 * p.row_pitch + g2;
                                 bulk_prefetch(p.nlse2_t + off2, kSub * 4);
@@ -1376,7 +1378,7 @@ int launch_kv_as(const TcBwdParams &p, const CUtensorMap *tm, int64_t grid, bool
         ++cfg.numAttrs;
     }
     cfg.attrs = attr;
-    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_kv_kernel<D, MODE, SPLIT>, tm[0], tm[1], tm[2], tm[3], tm[4], p));
+    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_kv_kernel<D, MODE, SPLIT>, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], p));
     return ba_check_launch();
 }
 
@@ -1437,13 +1439,19 @@ int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
     const uint64_t qm_rows = depth ? (uint64_t)pr.num_branches : q_main ? (uint64_t)pr.n_main : (uint64_t)pr.n_branch;
     const uint64_t qb_rows = depth ? (uint64_t)pr.num_branches
                              : (q_branch && pr.n_branch > 0) ? (uint64_t)pr.n_branch : (uint64_t)pr.n_main;
-    // maps in the order q_main, q_branch, dO, K, V; boxes of `qr` query rows x `qh` heads and `kr` key rows
+    // dO of the branch rows alone: whatever lies in front of branch row 0 (rows of dO that a call without main
+    // queries leaves unset) is not loaded
+    const bool go_split = !depth && pr.n_branch > 0;
+    const void *gob = go_split ? (const char *)d_o + (size_t)pr.n_main * pr.h_q * D * 2 : d_o;
+    const uint64_t gob_rows = go_split ? (uint64_t)pr.n_branch : go_rows;
+    // maps in the order q_main, q_branch, dO, K, V, branch rows of dO; boxes of `qr` query rows x `qh` heads and
+    // `kr` key rows
     auto maps = [&](CUtensorMap *tm, uint32_t qr, uint32_t qh, uint32_t kr) {
         return make_tmap_rhd(&tm[0], qm, qm_rows, pr.h_q, D, qr, qh) && make_tmap_rhd(&tm[1], qb, qb_rows, pr.h_q, D, qr, qh) &&
                make_tmap_rhd(&tm[2], d_o, go_rows, pr.h_q, D, qr, qh) && make_tmap_rhd(&tm[3], k, kv_rows, pr.h_kv, D, kr) &&
-               make_tmap_rhd(&tm[4], v, kv_rows, pr.h_kv, D, kr);
+               make_tmap_rhd(&tm[4], v, kv_rows, pr.h_kv, D, kr) && make_tmap_rhd(&tm[5], gob, gob_rows, pr.h_q, D, qr, qh);
     };
-    CUtensorMap tm[5];
+    CUtensorMap tm[6];
     const int64_t qm_n = q_main ? r.qm_end - r.qm_begin : 0, br_n = r.tok_end - r.tok_begin;
     if (stages & BA_STAGE_DQ) {
         if (D == 64) {

@@ -155,7 +155,7 @@ template <bool SPLIT>
 __global__ void __launch_bounds__(kFusedThreads, 1)
 tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constant__ CUtensorMap tm_q_branch,
                     const __grid_constant__ CUtensorMap tm_go, const __grid_constant__ CUtensorMap tm_k,
-                    const __grid_constant__ CUtensorMap tm_v, const TcBwdParams p) {
+                    const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_go_branch, const TcBwdParams p) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     FusedSmem &sm = *reinterpret_cast<FusedSmem *>(smem_raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -287,11 +287,12 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_
                 const bool seg_main = u < n_sub_main;
                 const int64_t r0 = seg_main ? ma + (int64_t)u * kTile : ba + (int64_t)(u - n_sub_main) * kTile;
                 const int64_t grow0 = seg_main ? r0 : n + r0;
-                const CUtensorMap *tq = seg_main ? &tm_q_main : &tm_q_branch;
+                // (a branch tile may start up to three rows before branch row 0: no rows of these maps)
+                const CUtensorMap *tq = seg_main ? &tm_q_main : &tm_q_branch, *tg = seg_main ? &tm_go : &tm_go_branch;
                 mbar_expect_tx(&sm.q_full[st], 2 * kTileBytes + 2 * kTile * 4);
                 for (int half = 0; half < 2; ++half) {
                     tma_load_3d(sm.q[st] + half * 16384, tq, half * 64, h, (int)r0, &sm.q_full[st]);
-                    tma_load_3d(sm.go[st] + half * 16384, &tm_go, half * 64, h, (int)grow0, &sm.q_full[st]);
+                    tma_load_3d(sm.go[st] + half * 16384, tg, half * 64, h, (int)r0, &sm.q_full[st]);
                 }
                 const size_t off = (size_t)h * p.row_pitch + grow0;
                 bulk_load(sm.neg_lse2[st], p.nlse2_t + off, kTile * 4, &sm.q_full[st]);
@@ -303,10 +304,10 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_
                     const bool main2 = u2 < n_sub_main;
                     const int64_t r2 = main2 ? ma + (int64_t)u2 * kTile : ba + (int64_t)(u2 - n_sub_main) * kTile;
                     const int64_t g2 = main2 ? r2 : n + r2;
-                    const CUtensorMap *tq2 = main2 ? &tm_q_main : &tm_q_branch;
+                    const CUtensorMap *tq2 = main2 ? &tm_q_main : &tm_q_branch, *tg2 = main2 ? &tm_go : &tm_go_branch;
                     for (int half = 0; half < 2; ++half) {
                         tma_prefetch_3d(tq2, half * 64, h2, (int)r2);
-                        tma_prefetch_3d(&tm_go, half * 64, h2, (int)g2);
+                        tma_prefetch_3d(tg2, half * 64, h2, (int)r2);
                     }
                     const size_t off2 = (size_t)h2 * p.row_pitch + g2;
                     bulk_prefetch(p.nlse2_t + off2, kTile * 4);
@@ -688,7 +689,7 @@ int ba_tc_bwd_fused(const ba_plan *pl, const BaRange &r, const void *q_main, con
         }
     p.total_key_tiles = (int)(kmt + (kbt + p.splits - 1) / p.splits);    // work items (clusters) per KV head
 
-    CUtensorMap tq_main, tq_branch, tgo, tk, tv;
+    CUtensorMap tq_main, tq_branch, tgo, tgo_branch, tk, tv;
     const uint64_t all_rows = (uint64_t)(pr.n_main + pr.n_branch);
     // without own-branch keys nothing beyond kv_end is needed (a received shard ends there)
     const uint64_t kv_rows = (r.parts & BA_PART_BRANCH) ? all_rows : (uint64_t)(r.kv_end > r.kv_base ? r.kv_end - r.kv_base : 1);
@@ -698,7 +699,10 @@ int ba_tc_bwd_fused(const ba_plan *pl, const BaRange &r, const void *q_main, con
     const uint64_t qb_rows = (q_branch && pr.n_branch > 0) ? (uint64_t)pr.n_branch : (uint64_t)pr.n_main;
     if (!make_tmap_rhd(&tk, k, kv_rows, pr.h_kv, 128, kTile) || !make_tmap_rhd(&tv, v, kv_rows, pr.h_kv, 128, kTile) ||
         !make_tmap_rhd(&tgo, d_o, all_rows, pr.h_q, 128, kTile) || !make_tmap_rhd(&tq_main, qm, qm_rows, pr.h_q, 128, kTile) ||
-        !make_tmap_rhd(&tq_branch, qb, qb_rows, pr.h_q, 128, kTile))
+        !make_tmap_rhd(&tq_branch, qb, qb_rows, pr.h_q, 128, kTile) ||
+        // dO of the branch rows alone: what lies in front of branch row 0 is not loaded
+        !make_tmap_rhd(&tgo_branch, (const char *)d_o + (pr.n_branch > 0 ? (size_t)pr.n_main * pr.h_q * 256 : 0),
+                       pr.n_branch > 0 ? (uint64_t)pr.n_branch : all_rows, pr.h_q, 128, kTile))
         return BA_EINVAL;
     const int64_t grid = (int64_t)p.total_key_tiles * pr.h_kv * p.splits;
     if (grid > INT_MAX) return BA_EUNSUPPORTED;
@@ -715,6 +719,6 @@ int ba_tc_bwd_fused(const ba_plan *pl, const BaRange &r, const void *q_main, con
     cfg.attrs = &attr;
     cfg.numAttrs = p.splits > 1 ? 1 : 0;
     auto kernel = p.splits > 1 ? &tc_bwd_fused_kernel<true> : &tc_bwd_fused_kernel<false>;
-    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kernel, tq_main, tq_branch, tgo, tk, tv, p));
+    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kernel, tq_main, tq_branch, tgo, tk, tv, tgo_branch, p));
     return ba_check_launch();
 }

@@ -32,9 +32,10 @@ def problem(kind, head_dim, dtype, lens, anchors, blen, h_q=4, h_kv=2):
 # middle of 32-, 64- and 128-row tiles; few rows (tiles shared by clusters) and enough rows to leave tiles whole
 SMALL = dict(lens=[70, 131, 300], anchors=list(range(0, 501, 9)), blen=5)
 LARGE = dict(lens=[1500, 333, 2200], anchors=list(range(0, 4033, 5)), blen=3, h_q=8, h_kv=8)
+SHARED = dict(lens=[40, 600, 5], anchors=list(range(645)), blen=3, h_q=8, h_kv=1)     # dK/dV in clusters of four
 CASES = [(W.CHAIN, 64, "fp32", False, SMALL), (W.TREE, 128, "fp32", False, SMALL), (W.BLOCK, 64, "fp32", False, LARGE),
          (W.TREE, 64, "bf16", False, SMALL), (W.CHAIN, 64, "bf16", False, LARGE), (W.CHAIN, 64, "bf16", True, SMALL),
-         (W.BLOCK, 128, "bf16", True, SMALL)]
+         (W.CHAIN, 64, "bf16", False, SHARED), (W.BLOCK, 128, "bf16", True, SMALL)]
 
 
 def poisoned(p, d, name, row, value):
@@ -103,3 +104,21 @@ def test_a_poisoned_row_reaches_what_contains_it_only(ba, oracle, kind, head_dim
             check(f"dK, poisoned {name}[{r}]", dk, clean[1], k_hit, dtype)
             check(f"dV, poisoned {name}[{r}]", dv, clean[2], k_hit, dtype)
     plan.check()
+
+
+@pytest.mark.parametrize("head_dim,dtype,stages", [(64, "fp32", 7), (64, "bf16", 7), (128, "bf16", 7), (128, "bf16", 9)])
+@pytest.mark.parametrize("lens", [[130, 91], [130, 92], [3, 222, 66]])     # N = 221, 222, 291
+def test_a_call_without_main_queries_reads_no_main_row_of_d_o(ba, head_dim, dtype, stages, lens):
+    p = problem(W.CHAIN, head_dim, dtype, lens, list(range(sum(lens))), 4)
+    d = to_dev(p, W.make_tensors(p, seed=63, std=0.5))
+    plan, n = ba.Plan(p), p.n_main
+    o, lse = ba.branch_attn_fwd(plan, d["q_main"], d["q_branch"], d["k"], d["v"])
+    results = []
+    for fill in (0.0, float("nan")):
+        d["d_o"][:n] = fill
+        g = ba.branch_attn_bwd(plan, None, d["q_branch"], d["k"], d["v"], o, lse, d["d_o"], stages=stages)
+        results.append([f32(x) for x in g[1:]])
+    plan.check()
+    for name, a, b in zip(("dQ", "dK", "dV"), *results):
+        assert np.isfinite(b).all(), name
+        assert np.abs(a - b).max() <= (1e-3 * np.abs(a).max() if stages == 9 else 0.0), name    # (atomic adds, rounded to bf16)
