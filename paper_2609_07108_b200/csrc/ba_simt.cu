@@ -537,7 +537,7 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const __grid_constant
             for (int s = 0; s < a.splits; ++s) mx = fmaxf(mx, cluster_ld_f2(cluster_map(src_ml, s)).x);
             for (int s = 0; s < a.splits; ++s) {
                 const float2 ml = cluster_ld_f2(cluster_map(src_ml, s));
-                if (ml.x == -INFINITY) continue;
+                if (ml.y == 0.f) continue;      // sees nothing (a sum that is NaN is not an empty part)
                 const float w = exp2f(ml.x - mx);
                 const float4 v = cluster_ld_f4(cluster_map(src0, s));
                 l += w * ml.y;

@@ -244,7 +244,7 @@ __device__ __forceinline__ void combine_parts(const TcFwdParams &p, FwdSmem<D> &
     const uint64_t nans = D == 64 && valid ? nan_mask(acc) : 0;
     if (D == 64) not_finite = __any_sync(0xffffffffu, nans != 0);
     if (!valid && !not_finite) return;
-    const float inv = sum > 0.f ? 1.0f / sum : 0.f;
+    const float inv = sum > 0.f ? 1.0f / sum : sum;      // 0, or NaN although the part that is NaN may weigh nothing
     const float lse_p = sum > 0.f ? (mx + log2f(sum)) * kLn2 : -INFINITY;
     float lse_out = lse_p, w_new = inv, w_old = 0.f;
     if (p.partial_out == 2) merge_weights(lse_a, lse_p, inv, lse_out, w_old, w_new);
@@ -752,7 +752,9 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
             if (SPLIT) {
                 // unnormalised O and (max, sum) of my part into shared memory (o_full covers every MMA of
                 // this CTA, so the K / V stages are idle)
-                sm.ml(i)[r_in] = make_float2(started && l_run > 0.f ? m_run * sl2 : -INFINITY, started ? l_run : 0.f);
+                // (a sum that is NaN is not an empty part; its maximum may be none)
+                const bool any = started && l_run != 0.f;
+                sm.ml(i)[r_in] = make_float2(any ? (m_run == -INFINITY ? 0.f : m_run * sl2) : -INFINITY, any ? l_run : 0.f);
                 if (started) {
                     float4 *dst = reinterpret_cast<float4 *>(sm.kv[0]) + (size_t)(i * kTile + r_in) * (D / 4);
 #pragma unroll

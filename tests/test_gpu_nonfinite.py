@@ -106,6 +106,42 @@ def test_a_poisoned_row_reaches_what_contains_it_only(ba, oracle, kind, head_dim
     plan.check()
 
 
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+@pytest.mark.parametrize("head_dim,dtype", [(64, "bf16"), (128, "bf16"), (64, "fp32")])
+def test_a_poisoned_key_of_few_rows_on_long_sequences(ba, oracle, head_dim, dtype, value):
+    """Draft rows only: the keys of an item are split over a cluster, both query tiles hold one sequence's rows.  Rows
+    that see the poison are not finite, whichever part it is in (head_dim 128: others may be, see branch_attn.h)."""
+    p = problem(W.TREE, head_dim, dtype, [2100, 1900], [1800, 2099, 3999], 6)
+    d = to_dev(p, W.make_tensors(p, seed=62, std=0.5))
+    plan, n, q_head = ba.Plan(p), p.n_main, np.arange(p.h_q) >= p.h_q // 2
+    vis = oracle.visibility(p)[n:]
+    o, _ = ba.branch_attn_fwd(plan, None, d["q_branch"], d["k"], d["v"])
+    for x in (7, 1900, 2050, 2099, 2101, n + 8):
+        for name in ("k", "v"):
+            dd = poisoned(p, d, name, x, value)
+            po, _ = ba.branch_attn_fwd(plan, None, dd["q_branch"], dd["k"], dd["v"])
+            hit = vis[:, x][:, None] & q_head
+            if name == "v" or np.isnan(value):      # (an infinite key may also make a score of -inf)
+                assert not np.isfinite(f32(po)[n:][hit]).all(axis=-1).any(), f"poisoned {name}[{x}] is lost"
+            if head_dim == 64:
+                check(f"O, poisoned {name}[{x}]", f32(po)[n:], f32(o)[n:], hit, dtype)
+    plan.check()
+
+
+
+@pytest.mark.parametrize("head_dim,dtype,simt", [(64, "fp32", False), (128, "fp32", False), (64, "bf16", True), (64, "bf16", False), (128, "bf16", False)])
+def test_rows_that_see_nan_alone_are_nan(ba, head_dim, dtype, simt):
+    """Every key of one KV head is NaN: no score of its rows is a maximum.  O is NaN, not an empty row's zero."""
+    p = problem(W.CHAIN, head_dim, dtype, [90, 1], [0, 60, 90], 3)
+    d = to_dev(p, W.make_tensors(p, seed=64, std=0.5))
+    d["k"][:, -1] = float("nan")
+    plan = ba.Plan(p, impl=ba.IMPL_SIMT if simt else ba.IMPL_AUTO)
+    o, _ = ba.branch_attn_fwd(plan, d["q_main"], d["q_branch"], d["k"], d["v"])
+    plan.check()
+    half = p.h_q // 2
+    assert np.isnan(f32(o)[:, half:]).all() and np.isfinite(f32(o)[:, :half]).all()
+
+
 @pytest.mark.parametrize("head_dim,dtype,stages", [(64, "fp32", 7), (64, "bf16", 7), (128, "bf16", 7), (128, "bf16", 9)])
 @pytest.mark.parametrize("lens", [[130, 91], [130, 92], [3, 222, 66]])     # N = 221, 222, 291
 def test_a_call_without_main_queries_reads_no_main_row_of_d_o(ba, head_dim, dtype, stages, lens):
