@@ -112,10 +112,17 @@ int ba_plan_destroy(ba_plan_t *plan);
  * device arrays are read by one kernel on `stream`, after the copies that the caller
  * queued there.  Nothing is synchronised, so a caller that builds a plan per step keeps
  * the GPU busy.  The device arrays must hold the host values and stay alive until the
- * work queued on `stream` has run.
+ * work queued on `stream` has run; calls on another stream must wait for that work.  Not
+ * while `stream` is capturing (BA_EINVAL): the plan would not exist before a replay.
  */
 int ba_plan_create_host(const ba_problem_t *host, const ba_problem_t *dev, void *plan_mem,
                         size_t plan_bytes, void *stream, ba_plan_t **out);
+
+/* Blocks the host until `event` (a cudaEvent_t recorded outside any capture) has completed; also
+ * allowed while this thread captures a stream.  A stream under capture cannot be made to wait for
+ * work outside the capture, such as the kernel of ba_plan_create_host on another stream: record an
+ * event behind it and call this before (or during) the capture of calls that use the plan. */
+int ba_host_wait(void *event);
 
 /* Scratch bytes (device, 256-byte aligned) that `op` needs; may be 0.
  * BA_OP_BWD_FUSED = BA_OP_BWD plus an fp32 dQ accumulator of (N + M) * h_q * head_dim

@@ -46,7 +46,7 @@ class _Problem(C.Structure):
 
 _LIB = None
 EXPORTS = ("ba_status_string", "ba_last_cuda_error", "ba_plan_bytes", "ba_plan_create", "ba_plan_create_host",
-           "ba_plan_destroy", "ba_workspace_bytes", "ba_plan_pairs", "ba_plan_impl", "ba_plan_check", "branch_attn_fwd",
+           "ba_plan_destroy", "ba_host_wait", "ba_workspace_bytes", "ba_plan_pairs", "ba_plan_impl", "ba_plan_check", "branch_attn_fwd",
            "branch_attn_fwd_partial", "branch_attn_fwd_partial_merge", "lse_merge", "branch_attn_bwd", "branch_attn_bwd_stages",
            "branch_attn_bwd_static", "ba_finalize_grads", "ba_selftest_bounded_wait",
            "branch_attn_fwd_depth", "branch_attn_bwd_depth", "branch_attn_fwd_shard", "branch_attn_bwd_shard")
@@ -74,6 +74,8 @@ def _lib():
                                             C.c_void_p, C.POINTER(C.c_void_p)]
         lib.ba_plan_destroy.restype = C.c_int
         lib.ba_plan_destroy.argtypes = [C.c_void_p]
+        lib.ba_host_wait.restype = C.c_int
+        lib.ba_host_wait.argtypes = [C.c_void_p]
         lib.ba_workspace_bytes.restype = C.c_size_t
         lib.ba_workspace_bytes.argtypes = [C.c_void_p, C.c_int]
         lib.ba_plan_pairs.restype = C.c_int64
@@ -154,13 +156,14 @@ def _stream():
 
 def _plan_stream(plan):
     """The current stream, made to wait for the plan's metadata if it was built on another one.
-    (A stream under capture cannot wait for work outside the capture; capture starts synchronised.)"""
+    (Without an event query: it would end a capture that another thread has begun.)"""
     st = torch.cuda.current_stream()
-    if plan._ready is not None and st.cuda_stream != plan._built_on and not torch.cuda.is_current_stream_capturing():
-        if plan._ready.query():
-            plan._ready = None
+    if plan._ready is not None and st.cuda_stream not in plan._ordered:
+        if torch.cuda.is_current_stream_capturing():
+            plan.wait()          # inside a capture no stream can wait for work outside it
         else:
             st.wait_event(plan._ready)
+            plan._ordered.add(st.cuda_stream)
     return C.c_void_p(st.cuda_stream)
 
 
@@ -179,11 +182,15 @@ class Plan:
     `problem` is a `workloads.Problem` (host numpy metadata); the arrays are
     validated on the host, copied to the device in one piece and expanded there.
     Nothing waits for the GPU: the copy is queued from pinned memory on the current
-    stream, behind whatever runs there.
+    stream, behind whatever runs there.  Calls on other streams wait for it by
+    themselves; a call that is captured into a graph makes the host wait (`wait()`
+    does that ahead of time).  A plan cannot be built while the stream is capturing.
     """
 
     def __init__(self, problem, device="cuda", impl=IMPL_AUTO):
         lib = _lib()
+        if torch.cuda.is_current_stream_capturing():
+            raise RuntimeError("ba_plan_create: the stream is capturing (build the plan before the capture)")
         self.problem = problem
         self.device = torch.device(device)
         if self.device.type == "cuda" and self.device.index is None:
@@ -218,7 +225,7 @@ class Plan:
             st = torch.cuda.current_stream()
             rc = lib.ba_plan_create_host(C.byref(host), C.byref(self.c), _p(self._mem), nbytes,
                                          C.c_void_p(st.cuda_stream), C.byref(handle))
-            self._built_on, self._ready = st.cuda_stream, torch.cuda.Event()
+            self._ready, self._ordered = torch.cuda.Event(), {st.cuda_stream}    # streams whose work comes after the plan
             self._ready.record(st)
         _check(rc, "ba_plan_create")
         self.handle = handle
@@ -231,6 +238,12 @@ class Plan:
             n = _lib().ba_workspace_bytes(self.handle, op)
             self._ws[op] = torch.empty(max(n, 256), dtype=torch.uint8, device=self.device)
         return self._ws[op]
+
+    def wait(self):
+        """Blocks the host until the metadata is on the device."""
+        if self._ready is not None:
+            _check(_lib().ba_host_wait(C.c_void_p(self._ready.cuda_event)), "ba_host_wait")
+            self._ready = None
 
     def check(self):
         """Synchronise and raise if a kernel of this plan gave up a bounded wait."""

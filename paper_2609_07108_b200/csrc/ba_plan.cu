@@ -402,6 +402,9 @@ extern "C" int ba_plan_create_host(const ba_problem_t *host, const ba_problem_t 
     if (host->n_main != dev->n_main || host->n_branch != dev->n_branch || host->num_seqs != dev->num_seqs ||
         host->num_branches != dev->num_branches || host->uniform_len != dev->uniform_len || host->mask_kind != dev->mask_kind)
         return BA_EINVAL;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    BA_CUDA_CHECK(cudaStreamIsCapturing((cudaStream_t)stream, &capture));
+    if (capture != cudaStreamCaptureStatusNone) return BA_EINVAL;
     int64_t pairs = 0;
     ba_problem_t pr = *dev;
     if ((rc = check_metadata(host, &pairs, &pr.uniform_len)) != BA_OK) return rc;
@@ -423,6 +426,16 @@ extern "C" int ba_plan_create_host(const ba_problem_t *host, const ba_problem_t 
     ba_plan *pl = new_plan(&pr, a, pairs, offsets);
     if (!pl) return BA_EINVAL;
     *out = pl;
+    return BA_OK;
+}
+
+extern "C" int ba_host_wait(void *event) {
+    // relaxed: another stream of this thread may be capturing, and the event lies outside that capture
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    BA_CUDA_CHECK(cudaThreadExchangeStreamCaptureMode(&mode));
+    const cudaError_t e = cudaEventSynchronize((cudaEvent_t)event);
+    BA_CUDA_CHECK(cudaThreadExchangeStreamCaptureMode(&mode));
+    BA_CUDA_CHECK(e);
     return BA_OK;
 }
 

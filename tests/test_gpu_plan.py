@@ -63,3 +63,43 @@ def test_plan_used_from_another_stream(ba, kind):
         o, _ = ba.branch_attn_fwd(plan, d["q_main"], d["q_branch"], d["k"], d["v"])
     torch.cuda.synchronize()
     assert (f32(o) == want).all()
+
+
+@pytest.mark.parametrize("error_mode", ["global", "thread_local", "relaxed"])
+def test_plan_captured_right_after_it_was_built(ba, error_mode):
+    """A capture that does not begin with a synchronisation: the plan's kernel waits behind other work on its stream
+    while calls that use the plan are captured on another one.  The replay must find the metadata."""
+    p = W.odd_shapes(W.TREE, head_dim=128, dtype="bf16")
+    d = to_dev(p, W.make_tensors(p, seed=2, std=0.5))
+    want = f32(ba.branch_attn_fwd(ba.Plan(p), d["q_main"], d["q_branch"], d["k"], d["v"])[0])
+    busy = torch.randn(4096, 4096, device="cuda")
+    side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    o, lse = torch.zeros((p.rows, p.h_q, 128), dtype=torch.bfloat16, device="cuda"), torch.zeros((p.rows, p.h_q), device="cuda")
+    torch.cuda.synchronize()
+    for _ in range(20):
+        busy = busy @ busy.clamp(-1e-3, 1e-3)
+    plan = ba.Plan(p)
+    with torch.cuda.stream(side):
+        graph.capture_begin(capture_error_mode=error_mode)
+        ba.branch_attn_fwd(plan, d["q_main"], d["q_branch"], d["k"], d["v"], out=o, lse=lse)
+        with pytest.raises(RuntimeError):
+            ba.Plan(p)                                 # its copy and kernel would run at each replay only
+        graph.capture_end()
+        assert plan._ready is None                     # the host has waited
+        graph.replay()
+    torch.cuda.synchronize()
+    assert (f32(o) == want).all()
+
+
+def test_plan_wait(ba):
+    p = W.odd_shapes(W.CHAIN)
+    busy = torch.randn(4096, 4096, device="cuda")
+    for _ in range(20):
+        busy = busy @ busy.clamp(-1e-3, 1e-3)
+    plan = ba.Plan(p)
+    done = torch.cuda.Event()
+    done.record()
+    plan.wait()
+    plan.wait()
+    assert plan._ready is None and plan.pairs == W.useful_pairs(p)
+    assert ba._lib().ba_host_wait(ba.C.c_void_p(done.cuda_event)) == 0 and done.query()
