@@ -21,6 +21,7 @@ OP_FWD, OP_BWD, OP_BWD_FUSED, OP_BWD_DEPTH = 0, 1, 2, 3
 STAGE_PREP, STAGE_DQ, STAGE_DKDV, STAGE_ALL = 1, 2, 4, 7
 STAGE_FUSED, STAGE_ALL_FUSED = 8, 9
 IMPL_AUTO, IMPL_SIMT, IMPL_TC = 0, 1, 2
+MASK_TREE = 2
 
 _DT = {"bf16": (BA_BF16, torch.bfloat16), "fp32": (BA_FP32, torch.float32)}
 
@@ -198,7 +199,9 @@ class Plan:
         self.dtype_code, self.torch_dtype = _DT[problem.dtype]
         arrays = [_i32(problem.cu_seqlens), _i32(problem.anchor_idx), _i32(problem.branch_offsets),
                   _i32(problem.parent) if problem.parent is not None else np.zeros(0, np.int32)]
-        if len(arrays[2]) != problem.num_branches + 1 or (problem.parent is not None and len(arrays[3]) < problem.n_branch):
+        # (a length that the library cannot see: it would read past the end)
+        short_parent = int(problem.kind) == MASK_TREE and problem.parent is not None and len(arrays[3]) < problem.n_branch
+        if len(arrays[2]) != problem.num_branches + 1 or short_parent:
             raise BranchAttnError(-4, "ba_plan_create")
         ends = np.cumsum([len(a) for a in arrays]).tolist()
         packed = torch.empty(ends[-1], dtype=torch.int32, pin_memory=True)

@@ -103,3 +103,10 @@ def test_plan_wait(ba):
     plan.wait()
     assert plan._ready is None and plan.pairs == W.useful_pairs(p)
     assert ba._lib().ba_host_wait(ba.C.c_void_p(done.cuda_event)) == 0 and done.query()
+
+
+@pytest.mark.parametrize("kind", [W.CHAIN, W.BLOCK])
+@pytest.mark.parametrize("length", [0, 3])
+def test_parents_of_chains_and_blocks_are_not_looked_at(ba, kind, length):
+    p = W.odd_shapes(kind)
+    assert ba.Plan(bad(p, parent=np.full(length, 7))).pairs == W.useful_pairs(p)
