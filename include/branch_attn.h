@@ -41,7 +41,7 @@ typedef enum ba_status {
     BA_EINVAL = -1,        /* bad argument (NULL pointer, negative size, bad range) */
     BA_EUNSUPPORTED = -2,  /* dtype / head_dim / branch length not supported */
     BA_EWORKSPACE = -3,    /* plan memory or workspace too small / misaligned */
-    BA_EMETA = -4,         /* device-side validation of the metadata failed */
+    BA_EMETA = -4,         /* validation of the metadata failed */
     BA_ECUDA = -5,         /* a CUDA runtime call failed; see ba_last_cuda_error */
     BA_ETIMEOUT = -6       /* a bounded device-side wait expired */
 } ba_status;
@@ -112,7 +112,9 @@ int ba_plan_destroy(ba_plan_t *plan);
  * device arrays are read by one kernel on `stream`, after the copies that the caller
  * queued there.  Nothing is synchronised, so a caller that builds a plan per step keeps
  * the GPU busy.  The device arrays must hold the host values and stay alive until the
- * work queued on `stream` has run; calls on another stream must wait for that work.  Not
+ * work queued on `stream` has run; calls on another stream must wait for that work.
+ * Branches of one length are recognised from the offsets (as if uniform_len had been given,
+ * which the per-depth calls need); ba_plan_create takes uniform_len as it is.  Not
  * while `stream` is capturing (BA_EINVAL): the plan would not exist before a replay.
  */
 int ba_plan_create_host(const ba_problem_t *host, const ba_problem_t *dev, void *plan_mem,
