@@ -57,7 +57,8 @@ static int fwd_common(const ba_plan_t *plan, const BaRange &r, const void *q_mai
     if (!k || !v || !o || !lse) return BA_EINVAL;
     if (has_branch_q && !q_branch) return BA_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
-    if (ba_use_tc(plan, partial != 0)) return ba_tc_fwd(plan, r, q_main, q_branch, k, v, o, lse, partial, st);
+    const uintptr_t addresses = (uintptr_t)q_main | (uintptr_t)q_branch | (uintptr_t)k | (uintptr_t)v | (uintptr_t)o;
+    if (ba_use_tc(plan, partial != 0, addresses)) return ba_tc_fwd(plan, r, q_main, q_branch, k, v, o, lse, partial, st);
     if (partial == 2 && plan->impl != BA_IMPL_TC) return BA_EUNSUPPORTED;   // merge in the epilogue: tensor-core plans only
     return ba_simt_fwd(plan, r, q_main, q_branch, k, v, o, lse, partial, st);
 }
@@ -178,7 +179,9 @@ static int bwd_common(const ba_plan_t *plan, const void *q_main, const void *q_b
             return rc;
         return BA_OK;
     }
-    if (ba_use_tc(plan, accumulate != 0))
+    const uintptr_t addresses = (uintptr_t)q_main | (uintptr_t)q_branch | (uintptr_t)k | (uintptr_t)v | (uintptr_t)dQ_main |
+                                (uintptr_t)dQ_branch | (uintptr_t)dK | (uintptr_t)dV;
+    if (ba_use_tc(plan, accumulate != 0, addresses))
         return ba_tc_bwd(plan, r, qm, q_branch, k, v, LSE, delta, dO, accumulate, dQ_main, dQ_branch, dK,
                          dV, st, stages);
     return ba_simt_bwd(plan, r, qm, q_branch, k, v, LSE, delta, dO, accumulate, dQ_main, dQ_branch, dK, dV,

@@ -104,8 +104,10 @@ bool ba_tc_supported(const ba_problem_t *p);
 // tensor-core kernels carry P and dS as bf16 pairs (16 bits of mantissa), which bf16 results do not show and fp32
 // results do.  Against fp64, 1,600 .. 3,000 tokens with chains, plain FMA / tensor cores, 2-norm: O 1e-7 .. 3e-7 /
 // 2e-6, dQ 2e-7 .. 5e-7 / 3e-6, dK and dV 4e-7 .. 7e-7 / 4e-6 .. 1.4e-5.
-static inline bool ba_use_tc(const ba_plan *pl, bool fp32_out) {
-    return pl->impl == BA_IMPL_TC && !(pl->prob.head_dim == 64 && fp32_out);
+// So do, as ever, tensors that are not 16-byte aligned (`addresses`: theirs, or-ed): tensor maps need that, the
+// plain-FMA kernels 8 bytes.
+static inline bool ba_use_tc(const ba_plan *pl, bool fp32_out, uintptr_t addresses) {
+    return pl->impl == BA_IMPL_TC && !(pl->prob.head_dim == 64 && (fp32_out || (addresses & 15)));
 }
 // Elementwise (ba_elementwise.cu)
 // Backward preprocess into head-major scratch [h_q, row_pitch]:

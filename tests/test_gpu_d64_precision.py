@@ -50,3 +50,28 @@ def test_fp32_results_keep_fp32_probabilities(ba, oracle, kind):
     for name, a, b in zip(("dQ_main", "dQ_branch", "dK", "dV"), *grads):
         assert float(a.abs().max()) > 0 and torch.equal(a, b), name
     auto.check()
+
+
+def test_tensors_on_8_byte_boundaries(ba):
+    """Views that begin 8 bytes into an allocation: no tensor map can start there, the plain-FMA kernels can."""
+    p = W.odd_shapes(W.TREE, head_dim=64, dtype="bf16")
+    d = to_dev(p, W.make_tensors(p, seed=72, std=0.5))
+
+    def shifted(x):
+        buf = torch.zeros(x.numel() + 4, dtype=x.dtype, device="cuda")
+        buf[4:] = x.flatten()
+        return buf[4:].view(x.shape)
+
+    results = []
+    for move, impl in ((lambda x: x, ba.IMPL_SIMT), (shifted, ba.IMPL_AUTO)):
+        plan = ba.Plan(p, impl=impl)
+        qkv = [move(d[x]) for x in ("q_main", "q_branch", "k", "v")]
+        o, lse = ba.branch_attn_fwd(plan, *qkv, out=move(torch.zeros_like(d["d_o"])))
+        o = o.clone()                                   # (the backward's own pass over O and dO needs 16 bytes)
+        grads = [move(torch.zeros_like(x)) for x in qkv]
+        ba.branch_attn_bwd(plan, *qkv, o, lse, d["d_o"], grads=grads)
+        plan.check()
+        results.append((o, lse, *grads))
+    assert results[1][2].data_ptr() % 16 == 8
+    for a, b in zip(*results):
+        assert torch.equal(a, b)
