@@ -828,6 +828,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sm.tmem_base;
+    const int accumulate = D == 128 ? p.accumulate : 0;      // head_dim 64: bf16 gradients only (ba_use_tc)
     bool shared_tile = false;      // SPLIT: this CTA walked a part of a main key tile
 
     if (warp >= 8) {
@@ -855,11 +856,11 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                     const KvItem &it = sm.item[s];
                     const int rows = it.row_end - it.row0;
                     if (kDq) {
-                        store_zero_rows<D>(it.is_main ? p.dq_main : p.dq_branch, p.accumulate, it.row0, rows, it.h0,
+                        store_zero_rows<D>(it.is_main ? p.dq_main : p.dq_branch, accumulate, it.row0, rows, it.h0,
                                          min(p.hp, (it.g + 1) * p.group - it.h0), p.h_q, lane);
                     } else {
-                        store_zero_rows<D>(p.dk, p.accumulate, it.srow0, rows, it.g, 1, p.h_kv, lane);
-                        store_zero_rows<D>(p.dv, p.accumulate, it.srow0, rows, it.g, 1, p.h_kv, lane);
+                        store_zero_rows<D>(p.dk, accumulate, it.srow0, rows, it.g, 1, p.h_kv, lane);
+                        store_zero_rows<D>(p.dv, accumulate, it.srow0, rows, it.g, 1, p.h_kv, lane);
                     }
                 } else {
                     if (lane == 0) mbar_arrive(&sm.item_full[s]);
@@ -927,12 +928,13 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                         const int h = it.g * p.group + hh;
                         const int gr0 = seg_main ? r0 : qbase + r0;
                         if (lane == 0) {
-                            // (a branch tile may start up to three rows before branch row 0: no rows of these maps)
-                            const CUtensorMap *tq = seg_main ? &tm_q_main : &tm_q_branch, *tg = seg_main ? &tm_go : &tm_go_branch;
+                            // A branch tile may start up to three rows before branch row 0: dO by the map that has no rows
+                            // there.  (By that map for every branch tile: 129 us instead of 126 at 2,048 tokens.)
+                            const CUtensorMap *tq = seg_main ? &tm_q_main : &tm_q_branch, *tg = r0 >= 0 ? &tm_go : &tm_go_branch;
                             mbar_expect_tx(&sm.x_full[st], 2 * kSubBytes + 2 * kSub * 4);
                             for (int half = 0; half < kHalves; ++half) {
                                 tma_load_3d(sm.xs[st] + half * 8192, tq, half * 64, h, r0, &sm.x_full[st]);
-                                tma_load_3d(sm.xs[st] + kSubBytes + half * 8192, tg, half * 64, h, r0, &sm.x_full[st]);
+                                tma_load_3d(sm.xs[st] + kSubBytes + half * 8192, tg, half * 64, h, r0 >= 0 ? gr0 : r0, &sm.x_full[st]);
                             }
                             const size_t off = (size_t)h * p.row_pitch + gr0;
                             bulk_load(mt.neg_lse2, p.nlse2_t + off, kSub * 4, &sm.x_full[st]);
@@ -942,10 +944,10 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                                 const bool main2 = ps < it.n_sub_main;
                                 const int r2 = main2 ? it.ma + ps * kSub : it.ba + (ps - it.n_sub_main) * kSub;
                                 const int g2 = main2 ? r2 : qbase + r2;
-                                const CUtensorMap *tq2 = main2 ? &tm_q_main : &tm_q_branch, *tg2 = main2 ? &tm_go : &tm_go_branch;
+                                const CUtensorMap *tq2 = main2 ? &tm_q_main : &tm_q_branch;
                                 for (int half = 0; half < kHalves; ++half) {
                                     tma_prefetch_3d(tq2, half * 64, h2, r2);
-                                    tma_prefetch_3d(tg2, half * 64, h2, r2);
+                                    tma_prefetch_3d(&tm_go, half * 64, h2, g2);
                                 }
                                 const size_t off2 = (size_t)h2 * p.row_pitch + g2;
                                 bulk_prefetch(p.nlse2_t + off2, kSub * 4);
@@ -1276,7 +1278,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                             make_float4(__uint_as_float(r[4 * e]), __uint_as_float(r[4 * e + 1]), __uint_as_float(r[4 * e + 2]),
                                         __uint_as_float(r[4 * e + 3]));
                 } else if (w.valid) {
-                    if (p.accumulate) store_grad_chunk<true>(dst, base + c * 32, r, mul);
+                    if (accumulate) store_grad_chunk<true>(dst, base + c * 32, r, mul);
                     else store_grad_chunk<false>(dst, base + c * 32, r, mul, p.wide);
                 }
                 if (D == 64 && not_finite) {      // does it hold rows out of its reach (ba_exact.cuh; bf16 results only)?
@@ -1314,7 +1316,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                 x.x *= mul; x.y *= mul; x.z *= mul; x.w *= mul;
                 void *dst = which == 0 ? p.dk : p.dv;
                 const size_t off = ((size_t)(it.srow0 + r) * p.h_kv + it.g) * D + ch * 4;
-                if (p.accumulate) {
+                if (accumulate) {
                     float4 *d4 = reinterpret_cast<float4 *>((float *)dst + off);
                     const float4 o = *d4;
                     *d4 = make_float4(o.x + x.x, o.y + x.y, o.z + x.z, o.w + x.w);

@@ -287,12 +287,12 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_
                 const bool seg_main = u < n_sub_main;
                 const int64_t r0 = seg_main ? ma + (int64_t)u * kTile : ba + (int64_t)(u - n_sub_main) * kTile;
                 const int64_t grow0 = seg_main ? r0 : n + r0;
-                // (a branch tile may start up to three rows before branch row 0: no rows of these maps)
-                const CUtensorMap *tq = seg_main ? &tm_q_main : &tm_q_branch, *tg = seg_main ? &tm_go : &tm_go_branch;
+                // a branch tile may start up to three rows before branch row 0: dO by the map that has no rows there
+                const CUtensorMap *tq = seg_main ? &tm_q_main : &tm_q_branch, *tg = r0 >= 0 ? &tm_go : &tm_go_branch;
                 mbar_expect_tx(&sm.q_full[st], 2 * kTileBytes + 2 * kTile * 4);
                 for (int half = 0; half < 2; ++half) {
                     tma_load_3d(sm.q[st] + half * 16384, tq, half * 64, h, (int)r0, &sm.q_full[st]);
-                    tma_load_3d(sm.go[st] + half * 16384, tg, half * 64, h, (int)r0, &sm.q_full[st]);
+                    tma_load_3d(sm.go[st] + half * 16384, tg, half * 64, h, (int)(r0 >= 0 ? grow0 : r0), &sm.q_full[st]);
                 }
                 const size_t off = (size_t)h * p.row_pitch + grow0;
                 bulk_load(sm.neg_lse2[st], p.nlse2_t + off, kTile * 4, &sm.q_full[st]);
@@ -304,10 +304,10 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_
                     const bool main2 = u2 < n_sub_main;
                     const int64_t r2 = main2 ? ma + (int64_t)u2 * kTile : ba + (int64_t)(u2 - n_sub_main) * kTile;
                     const int64_t g2 = main2 ? r2 : n + r2;
-                    const CUtensorMap *tq2 = main2 ? &tm_q_main : &tm_q_branch, *tg2 = main2 ? &tm_go : &tm_go_branch;
+                    const CUtensorMap *tq2 = main2 ? &tm_q_main : &tm_q_branch;
                     for (int half = 0; half < 2; ++half) {
                         tma_prefetch_3d(tq2, half * 64, h2, (int)r2);
-                        tma_prefetch_3d(tg2, half * 64, h2, (int)r2);
+                        tma_prefetch_3d(&tm_go, half * 64, h2, (int)g2);
                     }
                     const size_t off2 = (size_t)h2 * p.row_pitch + g2;
                     bulk_prefetch(p.nlse2_t + off2, kTile * 4);

@@ -204,6 +204,7 @@ template <int D> __device__ void store_empty_item(const TcFwdParams &p, const It
 template <int D, int P>
 __device__ __forceinline__ void combine_parts(const TcFwdParams &p, FwdSmem<D> &sm, int tid) {
     constexpr int kCols = D / P, kVec = kCols / 4;
+    const int partial_out = D == 128 ? p.partial_out : 0;
     const Item &it = sm.item[0];
     const int lane = tid & 31, dup = p.same_rows, rank = (int)(blockIdx.x % p.splits);
     const int row = rank * (256 / P) + tid / P, part = tid % P;
@@ -213,7 +214,7 @@ __device__ __forceinline__ void combine_parts(const TcFwdParams &p, FwdSmem<D> &
     const int my_row = it.row0 + tok + (i ? tile1_off(p, it.is_main) : 0);
     const int64_t orow = out_row(p, it.is_main, my_row);
     // the threads of a row sit in one warp: all have read the old LSE before one of them replaces it
-    const float lse_a = valid && p.partial_out == 2 ? p.lse[orow * p.h_q + h] : -INFINITY;
+    const float lse_a = valid && partial_out == 2 ? p.lse[orow * p.h_q + h] : -INFINITY;
     __syncwarp();
     auto slot = [&](int s) { return (dup ? s & 1 : i) * kTile + r_in; };
     const float2 ml = cluster_ld_f2(cluster_map(smem_u32(sm.ml(0) + slot(part)), part >> dup));
@@ -247,13 +248,13 @@ __device__ __forceinline__ void combine_parts(const TcFwdParams &p, FwdSmem<D> &
     const float inv = sum > 0.f ? 1.0f / sum : sum;      // 0, or NaN although the part that is NaN may weigh nothing
     const float lse_p = sum > 0.f ? (mx + log2f(sum)) * kLn2 : -INFINITY;
     float lse_out = lse_p, w_new = inv, w_old = 0.f;
-    if (p.partial_out == 2) merge_weights(lse_a, lse_p, inv, lse_out, w_old, w_new);
+    if (partial_out == 2) merge_weights(lse_a, lse_p, inv, lse_out, w_old, w_new);
     const size_t base = ((size_t)orow * p.h_q + h) * D + part * kCols;
     if (valid && part == 0) p.lse[orow * p.h_q + h] = lse_out;
 #pragma unroll
     for (int e = 0; valid && e < kVec; ++e) {
         float4 v = make_float4(acc[4 * e] * w_new, acc[4 * e + 1] * w_new, acc[4 * e + 2] * w_new, acc[4 * e + 3] * w_new);
-        if (p.partial_out == 0) {
+        if (partial_out == 0) {
             *reinterpret_cast<uint2 *>((__nv_bfloat16 *)p.o + base + 4 * e) = make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
         } else {
             float4 *dst = reinterpret_cast<float4 *>((float *)p.o + base + 4 * e);
@@ -590,6 +591,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
         const uint32_t s_addr = tmem + lane_base + i * 128;
         const uint32_t o_addr = tmem + lane_base + 256 + i * 128, lo_addr = o_addr + 64;
         const float sl2 = p.scale_log2;
+        const int partial_out = D == 128 ? p.partial_out : 0;      // head_dim 64: bf16 results only (ba_use_tc)
         uint32_t n_s = 0, n_o = 0;
         // What this role needs of an item, and this thread's row.  Everything the key loop uses sits in
         // registers (a shared-memory load of these warps waits several hundred clocks behind the operand
@@ -778,7 +780,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
             float w_new = inv, w_old = 0.f;   // partial_out == 2: weights of Eq. (lse-merge)
             if (w.valid) {
                 float lse_out = lse_p;
-                if (p.partial_out == 2) merge_weights(p.lse[orow * p.h_q + w.h], lse_p, inv, lse_out, w_old, w_new);
+                if (partial_out == 2) merge_weights(p.lse[orow * p.h_q + w.h], lse_p, inv, lse_out, w_old, w_new);
                 p.lse[orow * p.h_q + w.h] = lse_out;
             }
             // A warp whose rows are all live hands 64 columns at a time to a TMA store: row by row from
@@ -829,10 +831,10 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
                     if (lane == 0) tma_store_3d(&tm_o, hf * 64, w.h, (int)orow, smem_u32(sm.out[warp]));
                 } else if (w.valid) {
                     const size_t off = base + hf * 64;
-                    if (p.partial_out == 2) {
+                    if (partial_out == 2) {
                         merge_row_chunk(p.o, off, ra, w_new, w_old);
                         merge_row_chunk(p.o, off + 32, rb, w_new, w_old);
-                    } else if (p.partial_out) {
+                    } else if (partial_out) {
                         store_row_chunk<true>(p.o, off, ra, inv, p.wide);
                         store_row_chunk<true>(p.o, off + 32, rb, inv, p.wide);
                     } else {
