@@ -428,7 +428,8 @@ def run_ours(args):
     impl = {"auto": ba.IMPL_AUTO, "simt": ba.IMPL_SIMT, "tc": ba.IMPL_TC}[args.kernels]
     plan = ba.Plan(p, device=device, impl=impl)
     # metadata builder, timed on its own (it is reused by the forward, the backward and, in a
-    # model, every layer): host wall clock around ba_plan_create incl. its stream synchronisations
+    # model, every layer): host wall clock around ba_plan_create_host, which validates and counts on the host and
+    # queues one copy and one kernel, and the wait for them
     plan_times = []
     for _ in range(3):
         torch.cuda.synchronize()

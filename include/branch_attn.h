@@ -24,6 +24,13 @@
  *     KV head h / (h_q / h_kv).
  *   - Element type of q/k/v/O/dO is ba_problem_t.dtype.  Supported: BA_FP32 and
  *     BA_BF16 with head_dim 64 or 128; a branch holds at most 64 tokens.
+ *   - NaN and infinities: on the plain-FMA kernels, and at head_dim 64 throughout, a row of
+ *     an input reaches the results whose definition contains it and no others (which of them
+ *     come out as NaN and which as infinity is not specified).  On the tensor-core kernels at
+ *     head_dim 128 it may also reach rows that share a tile of 128 with them, of other
+ *     sequences too, so every row of q, k, v, O, dO that a call can read must be finite: all
+ *     rows, except those of later depths (per-depth calls), those outside a received shard,
+ *     and, without main queries (q_main NULL), the main rows of O and dO.
  *   - Every function returns BA_OK (0) or a negative ba_status; nothing throws.
  */
 #ifndef BRANCH_ATTN_H_

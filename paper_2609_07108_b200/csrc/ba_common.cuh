@@ -21,6 +21,8 @@ struct BaMeta {
     const int32_t *key_bq_end;    // [N] first branch token anchored beyond x's sequence
 };
 
+constexpr int kSms = 148;          // B200
+
 struct ba_plan {
     ba_problem_t prob;            // copy; the metadata pointers in it are NOT kept alive
     BaMeta meta;

@@ -1,13 +1,13 @@
 // HBM-bound elementwise kernels: Eq. (lse-merge), the backward preprocess
 // delta = rowsum(dO * O), and the fp32 -> output-dtype conversion of gradient
-// accumulators.  All are grid-stride, 16-byte vectorised, one pass over memory.
+// accumulators.  All are 16-byte vectorised, one pass over memory; merge and conversion
+// are grid-stride, delta has one CTA per tile of rows and heads.
 #include "ba_common.cuh"
 
 namespace {
 
 constexpr int kThreads = 256;
 constexpr int kBlocksPerSm = 8;
-constexpr int kSms = 148;
 
 inline int stream_grid(int64_t work_items) {
     int64_t g = (work_items + kThreads - 1) / kThreads;

@@ -190,7 +190,7 @@ __global__ void plan_rows_kernel(PlanArgs p, int main_blocks) {
 int grid_for(int64_t n, int block) {
     int64_t g = (n + block - 1) / block;
     if (g < 1) g = 1;
-    if (g > 148 * 16) g = 148 * 16;
+    if (g > kSms * 16) g = kSms * 16;
     return (int)g;
 }
 

@@ -675,8 +675,8 @@ int launch_tiles(const ba_plan *pl, SimtArgs a, bool after_dq, cudaStream_t st) 
     // 303 us with eight, 270 with sixteen; 3,500 tokens, 200 chains of 20, 8/4 heads, D 64: 1625 and 980; 1,000
     // tokens with 60 trees, dQ: 138 us in parts of four, 162 in parts of two).
     a.splits = 1;
-    while (a.splits < 8 && ((work * a.splits * 2 <= 148 * 8 && est >= 2 * 2 * a.splits) ||
-                            (work * a.splits * 2 <= 148 * 16 && est >= 2 * 4 * a.splits)))
+    while (a.splits < 8 && ((work * a.splits * 2 <= kSms * 8 && est >= 2 * 2 * a.splits) ||
+                            (work * a.splits * 2 <= kSms * 16 && est >= 2 * 4 * a.splits)))
         a.splits *= 2;
     if (work * a.splits > INT_MAX) return BA_EUNSUPPORTED;
     return launch<T, D, MODE>(a, work, after_dq, st);

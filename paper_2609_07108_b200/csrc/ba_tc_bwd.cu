@@ -583,10 +583,13 @@ tc_dq_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
 // blocks of 16 on 32,768 tokens, draft rows, 439 -> 387 us; dQ of the head_dim 64 batch below 285 -> 205).
 //   TMEM: acc1 [0,D) acc2 [D,2D); set b: XS_b = 256 + 128 b (64 cols: S, its first 32 columns then hold P as
 //   bf16), XD_b = XS_b + 64 (dP, then dS); head_dim 64: P_lo, dS_lo of set b in 32 columns each from 128 + 64 b.
-// head_dim 64 runs in place of plain-FMA kernels that kept P and dS in fp32.  To give up none of that, P and
-// dS go in as bf16 pairs hi + lo (16 bits of mantissa), two products each; against fp64 the gradients are
-// then off by exactly what those kernels show.  4,096 tokens, 6 sequences, chains of three, 32/8 heads:
-// dQ / dK/dV 282 / 368 us (were 3052 / 8978).
+// head_dim 64 runs in place of plain-FMA kernels that kept P and dS in fp32.  P and dS go in as bf16 pairs hi + lo (16
+// bits of mantissa), two products each: against fp64, gradients rounded to bf16 are then off by what those kernels'
+// are (dQ, dK, dV 1.64e-3 .. 1.66e-3 in the 2-norm, the same to 1 part in 10,000).  Gradients accumulated in fp32
+// would not be, so they stay with those kernels (ba_use_tc).  4,096 tokens, 6 sequences, chains of three, 32/8 heads:
+// dQ / dK/dV 189 / 342 us (were 3052 / 8978).
+// dQ at head_dim 64 is here and not in tc_dq_kernel because that kernel was written for 128 columns of dQ and keeps P
+// in registers as bf16; a form of it with hi + lo pairs has not been tried.
 //
 // Key tiles of dK/dV differ in length (causal) and are few in small batches: the CTAs of a cluster then share
 // a main key tile, each walks a contiguous part of its (head, row tile) steps, and the parts are summed through
@@ -1509,7 +1512,7 @@ int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
         const int64_t keys = kmt * kTile, viewers = qm_n + br_n;
         const int64_t seq = pr.num_seqs > 0 ? pr.n_main / pr.num_seqs : 0;
         const int64_t est = keys > 0 ? (seq < keys ? seq : keys) / 2 * viewers / (keys < pr.n_main ? pr.n_main : keys) * p.group / kSub : 0;
-        while (p.splits < 8 && kmt * pr.h_kv * p.splits * 2 <= 148 && est >= 8 * 2 * p.splits) p.splits *= 2;
+        while (p.splits < 8 && kmt * pr.h_kv * p.splits * 2 <= kSms && est >= 8 * 2 * p.splits) p.splits *= 2;
         p.main_key_tiles = (int)kmt;
         const int64_t tiles = kmt + (kbt + p.splits - 1) / p.splits;    // work items (clusters) per KV head
         p.total_key_tiles = (int)tiles;
@@ -1517,13 +1520,14 @@ int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
         // tokens with chains 830 us against 1030 KV-head-major, 32,768 tokens with blocks 1616 against 1711);
         // beyond that KV-head-major, whose resident CTAs share one query stream through L2 (65,536-token trees 7862
         // us against 7953, 73,728 tokens with chains 48.4 ms against 48.9).
-        p.tile_major = tiles * pr.h_kv <= 24 * 148;
+        p.tile_major = tiles * pr.h_kv <= 24 * kSms;
         if (!maps(tm, kSub, 1, kTile)) return BA_EINVAL;
         const int64_t grid = tiles * pr.h_kv * p.splits;
         // The two kernels write different tensors and need the same inputs: the second may start on the SMs that the
         // last items of the first leave idle (not when no row of dQ was launched: the kernel before is then the
         // caller's, or delta).  Both kernels, overlapped / one after the other: 2,048-token chains 222 / 231 us, draft
-        // rows of 512 blocks 658 / 680; head_dim 64, 4,096-token chains 605 / 548, so not there.
+        // rows of 512 blocks 658 / 680; head_dim 64, 4,096-token chains 605 / 548 (that shape alone was measured), so not
+        // there.
         const bool after_dq = D == 128 && (stages & BA_STAGE_DQ) && qm_n + br_n > 0;
         const int rc = D == 64 ? launch_kv<64, kModeDkdv>(p, tm, grid, after_dq, dev, st)
                                : launch_kv<128, kModeDkdv>(p, tm, grid, after_dq, dev, st);

@@ -680,8 +680,8 @@ int ba_tc_bwd_fused(const ba_plan *pl, const BaRange &r, const void *q_main, con
     const int64_t steps = viewers / kTile * p.group;
     p.splits = 1;
     auto waves = [&](int64_t split, int64_t sms) { return (double)((kmt * pr.h_kv * split + sms - 1) / sms) / (double)split; };
-    double best = waves(1, 148);
-    const int64_t sms[3] = {148, 136, 128};      // SMs that clusters of two, four, eight can use
+    double best = waves(1, kSms);
+    const int64_t sms[3] = {kSms, 136, 128};      // SMs that clusters of two, four, eight can use
     for (int i = 0; i < 3; ++i)
         if (steps >= 8 << (i + 1) && waves(2 << i, sms[i]) < 0.9 * best) {
             p.splits = 2 << i;

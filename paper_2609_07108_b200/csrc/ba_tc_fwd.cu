@@ -22,9 +22,10 @@
 //                    next item run behind the softmax and the output stores of the current one
 // TMEM (512 columns): S_0 [0,128) S_1 [128,256) O_0 [256,256+D) O_1 [384,384+D); P_i occupies the
 // first 64 columns of S_i; head_dim 64: the 64 columns after O_i hold P_lo.
-// head_dim 64 runs in place of a plain-FMA kernel that kept P in fp32.  To give up none of that, P goes in as
-// a bf16 pair hi + lo (16 bits of mantissa), two products each; against fp64 O is then off by exactly what
-// that kernel shows.  4,096 tokens, 6 sequences, chains of three, 32/8 heads: 176 us (was 2619).
+// head_dim 64 runs in place of a plain-FMA kernel that kept P in fp32.  P goes in as a bf16 pair hi + lo (16 bits of
+// mantissa), two products each: against fp64, O rounded to bf16 is then off by what that kernel's is (1.5803e-3
+// against 1.5803e-3 in the 2-norm).  O in fp32 would not be, so partial forwards stay with that kernel (ba_use_tc).
+// 4,096 tokens, 6 sequences, chains of three, 32/8 heads: 173 us (was 2619).
 //
 // What bounds it: the chain scores -> maximum -> exponentials -> P -> P V, next Q K^T of each of the
 // two tiles (about 2000 clocks of softmax and 1000 of MMA and handoffs per 128 x 128 tile), so the
@@ -949,11 +950,11 @@ int ba_tc_fwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
     auto split = [&](bool same_rows_ok) {
         work = fill_items(p, pl, r, q_main != nullptr, depth, same_rows_ok);
         p.splits = 1;
-        while (p.splits < 8 && work * p.splits * 2 <= 2 * 148 && est_tiles >= 4 * 2 * p.splits) p.splits *= 2;
+        while (p.splits < 8 && work * p.splits * 2 <= 2 * kSms && est_tiles >= 4 * 2 * p.splits) p.splits *= 2;
     };
     split(true);
     // (the kernel for whole items has different rows in its tiles)
-    if (p.same_rows && (p.splits == 1 || (work * 2 > 148 && est_tiles < 32))) split(false);
+    if (p.same_rows && (p.splits == 1 || (work * 2 > kSms && est_tiles < 32))) split(false);
     if (work == 0) return BA_OK;
     if (work > INT_MAX) return BA_EUNSUPPORTED;
 
