@@ -300,14 +300,14 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const __grid_constant
     const int n_iter = n_tiles * (MODE == kDkdv ? a.group : 1);
     const int t_beg = (int)((int64_t)n_iter * rank / a.splits), t_end = (int)((int64_t)n_iter * (rank + 1) / a.splits);
 
-    struct Tile { int64_t r0; int cnt, h; bool main; };
+    struct Tile { int r0, cnt, h; bool main; };
     auto tile_of = [&](int t) -> Tile {
         Tile x;
         const int s = MODE == kDkdv ? t % n_tiles : t;
         x.h = MODE == kDkdv ? g * a.group + t / n_tiles : g;
         x.main = s < nm;
-        x.r0 = x.main ? m0 + (int64_t)s * kBN : b0 + (int64_t)(s - nm) * kBN;
-        x.cnt = (int)min((int64_t)kBN, (x.main ? m1 : b1) - x.r0);
+        x.r0 = (int)(x.main ? m0 : b0) + (x.main ? s : s - nm) * kBN;
+        x.cnt = min(kBN, (int)(x.main ? m1 : b1) - x.r0);
         return x;
     };
     auto load_x1 = [&](int t) {
@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const __grid_constant
         float *dst = sm.x1[t % Smem::kX1];
         if (MODE == kDkdv) {
             load_rows<T, D, kBN>(dst, x.main ? (const T *)a.q_main : (const T *)a.q_branch,
-                            [&](int r) -> int64_t { return r < x.cnt ? ((x.r0 + r) * a.h_q + x.h) * D : -1; });
+                            [&](int r) -> int64_t { return r < x.cnt ? ((int64_t)(x.r0 + r) * a.h_q + x.h) * D : -1; });
             if (tid < kBN) {
                 const bool live = tid < x.cnt;
                 const int64_t row = x.r0 + tid, gr = (x.main ? 0 : n) + row;
@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const __grid_constant
                 sm.mask[tid] = live && !x.main ? a.meta.br_mask[row] : 0ull;
             }
         } else {
-            const int row0 = (int)((x.main ? -a.r.kv_base : n) + x.r0);      // in the key tensors
+            const int row0 = (int)(x.main ? -a.r.kv_base : n) + x.r0;      // in the key tensors
             load_rows<T, D, kBN>(dst, (const T *)a.k,
                             [&](int r) -> int64_t { return r < x.cnt ? ((int64_t)(row0 + r) * a.h_kv + g) * D : -1; });
         }
@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const __grid_constant
     auto load_x2 = [&](int t) {
         if (t >= t_end) return;
         const Tile x = tile_of(t);
-        const int heads = MODE == kDkdv ? a.h_q : a.h_kv, row0 = (int)((!x.main ? n : MODE == kDkdv ? 0 : -a.r.kv_base) + x.r0);
+        const int heads = MODE == kDkdv ? a.h_q : a.h_kv, row0 = (int)(!x.main ? n : MODE == kDkdv ? 0 : -a.r.kv_base) + x.r0;
         load_rows<T, D, kBN>(sm.x2, MODE == kDkdv ? (const T *)a.d_o : (const T *)a.v,
                         [&](int r) -> int64_t { return r < x.cnt ? ((int64_t)(row0 + r) * heads + x.h) * D : -1; });
     };
@@ -383,8 +383,8 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const __grid_constant
     auto visible = [&](const Tile &x, int i, int c) -> bool {
         if (!valid[i]) return false;
         if (MODE != kDkdv) {
-            if (x.main) { const int kk = (int)x.r0 + c; return kk >= lo[i] && kk <= hi[i]; }
-            const int rel = (int)x.r0 + c - bst[i];
+            if (x.main) { const int kk = x.r0 + c; return kk >= lo[i] && kk <= hi[i]; }
+            const int rel = x.r0 + c - bst[i];
             return c < x.cnt && rel >= 0 && rel < 64 && ((mask[i] >> rel) & 1ull);
         }
         if (is_main) return key[i] >= sm.lo[c] && key[i] <= sm.hi[c];
