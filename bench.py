@@ -276,7 +276,7 @@ class Recorder:
     def branch_attn_fwd_depth(self, *a, **k):
         return self._wrap("fwd", 1, self.ba.branch_attn_fwd_depth, *a, **k)
 
-    def branch_attn_bwd_depth(self, *a, **k):     # delta, the one-kernel backward, conversion of dQ
+    def branch_attn_bwd_depth(self, *a, **k):     # delta, dQ, dK/dV
         return self._wrap("bwd_depth", 3, self.ba.branch_attn_bwd_depth, *a, **k)
 
     def totals(self):
@@ -555,10 +555,10 @@ def run_ours(args):
         # algorithmic flop of all launches of that kind over the timed steps
         # flop per visible pair and query head that the kernel itself executes, in
         # units of head_dim: forward 2 GEMMs (QK^T, PV); dQ kernel 3 (S, dP, dQ);
-        # dK/dV kernel 4 (S^T and dP^T recomputed, dV, dK)
-        share = {"fwd": 4.0, "bwd_dq": 6.0, "bwd_dkdv": 8.0, "bwd_fused": 10.0, "bwd_depth": 10.0}.get(kind)
-        kernel_name = {"fwd": "tc_fwd_kernel", "bwd_dq": "tc_dq_kernel", "bwd_dkdv": "tc_dkdv_kernel",
-                       "bwd_fused": "tc_bwd_fused_kernel", "bwd_depth": "tc_bwd_fused_kernel"}.get(kind, kind)
+        # dK/dV kernel 4 (S^T and dP^T recomputed, dV, dK); a per-depth backward runs these two
+        share = {"fwd": 4.0, "bwd_dq": 6.0, "bwd_dkdv": 8.0, "bwd_fused": 10.0, "bwd_depth": 14.0}.get(kind)
+        kernel_name = {"fwd": "tc_fwd_kernel", "bwd_dq": "tc_dq_kernel", "bwd_dkdv": "tc_kv_kernel",
+                       "bwd_fused": "tc_bwd_fused_kernel", "bwd_depth": "tc_dq_kernel + tc_kv_kernel"}.get(kind, kind)
         if share is not None:
             kpairs = pairs
             if mode == "stepwise" and kind != "fwd":    # the per-depth calls cover the branch rows only

@@ -17,8 +17,9 @@
 // products.  All operands stay in their natural [row][D] layout, padded by 16 bytes per row: 16-byte reads
 // of 8 consecutive rows then touch all 32 banks once.
 //
-// Bound: latency, with three CTAs (twelve warps) per SM by registers: the schedulers issue in under half of the
-// cycles, FMA pipe and shared memory are 30 to 50 % busy.  So more warps beat bigger tiles: 64 stationary rows (two
+// Bound: latency, with three CTAs (twelve warps) per SM by registers: forward / dK/dV of the 2,048-token batch below
+// issue in 49 / 42 % of the cycles, the FMA pipe is 48 / 48 % busy (60 / 61 % on the fullest SM), shared memory 40 /
+// 50 %.  So more warps beat bigger tiles: 64 stationary rows (two
 // CTAs per SM) read less shared memory per FMA and are slower, 8,192 tokens, 300 blocks of 8, 8/8 heads, D 128,
 // forward / dQ / dK/dV: 1390 / 1837 / 2416 us against 1193 / 1725 / 2029.  Measured against kernels that walked the
 // keys one by one with a row's dot product spread over D/32 lanes: 2,048 tokens with 64 blocks of 16, 8/2 heads,
