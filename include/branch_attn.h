@@ -30,7 +30,9 @@
  *     head_dim 128 it may also reach rows that share a tile of 128 with them, of other
  *     sequences too, so every row of q, k, v, O, dO that a call can read must be finite: all
  *     rows, except those of later depths (per-depth calls), those outside a received shard,
- *     and, without main queries (q_main NULL), the main rows of O and dO.
+ *     and, without main queries (q_main NULL), the main rows of O and dO.  A score of minus
+ *     infinity has weight 0; a row without any other score gets O = 0 and LSE = -inf, as a
+ *     row that sees no key does.
  *   - Every function returns BA_OK (0) or a negative ba_status; nothing throws.
  */
 #ifndef BRANCH_ATTN_H_

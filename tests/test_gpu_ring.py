@@ -76,6 +76,29 @@ def test_shard_calls_check_their_ranges(ba):
     torch.cuda.synchronize()
 
 
+def test_ring_and_zigzag_at_head_dim_64(ba):
+    """The steps' fp32 results come from the plain-FMA kernels, merged in their epilogue; the full call is on the
+    tensor cores.  Both round O and the gradients to bf16 once."""
+    n, cp = 1024, 2
+    p = W.Problem(np.array([0, n], np.int32), np.arange(0, n, 3, dtype=np.int32), W.uniform_branch_offsets(342, 3), W.CHAIN, None,
+                  4, 2, 64, dtype="bf16")
+    plan = ba.Plan(p)
+    g = torch.Generator(device="cuda").manual_seed(54)
+    draw = lambda rows, heads, std: (torch.randn((rows, heads, 64), generator=g, device="cuda") * std).to(torch.bfloat16)
+    qm, qb, k, v, go = draw(n, 4, 0.5), draw(p.n_branch, 4, 0.5), draw(p.rows, 2, 0.5), draw(p.rows, 2, 0.5), draw(p.rows, 4, 0.1)
+    o, lse = ba.branch_attn_fwd(plan, qm, qb, k, v)
+    want = ba.branch_attn_bwd(plan, qm, qb, k, v, o, lse, go)
+    o1, l1, _ = zigzag.forward(ba, plan, qm, qb, k, v, cp)
+    o2, l2, _ = ring.forward(ba, plan, qm, qb, k, v, cp)
+    assert torch.equal(o1, o2) and torch.equal(l1, l2)
+    assert float((o1.float() - o.float()).norm()) <= 4e-3 * float(o.float().norm()) and float((l1 - lse).abs().max()) <= 1e-5
+    g1 = [x.clone() for x in zigzag.backward(ba, plan, qm, qb, k, v, o, lse, go, cp)[:4]]
+    g2 = ring.backward(ba, plan, qm, qb, k, v, o, lse, go, cp)[:4]
+    plan.check()
+    for a, b, c in zip(g1, g2, want):      # (2^-9 per rounding)
+        assert torch.equal(a, b) and float((a.float() - c.float()).norm()) <= 4e-3 * float(c.float().norm())
+
+
 # Two sequences, the second one starting inside a shard; N no multiple of 32 or 128.  Behind each shard (in the same
 # allocation) lie rows of NaN: a kernel that read them, and multiplied them with a weight of zero, would show.
 @pytest.mark.parametrize("head_dim", [64, 128])
