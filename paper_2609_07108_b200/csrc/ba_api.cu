@@ -182,7 +182,7 @@ static int bwd_common(const ba_plan_t *plan, const void *q_main, const void *q_b
     const uintptr_t addresses = (uintptr_t)q_main | (uintptr_t)q_branch | (uintptr_t)k | (uintptr_t)v | (uintptr_t)dQ_main |
                                 (uintptr_t)dQ_branch | (uintptr_t)dK | (uintptr_t)dV;
     if (ba_use_tc(plan, accumulate != 0, addresses))
-        return ba_tc_bwd(plan, r, qm, q_branch, k, v, LSE, delta, dO, accumulate, dQ_main, dQ_branch, dK,
+        return ba_tc_bwd(plan, r, qm, q_branch, k, v, delta, dO, accumulate, dQ_main, dQ_branch, dK,
                          dV, st, stages);
     return ba_simt_bwd(plan, r, qm, q_branch, k, v, LSE, delta, dO, accumulate, dQ_main, dQ_branch, dK, dV,
                        st, stages);
@@ -245,7 +245,7 @@ extern "C" int branch_attn_bwd_depth(const ba_plan_t *plan, int depth, const voi
     if ((rc = ba_delta(O_depth, dO_depth, LSE_depth, delta, nlse2, plan->row_pitch, 0, 0, br_begin, br_end,
                        pr.h_q, pr.head_dim, pr.dtype, st)) != BA_OK)
         return rc;
-    return ba_tc_bwd(plan, r, nullptr, q_depth, k, v, LSE_depth, delta, dO_depth, 1, nullptr, dQ_depth, dK, dV, st,
+    return ba_tc_bwd(plan, r, nullptr, q_depth, k, v, delta, dO_depth, 1, nullptr, dQ_depth, dK, dV, st,
                      BA_STAGE_DQ | BA_STAGE_DKDV, depth);
 }
 

@@ -85,7 +85,7 @@ int ba_simt_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const v
                 const void *k, const void *v, const float *lse, const float *delta,
                 const void *d_o, int accumulate, void *dq_main, void *dq_branch, void *dk,
                 void *dv, cudaStream_t st, int stages);
-// Tensor-core path (ba_tc_fwd.cu / ba_tc_bwd.cu)
+// Tensor-core path (ba_tc_fwd.cu / ba_tc_bwd.cu / ba_tc_dkdv.cu)
 // partial_out: 0 = final layout in the input dtype, 1 = compact fp32, 2 = compact fp32 merged in place
 // depth > 0: step-major call (queries = the depth-`depth` tokens of branches [r.tok_begin, r.tok_end),
 // q_branch / o / lse indexed by branch, branch keys stored depth-major after the main rows)
@@ -93,7 +93,7 @@ int ba_tc_fwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
               const void *k, const void *v, void *o, float *lse, int partial_out,
               cudaStream_t st, int depth = 0);
 int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const void *q_branch,
-              const void *k, const void *v, const float *lse, const float *delta,
+              const void *k, const void *v, const float *delta,
               const void *d_o, int accumulate, void *dq_main, void *dq_branch, void *dk,
               void *dv, cudaStream_t st, int stages, int depth = 0);
 // One-kernel backward (ba_tc_bwd_fused.cu): dq_* are fp32 accumulators (atomic adds) in either mode

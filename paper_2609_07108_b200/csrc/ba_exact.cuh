@@ -15,8 +15,6 @@
 
 #include "ba_common.cuh"
 
-namespace {
-
 // What the sums read.
 struct RowArgs {
     BaMeta meta;
@@ -27,6 +25,8 @@ struct RowArgs {
     int h_q, h_kv, group;
     float scale, scale_log2;
 };
+
+namespace {
 
 template <int C> struct Cols {
     float v[C];

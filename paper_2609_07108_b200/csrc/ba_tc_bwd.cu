@@ -1,4 +1,4 @@
-// Tensor-core backward (sm_100a, bf16, head_dim 64 or 128): dQ and dK/dV kernels.
+// Tensor-core backward (sm_100a, bf16): dQ at head_dim 64 and 128, dK/dV at head_dim 64 (128: ba_tc_dkdv.cu).
 //
 // Gradients of the attention of paper Section 3.2, accumulated over key chunks
 // ("replays the same K/V ring and accumulates gradients locally").  With the
@@ -57,18 +57,6 @@ struct TcDqParams : ItemParams {
     int accumulate, wide;             // wide: bf16 gradients are 32-byte aligned
     int *status;
 };
-
-// One warp: gradient rows [row0, row0 + rows) x heads [h0, h0 + heads) that receive no term (bf16: zeros;
-// accumulated: unchanged)
-template <int D> __device__ void store_zero_rows(void *dst, int accumulate, int row0, int rows, int h0, int heads, int h_all, int lane) {
-    if (accumulate) return;
-    constexpr int kChunks = D / 8;        // 16 bytes each
-    for (int idx = lane; idx < rows * heads * kChunks; idx += 32) {
-        const int r = idx / kChunks;
-        const int64_t o = (int64_t)(row0 + r / heads) * h_all + h0 + r % heads;
-        reinterpret_cast<uint4 *>(dst)[o * kChunks + idx % kChunks] = make_uint4(0u, 0u, 0u, 0u);
-    }
-}
 
 // P = 2^(s * sl2 + neg_lse2) for one 32-column chunk, as 16 packed bf16 pairs (invisible columns: 0)
 template <bool MASKED>
@@ -568,7 +556,7 @@ tc_dq_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
 
 
 // ============================================================================
-// 64-row streamed tiles: dK / dV (head_dim 64 and 128), dQ (head_dim 64)
+// head_dim 64: 64-row streamed tiles, dQ and dK/dV
 // ============================================================================
 // A CTA keeps 128 stationary rows (pair st1, st2) in shared memory and their gradients (fp32) in TMEM and
 // walks the rows of the other side that can see them, or that they see, as 64-row tiles (pair x1, x2):
@@ -579,16 +567,16 @@ tc_dq_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
 //   acc1 += dS x1 (dK / dQ), acc2 += P x2 (dV); P, dS are TMEM A operands.
 // Two tiles are in flight (sets 0 / 1, one P / dS warpgroup each).  CTAs fetch further items as in the forward: the
 // next stationary pair is loaded and its first S, dP formed behind the last steps and the output of the current
-// item (set-up, first loads and output took 7 us per CTA, a quarter of the time of the smaller calls: dK/dV of 512
-// blocks of 16 on 32,768 tokens, draft rows, 439 -> 387 us; dQ of the head_dim 64 batch below 285 -> 205).
-//   TMEM: acc1 [0,D) acc2 [D,2D); set b: XS_b = 256 + 128 b (64 cols: S, its first 32 columns then hold P as
-//   bf16), XD_b = XS_b + 64 (dP, then dS); head_dim 64: P_lo, dS_lo of set b in 32 columns each from 128 + 64 b.
-// head_dim 64 runs in place of plain-FMA kernels that kept P and dS in fp32.  P and dS go in as bf16 pairs hi + lo (16
+// item (dQ of the batch below 285 -> 205 us).
+//   TMEM: acc1 [0,64) acc2 [64,128); set b: XS_b = 256 + 128 b (64 cols: S, its first 32 columns then hold P as
+//   bf16), XD_b = XS_b + 64 (dP, then dS); P_lo, dS_lo of set b in 32 columns each from 128 + 64 b.
+// This runs in place of plain-FMA kernels that kept P and dS in fp32.  P and dS go in as bf16 pairs hi + lo (16
 // bits of mantissa), two products each: against fp64, gradients rounded to bf16 are then off by what those kernels'
 // are (dQ, dK, dV 1.64e-3 .. 1.66e-3 in the 2-norm, the same to 1 part in 10,000).  Gradients accumulated in fp32
 // would not be, so they stay with those kernels (ba_use_tc).  4,096 tokens, 6 sequences, chains of three, 32/8 heads:
-// dQ / dK/dV 189 / 342 us (were 3052 / 8978).
-// dQ at head_dim 64 is here and not in tc_dq_kernel because that kernel was written for 128 columns of dQ and keeps P
+// dQ / dK/dV 189 / 342 us (were 3052 / 8978).  The 128-row tiles of ba_tc_dkdv.cu take 359 us for that dK/dV against
+// 336: twice the conversions per flop make the warps the limit, and two tiles in flight hide them better.
+// dQ is here and not in tc_dq_kernel because that kernel was written for 128 columns of dQ and keeps P
 // in registers as bf16; a form of it with hi + lo pairs has not been tried.
 //
 // Key tiles of dK/dV differ in length (causal) and are few in small batches: the CTAs of a cluster then share
@@ -621,8 +609,9 @@ struct KvItem {
     int ma, ba;                  // first rows of the two parts' tiles
 };
 
-template <int D> struct KvSmem {
-    static constexpr uint32_t kStatBytes = kTile * D * 2, kSubBytes = kSub * D * 2;
+constexpr int kD = 64;
+struct KvSmem {
+    static constexpr uint32_t kStatBytes = kTile * kD * 2, kSubBytes = kSub * kD * 2;
     alignas(1024) uint8_t st1[kStatBytes];
     alignas(1024) uint8_t st2[kStatBytes];
     alignas(1024) uint8_t xs[kQStages][2 * kSubBytes];  // x1 tile, then x2 tile
@@ -636,16 +625,12 @@ template <int D> struct KvSmem {
     uint32_t tmem_base;
     int abort_flag;
 };
-static_assert(sizeof(KvSmem<128>) <= 232448, "shared memory of the dK/dV kernel");
+static_assert(sizeof(KvSmem) <= 232448, "shared memory of the head_dim 64 backward");
 static_assert(kQStages * 2 * kSub * 2 == 2 * kTile * 4, "a cluster's partial accumulators fill the streamed stages exactly");
 
-__device__ __forceinline__ uint32_t bf16_rest(float2 x, uint32_t hi) {    // x - hi as a bf16 pair
-    return pack_bf16(x.x - __uint_as_float(hi << 16), x.y - __uint_as_float(hi & 0xffff0000u));
-}
-
-// 16 columns of a tile: P and dS as 8 packed bf16 pairs each (HL: and the pairs of what rounding left);
+// 16 columns of a tile: P and dS as 8 packed bf16 pairs each, and the pairs of what rounding left;
 // COLS: nl / dl point at the columns' -lse2 and delta in shared memory, otherwise they are the row's own
-template <bool MASKED, bool COLS, bool HL>
+template <bool MASKED, bool COLS>
 __device__ __forceinline__ void quarter_pds(const uint32_t (&rs)[16], const uint32_t (&rd)[16], uint32_t mk, float sl2,
                                             const float *nl, const float *dl, float row_nl, float row_dl,
                                             uint32_t (&pk)[8], uint32_t (&dk8)[8], uint32_t (&pl)[8], uint32_t (&dl8)[8]) {
@@ -682,12 +667,10 @@ __device__ __forceinline__ void quarter_pds(const uint32_t (&rs)[16], const uint
         pk[q + 1] = pack_bf16(p1.x, p1.y);
         dk8[q] = pack_bf16(d0.x, d0.y);
         dk8[q + 1] = pack_bf16(d1.x, d1.y);
-        if (HL) {
-            pl[q] = bf16_rest(p0, pk[q]);
-            pl[q + 1] = bf16_rest(p1, pk[q + 1]);
-            dl8[q] = bf16_rest(d0, dk8[q]);
-            dl8[q + 1] = bf16_rest(d1, dk8[q + 1]);
-        }
+        pl[q] = bf16_rest(p0, pk[q]);
+        pl[q + 1] = bf16_rest(p1, pk[q + 1]);
+        dl8[q] = bf16_rest(d0, dk8[q]);
+        dl8[q + 1] = bf16_rest(d1, dk8[q + 1]);
     }
 }
 
@@ -723,7 +706,7 @@ template <int MODE> __device__ void make_kv_item(const TcBwdParams &p, uint32_t 
     }
     const bool is_main = tile < (kDq ? p.main_tiles : p.main_key_tiles);
     it.is_main = is_main;
-    int step, kdepth = 0;
+    int step;
     if (kDq) {
         step = p.tok;
         it.row0 = is_main ? (int)p.r.qm_begin + tile * step : (int)p.r.tok_begin + (tile - p.main_tiles) * step;
@@ -732,12 +715,11 @@ template <int MODE> __device__ void make_kv_item(const TcBwdParams &p, uint32_t 
         int bt = tile - p.main_key_tiles;
         if (!is_main && S > 1) bt = bt * S + rank;           // a cluster holds S branch key tiles
         const bool past = !is_main && bt >= p.branch_key_tiles;      // the last cluster has ranks to spare: no rows
-        if (!is_main && p.depth) { kdepth = bt / p.branch_tiles_per_depth; bt %= p.branch_tiles_per_depth; }
         step = is_main ? kTile : p.step_kb;
         it.row0 = is_main ? (int)p.r.kv_begin + tile * step : (int)p.r.tok_begin + bt * step;
         it.row_end = past ? it.row0 : min(it.row0 + step, (int)(is_main ? p.r.kv_end : p.r.tok_end));
     }
-    it.srow0 = is_main ? it.row0 - (kDq ? 0 : (int)p.r.kv_base) : n + (kDq ? 0 : kdepth * p.num_branches) + it.row0;
+    it.srow0 = is_main ? it.row0 - (kDq ? 0 : (int)p.r.kv_base) : n + it.row0;
     it.m0 = it.m1 = it.b0 = it.b1 = 0;
     const int first = it.row0, last = it.row_end - 1;
     if (last >= first) {
@@ -756,9 +738,6 @@ template <int MODE> __device__ void make_kv_item(const TcBwdParams &p, uint32_t 
                 }
                 it.b0 = p.meta.key_bq_begin[first];
                 it.b1 = p.meta.key_bq_end[last];
-                if (p.depth) { it.b0 /= p.branch_len; it.b1 /= p.branch_len; }    // token ranges -> branch ranges
-            } else if (p.depth) {
-                it.b0 = first; it.b1 = last + 1;             // seen by the query of its own branch only
             } else {
                 it.b0 = p.meta.br_start[first];
                 it.b1 = p.meta.br_end[last];
@@ -770,9 +749,8 @@ template <int MODE> __device__ void make_kv_item(const TcBwdParams &p, uint32_t 
     // In dK/dV the streamed tiles start at ma / ba: the parts' starts moved back (by < 4 rows) so that every
     // tile's first row is a multiple of 4 in the row numbering of the per-row scalars, whose bulk copies are then
     // 16-byte aligned.  The extra leading rows are masked like any other invisible row.
-    const int qbase = p.depth ? 0 : n;
     it.ma = kDq ? it.m0 : it.m0 & ~3;
-    it.ba = kDq ? it.b0 : ((qbase + it.b0) & ~3) - qbase;   // may be as low as -3
+    it.ba = kDq ? it.b0 : ((n + it.b0) & ~3) - n;   // may be as low as -3
     it.n_sub_main = it.m1 > it.m0 ? (it.m1 - it.ma + kSub - 1) / kSub : 0;
     it.n_sub = it.n_sub_main + (it.b1 > it.b0 ? (it.b1 - it.ba + kSub - 1) / kSub : 0);
     const int n_all = it.n_sub * (kDq ? 1 : p.group);
@@ -783,29 +761,27 @@ template <int MODE> __device__ void make_kv_item(const TcBwdParams &p, uint32_t 
     it.hh_beg = it.n_sub > 0 ? t_beg / it.n_sub : 0;
 }
 
-template <int D, int MODE, bool SPLIT>
+template <int MODE, bool SPLIT>
 __global__ void __launch_bounds__(kKvThreads, 1)
 tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constant__ CUtensorMap tm_q_branch,
              const __grid_constant__ CUtensorMap tm_go, const __grid_constant__ CUtensorMap tm_k,
              const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_go_branch,
              const __grid_constant__ TcBwdParams p) {
-    using Smem = KvSmem<D>;
-    constexpr bool kDq = MODE == kModeDq, kHL = D == 64;
+    using Smem = KvSmem;
+    constexpr bool kDq = MODE == kModeDq;
+    constexpr int D = kD;
     constexpr uint32_t kSubBytes = Smem::kSubBytes;
-    constexpr int kHalves = D / 64;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     volatile int *abort_flag = &sm.abort_flag;
-    constexpr long long kLimit = D == 64 ? kSlowWaitLimitCycles : kWaitLimitCycles;
+    constexpr long long kLimit = kSlowWaitLimitCycles;
     if (smem_u32(smem_raw) & 1023u) {   // the swizzled tiles need 1024-byte alignment
         if (tid == 0) atomicExch(p.status, BA_EUNSUPPORTED);
         return;
     }
     const int S = SPLIT ? p.splits : 1, rank = SPLIT ? (int)(blockIdx.x % S) : 0;
-    // global row number of branch query 0 (rows of dO and of the per-row scalars): branch rows follow the main
-    // rows, except in depth mode, where those tensors hold one row per branch
-    const int qbase = p.depth ? 0 : (int)p.meta.n_main;
+    const int n = (int)p.meta.n_main;      // global row number of branch row 0
 
     if (tid == 0) {
         mbar_init(&sm.st_full, 1); mbar_init(&sm.st_empty, 1);
@@ -831,7 +807,6 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sm.tmem_base;
-    const int accumulate = D == 128 ? p.accumulate : 0;      // head_dim 64: bf16 gradients only (ba_use_tc)
     bool shared_tile = false;      // SPLIT: this CTA walked a part of a main key tile
 
     if (warp >= 8) {
@@ -859,11 +834,11 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                     const KvItem &it = sm.item[s];
                     const int rows = it.row_end - it.row0;
                     if (kDq) {
-                        store_zero_rows<D>(it.is_main ? p.dq_main : p.dq_branch, accumulate, it.row0, rows, it.h0,
+                        store_zero_rows<D>(it.is_main ? p.dq_main : p.dq_branch, 0, it.row0, rows, it.h0,
                                          min(p.hp, (it.g + 1) * p.group - it.h0), p.h_q, lane);
                     } else {
-                        store_zero_rows<D>(p.dk, accumulate, it.srow0, rows, it.g, 1, p.h_kv, lane);
-                        store_zero_rows<D>(p.dv, accumulate, it.srow0, rows, it.g, 1, p.h_kv, lane);
+                        store_zero_rows<D>(p.dk, 0, it.srow0, rows, it.g, 1, p.h_kv, lane);
+                        store_zero_rows<D>(p.dv, 0, it.srow0, rows, it.g, 1, p.h_kv, lane);
                     }
                 } else {
                     if (lane == 0) mbar_arrive(&sm.item_full[s]);
@@ -922,23 +897,19 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                         if (lane == 0) {
                             const int kr = seg_main ? r0 - (int)p.r.kv_base : (int)p.meta.n_main + r0;
                             mbar_expect_tx(&sm.x_full[st], 2 * kSubBytes);
-                            for (int half = 0; half < kHalves; ++half) {
-                                tma_load_3d(sm.xs[st] + half * 8192, &tm_k, half * 64, it.g, kr, &sm.x_full[st]);
-                                tma_load_3d(sm.xs[st] + kSubBytes + half * 8192, &tm_v, half * 64, it.g, kr, &sm.x_full[st]);
-                            }
+                            tma_load_3d(sm.xs[st], &tm_k, 0, it.g, kr, &sm.x_full[st]);
+                            tma_load_3d(sm.xs[st] + kSubBytes, &tm_v, 0, it.g, kr, &sm.x_full[st]);
                         }
                     } else {
                         const int h = it.g * p.group + hh;
-                        const int gr0 = seg_main ? r0 : qbase + r0;
+                        const int gr0 = seg_main ? r0 : n + r0;
                         if (lane == 0) {
                             // A branch tile may start up to three rows before branch row 0: dO by the map that has no rows
                             // there.  (By that map for every branch tile: 129 us instead of 126 at 2,048 tokens.)
                             const CUtensorMap *tq = seg_main ? &tm_q_main : &tm_q_branch, *tg = r0 >= 0 ? &tm_go : &tm_go_branch;
                             mbar_expect_tx(&sm.x_full[st], 2 * kSubBytes + 2 * kSub * 4);
-                            for (int half = 0; half < kHalves; ++half) {
-                                tma_load_3d(sm.xs[st] + half * 8192, tq, half * 64, h, r0, &sm.x_full[st]);
-                                tma_load_3d(sm.xs[st] + kSubBytes + half * 8192, tg, half * 64, h, r0 >= 0 ? gr0 : r0, &sm.x_full[st]);
-                            }
+                            tma_load_3d(sm.xs[st], tq, 0, h, r0, &sm.x_full[st]);
+                            tma_load_3d(sm.xs[st] + kSubBytes, tg, 0, h, r0 >= 0 ? gr0 : r0, &sm.x_full[st]);
                             const size_t off = (size_t)h * p.row_pitch + gr0;
                             bulk_load(mt.neg_lse2, p.nlse2_t + off, kSub * 4, &sm.x_full[st]);
                             bulk_load(mt.delta, p.delta_t + off, kSub * 4, &sm.x_full[st]);
@@ -946,18 +917,16 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                                 const int h2 = it.g * p.group + ph;
                                 const bool main2 = ps < it.n_sub_main;
                                 const int r2 = main2 ? it.ma + ps * kSub : it.ba + (ps - it.n_sub_main) * kSub;
-                                const int g2 = main2 ? r2 : qbase + r2;
+                                const int g2 = main2 ? r2 : n + r2;
                                 const CUtensorMap *tq2 = main2 ? &tm_q_main : &tm_q_branch;
-                                for (int half = 0; half < kHalves; ++half) {
-                                    tma_prefetch_3d(tq2, half * 64, h2, r2);
-                                    tma_prefetch_3d(&tm_go, half * 64, h2, g2);
-                                }
+                                tma_prefetch_3d(tq2, 0, h2, r2);
+                                tma_prefetch_3d(&tm_go, 0, h2, g2);
                                 const size_t off2 = (size_t)h2 * p.row_pitch + g2;
                                 bulk_prefetch(p.nlse2_t + off2, kSub * 4);
                                 bulk_prefetch(p.delta_t + off2, kSub * 4);
                             }
                         }
-                        if (!it.is_main && !p.depth) {
+                        if (!it.is_main) {
                             // own-branch tiles: branch start and mask of each query token
                             for (int c = lane; c < kSub; c += 32) {
                                 const int tok = r0 + c;
@@ -978,16 +947,12 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                             if (kDq) {
                                 const CUtensorMap *tq = it.is_main ? &tm_q_main : &tm_q_branch;
                                 mbar_expect_tx(&sm.st_full, (uint32_t)(2 * p.hp * p.tok * D * 2));
-                                for (int half = 0; half < kHalves; ++half) {
-                                    tma_load_3d(sm.st1 + half * 16384, tq, half * 64, it.h0, it.row0, &sm.st_full);
-                                    tma_load_3d(sm.st2 + half * 16384, &tm_go, half * 64, it.h0, it.srow0, &sm.st_full);
-                                }
+                                tma_load_3d(sm.st1, tq, 0, it.h0, it.row0, &sm.st_full);
+                                tma_load_3d(sm.st2, &tm_go, 0, it.h0, it.srow0, &sm.st_full);
                             } else {
                                 mbar_expect_tx(&sm.st_full, 2 * Smem::kStatBytes);
-                                for (int half = 0; half < kHalves; ++half) {
-                                    tma_load_3d(sm.st1 + half * 16384, &tm_k, half * 64, it.g, it.srow0, &sm.st_full);
-                                    tma_load_3d(sm.st2 + half * 16384, &tm_v, half * 64, it.g, it.srow0, &sm.st_full);
-                                }
+                                tma_load_3d(sm.st1, &tm_k, 0, it.g, it.srow0, &sm.st_full);
+                                tma_load_3d(sm.st2, &tm_v, 0, it.g, it.srow0, &sm.st_full);
                             }
                         }
                         ++n_st;
@@ -1079,10 +1044,8 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                     tc_fence_after();
                     if (!kDq) issue_acc(tmem + D, xs, stage_mn + kHalfStage, !s0.first);     // dV += P^T dO
                     issue_acc(tmem, xs + 64, stage_mn, !s0.first);                           // dK += dS^T Q / dQ += dS K
-                    if (kHL) {
-                        if (!kDq) issue_acc(tmem + D, tmem + 128 + b * 64, stage_mn + kHalfStage, true);
-                        issue_acc(tmem, tmem + 128 + b * 64 + 32, stage_mn, true);
-                    }
+                    if (!kDq) issue_acc(tmem + D, tmem + 128 + b * 64, stage_mn + kHalfStage, true);         // + P_lo, dS_lo
+                    issue_acc(tmem, tmem + 128 + b * 64 + 32, stage_mn, true);
                     tc_commit(&sm.x_empty[t % kQStages]);
                     if (s0.last) {
                         tc_commit(&sm.acc_full);
@@ -1146,9 +1109,6 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                     f.hi = p.meta.key_qend[f.row] - 1;
                     f.rb0 = p.meta.key_bq_begin[f.row];
                     f.rb1 = p.meta.key_bq_end[f.row];
-                    if (p.depth) { f.rb0 /= p.branch_len; f.rb1 /= p.branch_len; }
-                } else if (p.depth) {
-                    f.rb0 = f.row; f.rb1 = f.row + 1;
                 } else {
                     f.rb0 = p.meta.br_start[f.row];
                     f.rb1 = p.meta.br_end[f.row];
@@ -1180,9 +1140,9 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                 if (w.valid) {
                     if (kDq) {
                         vis = seg_main ? bit_range(w.lo - r0, w.hi - r0) : shift_mask(w.mask, r0 - w.rb0);
-                    } else if (w.is_main || p.depth) {
+                    } else if (w.is_main) {
                         // main rows: same sequence, causal: key <= row < end of the key's sequence; branch tokens
-                        // anchored at or after the key, inside its sequence (depth mode: branches)
+                        // anchored at or after the key, inside its sequence
                         const int v0 = seg_main ? w.lo : w.rb0, v1 = seg_main ? w.hi + 1 : w.rb1;
                         const int rbeg = seg_main ? w.m0 : w.b0, rend = seg_main ? w.m1 : w.b1;
                         vis = bit_range(max(v0, rbeg) - r0, min(v1, rend) - 1 - r0);
@@ -1205,14 +1165,12 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                     auto quarters = [&](auto msk) {
                         constexpr bool MASKED = decltype(msk)::value;
                         auto quarter = [&](const uint32_t (&rs)[16], const uint32_t (&rd)[16], int q) {
-                            quarter_pds<MASKED, !kDq, kHL>(rs, rd, (uint32_t)(vis >> (16 * q)) & 0xffffu, sl2, mt.neg_lse2 + 16 * q,
+                            quarter_pds<MASKED, !kDq>(rs, rd, (uint32_t)(vis >> (16 * q)) & 0xffffu, sl2, mt.neg_lse2 + 16 * q,
                                                            mt.delta + 16 * q, w.nl, w.dl, pk, dk8, pl, dl8);
                             if (!kDq) tmem_st8(xs_addr + 8 * q, pk);
                             tmem_st8(xd_addr + 8 * q, dk8);
-                            if (kHL) {
-                                if (!kDq) tmem_st8(lo_addr + 8 * q, pl);
-                                tmem_st8(lo_addr + 32 + 8 * q, dl8);
-                            }
+                            if (!kDq) tmem_st8(lo_addr + 8 * q, pl);
+                            tmem_st8(lo_addr + 32 + 8 * q, dl8);
                         };
                         tmem_ld16(xs_addr, sa);
                         tmem_ld16(xd_addr, da);
@@ -1269,7 +1227,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                 }
                 bool not_finite = false;
                 uint64_t nans = 0;
-                if (D == 64 && !shared_tile) {
+                if (!shared_tile) {
                     const float s = sum32(r);
                     not_finite = __any_sync(0xffffffffu, w.valid && s != s);
                     if (not_finite && w.valid) nans = nan_mask(r);
@@ -1281,10 +1239,9 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                             make_float4(__uint_as_float(r[4 * e]), __uint_as_float(r[4 * e + 1]), __uint_as_float(r[4 * e + 2]),
                                         __uint_as_float(r[4 * e + 3]));
                 } else if (w.valid) {
-                    if (accumulate) store_grad_chunk<true>(dst, base + c * 32, r, mul);
-                    else store_grad_chunk<false>(dst, base + c * 32, r, mul, p.wide);
+                    store_grad_chunk<false>(dst, base + c * 32, r, mul, p.wide);
                 }
-                if (D == 64 && not_finite) {      // does it hold rows out of its reach (ba_exact.cuh; bf16 results only)?
+                if (not_finite) {      // does it hold rows out of its reach (ba_exact.cuh; bf16 results only)?
                     __nv_bfloat16 *row = (__nv_bfloat16 *)dst + base + c * 32;
                     if (kDq) repair_query_row<true, 8>(p.rows, w.is_main, w.row, w.h, w.g, w.nl, b * 32, 32, nans, mul, row);
                     else repair_key_row<8>(p.rows, w.is_main, w.row, w.g, b == 1, c * 32, 32, nans, mul, row);
@@ -1319,16 +1276,10 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                 x.x *= mul; x.y *= mul; x.z *= mul; x.w *= mul;
                 void *dst = which == 0 ? p.dk : p.dv;
                 const size_t off = ((size_t)(it.srow0 + r) * p.h_kv + it.g) * D + ch * 4;
-                if (accumulate) {
-                    float4 *d4 = reinterpret_cast<float4 *>((float *)dst + off);
-                    const float4 o = *d4;
-                    *d4 = make_float4(o.x + x.x, o.y + x.y, o.z + x.z, o.w + x.w);
-                } else {
-                    *reinterpret_cast<uint2 *>((__nv_bfloat16 *)dst + off) = make_uint2(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w));
-                }
-                if (D == 64) chk += x.x + x.y + x.z + x.w;
+                *reinterpret_cast<uint2 *>((__nv_bfloat16 *)dst + off) = make_uint2(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w));
+                chk += x.x + x.y + x.z + x.w;
             }
-            if (D == 64 && __any_sync(0xffffffffu, chk != chk)) {      // do they hold rows out of their reach (ba_exact.cuh; bf16 results only)?
+            if (__any_sync(0xffffffffu, chk != chk)) {      // do they hold rows out of their reach (ba_exact.cuh; bf16 results only)?
 #pragma unroll 1
                 for (int idx = tid; idx < 2 * rows_mine * (D / 4); idx += 256) {
                     const int ch = idx % (D / 4), rr = idx / (D / 4), which = rr / rows_mine, r = rank * rows_mine + rr % rows_mine;
@@ -1347,21 +1298,22 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
     tc_fence_before();
     __syncthreads();
     if (warp == 8) tmem_dealloc(tmem, 512);
-    if (!kDq) wait_prerequisites();      // never done before the dQ kernel that it may overlap
     if (tid == 0 && sm.abort_flag) atomicExch(p.status, BA_ETIMEOUT);
 }
 
-template <int D, int MODE, bool SPLIT>
-int launch_kv_as(const TcBwdParams &p, const CUtensorMap *tm, int64_t grid, bool after_dq, int dev, cudaStream_t st) {
+template <int MODE, bool SPLIT>
+int launch_kv(const TcBwdParams &p, const CUtensorMap *tm, int64_t grid, int dev, cudaStream_t st) {
+    if (grid <= 0) return BA_OK;
+    if (grid > INT_MAX) return BA_EUNSUPPORTED;
     // the dynamic shared-memory limit is a per-device attribute of the kernel
     static bool attr_set[64] = {};
-    const size_t smem = sizeof(KvSmem<D>);
+    const size_t smem = sizeof(KvSmem);
     if (!attr_set[dev]) {
         // the register re-split hands out what a launch with kKvRegsLaunch registers per thread owns
         cudaFuncAttributes fa;
-        BA_CUDA_CHECK(cudaFuncGetAttributes(&fa, tc_kv_kernel<D, MODE, SPLIT>));
+        BA_CUDA_CHECK(cudaFuncGetAttributes(&fa, tc_kv_kernel<MODE, SPLIT>));
         if (fa.numRegs * kKvThreads < 256 * kKvRegsCompute + 128 * kKvRegsIssue) return BA_EUNSUPPORTED;
-        BA_CUDA_CHECK(cudaFuncSetAttribute(tc_kv_kernel<D, MODE, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        BA_CUDA_CHECK(cudaFuncSetAttribute(tc_kv_kernel<MODE, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         attr_set[dev] = true;
     }
     cudaLaunchConfig_t cfg;
@@ -1370,168 +1322,87 @@ int launch_kv_as(const TcBwdParams &p, const CUtensorMap *tm, int64_t grid, bool
     cfg.blockDim = dim3(kKvThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    if (SPLIT) {
-        attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
-        attr[cfg.numAttrs].val.clusterDim.x = (unsigned)p.splits;
-        attr[cfg.numAttrs].val.clusterDim.y = attr[cfg.numAttrs].val.clusterDim.z = 1;
-        ++cfg.numAttrs;
-    }
-    if (after_dq) {     // start when every CTA of the dQ kernel queued just before has started or been taken over
-        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
-        ++cfg.numAttrs;
-    }
-    cfg.attrs = attr;
-    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_kv_kernel<D, MODE, SPLIT>, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], p));
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)p.splits;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = SPLIT ? 1 : 0;
+    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_kv_kernel<MODE, SPLIT>, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], p));
     return ba_check_launch();
-}
-
-template <int D, int MODE>
-int launch_kv(const TcBwdParams &p, const CUtensorMap *tm, int64_t grid, bool after_dq, int dev, cudaStream_t st) {
-    if (grid <= 0) return BA_OK;
-    if (grid > INT_MAX) return BA_EUNSUPPORTED;
-    if (MODE == kModeDkdv && p.splits > 1) return launch_kv_as<D, kModeDkdv, true>(p, tm, grid, after_dq, dev, st);
-    return launch_kv_as<D, MODE, false>(p, tm, grid, after_dq, dev, st);
 }
 
 }  // namespace
 
 int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const void *q_branch, const void *k,
-              const void *v, const float *lse, const float *delta, const void *d_o, int accumulate,
+              const void *v, const float *delta, const void *d_o, int accumulate,
               void *dq_main, void *dq_branch, void *dk, void *dv, cudaStream_t st, int stages, int depth) {
     // depth > 0: dQ is written (bf16, one row per branch), dK / dV accumulate
     int dev = 0;
     BA_CUDA_CHECK(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return BA_EUNSUPPORTED;
     const ba_problem_t &pr = pl->prob;
-    const int D = pr.head_dim;
-    TcBwdParams p;
-    memset(&p, 0, sizeof p);
-    p.meta = pl->meta;
-    p.r = r;
-    (void)lse;
-    p.delta_t = delta;
-    p.nlse2_t = delta + (size_t)pl->row_pitch * pr.h_q;
-    p.row_pitch = pl->row_pitch;
-    p.dq_main = dq_main; p.dq_branch = dq_branch; p.dk = dk; p.dv = dv;
-    p.h_q = pr.h_q; p.h_kv = pr.h_kv;
-    p.group = pr.h_q / pr.h_kv;
-    p.scale = pl->scale;
-    p.scale_log2 = pl->scale * kLog2e;
-    p.accumulate = accumulate;
-    p.wide = (((uintptr_t)dq_main | (uintptr_t)dq_branch | (uintptr_t)dk | (uintptr_t)dv) & 31) == 0;
-    p.has_main_q = q_main != nullptr;
-    p.status = pl->dev_status;
-    p.splits = 1;
-    p.rows.meta = pl->meta; p.rows.r = r;
-    p.rows.q_main = q_main; p.rows.q_branch = q_branch; p.rows.k = k; p.rows.v = v; p.rows.d_o = d_o;
-    p.rows.nlse2_t = p.nlse2_t; p.rows.delta_t = p.delta_t; p.rows.row_pitch = p.row_pitch;
-    p.rows.h_q = p.h_q; p.rows.h_kv = p.h_kv; p.rows.group = p.group;
-    p.rows.scale_log2 = p.scale_log2;
-
-    // depth mode: key rows of depths <= depth only (later rows read as zero); Q, dO hold one row per branch
-    p.depth = depth;
-    p.num_branches = pr.num_branches;
-    p.branch_len = pr.uniform_len;
-    const uint64_t all_rows = (uint64_t)(pr.n_main + pr.n_branch);
-    // (without own-branch keys nothing beyond kv_end is needed: a received shard ends there)
-    const uint64_t kv_rows = depth ? (uint64_t)(pr.n_main + (int64_t)depth * pr.num_branches)
-                             : (r.parts & BA_PART_BRANCH) ? all_rows : (uint64_t)(r.kv_end > r.kv_base ? r.kv_end - r.kv_base : 1);
-    const uint64_t go_rows = depth ? (uint64_t)pr.num_branches : all_rows;
-    const void *qm = q_main ? q_main : q_branch;
-    const void *qb = (q_branch && pr.n_branch > 0) ? q_branch : q_main;
-    const uint64_t qm_rows = depth ? (uint64_t)pr.num_branches : q_main ? (uint64_t)pr.n_main : (uint64_t)pr.n_branch;
-    const uint64_t qb_rows = depth ? (uint64_t)pr.num_branches
-                             : (q_branch && pr.n_branch > 0) ? (uint64_t)pr.n_branch : (uint64_t)pr.n_main;
-    // dO of the branch rows alone: whatever lies in front of branch row 0 (rows of dO that a call without main
-    // queries leaves unset) is not loaded
-    const bool go_split = !depth && pr.n_branch > 0;
-    const void *gob = go_split ? (const char *)d_o + (size_t)pr.n_main * pr.h_q * D * 2 : d_o;
-    const uint64_t gob_rows = go_split ? (uint64_t)pr.n_branch : go_rows;
-    // maps in the order q_main, q_branch, dO, K, V, branch rows of dO; boxes of `qr` query rows x `qh` heads and
-    // `kr` key rows
-    auto maps = [&](CUtensorMap *tm, uint32_t qr, uint32_t qh, uint32_t kr) {
-        return make_tmap_rhd(&tm[0], qm, qm_rows, pr.h_q, D, qr, qh) && make_tmap_rhd(&tm[1], qb, qb_rows, pr.h_q, D, qr, qh) &&
-               make_tmap_rhd(&tm[2], d_o, go_rows, pr.h_q, D, qr, qh) && make_tmap_rhd(&tm[3], k, kv_rows, pr.h_kv, D, kr) &&
-               make_tmap_rhd(&tm[4], v, kv_rows, pr.h_kv, D, kr) && make_tmap_rhd(&tm[5], gob, gob_rows, pr.h_q, D, qr, qh);
-    };
+    TcBwdParams p = bwd_params(pl, r, q_main, q_branch, k, v, delta, d_o, accumulate, dq_main, dq_branch, dk, dv, depth);
     CUtensorMap tm[6];
+    auto maps = [&](uint32_t qr, uint32_t qh, uint32_t kr) { return bwd_maps(tm, pl, r, q_main, q_branch, k, v, d_o, depth, qr, qh, kr); };
     const int64_t qm_n = q_main ? r.qm_end - r.qm_begin : 0, br_n = r.tok_end - r.tok_begin;
-    if (stages & BA_STAGE_DQ) {
-        if (D == 64) {
+    if (pr.head_dim == 64) {
+        if (stages & BA_STAGE_DQ) {
             p.hp = p.group < kTile ? p.group : kTile;
             p.head_chunks = (p.group + p.hp - 1) / p.hp;
             p.tok = kTile / p.hp;
             p.main_tiles = (int)((qm_n + p.tok - 1) / p.tok);
             p.total_tiles = p.main_tiles + (int)((br_n + p.tok - 1) / p.tok);
-            if (!maps(tm, p.tok, p.hp, kSub)) return BA_EINVAL;
-            int rc = launch_kv<64, kModeDq>(p, tm, (int64_t)p.total_tiles * pr.h_kv * p.head_chunks, false, dev, st);
+            if (!maps(p.tok, p.hp, kSub)) return BA_EINVAL;
+            int rc = launch_kv<kModeDq, false>(p, tm, (int64_t)p.total_tiles * pr.h_kv * p.head_chunks, dev, st);
             if (rc != BA_OK) return rc;
-        } else {
-            static bool attr_set[64] = {};
-            if (!attr_set[dev]) {
-                // the register re-split hands out what a launch with kDqRegsLaunch registers per thread owns
-                cudaFuncAttributes fa;
-                BA_CUDA_CHECK(cudaFuncGetAttributes(&fa, tc_dq_kernel));
-                if (fa.numRegs * kDqThreads < 256 * kDqRegsCompute + 128 * kDqRegsIssue) return BA_EUNSUPPORTED;
-                BA_CUDA_CHECK(cudaFuncSetAttribute(tc_dq_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DqSmem)));
-                attr_set[dev] = true;
-            }
-            TcDqParams q;
-            memset(&q, 0, sizeof q);
-            const int64_t grid = fill_items(q, pl, r, q_main != nullptr, depth);
-            q.nlse2_t = p.nlse2_t; q.delta_t = p.delta_t; q.row_pitch = p.row_pitch;
-            q.dq_main = dq_main; q.dq_branch = dq_branch;
-            q.scale = p.scale; q.scale_log2 = p.scale_log2;
-            q.accumulate = depth ? 0 : accumulate;
-            q.wide = p.wide;
-            q.status = p.status;
-            if (grid > INT_MAX) return BA_EUNSUPPORTED;
-            CUtensorMap k32, v32;
-            if (!maps(tm, q.tok, q.hp, kTile) || !make_tmap_rhd(&k32, k, kv_rows, pr.h_kv, D, 32) ||
-                !make_tmap_rhd(&v32, v, kv_rows, pr.h_kv, D, 32))
-                return BA_EINVAL;
-            if (grid > 0) {
-                tc_dq_kernel<<<(unsigned)grid, kDqThreads, sizeof(DqSmem), st>>>(tm[0], tm[1], tm[2], tm[3], tm[4], k32, v32, q);
-                int rc = ba_check_launch();
-                if (rc != BA_OK) return rc;
-            }
+        }
+        if (stages & BA_STAGE_DKDV) {
+            // (both kernels overlapped, as at head_dim 128: 605 us instead of 548 for the 4,096-token chains)
+            const int64_t grid = key_items(p, pl, r, q_main != nullptr);
+            if (!maps(kSub, 1, kTile)) return BA_EINVAL;
+            return p.splits > 1 ? launch_kv<kModeDkdv, true>(p, tm, grid, dev, st) : launch_kv<kModeDkdv, false>(p, tm, grid, dev, st);
+        }
+        return BA_OK;
+    }
+    if (stages & BA_STAGE_DQ) {
+        static bool attr_set[64] = {};
+        if (!attr_set[dev]) {
+            // the register re-split hands out what a launch with kDqRegsLaunch registers per thread owns
+            cudaFuncAttributes fa;
+            BA_CUDA_CHECK(cudaFuncGetAttributes(&fa, tc_dq_kernel));
+            if (fa.numRegs * kDqThreads < 256 * kDqRegsCompute + 128 * kDqRegsIssue) return BA_EUNSUPPORTED;
+            BA_CUDA_CHECK(cudaFuncSetAttribute(tc_dq_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DqSmem)));
+            attr_set[dev] = true;
+        }
+        TcDqParams q;
+        memset(&q, 0, sizeof q);
+        const int64_t grid = fill_items(q, pl, r, q_main != nullptr, depth);
+        q.nlse2_t = p.nlse2_t; q.delta_t = p.delta_t; q.row_pitch = p.row_pitch;
+        q.dq_main = dq_main; q.dq_branch = dq_branch;
+        q.scale = p.scale; q.scale_log2 = p.scale_log2;
+        q.accumulate = depth ? 0 : accumulate;
+        q.wide = p.wide;
+        q.status = p.status;
+        if (grid > INT_MAX) return BA_EUNSUPPORTED;
+        const uint64_t kv_rows = key_rows(pl, r, depth);
+        CUtensorMap k32, v32;
+        if (!maps(q.tok, q.hp, kTile) || !make_tmap_rhd(&k32, k, kv_rows, pr.h_kv, 128, 32) ||
+            !make_tmap_rhd(&v32, v, kv_rows, pr.h_kv, 128, 32))
+            return BA_EINVAL;
+        if (grid > 0) {
+            tc_dq_kernel<<<(unsigned)grid, kDqThreads, sizeof(DqSmem), st>>>(tm[0], tm[1], tm[2], tm[3], tm[4], k32, v32, q);
+            int rc = ba_check_launch();
+            if (rc != BA_OK) return rc;
         }
     }
     if (stages & BA_STAGE_DKDV) {
-        const int64_t kmt = (r.parts & BA_PART_MAIN) ? (r.kv_end - r.kv_begin + kTile - 1) / kTile : 0;
-        p.step_kb = depth ? kTile : branch_key_step(pr.uniform_len);
-        int64_t kbt = (r.parts & BA_PART_BRANCH) ? (br_n + p.step_kb - 1) / p.step_kb : 0;
-        p.branch_tiles_per_depth = (int)kbt;
-        if (depth) kbt *= depth;    // the tokens of depths 1 .. depth of the selected branches are keys
-        p.branch_key_tiles = (int)kbt;
-        // Share main key tiles between the CTAs of a cluster until they fill the SMs once, as long as an average
-        // part keeps eight 64-row steps: 2,048 tokens, 8 KV heads (128 tiles) take 122 us whole, 130 us in two
-        // parts, 153 us in four.
-        const int64_t keys = kmt * kTile, viewers = qm_n + br_n;
-        const int64_t seq = pr.num_seqs > 0 ? pr.n_main / pr.num_seqs : 0;
-        const int64_t est = keys > 0 ? (seq < keys ? seq : keys) / 2 * viewers / (keys < pr.n_main ? pr.n_main : keys) * p.group / kSub : 0;
-        while (p.splits < 8 && kmt * pr.h_kv * p.splits * 2 <= kSms && est >= 8 * 2 * p.splits) p.splits *= 2;
-        p.main_key_tiles = (int)kmt;
-        const int64_t tiles = kmt + (kbt + p.splits - 1) / p.splits;    // work items (clusters) per KV head
-        p.total_key_tiles = (int)tiles;
-        // Up to 24 work items per SM heaviest first over all KV heads, so that the last items are short (8,192
-        // tokens with chains 830 us against 1030 KV-head-major, 32,768 tokens with blocks 1616 against 1711);
-        // beyond that KV-head-major, whose resident CTAs share one query stream through L2 (65,536-token trees 7862
-        // us against 7953, 73,728 tokens with chains 48.4 ms against 48.9).
-        p.tile_major = tiles * pr.h_kv <= 24 * kSms;
-        if (!maps(tm, kSub, 1, kTile)) return BA_EINVAL;
-        const int64_t grid = tiles * pr.h_kv * p.splits;
         // The two kernels write different tensors and need the same inputs: the second may start on the SMs that the
         // last items of the first leave idle (not when no row of dQ was launched: the kernel before is then the
         // caller's, or delta).  Both kernels, overlapped / one after the other: 2,048-token chains 222 / 231 us, draft
-        // rows of 512 blocks 658 / 680; head_dim 64, 4,096-token chains 605 / 548 (that shape alone was measured), so not
-        // there.
-        const bool after_dq = D == 128 && (stages & BA_STAGE_DQ) && qm_n + br_n > 0;
-        const int rc = D == 64 ? launch_kv<64, kModeDkdv>(p, tm, grid, after_dq, dev, st)
-                               : launch_kv<128, kModeDkdv>(p, tm, grid, after_dq, dev, st);
-        if (rc != BA_OK) return rc;
+        // rows of 512 blocks 658 / 680.
+        const bool after_dq = (stages & BA_STAGE_DQ) && qm_n + br_n > 0;
+        return ba_tc_dkdv(p, pl, r, q_main, q_branch, k, v, d_o, after_dq, dev, st);
     }
     return BA_OK;
 }

@@ -23,6 +23,8 @@ __device__ __forceinline__ uint64_t bit_range(int lo, int hi) {
     return (~0ull >> (63 - hi)) & (~0ull << lo);
 }
 
+}  // namespace
+
 struct TcBwdParams {
     BaMeta meta;
     BaRange r;
@@ -46,6 +48,8 @@ struct TcBwdParams {
     int *status;
     RowArgs rows;                     // head_dim 64: rows that are formed again one by one
 };
+
+namespace {
 
 // Branch tokens per branch key tile.  Branches of one length: a tile that starts and ends with a branch is seen
 // by its own tokens only (chains of three: 126 keys and 128 query rows instead of 128 and up to 135, which
@@ -87,4 +91,115 @@ __device__ __forceinline__ void store_grad_chunk(void *dst, size_t elem_off, con
     }
 }
 
+// One warp: gradient rows [row0, row0 + rows) x heads [h0, h0 + heads) that receive no term (bf16: zeros;
+// accumulated: unchanged)
+template <int D> __device__ void store_zero_rows(void *dst, int accumulate, int row0, int rows, int h0, int heads, int h_all, int lane) {
+    if (accumulate) return;
+    constexpr int kChunks = D / 8;        // 16 bytes each
+    for (int idx = lane; idx < rows * heads * kChunks; idx += 32) {
+        const int r = idx / kChunks;
+        const int64_t o = (int64_t)(row0 + r / heads) * h_all + h0 + r % heads;
+        reinterpret_cast<uint4 *>(dst)[o * kChunks + idx % kChunks] = make_uint4(0u, 0u, 0u, 0u);
+    }
+}
+
+__device__ __forceinline__ uint32_t bf16_rest(float2 x, uint32_t hi) {    // x - hi as a bf16 pair
+    return sm100::pack_bf16(x.x - __uint_as_float(hi << 16), x.y - __uint_as_float(hi & 0xffff0000u));
+}
+
+// What every backward kernel of a call needs
+inline TcBwdParams bwd_params(const ba_plan *pl, const BaRange &r, const void *q_main, const void *q_branch, const void *k,
+                              const void *v, const float *delta, const void *d_o, int accumulate, void *dq_main,
+                              void *dq_branch, void *dk, void *dv, int depth) {
+    const ba_problem_t &pr = pl->prob;
+    TcBwdParams p;
+    memset(&p, 0, sizeof p);
+    p.meta = pl->meta;
+    p.r = r;
+    p.delta_t = delta;
+    p.nlse2_t = delta + (size_t)pl->row_pitch * pr.h_q;
+    p.row_pitch = pl->row_pitch;
+    p.dq_main = dq_main; p.dq_branch = dq_branch; p.dk = dk; p.dv = dv;
+    p.h_q = pr.h_q; p.h_kv = pr.h_kv;
+    p.group = pr.h_q / pr.h_kv;
+    p.scale = pl->scale;
+    p.scale_log2 = pl->scale * kLog2e;
+    p.accumulate = accumulate;
+    p.wide = (((uintptr_t)dq_main | (uintptr_t)dq_branch | (uintptr_t)dk | (uintptr_t)dv) & 31) == 0;
+    p.has_main_q = q_main != nullptr;
+    p.status = pl->dev_status;
+    p.splits = 1;
+    p.rows.meta = pl->meta; p.rows.r = r;
+    p.rows.q_main = q_main; p.rows.q_branch = q_branch; p.rows.k = k; p.rows.v = v; p.rows.d_o = d_o;
+    p.rows.nlse2_t = p.nlse2_t; p.rows.delta_t = p.delta_t; p.rows.row_pitch = p.row_pitch;
+    p.rows.h_q = p.h_q; p.rows.h_kv = p.h_kv; p.rows.group = p.group;
+    p.rows.scale_log2 = p.scale_log2;
+    // depth mode: key rows of depths <= depth only (later rows read as zero); Q, dO hold one row per branch
+    p.depth = depth;
+    p.num_branches = pr.num_branches;
+    p.branch_len = pr.uniform_len;
+    return p;
+}
+
+// rows of the key tensors that a call may read: without own-branch keys nothing beyond kv_end (a received shard ends there)
+inline uint64_t key_rows(const ba_plan *pl, const BaRange &r, int depth) {
+    const ba_problem_t &pr = pl->prob;
+    return depth ? (uint64_t)(pr.n_main + (int64_t)depth * pr.num_branches)
+           : (r.parts & BA_PART_BRANCH) ? (uint64_t)(pr.n_main + pr.n_branch) : (uint64_t)(r.kv_end > r.kv_base ? r.kv_end - r.kv_base : 1);
+}
+
+// Maps in the order q_main, q_branch, dO, K, V, branch rows of dO; boxes of `qr` query rows x `qh` heads and `kr` key rows
+inline bool bwd_maps(CUtensorMap *tm, const ba_plan *pl, const BaRange &r, const void *q_main, const void *q_branch,
+                     const void *k, const void *v, const void *d_o, int depth, uint32_t qr, uint32_t qh, uint32_t kr) {
+    using sm100::make_tmap_rhd;
+    const ba_problem_t &pr = pl->prob;
+    const int D = pr.head_dim;
+    const uint64_t go_rows = depth ? (uint64_t)pr.num_branches : (uint64_t)(pr.n_main + pr.n_branch);
+    const void *qm = q_main ? q_main : q_branch;
+    const void *qb = (q_branch && pr.n_branch > 0) ? q_branch : q_main;
+    const uint64_t qm_rows = depth ? (uint64_t)pr.num_branches : q_main ? (uint64_t)pr.n_main : (uint64_t)pr.n_branch;
+    const uint64_t qb_rows = depth ? (uint64_t)pr.num_branches
+                             : (q_branch && pr.n_branch > 0) ? (uint64_t)pr.n_branch : (uint64_t)pr.n_main;
+    // dO of the branch rows alone: whatever lies in front of branch row 0 (rows of dO that a call without main
+    // queries leaves unset) is not loaded
+    const bool go_split = !depth && pr.n_branch > 0;
+    const void *gob = go_split ? (const char *)d_o + (size_t)pr.n_main * pr.h_q * D * 2 : d_o;
+    const uint64_t gob_rows = go_split ? (uint64_t)pr.n_branch : go_rows, kv_rows = key_rows(pl, r, depth);
+    return make_tmap_rhd(&tm[0], qm, qm_rows, pr.h_q, D, qr, qh) && make_tmap_rhd(&tm[1], qb, qb_rows, pr.h_q, D, qr, qh) &&
+           make_tmap_rhd(&tm[2], d_o, go_rows, pr.h_q, D, qr, qh) && make_tmap_rhd(&tm[3], k, kv_rows, pr.h_kv, D, kr) &&
+           make_tmap_rhd(&tm[4], v, kv_rows, pr.h_kv, D, kr) && make_tmap_rhd(&tm[5], gob, gob_rows, pr.h_q, D, qr, qh);
+}
+
+// Work items (key tiles) of dK/dV and how they are shared out; returns the number of CTAs
+inline int64_t key_items(TcBwdParams &p, const ba_plan *pl, const BaRange &r, bool has_main) {
+    const ba_problem_t &pr = pl->prob;
+    const int64_t qm_n = has_main ? r.qm_end - r.qm_begin : 0, br_n = r.tok_end - r.tok_begin;
+    const int64_t kmt = (r.parts & BA_PART_MAIN) ? (r.kv_end - r.kv_begin + kTile - 1) / kTile : 0;
+    p.step_kb = p.depth ? kTile : branch_key_step(pr.uniform_len);
+    int64_t kbt = (r.parts & BA_PART_BRANCH) ? (br_n + p.step_kb - 1) / p.step_kb : 0;
+    p.branch_tiles_per_depth = (int)kbt;
+    if (p.depth) kbt *= p.depth;    // the tokens of depths 1 .. depth of the selected branches are keys
+    p.branch_key_tiles = (int)kbt;
+    // Share main key tiles between the CTAs of a cluster until they fill the SMs once, as long as an average
+    // part keeps eight 64-row steps: 2,048 tokens, 8 KV heads (128 tiles) take 122 us whole, 130 us in two
+    // parts, 153 us in four.
+    const int64_t keys = kmt * kTile, viewers = qm_n + br_n;
+    const int64_t seq = pr.num_seqs > 0 ? pr.n_main / pr.num_seqs : 0;
+    const int64_t est = keys > 0 ? (seq < keys ? seq : keys) / 2 * viewers / (keys < pr.n_main ? pr.n_main : keys) * p.group / 64 : 0;
+    while (p.splits < 8 && kmt * pr.h_kv * p.splits * 2 <= kSms && est >= 8 * 2 * p.splits) p.splits *= 2;
+    p.main_key_tiles = (int)kmt;
+    const int64_t tiles = kmt + (kbt + p.splits - 1) / p.splits;    // work items (clusters) per KV head
+    p.total_key_tiles = (int)tiles;
+    // Up to 24 work items per SM heaviest first over all KV heads, so that the last items are short (8,192
+    // tokens with chains 830 us against 1030 KV-head-major, 32,768 tokens with blocks 1616 against 1711);
+    // beyond that KV-head-major, whose resident CTAs share one query stream through L2 (65,536-token trees 7862
+    // us against 7953, 73,728 tokens with chains 48.4 ms against 48.9).
+    p.tile_major = tiles * pr.h_kv <= 24 * kSms;
+    return tiles * pr.h_kv * p.splits;
+}
+
 }  // namespace
+
+// dK / dV of a call at head_dim 128 (ba_tc_dkdv.cu); after_dq: it may start while the dQ kernel queued just before ends
+int ba_tc_dkdv(const TcBwdParams &call, const ba_plan *pl, const BaRange &r, const void *q_main, const void *q_branch,
+               const void *k, const void *v, const void *d_o, bool after_dq, int dev, cudaStream_t st);

@@ -649,22 +649,8 @@ int ba_tc_bwd_fused(const ba_plan *pl, const BaRange &r, const void *q_main, con
         attr_set[dev] = true;
     }
     const ba_problem_t &pr = pl->prob;
-    TcBwdParams p;
-    memset(&p, 0, sizeof p);
-    p.meta = pl->meta;
-    p.r = r;
-    p.delta_t = delta;
-    p.nlse2_t = delta + (size_t)pl->row_pitch * pr.h_q;
-    p.row_pitch = pl->row_pitch;
-    p.dq_main = dq_main; p.dq_branch = dq_branch; p.dk = dk; p.dv = dv;
-    p.h_q = pr.h_q; p.h_kv = pr.h_kv;
-    p.group = pr.h_q / pr.h_kv;
-    p.scale = pl->scale;
-    p.scale_log2 = pl->scale * kLog2e;
-    p.accumulate = accumulate;
+    TcBwdParams p = bwd_params(pl, r, q_main, q_branch, k, v, delta, d_o, accumulate, dq_main, dq_branch, dk, dv, 0);
     p.wide = (((uintptr_t)dk | (uintptr_t)dv) & 31) == 0;
-    p.has_main_q = q_main != nullptr;
-    p.status = pl->dev_status;
     const int64_t kmt = (r.parts & BA_PART_MAIN) ? (r.kv_end - r.kv_begin + kTile - 1) / kTile : 0;
     p.step_kb = branch_key_step(pr.uniform_len);
     const int64_t kbt = (r.parts & BA_PART_BRANCH) ? (r.tok_end - r.tok_begin + p.step_kb - 1) / p.step_kb : 0;
@@ -678,7 +664,6 @@ int ba_tc_bwd_fused(const ba_plan *pl, const BaRange &r, const void *q_main, con
     // 8 heads 2.46 / 1.95 ms.  At 65,536 tokens (256 tiles) the rule keeps one CTA per tile.
     const int64_t viewers = (q_main ? r.qm_end - r.qm_begin : 0) + r.tok_end - r.tok_begin;
     const int64_t steps = viewers / kTile * p.group;
-    p.splits = 1;
     auto waves = [&](int64_t split, int64_t sms) { return (double)((kmt * pr.h_kv * split + sms - 1) / sms) / (double)split; };
     double best = waves(1, kSms);
     const int64_t sms[3] = {kSms, 136, 128};      // SMs that clusters of two, four, eight can use
@@ -689,21 +674,8 @@ int ba_tc_bwd_fused(const ba_plan *pl, const BaRange &r, const void *q_main, con
         }
     p.total_key_tiles = (int)(kmt + (kbt + p.splits - 1) / p.splits);    // work items (clusters) per KV head
 
-    CUtensorMap tq_main, tq_branch, tgo, tgo_branch, tk, tv;
-    const uint64_t all_rows = (uint64_t)(pr.n_main + pr.n_branch);
-    // without own-branch keys nothing beyond kv_end is needed (a received shard ends there)
-    const uint64_t kv_rows = (r.parts & BA_PART_BRANCH) ? all_rows : (uint64_t)(r.kv_end > r.kv_base ? r.kv_end - r.kv_base : 1);
-    const void *qm = q_main ? q_main : q_branch;
-    const void *qb = (q_branch && pr.n_branch > 0) ? q_branch : q_main;
-    const uint64_t qm_rows = q_main ? (uint64_t)pr.n_main : (uint64_t)pr.n_branch;
-    const uint64_t qb_rows = (q_branch && pr.n_branch > 0) ? (uint64_t)pr.n_branch : (uint64_t)pr.n_main;
-    if (!make_tmap_rhd(&tk, k, kv_rows, pr.h_kv, 128, kTile) || !make_tmap_rhd(&tv, v, kv_rows, pr.h_kv, 128, kTile) ||
-        !make_tmap_rhd(&tgo, d_o, all_rows, pr.h_q, 128, kTile) || !make_tmap_rhd(&tq_main, qm, qm_rows, pr.h_q, 128, kTile) ||
-        !make_tmap_rhd(&tq_branch, qb, qb_rows, pr.h_q, 128, kTile) ||
-        // dO of the branch rows alone: what lies in front of branch row 0 is not loaded
-        !make_tmap_rhd(&tgo_branch, (const char *)d_o + (pr.n_branch > 0 ? (size_t)pr.n_main * pr.h_q * 256 : 0),
-                       pr.n_branch > 0 ? (uint64_t)pr.n_branch : all_rows, pr.h_q, 128, kTile))
-        return BA_EINVAL;
+    CUtensorMap tm[6];
+    if (!bwd_maps(tm, pl, r, q_main, q_branch, k, v, d_o, 0, kTile, 1, kTile)) return BA_EINVAL;
     const int64_t grid = (int64_t)p.total_key_tiles * pr.h_kv * p.splits;
     if (grid > INT_MAX) return BA_EUNSUPPORTED;
     cudaLaunchConfig_t cfg;
@@ -719,6 +691,6 @@ int ba_tc_bwd_fused(const ba_plan *pl, const BaRange &r, const void *q_main, con
     cfg.attrs = &attr;
     cfg.numAttrs = p.splits > 1 ? 1 : 0;
     auto kernel = p.splits > 1 ? &tc_bwd_fused_kernel<true> : &tc_bwd_fused_kernel<false>;
-    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kernel, tq_main, tq_branch, tgo, tk, tv, tgo_branch, p));
+    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kernel, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], p));
     return ba_check_launch();
 }

@@ -27,6 +27,16 @@ def test_sequence_lengths(ba, oracle, d, n):  # noqa: F811
     check_full(ba, oracle, problem([n], [0, n // 2, n - 1], 3, W.CHAIN, 4, 2, d), seed=n, std=0.5, impl=ba.IMPL_TC)
 
 
+# dK/dV walk the viewers of a key tile in tiles of 128 rows from a row that is a multiple of 4; a last tile of at most 64
+# rows is formed at half width.  A short sequence in front moves the start of the second one's tiles by up to three rows.
+# (Few viewers per key: dQ and dK are held to the absolute bound, as below.)
+@pytest.mark.parametrize("shift", [1, 2, 3, 4])
+@pytest.mark.parametrize("n", [61, 62, 64, 125, 127, 190, 193])
+def test_query_row_tiles(ba, oracle, n, shift):  # noqa: F811
+    p = problem([shift, n], [shift, shift + n // 3, shift + n - 1], 22, W.BLOCK, 3, 1, 128)
+    check_full(ba, oracle, p, seed=n + shift, std=0.5, impl=ba.IMPL_TC, relative_grads=False)
+
+
 # Trees are held to the absolute bound on dQ and dK.  The backward takes O in bf16, so delta = <dO, O> of a row
 # is off by up to 2^-9 sum |dO O|, about 1e-3 here, and each viewer moves a dK row by up to 1e-3 P |q| scale (2e-5
 # at P = 0.1, head_dim 64; 3e-6 at P = 1/40, head_dim 128) whatever the kernel; the dK of a tree's leaf has one
