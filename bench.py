@@ -280,11 +280,19 @@ class Recorder:
         return self._wrap("bwd_depth", 3, self.ba.branch_attn_bwd_depth, *a, **k)
 
     def totals(self):
-        out = {}
+        """Device time (ms) and calls by kind; what calls of one kind overlap (on two streams) is counted once."""
+        out, last = {}, {}
         for kind, s, e in self.events:
-            out.setdefault(kind, [0.0, 0])
-            out[kind][0] += s.elapsed_time(e)
-            out[kind][1] += 1
+            t = out.setdefault(kind, [0.0, 0])
+            t[1] += 1
+            end = last.get(kind)
+            if end is None or end.elapsed_time(s) >= 0:
+                t[0] += s.elapsed_time(e)
+            elif end.elapsed_time(e) > 0:
+                t[0] += end.elapsed_time(e)
+            else:
+                continue
+            last[kind] = e
         return out
 
 

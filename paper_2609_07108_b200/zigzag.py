@@ -122,6 +122,9 @@ class Workspace:
             self.outs = tuple(torch.empty(s, dtype=plan.torch_dtype, device=dev) for s in shapes)
 
 
+L2_BYTES = 126 << 20
+
+
 def chunk_order(cp: int) -> List[int]:
     """Query chunks in the order the drivers work through them (rank by rank)."""
     return [qc for rank in range(cp) for qc in rank_chunks(rank, cp)]
@@ -185,6 +188,29 @@ def forward(ba, plan, q_main, q_branch, k, v, cp, out=None, lse=None, ws=None, h
     return out, lse, launches
 
 
+class _Lanes:
+    """The caller's stream and `n - 1` further ones that take independent launches in turn: the CTAs of one launch
+    start on the SMs that the last wave of another leaves idle.  Everything between `fork` and `join` comes after what
+    the caller's stream held before and before what it gets afterwards."""
+
+    def __init__(self, n):
+        import torch
+        self._torch = torch
+        self.main = torch.cuda.current_stream()
+        self.streams = [self.main] + [torch.cuda.Stream() for _ in range(n - 1)]
+
+    def fork(self):
+        for st in self.streams[1:]:
+            st.wait_stream(self.main)
+
+    def use(self, i):
+        return self._torch.cuda.stream(self.streams[i % len(self.streams)])
+
+    def join(self):
+        for st in self.streams[1:]:
+            self.main.wait_stream(st)
+
+
 def backward(ba, plan, q_main, q_branch, k, v, o, lse, d_o, cp, fused=False, ws=None, hooks=None):
     """Emulated CP backward: the same (rank, step) blocks, gradients accumulated
     in fp32 and converted once at the end.  Returns (dQ_main, dQ_branch, dK, dV,
@@ -195,7 +221,13 @@ def backward(ba, plan, q_main, q_branch, k, v, o, lse, d_o, cp, fused=False, ws=
     complete when the chunk's last block is done (as on the rank that owns it) and is
     converted right then; `hooks.dq_done(qc, (q0, q1), (t0, t1))`, if given, is called
     after that (a caller that streams the gradients out starts there).  dK and dV
-    are complete, and converted, at the end."""
+    are complete, and converted, at the end.
+    The one-kernel blocks of a query chunk write different dK / dV rows and add into dQ atomically, so they are
+    independent and go to two streams in turn, as long as the query rows that they share (Q and dO, one KV head at a
+    time) take no more than half of the L2: the two launches read different tiles of them at a time.  A block of 65,536
+    tokens in 16 chunks is 256 equal CTAs, 1.73 waves of 148 SMs.  Whole backward, one stream / two: 65,536 tokens (34
+    MB) 441 / 412 ms, 98,304 (50 MB) 974 / 935, 131,072 (67 MB) 1,598 / 1,633, 262,144 (134 MB) 6,315 / 6,737; 16,384
+    in 8 chunks 31.4 / 28.5, 8,192 in 16 chunks 10.3 / 9.5 (three and four streams take the same)."""
     p = plan.problem
     if ws is None or ws.grads is None:
         ws = Workspace(ba, plan, cp, backward=True)
@@ -205,22 +237,30 @@ def backward(ba, plan, q_main, q_branch, k, v, o, lse, d_o, cp, fused=False, ws=
     launches = 0
     common = dict(accumulate=True, grads=grads)
     blocks = schedule(p, cp)
+    chunk_rows = p.rows // (2 * cp)
+    shared = chunk_rows * (p.h_q // p.h_kv) * p.head_dim * 2 * 2      # bytes
+    lanes = _Lanes(2 if fused and shared <= L2_BYTES // 2 else 1)
     for rank in range(cp):
         for qc in rank_chunks(rank, cp):
             mine = [b for b in blocks if b.rank == rank and b.q_chunk == qc]
             ba.branch_attn_bwd(plan, q_main, q_branch, k, v, o, lse, d_o, qm_range=mine[0].qm, br_range=mine[0].br,
                                kv_range=(0, 0), parts=0, stages=ba.STAGE_PREP, **common)
             launches += 1
-            for b in mine:
-                parts = ba.PART_MAIN | (ba.PART_BRANCH if b.branch_part else 0)
-                rng = dict(qm_range=b.qm, br_range=b.br, kv_range=b.kv, parts=parts)
-                if fused:
-                    ba.branch_attn_bwd(plan, q_main, q_branch, k, v, o, lse, d_o, stages=ba.STAGE_FUSED, **rng, **common)
-                    launches += 1
-                else:
-                    ba.branch_attn_bwd(plan, q_main, q_branch, k, v, o, lse, d_o, stages=ba.STAGE_DQ, **rng, **common)
-                    ba.branch_attn_bwd(plan, q_main, q_branch, k, v, o, lse, d_o, stages=ba.STAGE_DKDV, **rng, **common)
-                    launches += 2
+            lanes.fork()
+            try:
+                for i, b in enumerate(mine):
+                    parts = ba.PART_MAIN | (ba.PART_BRANCH if b.branch_part else 0)
+                    rng = dict(qm_range=b.qm, br_range=b.br, kv_range=b.kv, parts=parts)
+                    if fused:
+                        with lanes.use(i):
+                            ba.branch_attn_bwd(plan, q_main, q_branch, k, v, o, lse, d_o, stages=ba.STAGE_FUSED, **rng, **common)
+                        launches += 1
+                    else:
+                        ba.branch_attn_bwd(plan, q_main, q_branch, k, v, o, lse, d_o, stages=ba.STAGE_DQ, **rng, **common)
+                        ba.branch_attn_bwd(plan, q_main, q_branch, k, v, o, lse, d_o, stages=ba.STAGE_DKDV, **rng, **common)
+                        launches += 2
+            finally:
+                lanes.join()
             q0, q1 = mine[0].qm
             t0, t1 = plan.token_range(*mine[0].br)
             ba.ba_finalize_grads(grads[0][q0:q1], dst=ws.outs[0][q0:q1])
