@@ -23,6 +23,28 @@ struct BaMeta {
 
 constexpr int kSms = 148;          // B200
 
+// The order in which a kernel takes the tiles of a call over everything: heaviest first, over all sequences, so that
+// the CTAs end together (the tiles' own numbering goes sequence by sequence).  Formed with the plan, handed to the
+// kernels by value.  n = 0: the kernel's own rule.
+constexpr int kMaxOrder = 1536;
+struct BaOrder {
+    int n;
+    uint16_t tile[kMaxOrder];
+};
+// What an order was formed for: query row tiles or key tiles; numbers of tiles and rows per tile, main part and
+// branch part; whether main rows are queries.
+enum { BA_ORDER_ROWS, BA_ORDER_KEYS };
+struct BaTiling {
+    int kind, has_main;
+    int64_t main_tiles, main_step, branch_tiles, branch_step;
+};
+constexpr int kMaxOrders = 8;
+struct BaOrders {
+    int count;
+    BaTiling tiling[kMaxOrders];
+    BaOrder order[kMaxOrders];
+};
+
 struct ba_plan {
     ba_problem_t prob;            // copy; the metadata pointers in it are NOT kept alive
     BaMeta meta;
@@ -32,6 +54,7 @@ struct ba_plan {
     int64_t row_pitch;            // rows per head of the head-major backward scratch (>= N + M + 128)
     int32_t *host_offsets;        // host copy of branch_offsets (NULL when uniform_len > 0)
     int32_t *dev_status;          // one int32 in plan_mem: device-side status word
+    BaOrders *orders;             // or NULL
 };
 
 // Query / key selection of one call (monolithic = everything).
@@ -42,6 +65,18 @@ struct BaRange {
     int64_t kv_base;              // first row that K, V (and dK, dV) hold: 0, or kv_begin on a received shard
     int parts;
 };
+
+static inline bool ba_whole_call(const ba_plan *pl, const BaRange &r, bool has_main) {
+    return (!has_main || (r.qm_begin == 0 && r.qm_end == pl->prob.n_main)) && r.tok_begin == 0 && r.tok_end == pl->prob.n_branch &&
+           r.kv_begin == 0 && r.kv_end == pl->prob.n_main && r.kv_base == 0 && r.parts == (BA_PART_MAIN | BA_PART_BRANCH);
+}
+// ba_plan.cu: forms an order (`host`: problem with host arrays) and keeps it; finds it again (or an empty one)
+void ba_add_order(ba_plan *pl, const ba_problem_t *host, const BaTiling &t);
+const BaOrder &ba_find_order(const ba_plan *pl, const BaTiling &t);
+// the tilings that the kernels use for calls over everything
+void ba_tc_fwd_orders(ba_plan *pl, const ba_problem_t *host);
+void ba_tc_bwd_orders(ba_plan *pl, const ba_problem_t *host);
+void ba_simt_orders(ba_plan *pl, const ba_problem_t *host);
 
 extern thread_local int g_ba_last_cuda_error;
 

@@ -11,6 +11,8 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
+
 #include "ba_common.cuh"
 
 thread_local int g_ba_last_cuda_error = 0;
@@ -345,6 +347,69 @@ static int check_metadata(const ba_problem_t *p, int64_t *pairs_out, int32_t *un
     return BA_OK;
 }
 
+constexpr int64_t kOrderMaxBytes = 160 << 20;
+
+// Number of keys that a query row tile walks, or of query rows that a key tile is walked by, per tile.
+static void tile_weights(const ba_problem_t *host, int32_t uniform, const BaTiling &t, int64_t *w) {
+    const int32_t *cu = host->cu_seqlens, *anchor = host->anchor_idx;
+    const int32_t ns = host->num_seqs, nb = host->num_branches;
+    const int64_t n = host->n_main, m = host->n_branch;
+    auto seq = [&](int64_t i) { return (int32_t)(std::upper_bound(cu + 1, cu + ns, (int32_t)i) - (cu + 1)); };      // of main row i
+    auto offset = [&](int64_t b) -> int64_t { return uniform > 0 ? b * uniform : host->branch_offsets[b]; };
+    auto branch = [&](int64_t tok) -> int64_t {
+        return uniform > 0 ? tok / uniform
+                           : std::upper_bound(host->branch_offsets + 1, host->branch_offsets + nb, (int32_t)tok) - (host->branch_offsets + 1);
+    };
+    auto anchored = [&](int64_t key) { return nb > 0 ? offset(std::lower_bound(anchor, anchor + nb, (int32_t)key) - anchor) : 0; };
+    for (int64_t i = 0; i < t.main_tiles; ++i) {
+        const int64_t a = i * t.main_step, b = std::min(a + t.main_step, n) - 1;
+        if (t.kind == BA_ORDER_ROWS) {
+            w[i] = b - cu[seq(a)] + 1;
+        } else {
+            const int64_t end = cu[seq(b) + 1];
+            w[i] = (t.has_main ? end - a : 0) + anchored(end) - anchored(a);
+        }
+    }
+    for (int64_t i = 0; i < t.branch_tiles; ++i) {
+        const int64_t a = i * t.branch_step, b = std::min(a + t.branch_step, m) - 1;
+        w[t.main_tiles + i] = b - a + 1;      // own-branch keys / rows
+        if (t.kind == BA_ORDER_ROWS) w[t.main_tiles + i] += anchor[branch(b)] - cu[seq(anchor[branch(a)])] + 1;
+    }
+}
+
+void ba_add_order(ba_plan *pl, const ba_problem_t *host, const BaTiling &t) {
+    const ba_problem_t &pr = pl->prob;
+    const int64_t tiles = t.main_tiles + t.branch_tiles, items = tiles * pr.h_kv;
+    if (tiles < 2 || tiles > kMaxOrder || ba_find_order(pl, t).n > 0) return;
+    // Not where the streamed rows (K and V, or Q and dO) are far larger than the L2, unless every item is resident or
+    // next: tiles of one sequence have to be taken together then, while that sequence's rows are there.  Nor for key tiles
+    // where the items are many and short enough as they are.
+    const int64_t rows = (t.kind == BA_ORDER_ROWS || t.has_main ? pr.n_main : 0) + pr.n_branch;
+    const int64_t streamed = 2 * rows * (t.kind == BA_ORDER_ROWS ? pr.h_kv : pr.h_q) * pr.head_dim * (pr.dtype == BA_FP32 ? 4 : 2);
+    if (items > 2 * kSms && (streamed > kOrderMaxBytes || (t.kind == BA_ORDER_KEYS && items > 12 * kSms))) return;
+    if (!pl->orders) pl->orders = (BaOrders *)calloc(1, sizeof(BaOrders));
+    if (!pl->orders || pl->orders->count == kMaxOrders) return;
+    int64_t w[kMaxOrder];
+    tile_weights(host, pl->prob.uniform_len, t, w);
+    BaOrder &o = pl->orders->order[pl->orders->count];
+    // equal weights in the kernels' own order: later query rows, earlier keys first
+    for (int64_t i = 0; i < tiles; ++i) o.tile[i] = (uint16_t)(t.kind == BA_ORDER_ROWS ? tiles - 1 - i : i);
+    std::stable_sort(o.tile, o.tile + tiles, [&](uint16_t a, uint16_t b) { return w[a] > w[b]; });
+    o.n = (int)tiles;
+    pl->orders->tiling[pl->orders->count++] = t;
+}
+
+const BaOrder &ba_find_order(const ba_plan *pl, const BaTiling &t) {
+    static const BaOrder none = {};
+    for (int i = 0; pl->orders && i < pl->orders->count; ++i) {
+        const BaTiling &x = pl->orders->tiling[i];
+        if (x.kind == t.kind && x.has_main == t.has_main && x.main_tiles == t.main_tiles && x.main_step == t.main_step &&
+            x.branch_tiles == t.branch_tiles && x.branch_step == t.branch_step)
+            return pl->orders->order[i];
+    }
+    return none;
+}
+
 extern "C" int ba_plan_create(const ba_problem_t *p, void *plan_mem, size_t plan_bytes, void *stream,
                               ba_plan_t **out) {
     if (!out) return BA_EINVAL;
@@ -425,6 +490,14 @@ extern "C" int ba_plan_create_host(const ba_problem_t *host, const ba_problem_t 
     }
     ba_plan *pl = new_plan(&pr, a, pairs, offsets);
     if (!pl) return BA_EINVAL;
+    if (pr.num_seqs > 1) {      // (one sequence: the tiles' own order is heaviest first)
+        if (pl->impl == BA_IMPL_TC) {
+            ba_tc_fwd_orders(pl, host);
+            ba_tc_bwd_orders(pl, host);
+        } else {
+            ba_simt_orders(pl, host);
+        }
+    }
     *out = pl;
     return BA_OK;
 }
@@ -442,6 +515,7 @@ extern "C" int ba_host_wait(void *event) {
 extern "C" int ba_plan_destroy(ba_plan_t *plan) {
     if (!plan) return BA_EINVAL;
     free(plan->host_offsets);
+    free(plan->orders);
     free(plan);
     return BA_OK;
 }

@@ -206,7 +206,7 @@ template <int D, int MODE> struct SimtSmem {
 };
 
 template <typename T, int D, int MODE>
-__global__ void __launch_bounds__(kThreads, 3) simt_kernel(const __grid_constant__ SimtArgs a) {
+__global__ void __launch_bounds__(kThreads, 3) simt_kernel(const __grid_constant__ SimtArgs a, const __grid_constant__ BaOrder order) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     using Smem = SimtSmem<D, MODE>;
     Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const __grid_constant
     // (longer prefixes), earlier keys (more viewers).
     const int per = MODE == kDkdv ? a.h_kv : a.h_kv * a.head_chunks;
     const int inner = work % per;
-    const int tile = MODE == kDkdv ? work / per : a.total_tiles - 1 - work / per;
+    const int tile = order.n > 0 ? order.tile[work / per] : MODE == kDkdv ? work / per : a.total_tiles - 1 - work / per;
     const bool is_main = tile < a.main_tiles;
     const int g = MODE == kDkdv ? inner : inner / a.head_chunks;
     const int h0 = MODE == kDkdv ? 0 : g * a.group + (inner % a.head_chunks) * a.hp;
@@ -607,7 +607,7 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const __grid_constant
 inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 template <typename T, int D, int MODE>
-int launch(SimtArgs &a, int64_t work, bool after_dq, cudaStream_t st) {
+int launch(SimtArgs &a, const BaOrder &order, int64_t work, bool after_dq, cudaStream_t st) {
     // the dynamic shared-memory limit is a per-device attribute of the kernel
     static bool attr_set[64] = {};
     int dev = 0;
@@ -637,7 +637,7 @@ int launch(SimtArgs &a, int64_t work, bool after_dq, cudaStream_t st) {
         ++cfg.numAttrs;
     }
     cfg.attrs = attr;
-    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, simt_kernel<T, D, MODE>, a));
+    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, simt_kernel<T, D, MODE>, a, order));
     return ba_check_launch();
 }
 
@@ -661,6 +661,11 @@ template <int MODE> int64_t tile_work(SimtArgs &a) {
     return (mt + bt) * per;
 }
 
+template <int MODE> BaTiling tiling(const SimtArgs &a, bool has_main) {
+    const int step = MODE == kDkdv ? kRows : a.tok;
+    return {MODE == kDkdv ? BA_ORDER_KEYS : BA_ORDER_ROWS, has_main, a.main_tiles, step, a.total_tiles - a.main_tiles, step};
+}
+
 template <typename T, int D, int MODE>
 int launch_tiles(const ba_plan *pl, SimtArgs a, bool after_dq, cudaStream_t st) {
     const ba_problem_t &pr = pl->prob;
@@ -680,7 +685,9 @@ int launch_tiles(const ba_plan *pl, SimtArgs a, bool after_dq, cudaStream_t st) 
                             (work * a.splits * 2 <= kSms * 16 && est >= 2 * 4 * a.splits)))
         a.splits *= 2;
     if (work * a.splits > INT_MAX) return BA_EUNSUPPORTED;
-    return launch<T, D, MODE>(a, work, after_dq, st);
+    const bool has_main = a.q_main != nullptr;
+    const BaOrder &order = ba_find_order(pl, ba_whole_call(pl, a.r, has_main) ? tiling<MODE>(a, has_main) : BaTiling{-1});
+    return launch<T, D, MODE>(a, order, work, after_dq, st);
 }
 
 template <int MODE> int dispatch(const ba_plan *pl, const SimtArgs &a, cudaStream_t st, bool after_dq = false) {
@@ -704,6 +711,18 @@ SimtArgs base_args(const ba_plan *pl, const BaRange &r) {
 }
 
 }  // namespace
+
+void ba_simt_orders(ba_plan *pl, const ba_problem_t *host) {
+    const BaRange r = {0, pl->prob.n_main, 0, pl->prob.n_branch, 0, pl->prob.n_main, 0, BA_PART_MAIN | BA_PART_BRANCH};
+    for (int has_main = 1; has_main >= 0; --has_main) {
+        SimtArgs a = base_args(pl, r);
+        a.q_main = has_main ? pl : nullptr;      // (only asked whether it is there)
+        tile_work<kFwd>(a);                      // forward and dQ
+        ba_add_order(pl, host, tiling<kFwd>(a, has_main));
+        tile_work<kDkdv>(a);
+        ba_add_order(pl, host, tiling<kDkdv>(a, has_main));
+    }
+}
 
 int ba_simt_fwd(const ba_plan *pl, const BaRange &r, const void *q_main, const void *q_branch,
                 const void *k, const void *v, void *o, float *lse, int partial_out,

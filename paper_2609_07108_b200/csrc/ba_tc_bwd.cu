@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(kDqThreads, 1)
 tc_dq_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constant__ CUtensorMap tm_q_branch,
              const __grid_constant__ CUtensorMap tm_go, const __grid_constant__ CUtensorMap tm_k,
              const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_k32,
-             const __grid_constant__ CUtensorMap tm_v32, const TcDqParams p) {
+             const __grid_constant__ CUtensorMap tm_v32, const TcDqParams p, const __grid_constant__ BaOrder order) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     DqSmem &sm = *reinterpret_cast<DqSmem *>(smem_raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -153,7 +153,7 @@ tc_dq_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                     }
                     break;
                 }
-                if (lane == 0) make_item(p, work, 0, sm.item[s]);
+                if (lane == 0) make_item(p, order, work, 0, sm.item[s]);
                 __syncwarp();
                 if (sm.item[s].T == 0) {
                     const Item &it = sm.item[s];
@@ -682,20 +682,20 @@ __device__ __forceinline__ uint64_t shift_mask(uint64_t m, int sh) {
 
 // Rows of one call are ordered by position (main) or anchor (branches), so the ranges of a tile are those of its
 // first and last row.
-template <int MODE> __device__ void make_kv_item(const TcBwdParams &p, uint32_t work, int rank, KvItem &it) {
+template <int MODE> __device__ void make_kv_item(const TcBwdParams &p, const BaOrder &order, uint32_t work, int rank, KvItem &it) {
     constexpr bool kDq = MODE == kModeDq;
     const int n = (int)p.meta.n_main, S = p.splits;
     int tile;
     // Heaviest first: earlier keys (more viewers), later query rows (longer prefixes)
     if (kDq) {
         const int per = p.h_kv * p.head_chunks;
-        tile = p.total_tiles - 1 - (int)(work / per);
+        tile = order.n > 0 ? order.tile[work / per] : p.total_tiles - 1 - (int)(work / per);
         it.g = (int)(work % per) / p.head_chunks;
         it.h0 = it.g * p.group + (int)(work % p.head_chunks) * p.hp;
     } else {
         it.h0 = 0;
         if (p.tile_major) {
-            tile = (int)(work / p.h_kv);
+            tile = order.n > 0 ? order.tile[work / p.h_kv] : (int)(work / p.h_kv);
             it.g = (int)(work % p.h_kv);
         } else {
             // KV-head-major: the CTAs running at one time belong to one or two KV heads and stream the same
@@ -766,7 +766,7 @@ __global__ void __launch_bounds__(kKvThreads, 1)
 tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constant__ CUtensorMap tm_q_branch,
              const __grid_constant__ CUtensorMap tm_go, const __grid_constant__ CUtensorMap tm_k,
              const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_go_branch,
-             const __grid_constant__ TcBwdParams p) {
+             const __grid_constant__ TcBwdParams p, const __grid_constant__ BaOrder order) {
     using Smem = KvSmem;
     constexpr bool kDq = MODE == kModeDq;
     constexpr int D = kD;
@@ -828,7 +828,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                     }
                     break;
                 }
-                if (lane == 0) make_kv_item<MODE>(p, work, rank, sm.item[s]);
+                if (lane == 0) make_kv_item<MODE>(p, order, work, rank, sm.item[s]);
                 __syncwarp();
                 if (!SPLIT && sm.item[s].n_iter == 0) {
                     const KvItem &it = sm.item[s];
@@ -1302,7 +1302,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
 }
 
 template <int MODE, bool SPLIT>
-int launch_kv(const TcBwdParams &p, const CUtensorMap *tm, int64_t grid, int dev, cudaStream_t st) {
+int launch_kv(const TcBwdParams &p, const BaOrder &order, const CUtensorMap *tm, int64_t grid, int dev, cudaStream_t st) {
     if (grid <= 0) return BA_OK;
     if (grid > INT_MAX) return BA_EUNSUPPORTED;
     // the dynamic shared-memory limit is a per-device attribute of the kernel
@@ -1328,11 +1328,39 @@ int launch_kv(const TcBwdParams &p, const CUtensorMap *tm, int64_t grid, int dev
     attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = SPLIT ? 1 : 0;
-    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_kv_kernel<MODE, SPLIT>, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], p));
+    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_kv_kernel<MODE, SPLIT>, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], p, order));
     return ba_check_launch();
 }
 
+// dQ at head_dim 64: 128-row tiles
+inline void row_tiles(TcBwdParams &p, int64_t qm_n, int64_t br_n) {
+    p.hp = p.group < kTile ? p.group : kTile;
+    p.head_chunks = (p.group + p.hp - 1) / p.hp;
+    p.tok = kTile / p.hp;
+    p.main_tiles = (int)((qm_n + p.tok - 1) / p.tok);
+    p.total_tiles = p.main_tiles + (int)((br_n + p.tok - 1) / p.tok);
+}
+inline BaTiling row_tiling(const TcBwdParams &p, bool has_main) {
+    return {BA_ORDER_ROWS, has_main, p.main_tiles, p.tok, p.total_tiles - p.main_tiles, p.tok};
+}
+inline const BaOrder &row_order(const TcBwdParams &p, const ba_plan *pl, bool has_main) {
+    return ba_find_order(pl, ba_whole_call(pl, p.r, has_main) ? row_tiling(p, has_main) : BaTiling{-1});
+}
+
 }  // namespace
+
+void ba_tc_bwd_orders(ba_plan *pl, const ba_problem_t *host) {
+    const int64_t n = pl->prob.n_main, m = pl->prob.n_branch;
+    const BaRange r = {0, n, 0, m, 0, n, 0, BA_PART_MAIN | BA_PART_BRANCH};
+    for (int has_main = 1; has_main >= 0; --has_main) {
+        TcBwdParams p = bwd_params(pl, r, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0, nullptr, nullptr, nullptr, nullptr, 0);
+        if (key_items(p, pl, r, has_main) > 0 && p.tile_major) ba_add_order(pl, host, key_tiling(p, has_main));
+        if (pl->prob.head_dim == 64) {
+            row_tiles(p, has_main ? n : 0, m);
+            ba_add_order(pl, host, row_tiling(p, has_main));
+        }
+    }
+}
 
 int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const void *q_branch, const void *k,
               const void *v, const float *delta, const void *d_o, int accumulate,
@@ -1348,20 +1376,17 @@ int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
     const int64_t qm_n = q_main ? r.qm_end - r.qm_begin : 0, br_n = r.tok_end - r.tok_begin;
     if (pr.head_dim == 64) {
         if (stages & BA_STAGE_DQ) {
-            p.hp = p.group < kTile ? p.group : kTile;
-            p.head_chunks = (p.group + p.hp - 1) / p.hp;
-            p.tok = kTile / p.hp;
-            p.main_tiles = (int)((qm_n + p.tok - 1) / p.tok);
-            p.total_tiles = p.main_tiles + (int)((br_n + p.tok - 1) / p.tok);
+            row_tiles(p, qm_n, br_n);
             if (!maps(p.tok, p.hp, kSub)) return BA_EINVAL;
-            int rc = launch_kv<kModeDq, false>(p, tm, (int64_t)p.total_tiles * pr.h_kv * p.head_chunks, dev, st);
+            int rc = launch_kv<kModeDq, false>(p, row_order(p, pl, q_main != nullptr), tm, (int64_t)p.total_tiles * pr.h_kv * p.head_chunks, dev, st);
             if (rc != BA_OK) return rc;
         }
         if (stages & BA_STAGE_DKDV) {
             // (both kernels overlapped, as at head_dim 128: 605 us instead of 548 for the 4,096-token chains)
             const int64_t grid = key_items(p, pl, r, q_main != nullptr);
             if (!maps(kSub, 1, kTile)) return BA_EINVAL;
-            return p.splits > 1 ? launch_kv<kModeDkdv, true>(p, tm, grid, dev, st) : launch_kv<kModeDkdv, false>(p, tm, grid, dev, st);
+            const BaOrder &order = key_order(p, pl, q_main != nullptr);
+            return p.splits > 1 ? launch_kv<kModeDkdv, true>(p, order, tm, grid, dev, st) : launch_kv<kModeDkdv, false>(p, order, tm, grid, dev, st);
         }
         return BA_OK;
     }
@@ -1391,7 +1416,8 @@ int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
             !make_tmap_rhd(&v32, v, kv_rows, pr.h_kv, 128, 32))
             return BA_EINVAL;
         if (grid > 0) {
-            tc_dq_kernel<<<(unsigned)grid, kDqThreads, sizeof(DqSmem), st>>>(tm[0], tm[1], tm[2], tm[3], tm[4], k32, v32, q);
+            tc_dq_kernel<<<(unsigned)grid, kDqThreads, sizeof(DqSmem), st>>>(tm[0], tm[1], tm[2], tm[3], tm[4], k32, v32, q,
+                                                                              item_order(q, pl, q_main != nullptr));
             int rc = ba_check_launch();
             if (rc != BA_OK) return rc;
         }

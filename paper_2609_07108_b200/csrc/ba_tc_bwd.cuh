@@ -198,6 +198,14 @@ inline int64_t key_items(TcBwdParams &p, const ba_plan *pl, const BaRange &r, bo
     return tiles * pr.h_kv * p.splits;
 }
 
+inline BaTiling key_tiling(const TcBwdParams &p, bool has_main) {
+    return {BA_ORDER_KEYS, has_main, p.main_key_tiles, kTile, p.total_key_tiles - p.main_key_tiles, (int64_t)p.step_kb * p.splits};
+}
+inline const BaOrder &key_order(const TcBwdParams &p, const ba_plan *pl, bool has_main) {
+    const bool any = !p.depth && p.tile_major && ba_whole_call(pl, p.r, has_main);
+    return ba_find_order(pl, any ? key_tiling(p, has_main) : BaTiling{-1});
+}
+
 }  // namespace
 
 // dK / dV of a call at head_dim 128 (ba_tc_dkdv.cu); after_dq: it may start while the dQ kernel queued just before ends

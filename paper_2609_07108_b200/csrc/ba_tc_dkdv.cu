@@ -70,12 +70,12 @@ __device__ __forceinline__ int walk(int n_sub, int s) { return n_sub - 1 - s; }
 
 // Rows of one call are ordered by position (main) or anchor (branches), so the ranges of a tile are those of its
 // first and last row.
-__device__ void make_key_item(const TcBwdParams &p, uint32_t work, int rank, KeyItem &it) {
+__device__ void make_key_item(const TcBwdParams &p, const BaOrder &order, uint32_t work, int rank, KeyItem &it) {
     const int n = (int)p.meta.n_main, S = p.splits;
     int tile;
     // Heaviest first: earlier keys (more viewers)
     if (p.tile_major) {
-        tile = (int)(work / p.h_kv);
+        tile = order.n > 0 ? order.tile[work / p.h_kv] : (int)(work / p.h_kv);
         it.g = (int)(work % p.h_kv);
     } else {
         // KV-head-major: the CTAs running at one time belong to one or two KV heads and stream the same
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 tc_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constant__ CUtensorMap tm_q_branch,
                const __grid_constant__ CUtensorMap tm_go, const __grid_constant__ CUtensorMap tm_k,
                const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_go_branch,
-               const __grid_constant__ TcBwdParams p) {
+               const __grid_constant__ TcBwdParams p, const __grid_constant__ BaOrder order) {
     using Smem = DkdvSmem;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
@@ -252,7 +252,7 @@ tc_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_const
                     }
                     break;
                 }
-                if (lane == 0) make_key_item(p, work, rank, sm.item[s]);
+                if (lane == 0) make_key_item(p, order, work, rank, sm.item[s]);
                 __syncwarp();
                 if (!SPLIT && sm.item[s].n_iter == 0) {
                     const KeyItem &it = sm.item[s];
@@ -683,7 +683,7 @@ tc_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_const
 }
 
 template <bool SPLIT>
-int launch(const TcBwdParams &p, const CUtensorMap *tm, int64_t grid, bool after_dq, int dev, cudaStream_t st) {
+int launch(const TcBwdParams &p, const BaOrder &order, const CUtensorMap *tm, int64_t grid, bool after_dq, int dev, cudaStream_t st) {
     // the dynamic shared-memory limit is a per-device attribute of the kernel
     static bool attr_set[64] = {};
     const size_t smem = sizeof(DkdvSmem);
@@ -714,7 +714,7 @@ int launch(const TcBwdParams &p, const CUtensorMap *tm, int64_t grid, bool after
         ++cfg.numAttrs;
     }
     cfg.attrs = attr;
-    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_dkdv_kernel<SPLIT>, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], p));
+    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_dkdv_kernel<SPLIT>, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], p, order));
     return ba_check_launch();
 }
 
@@ -729,5 +729,6 @@ int ba_tc_dkdv(const TcBwdParams &call, const ba_plan *pl, const BaRange &r, con
     if (grid > INT_MAX) return BA_EUNSUPPORTED;
     CUtensorMap tm[6];
     if (!bwd_maps(tm, pl, r, q_main, q_branch, k, v, d_o, p.depth, kTile, 1, kTile)) return BA_EINVAL;
-    return p.splits > 1 ? launch<true>(p, tm, grid, after_dq, dev, st) : launch<false>(p, tm, grid, after_dq, dev, st);
+    const BaOrder &order = key_order(p, pl, q_main != nullptr);
+    return p.splits > 1 ? launch<true>(p, order, tm, grid, after_dq, dev, st) : launch<false>(p, order, tm, grid, after_dq, dev, st);
 }

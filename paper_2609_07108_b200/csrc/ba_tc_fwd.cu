@@ -275,7 +275,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constant__ CUtensorMap tm_q_branch,
               const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
               const __grid_constant__ CUtensorMap tm_k32, const __grid_constant__ CUtensorMap tm_v32,
-              const __grid_constant__ CUtensorMap tm_o, const __grid_constant__ TcFwdParams p) {
+              const __grid_constant__ CUtensorMap tm_o, const __grid_constant__ TcFwdParams p,
+              const __grid_constant__ BaOrder order) {
     using Smem = FwdSmem<D>;
     constexpr int kStages = Smem::kStages;
     constexpr uint32_t kTileBytes = Smem::kTileBytes;
@@ -339,7 +340,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
                     }
                     break;
                 }
-                if (lane == 0) make_item(p, work, rank, sm.item[s]);
+                if (lane == 0) make_item(p, order, work, rank, sm.item[s]);
                 __syncwarp();
                 if (!SPLIT && sm.item[s].T == 0) {
                     store_empty_item<D>(p, sm.item[s], lane);
@@ -888,12 +889,12 @@ template <int D, bool SPLIT> int prepare_kernel(int dev) {
 }
 
 template <int D>
-int launch_fwd(TcFwdParams &p, const CUtensorMap *tm, int64_t work, int dev, cudaStream_t st) {
+int launch_fwd(TcFwdParams &p, const BaOrder &order, const CUtensorMap *tm, int64_t work, int dev, cudaStream_t st) {
     const size_t smem = sizeof(FwdSmem<D>);
     if (p.splits == 1) {
         int rc = prepare_kernel<D, false>(dev);
         if (rc != BA_OK) return rc;
-        tc_fwd_kernel<D, false><<<(unsigned)work, kThreads, smem, st>>>(tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], tm[6], p);
+        tc_fwd_kernel<D, false><<<(unsigned)work, kThreads, smem, st>>>(tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], tm[6], p, order);
         return ba_check_launch();
     }
     int rc = prepare_kernel<D, true>(dev);
@@ -910,7 +911,7 @@ int launch_fwd(TcFwdParams &p, const CUtensorMap *tm, int64_t work, int dev, cud
     attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_fwd_kernel<D, true>, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], tm[6], p));
+    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_fwd_kernel<D, true>, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], tm[6], p, order));
     return ba_check_launch();
 }
 
@@ -980,5 +981,14 @@ int ba_tc_fwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
     const uint64_t o_rows = depth ? (uint64_t)pr.num_branches : (uint64_t)(pr.n_main + pr.n_branch);
     if (!p.warp_tok) tm[6] = tm[0];
     else if (!make_tmap_rhd(&tm[6], o, o_rows, pr.h_q, D, p.warp_tok, p.hp)) return BA_EINVAL;
-    return D == 128 ? launch_fwd<128>(p, tm, work, dev, st) : launch_fwd<64>(p, tm, work, dev, st);
+    const BaOrder &order = item_order(p, pl, q_main != nullptr);
+    return D == 128 ? launch_fwd<128>(p, order, tm, work, dev, st) : launch_fwd<64>(p, order, tm, work, dev, st);
+}
+
+void ba_tc_fwd_orders(ba_plan *pl, const ba_problem_t *host) {
+    const BaRange r = {0, pl->prob.n_main, 0, pl->prob.n_branch, 0, pl->prob.n_main, 0, BA_PART_MAIN | BA_PART_BRANCH};
+    for (int i = 0; i < 3; ++i) {      // with main queries; branch rows only, two or one tile of rows per item
+        ItemParams p;
+        if (fill_items(p, pl, r, i == 0, 0, i == 2) > 0) ba_add_order(pl, host, item_tiling(p, i == 0));
+    }
 }

@@ -73,10 +73,10 @@ __device__ __forceinline__ void row_bounds(const ItemParams &p, bool is_main, in
 
 // Rows of one call are ordered by position (main) or anchor (branches), so the bounds of a row range
 // are those of its first and last row.
-__device__ void make_item(const ItemParams &p, uint32_t work, int rank, Item &it) {
+__device__ void make_item(const ItemParams &p, const BaOrder &order, uint32_t work, int rank, Item &it) {
     const int per = p.h_kv * p.head_chunks;
-    // later (longer-prefix) rows first; the items of one row range (all KV heads) are adjacent
-    const int tile = p.total_items - 1 - (int)(work / per);
+    // longest prefixes first (without an order: later rows first); the items of one row range (all KV heads) are adjacent
+    const int tile = order.n > 0 ? order.tile[work / per] : p.total_items - 1 - (int)(work / per);
     const int inner = (int)(work % per);
     it.g = inner / p.head_chunks;
     it.h0 = it.g * p.group + (inner % p.head_chunks) * p.hp;
@@ -197,6 +197,14 @@ inline int64_t fill_items(ItemParams &p, const ba_plan *pl, const BaRange &r, bo
     p.main_items = (int)mt;
     p.total_items = (int)(mt + bt);
     return (mt + bt) * pr.h_kv * p.head_chunks;
+}
+
+inline BaTiling item_tiling(const ItemParams &p, bool has_main) {
+    return {BA_ORDER_ROWS, has_main, p.main_items, p.step_m, p.total_items - p.main_items, p.step_b};
+}
+inline const BaOrder &item_order(const ItemParams &p, const ba_plan *pl, bool has_main) {
+    static const BaOrder none = {};
+    return !p.depth && ba_whole_call(pl, p.r, has_main) ? ba_find_order(pl, item_tiling(p, has_main)) : none;
 }
 
 }  // namespace
