@@ -1390,6 +1390,10 @@ int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
         }
         return BA_OK;
     }
+    if (depth && (stages & BA_STAGE_DKDV)) {
+        const int rc = ba_tc_own_branch(p, q_branch, k, v, d_o, st);
+        if (rc != BA_OK) return rc;
+    }
     if (stages & BA_STAGE_DQ) {
         static bool attr_set[64] = {};
         if (!attr_set[dev]) {

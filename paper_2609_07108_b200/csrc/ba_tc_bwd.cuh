@@ -44,7 +44,7 @@ struct TcBwdParams {
     // depth-`depth` tokens of branches [r.tok_begin, r.tok_end) (branch indices), Q / dO / dQ and
     // the per-row scalars are indexed by branch, and branch keys are stored depth-major after the
     // main rows: token (depth j + 1, branch b) is key row N + j * num_branches + b.
-    int depth, num_branches, branch_len, branch_tiles_per_depth;
+    int depth, num_branches, branch_len;
     int *status;
     RowArgs rows;                     // head_dim 64: rows that are formed again one by one
 };
@@ -175,10 +175,9 @@ inline int64_t key_items(TcBwdParams &p, const ba_plan *pl, const BaRange &r, bo
     const ba_problem_t &pr = pl->prob;
     const int64_t qm_n = has_main ? r.qm_end - r.qm_begin : 0, br_n = r.tok_end - r.tok_begin;
     const int64_t kmt = (r.parts & BA_PART_MAIN) ? (r.kv_end - r.kv_begin + kTile - 1) / kTile : 0;
-    p.step_kb = p.depth ? kTile : branch_key_step(pr.uniform_len);
-    int64_t kbt = (r.parts & BA_PART_BRANCH) ? (br_n + p.step_kb - 1) / p.step_kb : 0;
-    p.branch_tiles_per_depth = (int)kbt;
-    if (p.depth) kbt *= p.depth;    // the tokens of depths 1 .. depth of the selected branches are keys
+    p.step_kb = branch_key_step(pr.uniform_len);
+    // (step-major: own_branch_kernel)
+    const int64_t kbt = (r.parts & BA_PART_BRANCH) && !p.depth ? (br_n + p.step_kb - 1) / p.step_kb : 0;
     p.branch_key_tiles = (int)kbt;
     // Share main key tiles between the CTAs of a cluster until they fill the SMs once, as long as an average
     // part keeps eight 64-row steps: 2,048 tokens, 8 KV heads (128 tiles) take 122 us whole, 130 us in two
@@ -211,3 +210,5 @@ inline const BaOrder &key_order(const TcBwdParams &p, const ba_plan *pl, bool ha
 // dK / dV of a call at head_dim 128 (ba_tc_dkdv.cu); after_dq: it may start while the dQ kernel queued just before ends
 int ba_tc_dkdv(const TcBwdParams &call, const ba_plan *pl, const BaRange &r, const void *q_main, const void *q_branch,
                const void *k, const void *v, const void *d_o, bool after_dq, int dev, cudaStream_t st);
+// step-major calls: dK / dV of the own-branch keys alone
+int ba_tc_own_branch(const TcBwdParams &p, const void *q, const void *k, const void *v, const void *d_o, cudaStream_t st);

@@ -85,14 +85,13 @@ __device__ void make_key_item(const TcBwdParams &p, const BaOrder &order, uint32
     }
     const bool is_main = tile < p.main_key_tiles;
     it.is_main = is_main;
-    int bt = tile - p.main_key_tiles, kdepth = 0;
+    int bt = tile - p.main_key_tiles;
     if (!is_main && S > 1) bt = bt * S + rank;           // a cluster holds S branch key tiles
     const bool past = !is_main && bt >= p.branch_key_tiles;      // the last cluster has ranks to spare: no rows
-    if (!is_main && p.depth) { kdepth = bt / p.branch_tiles_per_depth; bt %= p.branch_tiles_per_depth; }
     const int step = is_main ? kTile : p.step_kb;
     it.row0 = is_main ? (int)p.r.kv_begin + tile * step : (int)p.r.tok_begin + bt * step;
     it.row_end = past ? it.row0 : min(it.row0 + step, (int)(is_main ? p.r.kv_end : p.r.tok_end));
-    it.krow0 = is_main ? it.row0 - (int)p.r.kv_base : n + kdepth * p.num_branches + it.row0;
+    it.krow0 = is_main ? it.row0 - (int)p.r.kv_base : n + it.row0;
     it.m0 = it.m1 = it.b0 = it.b1 = 0;
     const int first = it.row0, last = it.row_end - 1;
     if (last >= first) {
@@ -104,8 +103,6 @@ __device__ void make_key_item(const TcBwdParams &p, const BaOrder &order, uint32
             it.b0 = p.meta.key_bq_begin[first];
             it.b1 = p.meta.key_bq_end[last];
             if (p.depth) { it.b0 /= p.branch_len; it.b1 /= p.branch_len; }    // token ranges -> branch ranges
-        } else if (p.depth) {
-            it.b0 = first; it.b1 = last + 1;             // seen by the query of its own branch only
         } else {
             it.b0 = p.meta.br_start[first];
             it.b1 = p.meta.br_end[last];
@@ -503,8 +500,6 @@ tc_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_const
                     f.rb0 = p.meta.key_bq_begin[f.row];
                     f.rb1 = p.meta.key_bq_end[f.row];
                     if (p.depth) { f.rb0 /= p.branch_len; f.rb1 /= p.branch_len; }
-                } else if (p.depth) {
-                    f.rb0 = f.row; f.rb1 = f.row + 1;
                 } else {
                     f.rb0 = p.meta.br_start[f.row];
                     f.rb1 = p.meta.br_end[f.row];
@@ -528,7 +523,7 @@ tc_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_const
                 uint64_t vis = 0ull;
                 if (w.valid && !idle) {
                     const int rbeg = seg_main ? w.m0 : w.b0, rend = seg_main ? w.m1 : w.b1;
-                    if (w.is_main || p.depth) {
+                    if (w.is_main) {
                         // main rows: same sequence, causal: key <= row < end of the key's sequence; branch tokens
                         // anchored at or after the key, inside its sequence (depth mode: branches)
                         const int v0 = seg_main ? w.row : w.rb0, v1 = seg_main ? w.qend : w.rb1;
@@ -682,6 +677,83 @@ tc_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_const
     if (tid == 0 && sm.abort_flag) atomicExch(p.status, BA_ETIMEOUT);
 }
 
+// Step-major calls: dK, dV of the own-branch keys.  Token (depth j + 1, branch b) is seen by one query row of the call,
+// that of branch b: a term per query head of the group, no contraction over rows.  Sixteen lanes per (branch, KV head),
+// 8 of the 128 columns each; P and dS in fp32.
+// Bound by memory: Q and dO once, K, V and the fp32 dK, dV of every depth <= depth once.  So everything a lane reads
+// of one depth, and Q and dO of four heads, are in flight together (with the heads one after another 280 / 436 / 578 us).
+// 18,432 branches, 32/8 heads, depth 1 / 2 / 3: 123 / 185 / 254 us (158 registers and one block per SM: 141 / 227 / 307); as key tiles of the kernel above, 128 keys against 128 rows
+// of which each sees one, 155 / 329 / 464 us.
+constexpr int kOwnThreads = 256, kOwnHeads = 4;
+__device__ __forceinline__ float bf16_at(const uint4 &x, int e) {      // element e of eight
+    const uint32_t w = e < 2 ? x.x : e < 4 ? x.y : e < 6 ? x.z : x.w;
+    return __uint_as_float((e & 1) ? w & 0xffff0000u : w << 16);
+}
+__global__ void __launch_bounds__(kOwnThreads, 2) own_branch_kernel(const uint4 *__restrict__ q, const uint4 *__restrict__ go,
+                                                                  const uint4 *__restrict__ k, const uint4 *__restrict__ v,
+                                                                  const TcBwdParams p) {
+    const int64_t unit = ((int64_t)blockIdx.x * kOwnThreads + threadIdx.x) / 16, units = (p.r.tok_end - p.r.tok_begin) * p.h_kv;
+    const int sub = threadIdx.x & 15;
+    const bool live = unit < units;      // (whole warps go through the shuffles)
+    const int64_t b = p.r.tok_begin + (live ? unit / p.h_kv : 0);
+    const int g = live ? (int)(unit % p.h_kv) : 0;
+    for (int h0 = g * p.group; h0 < (g + 1) * p.group; h0 += kOwnHeads) {
+        const int heads = min(kOwnHeads, (g + 1) * p.group - h0);
+        uint4 qq[kOwnHeads], gg[kOwnHeads];
+        float nl[kOwnHeads], dl[kOwnHeads];
+#pragma unroll
+        for (int i = 0; i < kOwnHeads; ++i) {
+            const int h = h0 + min(i, heads - 1);
+            qq[i] = q[((size_t)b * p.h_q + h) * 16 + sub];
+            gg[i] = go[((size_t)b * p.h_q + h) * 16 + sub];
+            nl[i] = i < heads ? p.nlse2_t[(size_t)h * p.row_pitch + b] : -INFINITY;      // no head: P = 0
+            dl[i] = p.delta_t[(size_t)h * p.row_pitch + b];
+        }
+        for (int j = 0; j < p.depth; ++j) {
+            const size_t krow = ((size_t)(p.meta.n_main + (int64_t)j * p.num_branches + b) * p.h_kv + g) * 16 + sub;
+            const uint4 kk = k[krow], vv = v[krow];
+            float4 *ak = reinterpret_cast<float4 *>(p.dk) + 2 * krow, *av = reinterpret_cast<float4 *>(p.dv) + 2 * krow;
+            const float4 k0 = ak[0], k1 = ak[1], v0 = av[0], v1 = av[1];
+            float s[kOwnHeads], dp[kOwnHeads], dk[8], dv[8];
+#pragma unroll
+            for (int i = 0; i < kOwnHeads; ++i) {
+                s[i] = dp[i] = 0.f;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    s[i] = fmaf(bf16_at(qq[i], e), bf16_at(kk, e), s[i]);
+                    dp[i] = fmaf(bf16_at(gg[i], e), bf16_at(vv, e), dp[i]);
+                }
+            }
+#pragma unroll
+            for (int off = 8; off; off >>= 1)
+#pragma unroll
+                for (int i = 0; i < kOwnHeads; ++i) {
+                    s[i] += __shfl_xor_sync(0xffffffffu, s[i], off);
+                    dp[i] += __shfl_xor_sync(0xffffffffu, dp[i], off);
+                }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) dk[e] = dv[e] = 0.f;
+#pragma unroll
+            for (int i = 0; i < kOwnHeads; ++i) {
+                if (i >= heads) break;
+                const float pr = ex2(fmaf(s[i], p.scale_log2, nl[i])), ds = pr * (dp[i] - dl[i]);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    dk[e] = fmaf(ds, bf16_at(qq[i], e), dk[e]);
+                    dv[e] = fmaf(pr, bf16_at(gg[i], e), dv[e]);
+                }
+            }
+            if (live) {
+                const float sc = p.scale;
+                ak[0] = make_float4(fmaf(sc, dk[0], k0.x), fmaf(sc, dk[1], k0.y), fmaf(sc, dk[2], k0.z), fmaf(sc, dk[3], k0.w));
+                ak[1] = make_float4(fmaf(sc, dk[4], k1.x), fmaf(sc, dk[5], k1.y), fmaf(sc, dk[6], k1.z), fmaf(sc, dk[7], k1.w));
+                av[0] = make_float4(v0.x + dv[0], v0.y + dv[1], v0.z + dv[2], v0.w + dv[3]);
+                av[1] = make_float4(v1.x + dv[4], v1.y + dv[5], v1.z + dv[6], v1.w + dv[7]);
+            }
+        }
+    }
+}
+
 template <bool SPLIT>
 int launch(const TcBwdParams &p, const BaOrder &order, const CUtensorMap *tm, int64_t grid, bool after_dq, int dev, cudaStream_t st) {
     // the dynamic shared-memory limit is a per-device attribute of the kernel
@@ -731,4 +803,12 @@ int ba_tc_dkdv(const TcBwdParams &call, const ba_plan *pl, const BaRange &r, con
     if (!bwd_maps(tm, pl, r, q_main, q_branch, k, v, d_o, p.depth, kTile, 1, kTile)) return BA_EINVAL;
     const BaOrder &order = key_order(p, pl, q_main != nullptr);
     return p.splits > 1 ? launch<true>(p, order, tm, grid, after_dq, dev, st) : launch<false>(p, order, tm, grid, after_dq, dev, st);
+}
+
+int ba_tc_own_branch(const TcBwdParams &p, const void *q, const void *k, const void *v, const void *d_o, cudaStream_t st) {
+    const int64_t blocks = ((p.r.tok_end - p.r.tok_begin) * p.h_kv * 16 + kOwnThreads - 1) / kOwnThreads;
+    if (blocks <= 0) return BA_OK;
+    if (blocks > INT_MAX) return BA_EUNSUPPORTED;
+    own_branch_kernel<<<(unsigned)blocks, kOwnThreads, 0, st>>>((const uint4 *)q, (const uint4 *)d_o, (const uint4 *)k, (const uint4 *)v, p);
+    return ba_check_launch();
 }

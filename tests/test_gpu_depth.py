@@ -101,6 +101,12 @@ def test_depth_calls_sparse_anchors_shared_anchors_and_branch_ranges(ba, oracle)
     run_depth_case(ba, oracle, p, seed=32, splits=[(0, 37), (37, 37), (37, 130), (130, a)])
 
 
+# dK / dV of the own-branch keys: four query heads of a group at a time, sixteen lanes per (branch, KV head)
+@pytest.mark.parametrize("h_q,h_kv", [(1, 1), (3, 1), (5, 1), (8, 1), (6, 3), (14, 2)])
+def test_depth_calls_head_groups(ba, oracle, h_q, h_kv):
+    run_depth_case(ba, oracle, chain_problem([40, 61], [0, 3, 3, 20, 39, 40, 77, 100], 2, h_q, h_kv), seed=h_q, splits=[(0, 5), (5, 8)])
+
+
 def test_depth_calls_reject_what_they_cannot_do(ba):
     p = W.odd_shapes(W.CHAIN, head_dim=128, dtype="bf16")          # branches of unequal length
     plan = ba.Plan(p, impl=ba.IMPL_TC)
