@@ -198,10 +198,10 @@ inline int64_t key_items(TcBwdParams &p, const ba_plan *pl, const BaRange &r, bo
 }
 
 inline BaTiling key_tiling(const TcBwdParams &p, bool has_main) {
-    return {BA_ORDER_KEYS, has_main, p.main_key_tiles, kTile, p.total_key_tiles - p.main_key_tiles, (int64_t)p.step_kb * p.splits};
+    return {BA_ORDER_KEYS, has_main, p.main_key_tiles, kTile, p.total_key_tiles - p.main_key_tiles, p.step_kb};
 }
 inline const BaOrder &key_order(const TcBwdParams &p, const ba_plan *pl, bool has_main) {
-    const bool any = !p.depth && p.tile_major && ba_whole_call(pl, p.r, has_main);
+    const bool any = !p.depth && p.splits == 1 && p.tile_major && ba_whole_call(pl, p.r, has_main);
     return ba_find_order(pl, any ? key_tiling(p, has_main) : BaTiling{-1});
 }
 

@@ -202,9 +202,11 @@ inline int64_t fill_items(ItemParams &p, const ba_plan *pl, const BaRange &r, bo
 inline BaTiling item_tiling(const ItemParams &p, bool has_main) {
     return {BA_ORDER_ROWS, has_main, p.main_items, p.step_m, p.total_items - p.main_items, p.step_b};
 }
+// (Items shared by clusters are few: taken longest first, trees at the ends of 8 sequences, 65,536 tokens, 32/8 heads,
+// 88.4 -> 85.4 us, of 9 sequences, 29,883 tokens, 8/8 heads, 80.6 -> 83.7.)
 inline const BaOrder &item_order(const ItemParams &p, const ba_plan *pl, bool has_main) {
     static const BaOrder none = {};
-    return !p.depth && ba_whole_call(pl, p.r, has_main) ? ba_find_order(pl, item_tiling(p, has_main)) : none;
+    return !p.depth && p.splits == 1 && ba_whole_call(pl, p.r, has_main) ? ba_find_order(pl, item_tiling(p, has_main)) : none;
 }
 
 }  // namespace
