@@ -98,6 +98,20 @@ static inline int ba_check_launch() {
     return BA_OK;
 }
 
+// Launch that may come ahead of the end of the kernel before it in the stream (which the new kernel has to wait for
+// itself, before it reads or writes anything)
+static inline void dependent_launch(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &attr, dim3 grid, unsigned threads, size_t smem, cudaStream_t st) {
+    cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+}
+
 // weights of Eq. (lse-merge) for merging (lse_p, O_p * inv) into the running pair with lse_a
 __device__ __forceinline__ void merge_weights(float lse_a, float lse_p, float inv, float &lse_out, float &w_old, float &w_new) {
     const float mx = fmaxf(lse_a, lse_p);

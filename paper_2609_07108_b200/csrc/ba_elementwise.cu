@@ -3,6 +3,7 @@
 // accumulators.  All are 16-byte vectorised, one pass over memory; merge and conversion
 // are grid-stride, delta has one CTA per tile of rows and heads.
 #include "ba_common.cuh"
+#include "ba_sm100.cuh"
 
 namespace {
 
@@ -116,6 +117,8 @@ __global__ void __launch_bounds__(kThreads)
 delta_kernel(const uint4 *__restrict__ o, const uint4 *__restrict__ d_o, const float *__restrict__ lse,
              float *__restrict__ delta_t, float *__restrict__ nlse2_t, DeltaSegment seg_a, DeltaSegment seg_b,
              int h_q, int64_t pitch) {
+    sm100::wait_prerequisites();      // (ba_delta: the launch may come ahead of the end of the forward)
+    sm100::launch_dependents();
     constexpr int kItems = kThreads / LPI;      // (row, head) items per pass
     __shared__ float s_delta[kDeltaHeads][kDeltaRows + 1], s_nlse2[kDeltaHeads][kDeltaRows + 1];
     const bool in_a = (int64_t)blockIdx.x < seg_a.tiles;
@@ -225,8 +228,15 @@ int ba_delta(const void *o, const void *d_o, const float *lse, float *delta_t, f
     const uint4 *op = (const uint4 *)o, *gp = (const uint4 *)d_o;
     const int lpi = (int)(d * esz / 16);
     const dim3 grid((unsigned)(seg_a.tiles + seg_b.tiles), (unsigned)((h_q + kDeltaHeads - 1) / kDeltaHeads));
+    // Forward, delta and dQ follow one another in a step: each may be launched while the one before ends, and waits for
+    // it at its head (640 tokens in fp32, whole step 65.5 -> 63.9 us, 4,096 in bf16 at head_dim 64 676 -> 660).  A larger
+    // delta is launched as usual: its blocks would crowd the SMs that are free first (8,192 rows: 27 us instead of 24).
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    dependent_launch(cfg, attr, grid, kThreads, 0, st);
+    if ((int64_t)grid.x * grid.y > 4 * kSms) cfg.numAttrs = 0;
 #define BA_DELTA_LAUNCH(T, L) \
-    delta_kernel<T, L><<<grid, kThreads, 0, st>>>(op, gp, lse, delta_t, nlse2_t, seg_a, seg_b, h_q, row_pitch)
+    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, delta_kernel<T, L>, op, gp, lse, delta_t, nlse2_t, seg_a, seg_b, h_q, row_pitch))
     if (dtype == BA_FP32 && lpi == 16) BA_DELTA_LAUNCH(float, 16);
     else if (dtype == BA_FP32 && lpi == 32) BA_DELTA_LAUNCH(float, 32);
     else if (dtype == BA_BF16 && lpi == 8) BA_DELTA_LAUNCH(__nv_bfloat16, 8);

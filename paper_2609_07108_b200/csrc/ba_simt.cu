@@ -213,6 +213,8 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const __grid_constant
     constexpr int WR = kRows / 4, AR = 4;     // rows per warp, per accumulator lane
     constexpr bool kMerges = MODE == kFwd && D == 64 && sizeof(T) == 2;      // partial results merged in place
     constexpr int P = pitch<D>();
+    if (MODE == kDq) wait_prerequisites();      // launched while delta ends
+    if (MODE != kDkdv) launch_dependents();     // dQ: dK/dV may start beside it; forward: delta may be launched
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t n = a.meta.n_main;
     const int rank = (int)(blockIdx.x % a.splits);
@@ -238,7 +240,6 @@ __global__ void __launch_bounds__(kThreads, 3) simt_kernel(const __grid_constant
     };
     auto row_tok = [&](int r) -> int64_t { return MODE == kDkdv ? base + r : base + r / a.hp; };
 
-    if (MODE == kDq) launch_dependents();      // the dK/dV kernel may start beside this one
     if (tid == 0) { sm.lo_min = INT_MAX; sm.hi_max = -1; sm.bs_min = INT_MAX; sm.be_max = -1; }
     __syncthreads();
     if (tid < kRows && live_row(tid)) {
@@ -631,7 +632,7 @@ int launch(SimtArgs &a, const BaOrder &order, int64_t work, bool after_dq, cudaS
         attr[cfg.numAttrs].val.clusterDim.y = attr[cfg.numAttrs].val.clusterDim.z = 1;
         ++cfg.numAttrs;
     }
-    if (after_dq) {     // start when every CTA of the dQ kernel queued just before has started
+    if (after_dq) {     // start when every CTA of the kernel queued just before has started (dQ: it then waits for delta)
         attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
         ++cfg.numAttrs;
@@ -743,7 +744,7 @@ int ba_simt_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const v
     a.nlse2_t = delta + (size_t)pl->row_pitch * a.h_q;
     a.dq_main = dq_main; a.dq_branch = dq_branch; a.dk = dk; a.dv = dv;
     int rc = BA_OK;
-    if (stages & BA_STAGE_DQ) rc = dispatch<kDq>(pl, a, st);
+    if (stages & BA_STAGE_DQ) rc = dispatch<kDq>(pl, a, st, (stages & BA_STAGE_PREP) != 0);
     // The two kernels write different tensors and need the same inputs: the second may run beside the first
     // (not when no row of dQ was launched: the kernel before is then the caller's, or delta)
     const bool dq_rows = (q_main && r.qm_end > r.qm_begin) || r.tok_end > r.tok_begin;

@@ -100,7 +100,6 @@ tc_dq_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
         if (tid == 0) atomicExch(p.status, BA_EUNSUPPORTED);
         return;
     }
-    launch_dependents();      // the dK/dV kernel may take the SMs that this one leaves
     // global row number of branch query 0 (rows of dO and of the per-row scalars): see tc_kv_kernel
     const int qbase = p.depth ? 0 : (int)p.meta.n_main;
 
@@ -133,6 +132,8 @@ tc_dq_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sm.tmem_base;
+    wait_prerequisites();     // launched while delta ends
+    launch_dependents();      // the dK/dV kernel may take the SMs that this one leaves; delta is there for it too
 
     if (warp >= 8) {
         reg_dec<kDqRegsIssue>();
@@ -808,6 +809,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
     tc_fence_after();
     const uint32_t tmem = sm.tmem_base;
     bool shared_tile = false;      // SPLIT: this CTA walked a part of a main key tile
+    if (kDq) wait_prerequisites();      // launched while delta ends
 
     if (warp >= 8) {
         reg_dec<kKvRegsIssue>();
@@ -1302,7 +1304,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
 }
 
 template <int MODE, bool SPLIT>
-int launch_kv(const TcBwdParams &p, const BaOrder &order, const CUtensorMap *tm, int64_t grid, int dev, cudaStream_t st) {
+int launch_kv(const TcBwdParams &p, const BaOrder &order, const CUtensorMap *tm, int64_t grid, int dev, cudaStream_t st, bool after_delta = false) {
     if (grid <= 0) return BA_OK;
     if (grid > INT_MAX) return BA_EUNSUPPORTED;
     // the dynamic shared-memory limit is a per-device attribute of the kernel
@@ -1317,17 +1319,15 @@ int launch_kv(const TcBwdParams &p, const BaOrder &order, const CUtensorMap *tm,
         attr_set[dev] = true;
     }
     cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof cfg);
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kKvThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
     cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = (unsigned)p.splits;
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = SPLIT ? 1 : 0;
+    dependent_launch(cfg, attr, dim3((unsigned)grid), kKvThreads, smem, st);
+    if (SPLIT) {
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = (unsigned)p.splits;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    } else if (!after_delta) {
+        cfg.numAttrs = 0;
+    }
     BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_kv_kernel<MODE, SPLIT>, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], p, order));
     return ba_check_launch();
 }
@@ -1354,7 +1354,7 @@ void ba_tc_bwd_orders(ba_plan *pl, const ba_problem_t *host) {
     const BaRange r = {0, n, 0, m, 0, n, 0, BA_PART_MAIN | BA_PART_BRANCH};
     for (int has_main = 1; has_main >= 0; --has_main) {
         TcBwdParams p = bwd_params(pl, r, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0, nullptr, nullptr, nullptr, nullptr, 0);
-        if (key_items(p, pl, r, has_main) > 0 && p.tile_major) ba_add_order(pl, host, key_tiling(p, has_main));
+        if (key_items(p, pl, r, has_main) > 0 && p.splits == 1 && p.tile_major) ba_add_order(pl, host, key_tiling(p, has_main));
         if (pl->prob.head_dim == 64) {
             row_tiles(p, has_main ? n : 0, m);
             ba_add_order(pl, host, row_tiling(p, has_main));
@@ -1378,7 +1378,8 @@ int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
         if (stages & BA_STAGE_DQ) {
             row_tiles(p, qm_n, br_n);
             if (!maps(p.tok, p.hp, kSub)) return BA_EINVAL;
-            int rc = launch_kv<kModeDq, false>(p, row_order(p, pl, q_main != nullptr), tm, (int64_t)p.total_tiles * pr.h_kv * p.head_chunks, dev, st);
+            int rc = launch_kv<kModeDq, false>(p, row_order(p, pl, q_main != nullptr), tm, (int64_t)p.total_tiles * pr.h_kv * p.head_chunks, dev, st,
+                                                (stages & BA_STAGE_PREP) != 0);
             if (rc != BA_OK) return rc;
         }
         if (stages & BA_STAGE_DKDV) {
@@ -1420,8 +1421,11 @@ int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
             !make_tmap_rhd(&v32, v, kv_rows, pr.h_kv, 128, 32))
             return BA_EINVAL;
         if (grid > 0) {
-            tc_dq_kernel<<<(unsigned)grid, kDqThreads, sizeof(DqSmem), st>>>(tm[0], tm[1], tm[2], tm[3], tm[4], k32, v32, q,
-                                                                              item_order(q, pl, q_main != nullptr));
+            cudaLaunchConfig_t cfg;
+            cudaLaunchAttribute attr;
+            dependent_launch(cfg, attr, dim3((unsigned)grid), kDqThreads, sizeof(DqSmem), st);
+            if (!(stages & BA_STAGE_PREP)) cfg.numAttrs = 0;
+            BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_dq_kernel, tm[0], tm[1], tm[2], tm[3], tm[4], k32, v32, q, item_order(q, pl, q_main != nullptr)));
             int rc = ba_check_launch();
             if (rc != BA_OK) return rc;
         }

@@ -292,6 +292,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_consta
         return;
     }
 
+    launch_dependents();      // delta of the backward may be launched (it waits for the end of this kernel)
     if (tid == 0) {
         mbar_init(&sm.q_full, 1);
         mbar_init(&sm.q_empty, 1);
@@ -987,8 +988,8 @@ int ba_tc_fwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
 
 void ba_tc_fwd_orders(ba_plan *pl, const ba_problem_t *host) {
     const BaRange r = {0, pl->prob.n_main, 0, pl->prob.n_branch, 0, pl->prob.n_main, 0, BA_PART_MAIN | BA_PART_BRANCH};
-    for (int i = 0; i < 3; ++i) {      // with main queries; branch rows only, two or one tile of rows per item
+    for (int has_main = 1; has_main >= 0; --has_main) {
         ItemParams p;
-        if (fill_items(p, pl, r, i == 0, 0, i == 2) > 0) ba_add_order(pl, host, item_tiling(p, i == 0));
+        if (fill_items(p, pl, r, has_main, 0) > 0) ba_add_order(pl, host, item_tiling(p, has_main));
     }
 }
