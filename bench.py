@@ -276,8 +276,8 @@ class Recorder:
     def branch_attn_fwd_depth(self, *a, **k):
         return self._wrap("fwd", 1, self.ba.branch_attn_fwd_depth, *a, **k)
 
-    def branch_attn_bwd_depth(self, *a, **k):     # delta, dQ, dK/dV
-        return self._wrap("bwd_depth", 3, self.ba.branch_attn_bwd_depth, *a, **k)
+    def branch_attn_bwd_depth(self, *a, **k):     # delta, dK/dV of own-branch keys, dQ, dK/dV
+        return self._wrap("bwd_depth", 4, self.ba.branch_attn_bwd_depth, *a, **k)
 
     def totals(self):
         """Device time (ms) and calls by kind; what calls of one kind overlap (on two streams) is counted once."""
@@ -565,8 +565,8 @@ def run_ours(args):
         # units of head_dim: forward 2 GEMMs (QK^T, PV); dQ kernel 3 (S, dP, dQ);
         # dK/dV kernel 4 (S^T and dP^T recomputed, dV, dK); a per-depth backward runs these two
         share = {"fwd": 4.0, "bwd_dq": 6.0, "bwd_dkdv": 8.0, "bwd_fused": 10.0, "bwd_depth": 14.0}.get(kind)
-        kernel_name = {"fwd": "tc_fwd_kernel", "bwd_dq": "tc_dq_kernel", "bwd_dkdv": "tc_kv_kernel",
-                       "bwd_fused": "tc_bwd_fused_kernel", "bwd_depth": "tc_dq_kernel + tc_kv_kernel"}.get(kind, kind)
+        kernel_name = {"fwd": "tc_fwd_kernel", "bwd_dq": "tc_dq_kernel", "bwd_dkdv": "tc_dkdv_kernel",
+                       "bwd_fused": "tc_bwd_fused_kernel", "bwd_depth": "tc_dq_kernel + tc_dkdv_kernel + own_branch_kernel"}.get(kind, kind)
         if share is not None:
             kpairs = pairs
             if mode == "stepwise" and kind != "fwd":    # the per-depth calls cover the branch rows only
