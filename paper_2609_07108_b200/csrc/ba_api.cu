@@ -144,13 +144,15 @@ static int bwd_common(const ba_plan_t *plan, const void *q_main, const void *q_b
     const int64_t rp = plan->row_pitch;
     const int64_t n = plan->prob.n_main;
     const int hq = plan->prob.h_q, d = plan->prob.head_dim, dt = plan->prob.dtype;
-    if (stages & BA_STAGE_PREP) {   // main rows and branch rows of the call in one launch
-        const int64_t ma = has_main_q ? r.qm_begin : 0, mb = has_main_q ? r.qm_end : 0;
-        const int64_t ba_ = has_branch_q ? n + r.tok_begin : 0, bb = has_branch_q ? n + r.tok_end : 0;
-        if ((rc = ba_delta(O, dO, LSE, delta, nlse2, rp, ma, mb, ba_, bb, hq, d, dt, st)) != BA_OK) return rc;
-    }
-    if (!(stages & (BA_STAGE_DQ | BA_STAGE_DKDV | BA_STAGE_FUSED))) return BA_OK;
+    // main rows and branch rows of the call in one launch
+    const BaDelta prep = {O, dO, LSE, delta, nlse2, rp, r.qm_begin, r.qm_end, n + r.tok_begin, n + r.tok_end, hq, d, dt};
     const void *qm = has_main_q ? q_main : nullptr;
+    const uintptr_t addresses = (uintptr_t)q_main | (uintptr_t)q_branch | (uintptr_t)k | (uintptr_t)v | (uintptr_t)dQ_main |
+                                (uintptr_t)dQ_branch | (uintptr_t)dK | (uintptr_t)dV;
+    if ((stages & (BA_STAGE_DQ | BA_STAGE_DKDV)) && ba_use_tc(plan, accumulate != 0, addresses))
+        return ba_tc_bwd(plan, r, qm, q_branch, k, v, prep, accumulate, dQ_main, dQ_branch, dK, dV, st, stages);
+    if ((stages & BA_STAGE_PREP) && (rc = ba_delta(prep, st)) != BA_OK) return rc;
+    if (!(stages & (BA_STAGE_DQ | BA_STAGE_DKDV | BA_STAGE_FUSED))) return BA_OK;
     if (stages & BA_STAGE_FUSED) {
         if (plan->impl != BA_IMPL_TC || d != 128) return BA_EUNSUPPORTED;
         if (accumulate)
@@ -179,11 +181,6 @@ static int bwd_common(const ba_plan_t *plan, const void *q_main, const void *q_b
             return rc;
         return BA_OK;
     }
-    const uintptr_t addresses = (uintptr_t)q_main | (uintptr_t)q_branch | (uintptr_t)k | (uintptr_t)v | (uintptr_t)dQ_main |
-                                (uintptr_t)dQ_branch | (uintptr_t)dK | (uintptr_t)dV;
-    if (ba_use_tc(plan, accumulate != 0, addresses))
-        return ba_tc_bwd(plan, r, qm, q_branch, k, v, delta, dO, accumulate, dQ_main, dQ_branch, dK,
-                         dV, st, stages);
     return ba_simt_bwd(plan, r, qm, q_branch, k, v, LSE, delta, dO, accumulate, dQ_main, dQ_branch, dK, dV,
                        st, stages);
 }
@@ -237,16 +234,18 @@ extern "C" int branch_attn_bwd_depth(const ba_plan_t *plan, int depth, const voi
     if (!q_depth || !k || !v || !O_depth || !LSE_depth || !dO_depth || !dQ_depth || !dK || !dV) return BA_EINVAL;
     if (!workspace || ws_bytes < ba_workspace_bytes(plan, BA_OP_BWD_DEPTH) || ((uintptr_t)workspace & 255))
         return BA_EWORKSPACE;
-    cudaStream_t st = (cudaStream_t)stream;
+    // every kernel of the call reads and writes its rows in pieces of 16 bytes
+    if (((uintptr_t)q_depth | (uintptr_t)k | (uintptr_t)v | (uintptr_t)O_depth | (uintptr_t)dO_depth | (uintptr_t)dQ_depth |
+         (uintptr_t)dK | (uintptr_t)dV) & 15)
+        return BA_EINVAL;
     const ba_problem_t &pr = plan->prob;
     float *delta = (float *)workspace;
     float *nlse2 = delta + (size_t)plan->row_pitch * pr.h_q;
     // per-row scalars of the selected branches' depth-`depth` rows (rows are indexed by branch here)
-    if ((rc = ba_delta(O_depth, dO_depth, LSE_depth, delta, nlse2, plan->row_pitch, 0, 0, br_begin, br_end,
-                       pr.h_q, pr.head_dim, pr.dtype, st)) != BA_OK)
-        return rc;
-    return ba_tc_bwd(plan, r, nullptr, q_depth, k, v, delta, dO_depth, 1, nullptr, dQ_depth, dK, dV, st,
-                     BA_STAGE_DQ | BA_STAGE_DKDV, depth);
+    const BaDelta prep = {O_depth, dO_depth, LSE_depth, delta, nlse2, plan->row_pitch, 0, 0, br_begin, br_end,
+                          pr.h_q, pr.head_dim, pr.dtype};
+    return ba_tc_bwd(plan, r, nullptr, q_depth, k, v, prep, 1, nullptr, dQ_depth, dK, dV, (cudaStream_t)stream,
+                     BA_STAGE_ALL, depth);
 }
 
 // ---------------------------------------------------------------- ring steps on a received K/V shard

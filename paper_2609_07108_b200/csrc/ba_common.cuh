@@ -66,6 +66,16 @@ struct BaRange {
     int parts;
 };
 
+// Backward preprocess of one call (ba_delta): inputs, head-major scratch, rows [a_begin, a_end) and [b_begin, b_end)
+// (either may be empty)
+struct BaDelta {
+    const void *o, *d_o;
+    const float *lse;
+    float *delta_t, *nlse2_t;
+    int64_t row_pitch, a_begin, a_end, b_begin, b_end;
+    int h_q, d, dtype;
+};
+
 static inline bool ba_whole_call(const ba_plan *pl, const BaRange &r, bool has_main) {
     return (!has_main || (r.qm_begin == 0 && r.qm_end == pl->prob.n_main)) && r.tok_begin == 0 && r.tok_end == pl->prob.n_branch &&
            r.kv_begin == 0 && r.kv_end == pl->prob.n_main && r.kv_base == 0 && r.parts == (BA_PART_MAIN | BA_PART_BRANCH);
@@ -137,14 +147,14 @@ int ba_simt_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const v
 // Tensor-core path (ba_tc_fwd.cu / ba_tc_bwd.cu / ba_tc_dkdv.cu)
 // partial_out: 0 = final layout in the input dtype, 1 = compact fp32, 2 = compact fp32 merged in place
 // depth > 0: step-major call (queries = the depth-`depth` tokens of branches [r.tok_begin, r.tok_end),
-// q_branch / o / lse indexed by branch, branch keys stored depth-major after the main rows)
+// q_branch / o / lse indexed by branch, branch keys stored depth-major after the main rows).
+// ba_tc_bwd runs BA_STAGE_PREP (`prep`) itself: whatever it refuses is refused before it launches anything.
 int ba_tc_fwd(const ba_plan *pl, const BaRange &r, const void *q_main, const void *q_branch,
               const void *k, const void *v, void *o, float *lse, int partial_out,
               cudaStream_t st, int depth = 0);
 int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const void *q_branch,
-              const void *k, const void *v, const float *delta,
-              const void *d_o, int accumulate, void *dq_main, void *dq_branch, void *dk,
-              void *dv, cudaStream_t st, int stages, int depth = 0);
+              const void *k, const void *v, const BaDelta &prep, int accumulate, void *dq_main,
+              void *dq_branch, void *dk, void *dv, cudaStream_t st, int stages, int depth = 0);
 // One-kernel backward (ba_tc_bwd_fused.cu): dq_* are fp32 accumulators (atomic adds) in either mode
 int ba_tc_bwd_fused(const ba_plan *pl, const BaRange &r, const void *q_main, const void *q_branch,
                     const void *k, const void *v, const float *delta, const void *d_o,
@@ -163,8 +173,6 @@ static inline bool ba_use_tc(const ba_plan *pl, bool fp32_out, uintptr_t address
 // Elementwise (ba_elementwise.cu)
 // Backward preprocess into head-major scratch [h_q, row_pitch]:
 //   delta_t[h, r] = <dO[r, h], O[r, h]>,  nlse2_t[h, r] = -LSE[r, h] * log2(e)
-// for two row segments [row_a_begin, row_a_end) and [row_b_begin, row_b_end) (either may be empty)
-int ba_delta(const void *o, const void *d_o, const float *lse, float *delta_t, float *nlse2_t,
-             int64_t row_pitch, int64_t row_a_begin, int64_t row_a_end, int64_t row_b_begin,
-             int64_t row_b_end, int h_q, int d, int dtype, cudaStream_t st);
+// for the two row segments of `x`
+int ba_delta(const BaDelta &x, cudaStream_t st);
 static inline int64_t ba_row_pitch(int64_t rows) { return (rows + 128 + 63) / 64 * 64; }

@@ -214,20 +214,16 @@ extern "C" int lse_merge(int64_t rows_heads, int d, const float *O_a, const floa
     return launch_merge<false>(d / 4, rows_heads, O_a, LSE_a, O_b, LSE_b, O_out, LSE_out, st);
 }
 
-int ba_delta(const void *o, const void *d_o, const float *lse, float *delta_t, float *nlse2_t,
-             int64_t row_pitch, int64_t row_a_begin, int64_t row_a_end, int64_t row_b_begin,
-             int64_t row_b_end, int h_q, int d, int dtype, cudaStream_t st) {
+int ba_delta(const BaDelta &x, cudaStream_t st) {
     auto segment = [](int64_t begin, int64_t end) {
         DeltaSegment g = {begin, end, 0};
         if (end > begin) g.tiles = (end - (begin & ~(int64_t)(kDeltaRows - 1)) + kDeltaRows - 1) / kDeltaRows;
         return g;
     };
-    const DeltaSegment seg_a = segment(row_a_begin, row_a_end), seg_b = segment(row_b_begin, row_b_end);
+    const DeltaSegment seg_a = segment(x.a_begin, x.a_end), seg_b = segment(x.b_begin, x.b_end);
     if (seg_a.tiles + seg_b.tiles == 0) return BA_OK;
-    const size_t esz = dtype == BA_FP32 ? 4 : 2;
-    const uint4 *op = (const uint4 *)o, *gp = (const uint4 *)d_o;
-    const int lpi = (int)(d * esz / 16);
-    const dim3 grid((unsigned)(seg_a.tiles + seg_b.tiles), (unsigned)((h_q + kDeltaHeads - 1) / kDeltaHeads));
+    const int lpi = x.d * (x.dtype == BA_FP32 ? 4 : 2) / 16;
+    const dim3 grid((unsigned)(seg_a.tiles + seg_b.tiles), (unsigned)((x.h_q + kDeltaHeads - 1) / kDeltaHeads));
     // Forward, delta and dQ follow one another in a step: each may be launched while the one before ends, and waits for
     // it at its head (640 tokens in fp32, whole step 65.5 -> 63.9 us, 4,096 in bf16 at head_dim 64 676 -> 660).  A larger
     // delta is launched as usual: its blocks would crowd the SMs that are free first (8,192 rows: 27 us instead of 24).
@@ -236,11 +232,12 @@ int ba_delta(const void *o, const void *d_o, const float *lse, float *delta_t, f
     dependent_launch(cfg, attr, grid, kThreads, 0, st);
     if ((int64_t)grid.x * grid.y > 4 * kSms) cfg.numAttrs = 0;
 #define BA_DELTA_LAUNCH(T, L) \
-    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, delta_kernel<T, L>, op, gp, lse, delta_t, nlse2_t, seg_a, seg_b, h_q, row_pitch))
-    if (dtype == BA_FP32 && lpi == 16) BA_DELTA_LAUNCH(float, 16);
-    else if (dtype == BA_FP32 && lpi == 32) BA_DELTA_LAUNCH(float, 32);
-    else if (dtype == BA_BF16 && lpi == 8) BA_DELTA_LAUNCH(__nv_bfloat16, 8);
-    else if (dtype == BA_BF16 && lpi == 16) BA_DELTA_LAUNCH(__nv_bfloat16, 16);
+    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, delta_kernel<T, L>, (const uint4 *)x.o, (const uint4 *)x.d_o, x.lse, x.delta_t, x.nlse2_t, seg_a, seg_b, x.h_q, \
+                                     x.row_pitch))
+    if (x.dtype == BA_FP32 && lpi == 16) BA_DELTA_LAUNCH(float, 16);
+    else if (x.dtype == BA_FP32 && lpi == 32) BA_DELTA_LAUNCH(float, 32);
+    else if (x.dtype == BA_BF16 && lpi == 8) BA_DELTA_LAUNCH(__nv_bfloat16, 8);
+    else if (x.dtype == BA_BF16 && lpi == 16) BA_DELTA_LAUNCH(__nv_bfloat16, 16);
     else return BA_EUNSUPPORTED;
 #undef BA_DELTA_LAUNCH
     return ba_check_launch();

@@ -1306,7 +1306,6 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
 template <int MODE, bool SPLIT>
 int launch_kv(const TcBwdParams &p, const BaOrder &order, const CUtensorMap *tm, int64_t grid, int dev, cudaStream_t st, bool after_delta = false) {
     if (grid <= 0) return BA_OK;
-    if (grid > INT_MAX) return BA_EUNSUPPORTED;
     // the dynamic shared-memory limit is a per-device attribute of the kernel
     static bool attr_set[64] = {};
     const size_t smem = sizeof(KvSmem);
@@ -1363,39 +1362,41 @@ void ba_tc_bwd_orders(ba_plan *pl, const ba_problem_t *host) {
 }
 
 int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const void *q_branch, const void *k,
-              const void *v, const float *delta, const void *d_o, int accumulate,
-              void *dq_main, void *dq_branch, void *dk, void *dv, cudaStream_t st, int stages, int depth) {
+              const void *v, const BaDelta &prep, int accumulate, void *dq_main, void *dq_branch, void *dk, void *dv,
+              cudaStream_t st, int stages, int depth) {
     // depth > 0: dQ is written (bf16, one row per branch), dK / dV accumulate
     int dev = 0;
     BA_CUDA_CHECK(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return BA_EUNSUPPORTED;
     const ba_problem_t &pr = pl->prob;
-    TcBwdParams p = bwd_params(pl, r, q_main, q_branch, k, v, delta, d_o, accumulate, dq_main, dq_branch, dk, dv, depth);
-    CUtensorMap tm[6];
-    auto maps = [&](uint32_t qr, uint32_t qh, uint32_t kr) { return bwd_maps(tm, pl, r, q_main, q_branch, k, v, d_o, depth, qr, qh, kr); };
-    const int64_t qm_n = q_main ? r.qm_end - r.qm_begin : 0, br_n = r.tok_end - r.tok_begin;
+    const void *d_o = prep.d_o;
+    TcBwdParams p = bwd_params(pl, r, q_main, q_branch, k, v, prep.delta_t, d_o, accumulate, dq_main, dq_branch, dk, dv, depth);
+    const bool has_main = q_main != nullptr, do_dq = stages & BA_STAGE_DQ, do_dkdv = stages & BA_STAGE_DKDV;
+    const int64_t qm_n = has_main ? r.qm_end - r.qm_begin : 0, br_n = r.tok_end - r.tok_begin;
+    auto maps = [&](CUtensorMap *tm, uint32_t qr, uint32_t qh, uint32_t kr) {
+        return bwd_maps(tm, pl, r, q_main, q_branch, k, v, d_o, depth, qr, qh, kr);
+    };
+    auto prepare_rows = [&] { return stages & BA_STAGE_PREP ? ba_delta(prep, st) : BA_OK; };
+    CUtensorMap tm[6];      // dQ
     if (pr.head_dim == 64) {
-        if (stages & BA_STAGE_DQ) {
-            row_tiles(p, qm_n, br_n);
-            if (!maps(p.tok, p.hp, kSub)) return BA_EINVAL;
-            int rc = launch_kv<kModeDq, false>(p, row_order(p, pl, q_main != nullptr), tm, (int64_t)p.total_tiles * pr.h_kv * p.head_chunks, dev, st,
-                                                (stages & BA_STAGE_PREP) != 0);
-            if (rc != BA_OK) return rc;
-        }
-        if (stages & BA_STAGE_DKDV) {
-            // (both kernels overlapped, as at head_dim 128: 605 us instead of 548 for the 4,096-token chains)
-            const int64_t grid = key_items(p, pl, r, q_main != nullptr);
-            if (!maps(kSub, 1, kTile)) return BA_EINVAL;
-            const BaOrder &order = key_order(p, pl, q_main != nullptr);
-            return p.splits > 1 ? launch_kv<kModeDkdv, true>(p, order, tm, grid, dev, st) : launch_kv<kModeDkdv, false>(p, order, tm, grid, dev, st);
-        }
-        return BA_OK;
+        CUtensorMap tk[6];  // dK/dV
+        TcBwdParams pq = p;
+        row_tiles(pq, qm_n, br_n);
+        const int64_t dq_grid = (int64_t)pq.total_tiles * pr.h_kv * pq.head_chunks, grid = key_items(p, pl, r, has_main);
+        if ((do_dq && dq_grid > INT_MAX) || (do_dkdv && grid > INT_MAX)) return BA_EUNSUPPORTED;
+        if ((do_dq && !maps(tm, pq.tok, pq.hp, kSub)) || (do_dkdv && !maps(tk, kSub, 1, kTile))) return BA_EINVAL;
+        int rc = prepare_rows();
+        if (rc == BA_OK && do_dq)
+            rc = launch_kv<kModeDq, false>(pq, row_order(pq, pl, has_main), tm, dq_grid, dev, st, (stages & BA_STAGE_PREP) != 0);
+        if (rc != BA_OK || !do_dkdv) return rc;
+        // (both kernels overlapped, as at head_dim 128: 605 us instead of 548 for the 4,096-token chains)
+        const BaOrder &order = key_order(p, pl, has_main);
+        return p.splits > 1 ? launch_kv<kModeDkdv, true>(p, order, tk, grid, dev, st) : launch_kv<kModeDkdv, false>(p, order, tk, grid, dev, st);
     }
-    if (depth && (stages & BA_STAGE_DKDV)) {
-        const int rc = ba_tc_own_branch(p, q_branch, k, v, d_o, st);
-        if (rc != BA_OK) return rc;
-    }
-    if (stages & BA_STAGE_DQ) {
+    TcDqParams q;
+    CUtensorMap k32, v32;
+    int64_t dq_grid = 0;
+    if (do_dq) {
         static bool attr_set[64] = {};
         if (!attr_set[dev]) {
             // the register re-split hands out what a launch with kDqRegsLaunch registers per thread owns
@@ -1405,38 +1406,37 @@ int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
             BA_CUDA_CHECK(cudaFuncSetAttribute(tc_dq_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DqSmem)));
             attr_set[dev] = true;
         }
-        TcDqParams q;
         memset(&q, 0, sizeof q);
-        const int64_t grid = fill_items(q, pl, r, q_main != nullptr, depth);
+        dq_grid = fill_items(q, pl, r, has_main, depth);
         q.nlse2_t = p.nlse2_t; q.delta_t = p.delta_t; q.row_pitch = p.row_pitch;
         q.dq_main = dq_main; q.dq_branch = dq_branch;
         q.scale = p.scale; q.scale_log2 = p.scale_log2;
         q.accumulate = depth ? 0 : accumulate;
         q.wide = p.wide;
         q.status = p.status;
-        if (grid > INT_MAX) return BA_EUNSUPPORTED;
+        if (dq_grid > INT_MAX) return BA_EUNSUPPORTED;
         const uint64_t kv_rows = key_rows(pl, r, depth);
-        CUtensorMap k32, v32;
-        if (!maps(q.tok, q.hp, kTile) || !make_tmap_rhd(&k32, k, kv_rows, pr.h_kv, 128, 32) ||
+        if (!maps(tm, q.tok, q.hp, kTile) || !make_tmap_rhd(&k32, k, kv_rows, pr.h_kv, 128, 32) ||
             !make_tmap_rhd(&v32, v, kv_rows, pr.h_kv, 128, 32))
             return BA_EINVAL;
-        if (grid > 0) {
-            cudaLaunchConfig_t cfg;
-            cudaLaunchAttribute attr;
-            dependent_launch(cfg, attr, dim3((unsigned)grid), kDqThreads, sizeof(DqSmem), st);
-            if (!(stages & BA_STAGE_PREP)) cfg.numAttrs = 0;
-            BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_dq_kernel, tm[0], tm[1], tm[2], tm[3], tm[4], k32, v32, q, item_order(q, pl, q_main != nullptr)));
-            int rc = ba_check_launch();
-            if (rc != BA_OK) return rc;
-        }
     }
-    if (stages & BA_STAGE_DKDV) {
-        // The two kernels write different tensors and need the same inputs: the second may start on the SMs that the
-        // last items of the first leave idle (not when no row of dQ was launched: the kernel before is then the
-        // caller's, or delta).  Both kernels, overlapped / one after the other: 2,048-token chains 222 / 231 us, draft
-        // rows of 512 blocks 658 / 680.
-        const bool after_dq = (stages & BA_STAGE_DQ) && qm_n + br_n > 0;
-        return ba_tc_dkdv(p, pl, r, q_main, q_branch, k, v, d_o, after_dq, dev, st);
+    TcDkdvCall dkdv;
+    int rc = do_dkdv ? ba_tc_dkdv_prepare(dkdv, p, pl, r, q_main, q_branch, k, v, d_o, dev) : BA_OK;
+    // nothing has been launched so far, and nothing is refused from here on
+    if (rc == BA_OK) rc = prepare_rows();
+    if (rc == BA_OK && depth && do_dkdv) rc = ba_tc_own_branch(p, q_branch, k, v, d_o, st);
+    if (rc != BA_OK) return rc;
+    if (dq_grid > 0) {
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attr;
+        dependent_launch(cfg, attr, dim3((unsigned)dq_grid), kDqThreads, sizeof(DqSmem), st);
+        if (!(stages & BA_STAGE_PREP) || depth) cfg.numAttrs = 0;
+        BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_dq_kernel, tm[0], tm[1], tm[2], tm[3], tm[4], k32, v32, q, item_order(q, pl, has_main)));
+        if ((rc = ba_check_launch()) != BA_OK) return rc;
     }
-    return BA_OK;
+    // dK/dV: the two kernels write different tensors and need the same inputs: the second may start on the SMs that the
+    // last items of the first leave idle (not when no row of dQ was launched: the kernel before is then the
+    // caller's, or delta).  Both kernels, overlapped / one after the other: 2,048-token chains 222 / 231 us, draft
+    // rows of 512 blocks 658 / 680.
+    return do_dkdv ? ba_tc_dkdv_launch(dkdv, do_dq && qm_n + br_n > 0, st) : BA_OK;
 }

@@ -207,8 +207,16 @@ inline const BaOrder &key_order(const TcBwdParams &p, const ba_plan *pl, bool ha
 
 }  // namespace
 
-// dK / dV of a call at head_dim 128 (ba_tc_dkdv.cu); after_dq: it may start while the dQ kernel queued just before ends
-int ba_tc_dkdv(const TcBwdParams &call, const ba_plan *pl, const BaRange &r, const void *q_main, const void *q_branch,
-               const void *k, const void *v, const void *d_o, bool after_dq, int dev, cudaStream_t st);
+// dK / dV of a call at head_dim 128 (ba_tc_dkdv.cu): all that can be refused, then the launch; after_dq: it may start
+// while the dQ kernel queued just before ends
+struct TcDkdvCall {
+    TcBwdParams p;
+    CUtensorMap tm[6];
+    int64_t grid;
+    const BaOrder *order;
+};
+int ba_tc_dkdv_prepare(TcDkdvCall &c, const TcBwdParams &call, const ba_plan *pl, const BaRange &r, const void *q_main,
+                       const void *q_branch, const void *k, const void *v, const void *d_o, int dev);
+int ba_tc_dkdv_launch(const TcDkdvCall &c, bool after_dq, cudaStream_t st);
 // step-major calls: dK / dV of the own-branch keys alone
 int ba_tc_own_branch(const TcBwdParams &p, const void *q, const void *k, const void *v, const void *d_o, cudaStream_t st);

@@ -755,28 +755,31 @@ __global__ void __launch_bounds__(kOwnThreads, 2) own_branch_kernel(const uint4 
 }
 
 template <bool SPLIT>
-int launch(const TcBwdParams &p, const BaOrder &order, const CUtensorMap *tm, int64_t grid, bool after_dq, int dev, cudaStream_t st) {
+int prepare(int dev) {
     // the dynamic shared-memory limit is a per-device attribute of the kernel
     static bool attr_set[64] = {};
-    const size_t smem = sizeof(DkdvSmem);
-    if (!attr_set[dev]) {
-        // the register re-split hands out what a launch with kRegsLaunch registers per thread owns
-        cudaFuncAttributes fa;
-        BA_CUDA_CHECK(cudaFuncGetAttributes(&fa, tc_dkdv_kernel<SPLIT>));
-        if (fa.numRegs * kThreads < 256 * kRegsCompute + 128 * kRegsIssue) return BA_EUNSUPPORTED;
-        BA_CUDA_CHECK(cudaFuncSetAttribute(tc_dkdv_kernel<SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        attr_set[dev] = true;
-    }
+    if (attr_set[dev]) return BA_OK;
+    // the register re-split hands out what a launch with kRegsLaunch registers per thread owns
+    cudaFuncAttributes fa;
+    BA_CUDA_CHECK(cudaFuncGetAttributes(&fa, tc_dkdv_kernel<SPLIT>));
+    if (fa.numRegs * kThreads < 256 * kRegsCompute + 128 * kRegsIssue) return BA_EUNSUPPORTED;
+    BA_CUDA_CHECK(cudaFuncSetAttribute(tc_dkdv_kernel<SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DkdvSmem)));
+    attr_set[dev] = true;
+    return BA_OK;
+}
+
+template <bool SPLIT>
+int launch(const TcDkdvCall &c, bool after_dq, cudaStream_t st) {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof cfg);
-    cfg.gridDim = dim3((unsigned)grid);
+    cfg.gridDim = dim3((unsigned)c.grid);
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = sizeof(DkdvSmem);
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     if (SPLIT) {
         attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
-        attr[cfg.numAttrs].val.clusterDim.x = (unsigned)p.splits;
+        attr[cfg.numAttrs].val.clusterDim.x = (unsigned)c.p.splits;
         attr[cfg.numAttrs].val.clusterDim.y = attr[cfg.numAttrs].val.clusterDim.z = 1;
         ++cfg.numAttrs;
     }
@@ -786,23 +789,28 @@ int launch(const TcBwdParams &p, const BaOrder &order, const CUtensorMap *tm, in
         ++cfg.numAttrs;
     }
     cfg.attrs = attr;
-    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_dkdv_kernel<SPLIT>, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], p, order));
+    const CUtensorMap *tm = c.tm;
+    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_dkdv_kernel<SPLIT>, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], c.p, *c.order));
     return ba_check_launch();
 }
 
 }  // namespace
 
-int ba_tc_dkdv(const TcBwdParams &call, const ba_plan *pl, const BaRange &r, const void *q_main, const void *q_branch,
-               const void *k, const void *v, const void *d_o, bool after_dq, int dev, cudaStream_t st) {
-    TcBwdParams p = call;
-    p.wide = (((uintptr_t)p.dk | (uintptr_t)p.dv) & 31) == 0;
-    const int64_t grid = key_items(p, pl, r, q_main != nullptr);
-    if (grid <= 0) return BA_OK;
-    if (grid > INT_MAX) return BA_EUNSUPPORTED;
-    CUtensorMap tm[6];
-    if (!bwd_maps(tm, pl, r, q_main, q_branch, k, v, d_o, p.depth, kTile, 1, kTile)) return BA_EINVAL;
-    const BaOrder &order = key_order(p, pl, q_main != nullptr);
-    return p.splits > 1 ? launch<true>(p, order, tm, grid, after_dq, dev, st) : launch<false>(p, order, tm, grid, after_dq, dev, st);
+int ba_tc_dkdv_prepare(TcDkdvCall &c, const TcBwdParams &call, const ba_plan *pl, const BaRange &r, const void *q_main,
+                       const void *q_branch, const void *k, const void *v, const void *d_o, int dev) {
+    c.p = call;
+    c.p.wide = (((uintptr_t)call.dk | (uintptr_t)call.dv) & 31) == 0;
+    c.grid = key_items(c.p, pl, r, q_main != nullptr);
+    if (c.grid <= 0) return BA_OK;
+    if (c.grid > INT_MAX) return BA_EUNSUPPORTED;
+    if (!bwd_maps(c.tm, pl, r, q_main, q_branch, k, v, d_o, call.depth, kTile, 1, kTile)) return BA_EINVAL;
+    c.order = &key_order(c.p, pl, q_main != nullptr);
+    return c.p.splits > 1 ? prepare<true>(dev) : prepare<false>(dev);
+}
+
+int ba_tc_dkdv_launch(const TcDkdvCall &c, bool after_dq, cudaStream_t st) {
+    if (c.grid <= 0) return BA_OK;
+    return c.p.splits > 1 ? launch<true>(c, after_dq, st) : launch<false>(c, after_dq, st);
 }
 
 int ba_tc_own_branch(const TcBwdParams &p, const void *q, const void *k, const void *v, const void *d_o, cudaStream_t st) {

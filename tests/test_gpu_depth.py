@@ -125,6 +125,34 @@ def test_depth_calls_reject_what_they_cannot_do(ba):
     torch.cuda.synchronize()
 
 
+def test_backward_of_a_depth_refuses_unaligned_tensors(ba):
+    """Contiguous views that begin 8 bytes into an allocation: refused on the host, before any kernel of the call
+    (the per-row scalars in the workspace included)."""
+    p = chain_problem([40, 61], [0, 3, 20, 77], 2)
+    a = p.num_branches
+    plan = ba.Plan(p, impl=ba.IMPL_TC)
+
+    def make(shape, dtype, unaligned):
+        elements, skip = int(np.prod(shape)), (8 // torch.empty((), dtype=dtype).element_size() if unaligned else 0)
+        return torch.full((elements + skip,), 0.5, dtype=dtype, device="cuda")[skip:].view(shape)
+
+    rows, keys, bf16, fp32 = (a, p.h_q, 128), (p.rows, p.h_kv, 128), torch.bfloat16, torch.float32
+    shapes = dict(q=(rows, bf16), k=(keys, bf16), v=(keys, bf16), o=(rows, bf16), d_o=(rows, bf16), dk=(keys, fp32),
+                  dv=(keys, fp32), dq=(rows, bf16))
+    lse = torch.zeros((a, p.h_q), device="cuda")
+    ws = plan.workspace(ba.OP_BWD_DEPTH).fill_(0x5a)
+    for name in shapes:
+        t = {n: make(*shape, n == name) for n, shape in shapes.items()}
+        assert t[name].is_contiguous() and t[name].data_ptr() % 16 == 8
+        with pytest.raises(ba.BranchAttnError) as e:
+            ba.branch_attn_bwd_depth(plan, 2, t["q"], t["k"], t["v"], t["o"], lse, t["d_o"], t["dk"], t["dv"], dq=t["dq"])
+        assert e.value.code == -1, name
+        for n in ("dk", "dv", "dq"):
+            assert bool((t[n] == 0.5).all()), (name, n)
+    assert bool((ws == 0x5a).all())
+    plan.check()
+
+
 def test_stepwise_equals_all_depths_call_full_size(ba):
     """The paper's packed variable-length benchmark shape at full size: depth 1, 2, 3 in turn
     against the all-depths forward and backward (itself checked against the oracle at this
@@ -180,8 +208,8 @@ def test_stepwise_equals_all_depths_call_full_size(ba):
     plan.check()
 
 
-# One sequence with few key tiles: clusters of two, four and eight CTAs share a main key tile, and the branch key
-# tiles (a multiple of 9, 17 or 11 per call) do not fill the last cluster.
+# One sequence with few key tiles: clusters of two, four and eight CTAs share a main key tile.  (Branch keys have a
+# kernel of their own: the terms of the call's branches, at every depth up to the call's, and no others.)
 @pytest.mark.parametrize("tokens,h_q,h_kv,length,br_range", [
     (600, 4, 1, 3, None), (1100, 32, 8, 3, None), (2100, 16, 2, 2, None), (1300, 16, 1, 4, None),
     (1100, 32, 8, 3, (130, 1001)), (2100, 16, 2, 2, (1, 1500)),
