@@ -14,6 +14,7 @@ local step (s = 0).
 """
 from __future__ import annotations
 
+import contextlib
 from dataclasses import dataclass
 from typing import List, Tuple
 
@@ -120,9 +121,23 @@ class Workspace:
                       (p.rows, p.h_kv, p.head_dim), (p.rows, p.h_kv, p.head_dim))
             self.grads = tuple(torch.empty(s, **f32) for s in shapes)
             self.outs = tuple(torch.empty(s, dtype=plan.torch_dtype, device=dev) for s in shapes)
+        self._device, self._side = dev, None
+
+    def side_stream(self):
+        """The second stream of the backward, made when it is first asked for."""
+        if self._side is None:
+            import torch
+            self._side = torch.cuda.Stream(device=self._device)
+        return self._side
 
 
 L2_BYTES = 126 << 20
+
+
+def two_streams(problem, rows: int) -> bool:
+    """Whether the one-kernel blocks of a query chunk of `rows` rows go to two streams: while Q and dO of those rows, one
+    KV head at a time, take no more than half of the L2."""
+    return rows * (problem.h_q // problem.h_kv) * problem.head_dim * 2 * 2 <= L2_BYTES // 2
 
 
 def chunk_order(cp: int) -> List[int]:
@@ -189,26 +204,36 @@ def forward(ba, plan, q_main, q_branch, k, v, cp, out=None, lse=None, ws=None, h
 
 
 class _Lanes:
-    """The caller's stream and `n - 1` further ones that take independent launches in turn: the CTAs of one launch
-    start on the SMs that the last wave of another leaves idle.  Everything between `fork` and `join` comes after what
+    """The caller's stream and a second one that take independent launches in turn: the CTAs of one launch
+    start on the SMs that the last wave of another leaves idle.  Everything inside the `with` block comes after what
     the caller's stream held before and before what it gets afterwards."""
 
-    def __init__(self, n):
+    def __init__(self, side):
         import torch
-        self._torch = torch
-        self.main = torch.cuda.current_stream()
-        self.streams = [self.main] + [torch.cuda.Stream() for _ in range(n - 1)]
+        self._torch, self.main, self.side = torch, torch.cuda.current_stream(), side
 
-    def fork(self):
-        for st in self.streams[1:]:
-            st.wait_stream(self.main)
+    def __enter__(self):
+        self.side.wait_stream(self.main)
+        return self
 
     def use(self, i):
-        return self._torch.cuda.stream(self.streams[i % len(self.streams)])
+        return self._torch.cuda.stream(self.side if i % 2 else self.main)
 
-    def join(self):
-        for st in self.streams[1:]:
-            self.main.wait_stream(st)
+    def __exit__(self, *_):
+        self.main.wait_stream(self.side)
+
+
+class _OneStream:
+    """All launches on the caller's stream."""
+
+    def __enter__(self):
+        return self
+
+    def use(self, i):
+        return contextlib.nullcontext()
+
+    def __exit__(self, *_):
+        pass
 
 
 def backward(ba, plan, q_main, q_branch, k, v, o, lse, d_o, cp, fused=False, ws=None, hooks=None):
@@ -223,8 +248,9 @@ def backward(ba, plan, q_main, q_branch, k, v, o, lse, d_o, cp, fused=False, ws=
     after that (a caller that streams the gradients out starts there).  dK and dV
     are complete, and converted, at the end.
     The one-kernel blocks of a query chunk write different dK / dV rows and add into dQ atomically, so they are
-    independent and go to two streams in turn, as long as the query rows that they share (Q and dO, one KV head at a
-    time) take no more than half of the L2: the two launches read different tiles of them at a time.  A block of 65,536
+    independent and go to two streams in turn (the order in which dQ's terms are added then varies over the key chunks
+    too, not only inside a launch), as long as the query rows that they share take no more than half of the L2
+    (`two_streams`, for each chunk by itself): the two launches read different tiles of them at a time.  A block of 65,536
     tokens in 16 chunks is 256 equal CTAs, 1.73 waves of 148 SMs.  Whole backward, one stream / two: 65,536 tokens (34
     MB) 441 / 412 ms, 98,304 (50 MB) 974 / 935, 131,072 (67 MB) 1,598 / 1,633, 262,144 (134 MB) 6,315 / 6,737; 16,384
     in 8 chunks 31.4 / 28.5, 8,192 in 16 chunks 10.3 / 9.5 (three and four streams take the same)."""
@@ -237,17 +263,15 @@ def backward(ba, plan, q_main, q_branch, k, v, o, lse, d_o, cp, fused=False, ws=
     launches = 0
     common = dict(accumulate=True, grads=grads)
     blocks = schedule(p, cp)
-    chunk_rows = p.rows // (2 * cp)
-    shared = chunk_rows * (p.h_q // p.h_kv) * p.head_dim * 2 * 2      # bytes
-    lanes = _Lanes(2 if fused and shared <= L2_BYTES // 2 else 1)
     for rank in range(cp):
         for qc in rank_chunks(rank, cp):
             mine = [b for b in blocks if b.rank == rank and b.q_chunk == qc]
             ba.branch_attn_bwd(plan, q_main, q_branch, k, v, o, lse, d_o, qm_range=mine[0].qm, br_range=mine[0].br,
                                kv_range=(0, 0), parts=0, stages=ba.STAGE_PREP, **common)
             launches += 1
-            lanes.fork()
-            try:
+            q0, q1 = mine[0].qm
+            t0, t1 = plan.token_range(*mine[0].br)
+            with _Lanes(ws.side_stream()) if fused and two_streams(p, q1 - q0 + t1 - t0) else _OneStream() as lanes:
                 for i, b in enumerate(mine):
                     parts = ba.PART_MAIN | (ba.PART_BRANCH if b.branch_part else 0)
                     rng = dict(qm_range=b.qm, br_range=b.br, kv_range=b.kv, parts=parts)
@@ -259,10 +283,6 @@ def backward(ba, plan, q_main, q_branch, k, v, o, lse, d_o, cp, fused=False, ws=
                         ba.branch_attn_bwd(plan, q_main, q_branch, k, v, o, lse, d_o, stages=ba.STAGE_DQ, **rng, **common)
                         ba.branch_attn_bwd(plan, q_main, q_branch, k, v, o, lse, d_o, stages=ba.STAGE_DKDV, **rng, **common)
                         launches += 2
-            finally:
-                lanes.join()
-            q0, q1 = mine[0].qm
-            t0, t1 = plan.token_range(*mine[0].br)
             ba.ba_finalize_grads(grads[0][q0:q1], dst=ws.outs[0][q0:q1])
             launches += 1
             if t1 > t0:

@@ -83,6 +83,58 @@ def test_zigzag_schedule_is_balanced_and_complete():
     assert max(per) - min(per) == 0 or (max(per) - min(per)) / max(per) < 1e-2
 
 
+class _CallRecorder:
+    """Stands in for the binding in `zigzag.backward`: records the stages, runs nothing."""
+    IMPL_TC, IMPL_SIMT, PART_MAIN, PART_BRANCH = 2, 1, 1, 2
+    STAGE_PREP, STAGE_DQ, STAGE_DKDV, STAGE_FUSED = 1, 2, 4, 8
+
+    def __init__(self):
+        self.calls = []
+
+    def branch_attn_bwd(self, *a, stages, qm_range, **k):
+        self.calls.append((stages, qm_range))
+
+    def ba_finalize_grads(self, src, dst):
+        assert src.shape == dst.shape
+
+
+def _recorded_backward(p, cp, fused):
+    import torch
+    from types import SimpleNamespace
+    offsets = p.branch_offsets
+    plan = SimpleNamespace(problem=p, device=torch.device("cpu"), impl=2, torch_dtype=torch.bfloat16,
+                           token_range=lambda a, b: (int(offsets[a]), int(offsets[b])))
+    ba = _CallRecorder()
+    zigzag.backward(ba, plan, *[None] * 7, cp, fused=fused)
+    return ba.calls
+
+
+def test_zigzag_backward_by_two_kernels_asks_for_no_stream():
+    p = W.Problem(np.array([0, 64], np.int32), np.arange(64, dtype=np.int32), W.uniform_branch_offsets(64, 3), W.CHAIN, None, 4, 2, 128)
+    calls = _recorded_backward(p, 2, fused=False)
+    assert sum(st == 1 for st, _ in calls) == 4 and sum(st == 2 for st, _ in calls) == sum(st == 4 for st, _ in calls) == 10
+
+
+def test_zigzag_backward_takes_two_streams_by_the_rows_of_each_chunk(monkeypatch):
+    """All branches are anchored in the last of four chunks: 4,096 rows there, 64 in the others."""
+    n, m = 256, 64 * 63
+    p = W.Problem(np.array([0, n], np.int32), np.full(63, n - 1, np.int32), W.uniform_branch_offsets(63, 64), W.BLOCK, None, 4, 1, 128)
+    used = []
+
+    class Lanes(zigzag._OneStream):
+        def __init__(self, side):
+            used.append(True)
+
+    monkeypatch.setattr(zigzag, "_Lanes", Lanes)
+    monkeypatch.setattr(zigzag.Workspace, "side_stream", lambda self: None)
+    limit = lambda rows: 2 * rows * 4 * 128 * 2 * 2
+    for rows, want in ((n // 4 + m, 4), (n // 4 + m - 1, 3), (n // 4, 3), (n // 4 - 1, 0)):
+        used.clear()
+        monkeypatch.setattr(zigzag, "L2_BYTES", limit(rows))
+        _recorded_backward(p, 2, fused=True)
+        assert len(used) == want, rows
+
+
 def test_library_exports_every_declared_symbol():
     from paper_2609_07108_b200 import build
     lib_path = build.build()
