@@ -132,6 +132,18 @@ __device__ __forceinline__ bool is_half(int half, int n_sub, int n_sub_main, int
     return (u == n_sub_main - 1 && (half & 1)) || (u == n_sub - 1 && u >= n_sub_main && (half & 2));
 }
 
+// Which of the rows r0 + [lo, hi] (columns lo .. hi of 64) of a branch see the key `rel` of that branch: bit `rel` of their
+// masks.  Eight reads in flight, of the one word of a mask that holds the bit.
+__device__ __forceinline__ uint64_t own_rows(const uint64_t *br_mask, int r0, int lo, int hi, int rel) {
+    const uint32_t *word = reinterpret_cast<const uint32_t *>(br_mask) + 2 * (int64_t)r0 + (rel >> 5);
+    uint32_t v[2] = {0u, 0u};
+#pragma unroll
+    for (int part = 0; part < 2; ++part)
+#pragma unroll 8
+        for (int c = max(lo, 32 * part); c <= min(hi, 32 * part + 31); ++c) v[part] |= ((word[2 * c] >> (rel & 31)) & 1u) << (c & 31);
+    return (uint64_t)v[1] << 32 | v[0];
+}
+
 // P of 32 columns (fp32 bits, in place of the scores) and its bf16 pairs
 template <bool MASKED>
 __device__ __forceinline__ void chunk_p(uint32_t (&x)[32], uint32_t mk, float sl2, const float *nl, uint32_t *pk) {
@@ -480,6 +492,9 @@ tc_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_const
             int n_iter, n_sub, n_sub_main, s_beg, half, g, row_end, krow, m0, m1, b0, b1, ma, ba, row;
             bool is_main, valid;
             int qend, rb0, rb1;          // main rows [row, qend) and branch rows [rb0, rb1) see my key
+            // Branch key: which of my rows of streamed tiles 0 and 1 see it, (rb0, rb1) and (qend, m0), and whether the first
+            // row of tile 2 does, m1 (its only one: see fetch).  In fields that only main keys need otherwise: with fields of
+            // their own the steps of every item got 1 % slower.
         } w, nx;
         auto fetch = [&](int n_item, Work &f) -> bool {
             const int sl = n_item & 1;
@@ -501,8 +516,17 @@ tc_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_const
                     f.rb1 = p.meta.key_bq_end[f.row];
                     if (p.depth) { f.rb0 /= p.branch_len; f.rb1 /= p.branch_len; }
                 } else {
-                    f.rb0 = p.meta.br_start[f.row];
-                    f.rb1 = p.meta.br_end[f.row];
+                    const int start = p.meta.br_start[f.row], rbeg = max(start, f.b0), rend = min(p.meta.br_end[f.row], f.b1);
+                    // which of my 64 rows from r0 see my key
+                    auto own = [&](int r0) { return own_rows(p.meta.br_mask, r0, max(rbeg - r0, 0), min(rend - 1 - r0, 63), f.row - start); };
+                    // Once for every head, and for most items while the item before ends (32/8 heads, 16,384 tokens, draft
+                    // rows of 256 trees of 48: dK/dV 494 us; found at every step, one row after the other, 625; blocks of 24
+                    // on 2,400 tokens 31 and 48).  The 128 keys' branches have at most 63 more rows on either side and the
+                    // tiles start at most 3 rows early: 257 rows.
+                    const uint64_t own0 = own(f.ba + 64 * hf), own1 = own(f.ba + kTile + 64 * hf);
+                    f.rb0 = (int)(uint32_t)own0; f.rb1 = (int)(uint32_t)(own0 >> 32);
+                    f.qend = (int)(uint32_t)own1; f.m0 = (int)(uint32_t)(own1 >> 32);
+                    f.m1 = hf == 0 && own(f.ba + 2 * kTile) != 0ull;
                 }
             }
             return true;
@@ -529,12 +553,7 @@ tc_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_const
                         const int v0 = seg_main ? w.row : w.rb0, v1 = seg_main ? w.qend : w.rb1;
                         vis = bit_range(max(v0, rbeg) - r0, min(v1, rend) - 1 - r0);
                     } else {
-                        // own-branch tokens whose mask has my bit (few, short tiles)
-                        const int lo_c = max(max(w.rb0, rbeg) - r0, 0), hi_c = min(min(w.rb1, rend) - 1 - r0, 63);
-                        for (int c = lo_c; c <= hi_c; ++c) {
-                            const int rel = w.row - p.meta.br_start[r0 + c];
-                            if (rel >= 0 && rel < 64 && ((p.meta.br_mask[r0 + c] >> rel) & 1ull)) vis |= 1ull << c;
-                        }
+                        vis = u < 2 ? (uint64_t)(uint32_t)(u ? w.m0 : w.rb1) << 32 | (uint32_t)(u ? w.qend : w.rb0) : (uint64_t)w.m1;
                     }
                 }
                 const bool masked = !__all_sync(0xffffffffu, vis == ~0ull);
