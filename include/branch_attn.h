@@ -24,6 +24,10 @@
  *     KV head h / (h_q / h_kv).
  *   - Element type of q/k/v/O/dO is ba_problem_t.dtype.  Supported: BA_FP32 and
  *     BA_BF16 with head_dim 64 or 128; a branch holds at most 64 tokens.
+ *   - Alignment: every row tensor starts on a 16-byte boundary.  Calls on the plain-FMA kernels, and at
+ *     head_dim 64 in bf16 any call without fp32 results, also take bf16 q, k, v, O (forward), dO
+ *     (without BA_STAGE_PREP) and bf16 gradients on 8-byte boundaries.  Other addresses: BA_EINVAL
+ *     before anything is launched.  LSE: 4 bytes.
  *   - NaN and infinities: on the plain-FMA kernels, and at head_dim 64 throughout, a row of
  *     an input reaches the results whose definition contains it and no others (which of them
  *     come out as NaN and which as infinity is not specified).  On the tensor-core kernels at

@@ -36,6 +36,16 @@ int make_range(const ba_plan *pl, int64_t qm_begin, int64_t qm_end, int64_t br_b
     return token_range(pl, br_begin, br_end, &r->tok_begin, &r->tok_end);
 }
 
+// The keys of a call are read (and their gradients written)
+bool any_keys(const BaRange &r, bool has_branch_q) {
+    return ((r.parts & BA_PART_MAIN) && r.kv_end > r.kv_begin) || ((r.parts & BA_PART_BRANCH) && has_branch_q);
+}
+// Rows in the problem's dtype move in pieces of 16 bytes, bf16 rows of the plain-FMA kernels in pieces of 8; fp32 results
+// (partial outputs, accumulated gradients) in pieces of 16.
+bool rows_aligned(const ba_plan *pl, bool tc, uintptr_t rows, uintptr_t rows16) {
+    return (rows & (tc || pl->prob.dtype == BA_FP32 ? 15 : 7)) == 0 && (rows16 & 15) == 0;
+}
+
 }  // namespace
 
 extern "C" size_t ba_workspace_bytes(const ba_plan_t *plan, int op) {
@@ -58,7 +68,13 @@ static int fwd_common(const ba_plan_t *plan, const BaRange &r, const void *q_mai
     if (has_branch_q && !q_branch) return BA_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
     const uintptr_t addresses = (uintptr_t)q_main | (uintptr_t)q_branch | (uintptr_t)k | (uintptr_t)v | (uintptr_t)o;
-    if (ba_use_tc(plan, partial != 0, addresses)) return ba_tc_fwd(plan, r, q_main, q_branch, k, v, o, lse, partial, st);
+    const bool tc = ba_use_tc(plan, partial != 0, addresses);
+    uintptr_t rows = partial ? 0 : (uintptr_t)o;
+    if (has_main_q) rows |= (uintptr_t)q_main;
+    if (has_branch_q) rows |= (uintptr_t)q_branch;
+    if (any_keys(r, has_branch_q)) rows |= (uintptr_t)k | (uintptr_t)v;
+    if (!rows_aligned(plan, tc, rows, partial ? (uintptr_t)o : 0)) return BA_EINVAL;
+    if (tc) return ba_tc_fwd(plan, r, q_main, q_branch, k, v, o, lse, partial, st);
     if (partial == 2 && plan->impl != BA_IMPL_TC) return BA_EUNSUPPORTED;   // merge in the epilogue: tensor-core plans only
     return ba_simt_fwd(plan, r, q_main, q_branch, k, v, o, lse, partial, st);
 }
@@ -149,7 +165,19 @@ static int bwd_common(const ba_plan_t *plan, const void *q_main, const void *q_b
     const void *qm = has_main_q ? q_main : nullptr;
     const uintptr_t addresses = (uintptr_t)q_main | (uintptr_t)q_branch | (uintptr_t)k | (uintptr_t)v | (uintptr_t)dQ_main |
                                 (uintptr_t)dQ_branch | (uintptr_t)dK | (uintptr_t)dV;
-    if ((stages & (BA_STAGE_DQ | BA_STAGE_DKDV)) && ba_use_tc(plan, accumulate != 0, addresses))
+    const bool tc = ba_use_tc(plan, accumulate != 0, addresses);
+    uintptr_t rows = 0, rows16 = stages & BA_STAGE_PREP ? (uintptr_t)O | (uintptr_t)dO : 0;
+    if (stages & (BA_STAGE_DQ | BA_STAGE_DKDV | BA_STAGE_FUSED)) {
+        rows |= (uintptr_t)dO;
+        uintptr_t &grads = accumulate ? rows16 : rows;
+        if (has_main_q) rows |= (uintptr_t)q_main;
+        if (has_branch_q) rows |= (uintptr_t)q_branch;
+        if (any_keys(r, has_branch_q)) rows |= (uintptr_t)k | (uintptr_t)v;
+        if (any_keys(r, has_branch_q) && (stages & (BA_STAGE_DKDV | BA_STAGE_FUSED))) grads |= (uintptr_t)dK | (uintptr_t)dV;
+        if (stages & BA_STAGE_DQ) grads |= (has_main_q ? (uintptr_t)dQ_main : 0) | (has_branch_q ? (uintptr_t)dQ_branch : 0);
+    }
+    if (!rows_aligned(plan, tc, rows, rows16)) return BA_EINVAL;
+    if ((stages & (BA_STAGE_DQ | BA_STAGE_DKDV)) && tc)
         return ba_tc_bwd(plan, r, qm, q_branch, k, v, prep, accumulate, dQ_main, dQ_branch, dK, dV, st, stages);
     if ((stages & BA_STAGE_PREP) && (rc = ba_delta(prep, st)) != BA_OK) return rc;
     if (!(stages & (BA_STAGE_DQ | BA_STAGE_DKDV | BA_STAGE_FUSED))) return BA_OK;
@@ -220,6 +248,7 @@ extern "C" int branch_attn_fwd_depth(const ba_plan_t *plan, int depth, const voi
     if (rc != BA_OK) return rc;
     if (br_end == br_begin) return BA_OK;
     if (!q_depth || !k || !v || !O_depth || !LSE_depth) return BA_EINVAL;
+    if (!rows_aligned(plan, true, (uintptr_t)q_depth | (uintptr_t)k | (uintptr_t)v | (uintptr_t)O_depth, 0)) return BA_EINVAL;
     return ba_tc_fwd(plan, r, nullptr, q_depth, k, v, O_depth, LSE_depth, 0, (cudaStream_t)stream, depth);
 }
 
@@ -234,9 +263,8 @@ extern "C" int branch_attn_bwd_depth(const ba_plan_t *plan, int depth, const voi
     if (!q_depth || !k || !v || !O_depth || !LSE_depth || !dO_depth || !dQ_depth || !dK || !dV) return BA_EINVAL;
     if (!workspace || ws_bytes < ba_workspace_bytes(plan, BA_OP_BWD_DEPTH) || ((uintptr_t)workspace & 255))
         return BA_EWORKSPACE;
-    // every kernel of the call reads and writes its rows in pieces of 16 bytes
-    if (((uintptr_t)q_depth | (uintptr_t)k | (uintptr_t)v | (uintptr_t)O_depth | (uintptr_t)dO_depth | (uintptr_t)dQ_depth |
-         (uintptr_t)dK | (uintptr_t)dV) & 15)
+    if (!rows_aligned(plan, true, (uintptr_t)q_depth | (uintptr_t)k | (uintptr_t)v | (uintptr_t)O_depth | (uintptr_t)dO_depth |
+                      (uintptr_t)dQ_depth, (uintptr_t)dK | (uintptr_t)dV))
         return BA_EINVAL;
     const ba_problem_t &pr = plan->prob;
     float *delta = (float *)workspace;
