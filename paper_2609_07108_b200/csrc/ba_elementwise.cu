@@ -112,11 +112,19 @@ struct DeltaSegment {
     int64_t begin, end, tiles;      // rows, tiles of kDeltaRows rows from begin rounded down
 };
 
+// 16 bytes with the evict-first hint; volatile, so that no read moves ahead of wait_prerequisites()
+__device__ __forceinline__ uint4 load_once(const uint4 *p) {
+    uint4 x;
+    asm volatile("ld.global.cs.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w) : "l"(p));
+    return x;
+}
+
+// (The kernel may be launched while the one that writes o and lse still runs: no pointer is __restrict__, which would let
+// the compiler read through it before the wait.)
 template <typename T, int LPI>
 __global__ void __launch_bounds__(kThreads)
-delta_kernel(const uint4 *__restrict__ o, const uint4 *__restrict__ d_o, const float *__restrict__ lse,
-             float *__restrict__ delta_t, float *__restrict__ nlse2_t, DeltaSegment seg_a, DeltaSegment seg_b,
-             int h_q, int64_t pitch) {
+delta_kernel(const uint4 *o, const uint4 *d_o, const float *lse, float *delta_t, float *nlse2_t, DeltaSegment seg_a,
+             DeltaSegment seg_b, int h_q, int64_t pitch) {
     sm100::wait_prerequisites();      // (ba_delta: the launch may come ahead of the end of the forward)
     sm100::launch_dependents();
     constexpr int kItems = kThreads / LPI;      // (row, head) items per pass
@@ -137,8 +145,8 @@ delta_kernel(const uint4 *__restrict__ o, const uint4 *__restrict__ d_o, const f
         for (int b = 0; b < kBatch; ++b) {
             const int i = min(i0 + b * kItems, items - 1);
             const int64_t e = ((r0 + i / heads) * h_q + h0 + i % heads) * LPI + sub;
-            x[b] = __ldcs(o + e);
-            y[b] = __ldcs(d_o + e);
+            x[b] = load_once(o + e);
+            y[b] = load_once(d_o + e);
         }
 #pragma unroll
         for (int b = 0; b < kBatch; ++b) {
