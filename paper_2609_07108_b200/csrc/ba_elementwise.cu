@@ -183,20 +183,21 @@ delta_kernel(const uint4 *o, const uint4 *d_o, const float *lse, float *delta_t,
 }
 static_assert(kDeltaRows * kDeltaHeads == kThreads, "one thread per (row, head) of a tile");
 
-template <bool OUT_BF16>
+// WIDE: src and dst on 16-byte boundaries; otherwise element by element (rows of LSE of an odd number of heads)
+template <bool OUT_BF16, bool WIDE>
 __global__ void __launch_bounds__(kThreads)
 finalize_kernel(int64_t chunks, int64_t count, const float *__restrict__ src, void *dst) {
     const int64_t stride = (int64_t)gridDim.x * kThreads;
     for (int64_t c = (int64_t)blockIdx.x * kThreads + threadIdx.x; c < chunks; c += stride) {
         const int64_t e = c * 4;
-        if (e + 4 <= count) {
+        if (WIDE && e + 4 <= count) {
             const float4 x = *reinterpret_cast<const float4 *>(src + e);
             if (OUT_BF16)
                 *reinterpret_cast<uint2 *>((__nv_bfloat16 *)dst + e) = pack_bf16x4(x);
             else
                 *reinterpret_cast<float4 *>((float *)dst + e) = x;
         } else {
-            for (int64_t j = e; j < count; ++j) {
+            for (int64_t j = e; j < min(e + 4, count); ++j) {
                 if (OUT_BF16) ((__nv_bfloat16 *)dst)[j] = __float2bfloat16_rn(src[j]);
                 else ((float *)dst)[j] = src[j];
             }
@@ -257,13 +258,13 @@ extern "C" int ba_finalize_grads(const float *src, void *dst, int64_t count, int
     if (count == 0) return BA_OK;
     if (!src || !dst) return BA_EINVAL;
     if (dst_dtype != BA_FP32 && dst_dtype != BA_BF16) return BA_EUNSUPPORTED;
-    if (((uintptr_t)src | (uintptr_t)dst) & 15) return BA_EINVAL;
+    if (((uintptr_t)src & 3) || ((uintptr_t)dst & (dst_dtype == BA_BF16 ? 1 : 3))) return BA_EINVAL;
+    const bool wide = (((uintptr_t)src | (uintptr_t)dst) & 15) == 0;
     const int64_t chunks = (count + 3) / 4;
     const int grid = stream_grid(chunks);
     cudaStream_t st = (cudaStream_t)stream;
-    if (dst_dtype == BA_BF16)
-        finalize_kernel<true><<<grid, kThreads, 0, st>>>(chunks, count, src, dst);
-    else
-        finalize_kernel<false><<<grid, kThreads, 0, st>>>(chunks, count, src, dst);
+    auto kernel = dst_dtype == BA_BF16 ? (wide ? finalize_kernel<true, true> : finalize_kernel<true, false>)
+                                       : (wide ? finalize_kernel<false, true> : finalize_kernel<false, false>);
+    kernel<<<grid, kThreads, 0, st>>>(chunks, count, src, dst);
     return ba_check_launch();
 }

@@ -1,9 +1,11 @@
 """Tensors that start off a 16-byte boundary: refused on the host before any kernel of the call, or (bf16 on the plain-FMA
-kernels) taken with the same results."""
+kernels, and what ba_finalize_grads converts) taken with the same results."""
+import numpy as np
 import pytest
 import torch
 
 from paper_2609_07108_b200 import workloads as W
+from paper_2609_07108_b200 import zigzag
 from helpers import to_dev
 
 pytestmark = pytest.mark.gpu
@@ -78,3 +80,37 @@ def test_calls_refuse_what_they_cannot_address(ba, dtype, d, simt, off, fwd, bwd
     plan.check()
     for x, w in zip(GRADS, want):      # (head_dim 64: the stages above ran on different kernels, one rounding to bf16 each)
         assert torch.equal(base[x], w) or (d == 64 and float((base[x] - w).float().norm()) <= 2.0 ** -8 * float(w.float().norm()))
+
+
+@pytest.mark.parametrize("dst", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("count", [1, 3, 4, 5, 4099])
+def test_finalize_at_any_element(ba, dst, count):
+    g = torch.Generator(device="cuda").manual_seed(count)
+    src = torch.randn(count + 8, generator=g, device="cuda")
+    for a in (0, 1, 2, 4, 7):
+        for b in (0, 1, 4, 7):
+            out = torch.full((count + 16,), 7.0, dtype=dst, device="cuda")
+            ba.ba_finalize_grads(src[a:a + count], dst=out[b:b + count])
+            assert torch.equal(out[b:b + count], src[a:a + count].to(dst))
+            assert bool((out[:b] == 7).all()) and bool((out[b + count:] == 7).all())
+
+
+@pytest.mark.parametrize("n,cp,h_q,h_kv", [(1092, 2, 5, 1), (1084, 2, 3, 1), (1020, 2, 1, 1)])
+def test_zigzag_with_rows_of_lse_off_16_bytes(ba, n, cp, h_q, h_kv):
+    """Chunks of 273, 271 and 255 rows: the rows of LSE of a chunk, or of its branches, start on any 4-byte boundary."""
+    p = W.Problem(np.array([0, n], np.int32), np.arange(0, n, 3, dtype=np.int32), W.uniform_branch_offsets((n + 2) // 3, 3), W.CHAIN,
+                  None, h_q, h_kv, 128)
+    t = to_dev(p, W.make_tensors(p, seed=7, std=0.5))
+    plan = ba.Plan(p)
+    qkv = [t[x] for x in ROWS]
+    o, lse = ba.branch_attn_fwd(plan, *qkv)
+    want = ba.branch_attn_bwd(plan, *qkv, o, lse, t["d_o"])
+    o1, lse1, _ = zigzag.forward(ba, plan, *qkv, cp)
+    assert float((lse1 - lse).abs().max()) <= 1e-5
+    assert float((o1.float() - o.float()).norm()) <= 4e-3 * float(o.float().norm())          # two roundings to bf16
+    for fused in (False, True):
+        got = zigzag.backward(ba, plan, *qkv, o, lse, t["d_o"], cp, fused=fused)[:4]
+        for a, b in zip(got, want):
+            # one rounding to bf16 each, and P, dS rounded to bf16 against another running order of the tiles
+            assert float((a.float() - b.float()).norm()) <= 6e-3 * float(b.float().norm())
+    plan.check()
