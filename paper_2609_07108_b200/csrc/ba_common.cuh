@@ -175,4 +175,6 @@ static inline bool ba_use_tc(const ba_plan *pl, bool fp32_out, uintptr_t address
 //   delta_t[h, r] = <dO[r, h], O[r, h]>,  nlse2_t[h, r] = -LSE[r, h] * log2(e)
 // for the two row segments of `x`
 int ba_delta(const BaDelta &x, cudaStream_t st);
+// at most four CTAs to an SM
+bool ba_delta_small(const BaDelta &x);
 static inline int64_t ba_row_pitch(int64_t rows) { return (rows + 128 + 63) / 64 * 64; }

@@ -223,25 +223,39 @@ extern "C" int lse_merge(int64_t rows_heads, int d, const float *O_a, const floa
     return launch_merge<false>(d / 4, rows_heads, O_a, LSE_a, O_b, LSE_b, O_out, LSE_out, st);
 }
 
+namespace {
+struct DeltaGrid {
+    DeltaSegment a, b;
+    dim3 grid;
+    explicit DeltaGrid(const BaDelta &x) {
+        auto segment = [](int64_t begin, int64_t end) {
+            DeltaSegment g = {begin, end, 0};
+            if (end > begin) g.tiles = (end - (begin & ~(int64_t)(kDeltaRows - 1)) + kDeltaRows - 1) / kDeltaRows;
+            return g;
+        };
+        a = segment(x.a_begin, x.a_end);
+        b = segment(x.b_begin, x.b_end);
+        grid = dim3((unsigned)(a.tiles + b.tiles), (unsigned)((x.h_q + kDeltaHeads - 1) / kDeltaHeads));
+    }
+    bool small() const { return (int64_t)grid.x * grid.y <= 4 * kSms; }
+};
+}  // namespace
+
+bool ba_delta_small(const BaDelta &x) { return DeltaGrid(x).small(); }
+
 int ba_delta(const BaDelta &x, cudaStream_t st) {
-    auto segment = [](int64_t begin, int64_t end) {
-        DeltaSegment g = {begin, end, 0};
-        if (end > begin) g.tiles = (end - (begin & ~(int64_t)(kDeltaRows - 1)) + kDeltaRows - 1) / kDeltaRows;
-        return g;
-    };
-    const DeltaSegment seg_a = segment(x.a_begin, x.a_end), seg_b = segment(x.b_begin, x.b_end);
-    if (seg_a.tiles + seg_b.tiles == 0) return BA_OK;
+    const DeltaGrid g(x);
+    if (g.grid.x == 0) return BA_OK;
     const int lpi = x.d * (x.dtype == BA_FP32 ? 4 : 2) / 16;
-    const dim3 grid((unsigned)(seg_a.tiles + seg_b.tiles), (unsigned)((x.h_q + kDeltaHeads - 1) / kDeltaHeads));
     // Forward, delta and dQ follow one another in a step: each may be launched while the one before ends, and waits for
     // it at its head (640 tokens in fp32, whole step 65.5 -> 63.9 us, 4,096 in bf16 at head_dim 64 676 -> 660).  A larger
     // delta is launched as usual: its blocks would crowd the SMs that are free first (8,192 rows: 27 us instead of 24).
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr;
-    dependent_launch(cfg, attr, grid, kThreads, 0, st);
-    if ((int64_t)grid.x * grid.y > 4 * kSms) cfg.numAttrs = 0;
+    dependent_launch(cfg, attr, g.grid, kThreads, 0, st);
+    if (!g.small()) cfg.numAttrs = 0;
 #define BA_DELTA_LAUNCH(T, L) \
-    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, delta_kernel<T, L>, (const uint4 *)x.o, (const uint4 *)x.d_o, x.lse, x.delta_t, x.nlse2_t, seg_a, seg_b, x.h_q, \
+    BA_CUDA_CHECK(cudaLaunchKernelEx(&cfg, delta_kernel<T, L>, (const uint4 *)x.o, (const uint4 *)x.d_o, x.lse, x.delta_t, x.nlse2_t, g.a, g.b, x.h_q, \
                                      x.row_pitch))
     if (x.dtype == BA_FP32 && lpi == 16) BA_DELTA_LAUNCH(float, 16);
     else if (x.dtype == BA_FP32 && lpi == 32) BA_DELTA_LAUNCH(float, 32);
