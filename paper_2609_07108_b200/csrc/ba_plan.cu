@@ -347,7 +347,7 @@ static int check_metadata(const ba_problem_t *p, int64_t *pairs_out, int32_t *un
     return BA_OK;
 }
 
-constexpr int64_t kOrderMaxBytes = 160 << 20;
+constexpr int64_t kL2Bytes = 126 << 20;
 
 // Number of keys that a query row tile walks, or of query rows that a key tile is walked by, per tile.
 static void tile_weights(const ba_problem_t *host, int32_t uniform, const BaTiling &t, int64_t *w) {
@@ -381,13 +381,16 @@ void ba_add_order(ba_plan *pl, const ba_problem_t *host, const BaTiling &t) {
     const ba_problem_t &pr = pl->prob;
     const int64_t tiles = t.main_tiles + t.branch_tiles, items = tiles * pr.h_kv;
     if (tiles < 2 || tiles > kMaxOrder || ba_find_order(pl, t).n > 0) return;
-    // Not where the streamed rows (K and V, or Q and dO) are far larger than the L2: tiles of one sequence have to be
-    // taken together then, while that sequence's rows are there (32,768 tokens with blocks, dK/dV 1,697 us without an
-    // order, 2,011 with; 65,536 with trees, forward 3,706 / 3,950).  Nor for key tiles where the items are many and short
-    // enough as they are.
+    // Not where the streamed rows (K and V, or Q and dO) take more than twice the L2: tiles of one sequence have to be taken
+    // together then, while that sequence's rows are there.  Time without an order against with one, chains, blocks and
+    // trees, four and twelve sequences, 32/8, 16/4, 16/2 and 8/8 heads.  Forward and dQ: 0.98 to 1.16 at 50 to 175 MB, 0.99 to
+    // 1.04 at 210 and 260 (one of 0.92), 0.95 to 1.04 at 330; 65,536 tokens with trees (403 MB) 0.94.  dK/dV at 32/8: 0.96 to
+    // 1.19 up to 190 MB, 0.98 to 1.10 at 240, 0.95 to 1.07 at 300, 0.92 to 1.01 at 400; with fewer KV heads the gain lasts longer
+    // (16/4: 1.01 to 1.12 at 300 MB, 0.97 to 1.06 at 400; 16/2: 0.96 to 1.11 at 550).  Nor for key tiles in more than 12 items
+    // per SM, whose last ones are short enough as they are (8/8 heads: 0.97 to 1.03 up to 10 items, 0.94 to 1.03 from 13 on).
     const int64_t rows = (t.kind == BA_ORDER_ROWS || t.has_main ? pr.n_main : 0) + pr.n_branch;
     const int64_t streamed = 2 * rows * (t.kind == BA_ORDER_ROWS ? pr.h_kv : pr.h_q) * pr.head_dim * (pr.dtype == BA_FP32 ? 4 : 2);
-    if (streamed > kOrderMaxBytes || (t.kind == BA_ORDER_KEYS && items > 12 * kSms)) return;
+    if (streamed > 2 * kL2Bytes || (t.kind == BA_ORDER_KEYS && items > 12 * kSms)) return;
     if (!pl->orders) pl->orders = (BaOrders *)calloc(1, sizeof(BaOrders));
     if (!pl->orders || pl->orders->count == kMaxOrders) return;
     int64_t w[kMaxOrder];
