@@ -179,21 +179,30 @@ inline int64_t key_items(TcBwdParams &p, const ba_plan *pl, const BaRange &r, bo
     // (step-major: own_branch_kernel)
     const int64_t kbt = (r.parts & BA_PART_BRANCH) && !p.depth ? (br_n + p.step_kb - 1) / p.step_kb : 0;
     p.branch_key_tiles = (int)kbt;
-    // Share main key tiles between the CTAs of a cluster until they fill the SMs once, as long as an average
-    // part keeps eight 64-row steps: 2,048 tokens, 8 KV heads (128 tiles) take 122 us whole, 130 us in two
-    // parts, 153 us in four.
+    // Share main key tiles between the CTAs of a cluster while the CTAs are few and a part keeps enough steps (64 streamed
+    // rows, by the mean sequence length): ever more of them the more CTAs there are already, because a part costs its
+    // set-up and the sum at the end.  Twice as many parts against as many as before, mean / worst of 493 batches (one to
+    // sixteen sequences, chains and blocks, five head counts; the same at head_dim 64): up to half a CTA per SM with 3 to 4
+    // steps 0.77 / 1.00; up to one with 6 to 8 0.82 / 1.00 (4 to 6: 0.89 / 1.10); up to 1.5 with 8 to 12 0.78 / 0.98 (6 to 8:
+    // 0.98 / 1.04); up to 2.5 with 24 to 32 0.76 / 0.96 (16 to 24: 0.88 / 1.24); up to three with 64 0.79 / 0.96 (48 to 64:
+    // 0.88 / 1.12); beyond that 1.12 / 1.15 and more.
     const int64_t keys = kmt * kTile, viewers = qm_n + br_n;
     const int64_t seq = pr.num_seqs > 0 ? pr.n_main / pr.num_seqs : 0;
     const int64_t est = keys > 0 ? (seq < keys ? seq : keys) / 2 * viewers / (keys < pr.n_main ? pr.n_main : keys) * p.group / 64 : 0;
-    while (p.splits < 8 && kmt * pr.h_kv * p.splits * 2 <= kSms && est >= 8 * 2 * p.splits) p.splits *= 2;
+    auto worth = [&](int64_t splits) {
+        const int64_t halves = (kmt * pr.h_kv * splits * 2 + kSms - 1) / kSms;      // CTAs per SM, in halves
+        const int steps = halves <= 1 ? 3 : halves <= 2 ? 6 : halves <= 3 ? 8 : halves <= 5 ? 24 : 64;
+        return halves <= 6 && est >= steps * splits;
+    };
+    while (p.splits < 8 && worth(2 * p.splits)) p.splits *= 2;
     p.main_key_tiles = (int)kmt;
     const int64_t tiles = kmt + (kbt + p.splits - 1) / p.splits;    // work items (clusters) per KV head
     p.total_key_tiles = (int)tiles;
-    // Up to 24 work items per SM heaviest first over all KV heads, so that the last items are short (8,192
-    // tokens with chains 830 us against 1030 KV-head-major, 32,768 tokens with blocks 1616 against 1711);
-    // beyond that KV-head-major, whose resident CTAs share one query stream through L2 (65,536-token trees 7862
-    // us against 7953, 73,728 tokens with chains 48.4 ms against 48.9).
-    p.tile_major = tiles * pr.h_kv <= 24 * kSms;
+    // Up to 96 work items per SM heaviest first over all KV heads, so that the last items are short; beyond that
+    // KV-head-major, whose resident CTAs share one query stream through L2.  KV-head-major against tile-major, chains, blocks
+    // and trees, 32/8, 16/4 and 8/8 heads, 1 to 12 sequences: 1.05 to 1.48 times the time at 10 to 14 items per SM, 1.00 to
+    // 1.24 at 24, 0.99 to 1.16 at 48, 1.00 to 1.06 at 90, 0.98 to 1.07 at 124.
+    p.tile_major = tiles * pr.h_kv <= 96 * kSms;
     return tiles * pr.h_kv * p.splits;
 }
 
