@@ -127,7 +127,10 @@ int ba_plan_destroy(ba_plan_t *plan);
  * the GPU busy.  The device arrays must hold the host values and stay alive until the
  * work queued on `stream` has run; calls on another stream must wait for that work.
  * Branches of one length are recognised from the offsets (as if uniform_len had been given,
- * which the per-depth calls need); ba_plan_create takes uniform_len as it is.  Not
+ * which the per-depth calls need); ba_plan_create takes uniform_len as it is.  Plans of several
+ * sequences made here also hold the order in which kernels take their tiles, heaviest first
+ * (ba_plan_tile_order); those of ba_plan_create give the same results, small and medium calls a few
+ * per cent slower.  Not
  * while `stream` is capturing (BA_EINVAL): the plan would not exist before a replay.
  */
 int ba_plan_create_host(const ba_problem_t *host, const ba_problem_t *dev, void *plan_mem,
@@ -151,6 +154,14 @@ int64_t ba_plan_pairs(const ba_plan_t *plan);
 
 /* Which kernels the plan resolved to: BA_IMPL_SIMT or BA_IMPL_TC. */
 int ba_plan_impl(const ba_plan_t *plan);
+
+/* The order in which a forward (stage 0) or the BA_STAGE_DQ / BA_STAGE_DKDV kernel of a call over
+ * everything takes its tiles, heaviest first: returns their number and writes the first `capacity` of
+ * them, or returns 0 where the kernel keeps the order of the rows.  tiling[4]: main tiles, rows per main
+ * tile, branch tiles, tokens per branch tile; branch tiles are numbered after the main ones.  Tiles are of
+ * query rows, for BA_STAGE_DKDV of keys.  has_main_q: whether the call has main queries. */
+int ba_plan_tile_order(const ba_plan_t *plan, int stage, int has_main_q, int64_t *tiling, uint16_t *order,
+                       int capacity);
 
 /* Synchronises `stream` and reports whether any kernel launched with this plan
  * gave up a bounded device-side wait since the last check: BA_OK or BA_ETIMEOUT

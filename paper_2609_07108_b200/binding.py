@@ -47,7 +47,7 @@ class _Problem(C.Structure):
 
 _LIB = None
 EXPORTS = ("ba_status_string", "ba_last_cuda_error", "ba_plan_bytes", "ba_plan_create", "ba_plan_create_host",
-           "ba_plan_destroy", "ba_host_wait", "ba_workspace_bytes", "ba_plan_pairs", "ba_plan_impl", "ba_plan_check", "branch_attn_fwd",
+           "ba_plan_destroy", "ba_host_wait", "ba_workspace_bytes", "ba_plan_pairs", "ba_plan_impl", "ba_plan_tile_order", "ba_plan_check", "branch_attn_fwd",
            "branch_attn_fwd_partial", "branch_attn_fwd_partial_merge", "lse_merge", "branch_attn_bwd", "branch_attn_bwd_stages",
            "branch_attn_bwd_static", "ba_finalize_grads", "ba_selftest_bounded_wait",
            "branch_attn_fwd_depth", "branch_attn_bwd_depth", "branch_attn_fwd_shard", "branch_attn_bwd_shard")
@@ -83,6 +83,8 @@ def _lib():
         lib.ba_plan_pairs.argtypes = [C.c_void_p]
         lib.ba_plan_impl.restype = C.c_int
         lib.ba_plan_impl.argtypes = [C.c_void_p]
+        lib.ba_plan_tile_order.restype = C.c_int
+        lib.ba_plan_tile_order.argtypes = [C.c_void_p, C.c_int, C.c_int, C.c_void_p, C.c_void_p, C.c_int]
         lib.ba_plan_check.restype = C.c_int
         lib.ba_plan_check.argtypes = [C.c_void_p, C.c_void_p]
         vp, i64 = C.c_void_p, C.c_int64

@@ -80,6 +80,9 @@ static inline bool ba_whole_call(const ba_plan *pl, const BaRange &r, bool has_m
     return (!has_main || (r.qm_begin == 0 && r.qm_end == pl->prob.n_main)) && r.tok_begin == 0 && r.tok_end == pl->prob.n_branch &&
            r.kv_begin == 0 && r.kv_end == pl->prob.n_main && r.kv_base == 0 && r.parts == (BA_PART_MAIN | BA_PART_BRANCH);
 }
+static inline BaRange ba_everything(const ba_plan *pl) {
+    return {0, pl->prob.n_main, 0, pl->prob.n_branch, 0, pl->prob.n_main, 0, BA_PART_MAIN | BA_PART_BRANCH};
+}
 // ba_plan.cu: forms an order (`host`: problem with host arrays) and keeps it; finds it again (or an empty one)
 void ba_add_order(ba_plan *pl, const ba_problem_t *host, const BaTiling &t);
 const BaOrder &ba_find_order(const ba_plan *pl, const BaTiling &t);
@@ -87,6 +90,10 @@ const BaOrder &ba_find_order(const ba_plan *pl, const BaTiling &t);
 void ba_tc_fwd_orders(ba_plan *pl, const ba_problem_t *host);
 void ba_tc_bwd_orders(ba_plan *pl, const ba_problem_t *host);
 void ba_simt_orders(ba_plan *pl, const ba_problem_t *host);
+// the order that the launch of such a call finds (stage: 0 forward, BA_STAGE_DQ, BA_STAGE_DKDV), and the tiling
+const BaOrder &ba_tc_fwd_order(const ba_plan *pl, bool has_main, BaTiling *t);
+const BaOrder &ba_tc_bwd_order(const ba_plan *pl, int stage, bool has_main, BaTiling *t);
+const BaOrder &ba_simt_order(const ba_plan *pl, int stage, bool has_main, BaTiling *t);
 
 extern thread_local int g_ba_last_cuda_error;
 

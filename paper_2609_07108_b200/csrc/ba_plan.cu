@@ -526,6 +526,18 @@ extern "C" int ba_plan_destroy(ba_plan_t *plan) {
 
 extern "C" int64_t ba_plan_pairs(const ba_plan_t *plan) { return plan ? plan->pairs : -1; }
 
+extern "C" int ba_plan_tile_order(const ba_plan_t *plan, int stage, int has_main_q, int64_t *tiling, uint16_t *order, int capacity) {
+    if (!plan || !tiling || (capacity > 0 && !order) || capacity < 0) return BA_EINVAL;
+    if (stage != 0 && stage != BA_STAGE_DQ && stage != BA_STAGE_DKDV) return BA_EINVAL;
+    BaTiling t;
+    const BaOrder &o = plan->impl != BA_IMPL_TC ? ba_simt_order(plan, stage, has_main_q != 0, &t)
+                       : stage == 0             ? ba_tc_fwd_order(plan, has_main_q != 0, &t)
+                                                : ba_tc_bwd_order(plan, stage, has_main_q != 0, &t);
+    tiling[0] = t.main_tiles; tiling[1] = t.main_step; tiling[2] = t.branch_tiles; tiling[3] = t.branch_step;
+    for (int i = 0; i < o.n && i < capacity; ++i) order[i] = o.tile[i];
+    return o.n;
+}
+
 extern "C" int ba_plan_impl(const ba_plan_t *plan) { return plan ? plan->impl : BA_EINVAL; }
 
 extern "C" int ba_plan_check(ba_plan_t *plan, void *stream) {

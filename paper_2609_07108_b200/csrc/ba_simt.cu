@@ -667,6 +667,11 @@ template <int MODE> BaTiling tiling(const SimtArgs &a, bool has_main) {
     return {MODE == kDkdv ? BA_ORDER_KEYS : BA_ORDER_ROWS, has_main, a.main_tiles, step, a.total_tiles - a.main_tiles, step};
 }
 
+template <int MODE> const BaOrder &tile_order(const ba_plan *pl, const SimtArgs &a) {
+    const bool has_main = a.q_main != nullptr;
+    return ba_find_order(pl, ba_whole_call(pl, a.r, has_main) ? tiling<MODE>(a, has_main) : BaTiling{-1});
+}
+
 template <typename T, int D, int MODE>
 int launch_tiles(const ba_plan *pl, SimtArgs a, bool after_dq, cudaStream_t st) {
     const ba_problem_t &pr = pl->prob;
@@ -686,9 +691,7 @@ int launch_tiles(const ba_plan *pl, SimtArgs a, bool after_dq, cudaStream_t st) 
                             (work * a.splits * 2 <= kSms * 16 && est >= 2 * 4 * a.splits)))
         a.splits *= 2;
     if (work * a.splits > INT_MAX) return BA_EUNSUPPORTED;
-    const bool has_main = a.q_main != nullptr;
-    const BaOrder &order = ba_find_order(pl, ba_whole_call(pl, a.r, has_main) ? tiling<MODE>(a, has_main) : BaTiling{-1});
-    return launch<T, D, MODE>(a, order, work, after_dq, st);
+    return launch<T, D, MODE>(a, tile_order<MODE>(pl, a), work, after_dq, st);
 }
 
 template <int MODE> int dispatch(const ba_plan *pl, const SimtArgs &a, cudaStream_t st, bool after_dq = false) {
@@ -714,15 +717,27 @@ SimtArgs base_args(const ba_plan *pl, const BaRange &r) {
 }  // namespace
 
 void ba_simt_orders(ba_plan *pl, const ba_problem_t *host) {
-    const BaRange r = {0, pl->prob.n_main, 0, pl->prob.n_branch, 0, pl->prob.n_main, 0, BA_PART_MAIN | BA_PART_BRANCH};
     for (int has_main = 1; has_main >= 0; --has_main) {
-        SimtArgs a = base_args(pl, r);
+        SimtArgs a = base_args(pl, ba_everything(pl));
         a.q_main = has_main ? pl : nullptr;      // (only asked whether it is there)
         tile_work<kFwd>(a);                      // forward and dQ
         ba_add_order(pl, host, tiling<kFwd>(a, has_main));
         tile_work<kDkdv>(a);
         ba_add_order(pl, host, tiling<kDkdv>(a, has_main));
     }
+}
+
+const BaOrder &ba_simt_order(const ba_plan *pl, int stage, bool has_main, BaTiling *t) {
+    SimtArgs a = base_args(pl, ba_everything(pl));
+    a.q_main = has_main ? pl : nullptr;
+    if (stage == BA_STAGE_DKDV) {
+        tile_work<kDkdv>(a);
+        *t = tiling<kDkdv>(a, has_main);
+        return tile_order<kDkdv>(pl, a);
+    }
+    tile_work<kFwd>(a);
+    *t = tiling<kFwd>(a, has_main);
+    return tile_order<kFwd>(pl, a);
 }
 
 int ba_simt_fwd(const ba_plan *pl, const BaRange &r, const void *q_main, const void *q_branch,

@@ -1350,7 +1350,7 @@ inline const BaOrder &row_order(const TcBwdParams &p, const ba_plan *pl, bool ha
 
 void ba_tc_bwd_orders(ba_plan *pl, const ba_problem_t *host) {
     const int64_t n = pl->prob.n_main, m = pl->prob.n_branch;
-    const BaRange r = {0, n, 0, m, 0, n, 0, BA_PART_MAIN | BA_PART_BRANCH};
+    const BaRange r = ba_everything(pl);
     for (int has_main = 1; has_main >= 0; --has_main) {
         TcBwdParams p = bwd_params(pl, r, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0, nullptr, nullptr, nullptr, nullptr, 0);
         if (key_items(p, pl, r, has_main) > 0 && p.splits == 1 && p.tile_major) ba_add_order(pl, host, key_tiling(p, has_main));
@@ -1359,6 +1359,26 @@ void ba_tc_bwd_orders(ba_plan *pl, const ba_problem_t *host) {
             ba_add_order(pl, host, row_tiling(p, has_main));
         }
     }
+}
+
+const BaOrder &ba_tc_bwd_order(const ba_plan *pl, int stage, bool has_main, BaTiling *t) {
+    BaRange r = ba_everything(pl);
+    if (!has_main) r.qm_end = 0;
+    TcBwdParams p = bwd_params(pl, r, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0, nullptr, nullptr, nullptr, nullptr, 0);
+    if (stage == BA_STAGE_DKDV) {
+        key_items(p, pl, r, has_main);
+        *t = key_tiling(p, has_main);
+        return key_order(p, pl, has_main);
+    }
+    if (pl->prob.head_dim == 64) {
+        row_tiles(p, r.qm_end, r.tok_end);
+        *t = row_tiling(p, has_main);
+        return row_order(p, pl, has_main);
+    }
+    ItemParams q;
+    fill_items(q, pl, r, has_main, 0);
+    *t = item_tiling(q, has_main);
+    return item_order(q, pl, has_main);
 }
 
 int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const void *q_branch, const void *k,

@@ -916,6 +916,29 @@ int launch_fwd(TcFwdParams &p, const BaOrder &order, const CUtensorMap *tm, int6
     return ba_check_launch();
 }
 
+// Work items of a call and their cluster splits; returns the number of items.
+// Few items and long key ranges (a handful of branches on long sequences): split the keys of an item over a
+// cluster until the SMs are busy, as long as a part keeps at least four tiles.  With branches of different
+// sequences in the two query tiles (same_rows), an item per sequence's rows and both tiles on them, unless two
+// parts per item already exceed one CTA per SM on short sequences.  Kernel times with the caches flushed, 31-node
+// trees at the end of each of 8 / 16 sequences of 8,192 tokens, two sequences per item / same_rows: 154 / 100 and
+// 177 / 137 us; 9-node trees, 12 sequences of 8,333: 196 / 88; 16 sequences of 1,024 tokens: 47 / 50, not taken.
+// With parts until there are four CTAs per SM: 159 us instead of 100.
+int64_t split_items(ItemParams &p, const ba_plan *pl, const BaRange &r, bool has_main, int depth) {
+    const ba_problem_t &pr = pl->prob;
+    const int64_t est_tiles = (r.parts & BA_PART_MAIN) && pr.num_seqs > 0 ? (r.kv_end - r.kv_begin) / pr.num_seqs / kTile : 0;
+    int64_t work;
+    auto split = [&](bool same_rows_ok) {
+        work = fill_items(p, pl, r, has_main, depth, same_rows_ok);
+        p.splits = 1;
+        while (p.splits < 8 && work * p.splits * 2 <= 2 * kSms && est_tiles >= 4 * 2 * p.splits) p.splits *= 2;
+    };
+    split(true);
+    // (the kernel for whole items has different rows in its tiles)
+    if (p.same_rows && (p.splits == 1 || (work * 2 > kSms && est_tiles < 32))) split(false);
+    return work;
+}
+
 }  // namespace
 
 bool ba_tc_supported(const ba_problem_t *p) {
@@ -940,23 +963,7 @@ int ba_tc_fwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
     p.rows.q_main = q_main; p.rows.q_branch = q_branch; p.rows.k = k; p.rows.v = v;
     p.rows.h_q = pr.h_q; p.rows.h_kv = pr.h_kv; p.rows.group = pr.h_q / pr.h_kv;
     p.rows.scale_log2 = p.scale_log2;
-    // Few items and long key ranges (a handful of branches on long sequences): split the keys of an item over a
-    // cluster until the SMs are busy, as long as a part keeps at least four tiles.  With branches of different
-    // sequences in the two query tiles (same_rows), an item per sequence's rows and both tiles on them, unless two
-    // parts per item already exceed one CTA per SM on short sequences.  Kernel times with the caches flushed, 31-node
-    // trees at the end of each of 8 / 16 sequences of 8,192 tokens, two sequences per item / same_rows: 154 / 100 and
-    // 177 / 137 us; 9-node trees, 12 sequences of 8,333: 196 / 88; 16 sequences of 1,024 tokens: 47 / 50, not taken.
-    // With parts until there are four CTAs per SM: 159 us instead of 100.
-    const int64_t est_tiles = (r.parts & BA_PART_MAIN) && pr.num_seqs > 0 ? (r.kv_end - r.kv_begin) / pr.num_seqs / kTile : 0;
-    int64_t work;
-    auto split = [&](bool same_rows_ok) {
-        work = fill_items(p, pl, r, q_main != nullptr, depth, same_rows_ok);
-        p.splits = 1;
-        while (p.splits < 8 && work * p.splits * 2 <= 2 * kSms && est_tiles >= 4 * 2 * p.splits) p.splits *= 2;
-    };
-    split(true);
-    // (the kernel for whole items has different rows in its tiles)
-    if (p.same_rows && (p.splits == 1 || (work * 2 > kSms && est_tiles < 32))) split(false);
+    const int64_t work = split_items(p, pl, r, q_main != nullptr, depth);
     if (work == 0) return BA_OK;
     if (work > INT_MAX) return BA_EUNSUPPORTED;
 
@@ -987,9 +994,15 @@ int ba_tc_fwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
 }
 
 void ba_tc_fwd_orders(ba_plan *pl, const ba_problem_t *host) {
-    const BaRange r = {0, pl->prob.n_main, 0, pl->prob.n_branch, 0, pl->prob.n_main, 0, BA_PART_MAIN | BA_PART_BRANCH};
     for (int has_main = 1; has_main >= 0; --has_main) {
         ItemParams p;
-        if (fill_items(p, pl, r, has_main, 0) > 0) ba_add_order(pl, host, item_tiling(p, has_main));
+        if (fill_items(p, pl, ba_everything(pl), has_main, 0) > 0) ba_add_order(pl, host, item_tiling(p, has_main));
     }
+}
+
+const BaOrder &ba_tc_fwd_order(const ba_plan *pl, bool has_main, BaTiling *t) {
+    ItemParams p;
+    split_items(p, pl, ba_everything(pl), has_main, 0);
+    *t = item_tiling(p, has_main);
+    return item_order(p, pl, has_main);
 }
