@@ -377,7 +377,8 @@ int branch_attn_bwd_shard(const ba_plan_t *plan, const void *q_main, const void 
  * Running depth = 1 .. n over all branches gives the rows of branch_attn_fwd;
  * the backward calls together (plus the main rows' own backward) give its
  * gradients.  All results are bit-reproducible (the dQ and dK/dV kernels of
- * branch_attn_bwd).  workspace: ba_workspace_bytes(plan, BA_OP_BWD_DEPTH).
+ * branch_attn_bwd; own-branch keys, each seen by one query row of the call, by a
+ * kernel of their own).  A call that is refused has changed nothing.  workspace: ba_workspace_bytes(plan, BA_OP_BWD_DEPTH).
  */
 int branch_attn_fwd_depth(const ba_plan_t *plan, int depth, const void *q_depth, const void *k,
                           const void *v, int64_t br_begin, int64_t br_end, void *O_depth,

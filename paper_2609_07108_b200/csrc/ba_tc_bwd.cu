@@ -100,7 +100,8 @@ tc_dq_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
         if (tid == 0) atomicExch(p.status, BA_EUNSUPPORTED);
         return;
     }
-    // global row number of branch query 0 (rows of dO and of the per-row scalars): see tc_kv_kernel
+    // global row number of branch query 0 (rows of dO and of the per-row scalars): branch rows follow the main
+    // rows, except in depth mode, where those tensors hold one row per branch
     const int qbase = p.depth ? 0 : (int)p.meta.n_main;
 
     if (tid == 0) {
@@ -575,8 +576,8 @@ tc_dq_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
 // bits of mantissa), two products each: against fp64, gradients rounded to bf16 are then off by what those kernels'
 // are (dQ, dK, dV 1.64e-3 .. 1.66e-3 in the 2-norm, the same to 1 part in 10,000).  Gradients accumulated in fp32
 // would not be, so they stay with those kernels (ba_use_tc).  4,096 tokens, 6 sequences, chains of three, 32/8 heads:
-// dQ / dK/dV 189 / 342 us (were 3052 / 8978).  The 128-row tiles of ba_tc_dkdv.cu take 359 us for that dK/dV against
-// 336: twice the conversions per flop make the warps the limit, and two tiles in flight hide them better.
+// dQ / dK/dV 187 / 287 us (were 3052 / 8978).  The 128-row tiles of ba_tc_dkdv.cu took 359 us for that dK/dV when this
+// form, then without an order of the tiles, took 336: twice the conversions per flop make the warps the limit, and two tiles in flight hide them better.
 // dQ is here and not in tc_dq_kernel because that kernel was written for 128 columns of dQ and keeps P
 // in registers as bf16; a form of it with hi + lo pairs has not been tried.
 //
@@ -906,8 +907,7 @@ tc_kv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_constan
                         const int h = it.g * p.group + hh;
                         const int gr0 = seg_main ? r0 : n + r0;
                         if (lane == 0) {
-                            // A branch tile may start up to three rows before branch row 0: dO by the map that has no rows
-                            // there.  (By that map for every branch tile: 129 us instead of 126 at 2,048 tokens.)
+                            // a branch tile may start up to three rows before branch row 0: dO by the map that has no rows there
                             const CUtensorMap *tq = seg_main ? &tm_q_main : &tm_q_branch, *tg = r0 >= 0 ? &tm_go : &tm_go_branch;
                             mbar_expect_tx(&sm.x_full[st], 2 * kSubBytes + 2 * kSub * 4);
                             tma_load_3d(sm.xs[st], tq, 0, h, r0, &sm.x_full[st]);

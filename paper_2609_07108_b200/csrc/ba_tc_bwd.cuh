@@ -53,7 +53,7 @@ namespace {
 
 // Branch tokens per branch key tile.  Branches of one length: a tile that starts and ends with a branch is seen
 // by its own tokens only (chains of three: 126 keys and 128 query rows instead of 128 and up to 135, which
-// costs a third 64-row step per head), unless more than an eighth of the lanes would stay empty.
+// costs a second 128-row step per head, at head_dim 64 a third 64-row one), unless more than an eighth of the lanes would stay empty.
 inline int branch_key_step(int len) {
     return len > 1 && 8 * (kTile / len * len) >= 7 * kTile ? kTile / len * len : kTile;
 }
