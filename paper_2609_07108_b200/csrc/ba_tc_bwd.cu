@@ -1397,7 +1397,8 @@ int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
         return bwd_maps(tm, pl, r, q_main, q_branch, k, v, d_o, depth, qr, qh, kr);
     };
     // dQ may be launched while delta ends, but not with about one item to an SM behind a delta that fills the SMs: the CTAs
-    // that start first take the items of those that cannot start yet, and work them off one after the other.  Whole steps of
+    // that start first take the items of those that cannot start yet, and work them off one after the other, while dK/dV
+    // takes the SMs that come free (not at head_dim 64, where it comes after dQ: 2,738 rows, 5/1 heads, 88 / 91).  Whole steps of
     // draft rows, launched early / behind delta: 3,045 rows, 12/4 heads (148 items) 331 / 277 us, 3,430, 8/8 (112) 734 /
     // 630, 7,347, 5/1 (147) 267 / 239; with more items or a small delta early is 1 to 4 % better (372 items 129 / 131,
     // 1,372 rows 77 / 80), at worst 1.5 % slower (1,048 items 364 / 359).
@@ -1413,7 +1414,7 @@ int ba_tc_bwd(const ba_plan *pl, const BaRange &r, const void *q_main, const voi
         if ((do_dq && !maps(tm, pq.tok, pq.hp, kSub)) || (do_dkdv && !maps(tk, kSub, 1, kTile))) return BA_EINVAL;
         int rc = prepare_rows();
         if (rc == BA_OK && do_dq)
-            rc = launch_kv<kModeDq, false>(pq, row_order(pq, pl, has_main), tm, dq_grid, dev, st, early_dq(dq_grid));
+            rc = launch_kv<kModeDq, false>(pq, row_order(pq, pl, has_main), tm, dq_grid, dev, st, (stages & BA_STAGE_PREP) != 0);
         if (rc != BA_OK || !do_dkdv) return rc;
         // (both kernels overlapped, as at head_dim 128: 605 us instead of 548 for the 4,096-token chains)
         const BaOrder &order = key_order(p, pl, has_main);
