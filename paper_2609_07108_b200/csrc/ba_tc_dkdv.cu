@@ -138,9 +138,13 @@ __device__ __forceinline__ uint64_t own_rows(const uint64_t *br_mask, int r0, in
     const uint32_t *word = reinterpret_cast<const uint32_t *>(br_mask) + 2 * (int64_t)r0 + (rel >> 5);
     uint32_t v[2] = {0u, 0u};
 #pragma unroll
-    for (int part = 0; part < 2; ++part)
-#pragma unroll 8
-        for (int c = max(lo, 32 * part); c <= min(hi, 32 * part + 31); ++c) v[part] |= ((word[2 * c] >> (rel & 31)) & 1u) << (c & 31);
+    for (int part = 0; part < 2; ++part) {
+        const int last = min(hi, 32 * part + 31);
+        for (int c = max(lo, 32 * part); c <= last; c += 8)      // (eight of short branches' rows too: no loop over a remainder)
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (c + i <= last) v[part] |= ((word[2 * (c + i)] >> (rel & 31)) & 1u) << ((c + i) & 31);
+    }
     return (uint64_t)v[1] << 32 | v[0];
 }
 
@@ -520,8 +524,8 @@ tc_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q_main, const __grid_const
                     // which of my 64 rows from r0 see my key
                     auto own = [&](int r0) { return own_rows(p.meta.br_mask, r0, max(rbeg - r0, 0), min(rend - 1 - r0, 63), f.row - start); };
                     // Once for every head, and for most items while the item before ends (32/8 heads, 16,384 tokens, draft
-                    // rows of 256 trees of 48: dK/dV 494 us; found at every step, one row after the other, 625; blocks of 24
-                    // on 2,400 tokens 31 and 48).  The 128 keys' branches have at most 63 more rows on either side and the
+                    // rows of 256 trees of 48: dK/dV 484 us; found at every step, one row after the other, 625; blocks of 24
+                    // on 2,400 tokens 29 and 48).  The 128 keys' branches have at most 63 more rows on either side and the
                     // tiles start at most 3 rows early: 257 rows.
                     const uint64_t own0 = own(f.ba + 64 * hf), own1 = own(f.ba + kTile + 64 * hf);
                     f.rb0 = (int)(uint32_t)own0; f.rb1 = (int)(uint32_t)(own0 >> 32);
